@@ -131,8 +131,15 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     const char *ao = std::getenv("TALON_ARGMAX_OVERSPLIT");
     c->argmax_oversplit = ao ? std::atoi(ao) : 4;
     if (c->argmax_oversplit < 1) c->argmax_oversplit = 1;
+    const char *sf = std::getenv("TALON_STEP_FUSE_MB"), *sr = std::getenv("TALON_STEP_ROUND_MB"), *sn = std::getenv("TALON_STEP_ROUNDS");
+    c->step_fuse_mb = sf ? std::atof(sf) : 128.0;
+    c->step_round_mb = sr ? std::atof(sr) : 128.0;
+    c->step_rounds = sn ? std::atoi(sn) : 4;
+    if (c->step_rounds < 1) c->step_rounds = 1;
     const char *e = std::getenv("TALON_PDL");
     c->pdl = !e ? -1 : (e[0] == '1' ? 1 : 0);
+    const char *rw = std::getenv("TALON_STEP_ROWS");
+    c->step_rows = (rw && rw[0] == '0') ? 0 : 1;
     const char *g = std::getenv("TALON_STEP_GRAPH");
     c->step_graph = (g && g[0] == '0') ? 0 : 1;
   }
@@ -155,6 +162,9 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
   alloc((void **)&c->d_row_score, sizeof(double) * (size_t)c->rows_cap * c->key_stride);
   alloc((void **)&c->d_row_count, sizeof(unsigned int) * (size_t)c->rows_cap);
   alloc((void **)&c->d_seq_count, sizeof(unsigned int) * (size_t)p->batch_max);
+  alloc((void **)&c->d_growing, sizeof(int32_t) * p->batch_max);
+  alloc((void **)&c->d_depth_at, sizeof(int32_t) * p->batch_max);
+  alloc((void **)&c->d_row_bad, sizeof(unsigned int) * nrow);
   alloc((void **)&c->d_argmax, sizeof(unsigned long long) * nrow);
   alloc((void **)&c->d_target_tok, sizeof(int32_t) * nrow);
   alloc((void **)&c->d_walk_count, sizeof(unsigned int) * (size_t)p->batch_max);
@@ -166,12 +176,13 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     ok = cudaMemset(c->d_status, 0, sizeof(int)) == cudaSuccess &&
          cudaMemset(c->d_row_count, 0, sizeof(unsigned int) * (size_t)c->rows_cap) == cudaSuccess &&
          cudaMemset(c->d_argmax, 0, sizeof(unsigned long long) * nrow) == cudaSuccess &&
+         cudaMemset(c->d_row_bad, 0, sizeof(unsigned int) * nrow) == cudaSuccess &&
          cudaMemset(c->d_seq_count, 0, sizeof(unsigned int) * (size_t)p->batch_max) == cudaSuccess &&
          cudaMemset(c->d_walk_count, 0, sizeof(unsigned int) * (size_t)p->batch_max) == cudaSuccess &&
          cudaMemset(c->d_part_keys, 0, sizeof(unsigned long long) * (size_t)c->items_cap * c->key_stride) == cudaSuccess &&
          talon::expand_setup(c) == TALON_OK && talon::attention_mma_setup() == TALON_OK &&
          talon::attention_tc_setup() == TALON_OK &&
-         (c->k_cap > 32 || talon::expand_fused_setup(c) == TALON_OK);
+         (c->k_cap > 32 || (talon::expand_fused_setup(c) == TALON_OK && talon::grow_step_setup(c) == TALON_OK));
   }
   if (!ok) {
     std::fprintf(stderr, "talon: context creation failed: %s\n", cudaGetErrorString(cudaGetLastError()));
@@ -187,6 +198,7 @@ talon_status talon_destroy(talon_ctx *c) {
   cudaSetDevice(c->device);
   cudaFree(c->d_status); cudaFree(c->d_prefix_len); cudaFree(c->d_part_keys); cudaFree(c->d_part_ms);
   cudaFree(c->d_row_keys); cudaFree(c->d_row_lse); cudaFree(c->d_row_score); cudaFree(c->d_row_count); cudaFree(c->d_seq_count); cudaFree(c->d_argmax);
+  cudaFree(c->d_growing); cudaFree(c->d_depth_at); cudaFree(c->d_row_bad);
   cudaFree(c->d_target_tok); cudaFree(c->d_walk_count); cudaFree(c->d_samp_ms); cudaFree(c->d_attn_o); cudaFree(c->d_attn_ml);
   free_stage(c->stage);
   talon_timing_enable(c, 0, 0u);
@@ -199,11 +211,35 @@ talon_status talon_destroy(talon_ctx *c) {
   return TALON_OK;
 }
 
-talon_status talon_reset(talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len,
-                         int32_t B, void *stream) {
+static talon_status check_reset(const talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len,
+                                int32_t B) {
   if (!c || !tree_complete(t) || !root_tok || !prefix_len) return TALON_ERR_INVALID_ARG;
   if (B < 1) return TALON_ERR_INVALID_ARG;
-  if (B > c->p.batch_max) return TALON_ERR_CAPACITY;
+  return B > c->p.batch_max ? TALON_ERR_CAPACITY : TALON_OK;
+}
+
+static talon_status check_rows(const talon_ctx *c, const float *logits, int64_t row_stride) {
+  return !logits || row_stride < c->p.vocab || (row_stride & 3) || !aligned16(logits) ? TALON_ERR_INVALID_ARG : TALON_OK;
+}
+
+static talon_status check_accept(const talon_ctx *c, const talon_tree *t, const float *target_logits, int64_t row_stride,
+                                 const int32_t *accept_len, const int32_t *accept_nodes, const int32_t *bonus_tok) {
+  if (!c || !tree_complete(t) || !accept_len || !accept_nodes || !bonus_tok) return TALON_ERR_INVALID_ARG;
+  return check_rows(c, target_logits, row_stride);
+}
+
+// Whether somebody is capturing the stream's work into a graph (or it cannot be told).
+static bool being_captured(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
+talon_status talon_reset(talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len,
+                         int32_t B, void *stream) {
+  const talon_status ok = check_reset(c, t, root_tok, prefix_len, B);
+  if (ok != TALON_OK) return ok;
   c->B = B;
   c->layers_run = 0;
   return talon::launch_reset(c, t, root_tok, prefix_len, B, (cudaStream_t)stream);
@@ -214,7 +250,7 @@ talon_status talon_expand_layer(talon_ctx *c, const talon_tree *t, const float *
   if (!c || !tree_complete(t) || !logits) return TALON_ERR_INVALID_ARG;
   if (c->B < 1) return TALON_ERR_INVALID_ARG;                      // no reset yet
   if (layout != TALON_ROWS_BY_NODE && layout != TALON_ROWS_PACKED) return TALON_ERR_INVALID_ARG;
-  if (row_stride < c->p.vocab || (row_stride & 3) || !aligned16(logits)) return TALON_ERR_INVALID_ARG;
+  if (check_rows(c, logits, row_stride) != TALON_OK) return TALON_ERR_INVALID_ARG;
   if (rows_per_seq < 1 || (layout == TALON_ROWS_BY_NODE && rows_per_seq < c->p.budget)) return TALON_ERR_INVALID_ARG;
   if (c->layers_run >= c->p.max_depth) return TALON_OK;            // depth stop: nothing to do
   talon_status s = talon::launch_expand(c, t, logits, row_stride, rows_per_seq, layout, (cudaStream_t)stream);
@@ -278,10 +314,9 @@ talon_status talon_tree_attention_paged(talon_ctx *c, const talon_tree *t, const
 static talon_status accept_checked(talon_ctx *c, const talon_tree *t, const float *target_logits, int64_t row_stride,
                                    int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes,
                                    int32_t *bonus_tok, void *stream, bool close_tree) {
-  if (!c || !tree_complete(t) || !target_logits || !accept_len || !accept_nodes || !bonus_tok)
-    return TALON_ERR_INVALID_ARG;
+  const talon_status ok = check_accept(c, t, target_logits, row_stride, accept_len, accept_nodes, bonus_tok);
+  if (ok != TALON_OK) return ok;
   if (c->B < 1) return TALON_ERR_INVALID_ARG;
-  if (row_stride < c->p.vocab || (row_stride & 3) || !aligned16(target_logits)) return TALON_ERR_INVALID_ARG;
   return talon::launch_accept(c, t, target_logits, row_stride, target_tok, accept_len, accept_nodes, bonus_tok,
                               (cudaStream_t)stream, close_tree);
 }
@@ -350,7 +385,7 @@ static talon_status step_enqueue(talon_ctx *c, const talon_tree *t, int32_t B, c
                                  int64_t kv_stride_t, int64_t kv_stride_h, int32_t max_prefix_len, float sm_scale,
                                  void *out, const float *target_logits, int64_t target_row_stride,
                                  int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes, int32_t *bonus_tok,
-                                 void *stream);
+                                 void *stream, bool layered);
 
 talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_steps, int32_t *root_tok,
                         int32_t *prefix_len, const float *draft_logits, int64_t draft_row_stride,
@@ -367,6 +402,8 @@ talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_
       result_step_stride < 0 || (q_step_stride & 7) || (kv_tree_step_stride & 7) || (draft_step_stride & 3) ||
       (target_step_stride & 3))
     return TALON_ERR_INVALID_ARG;
+  // a caller that captures the loop gets the layered launch sequence, as talon_step's callers do
+  const bool layered = being_captured((cudaStream_t)stream);
   const char *qb = static_cast<const char *>(q), *ktb = static_cast<const char *>(k_tree), *vtb = static_cast<const char *>(v_tree);
   for (int s = 0; s < n_steps; ++s) {
     // step s reads its own slice of the stand-ins for the two model forwards; the tree, the cache,
@@ -377,7 +414,7 @@ talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_
     talon_status r = step_enqueue(c, t, B, root_tok, prefix_len, draft_logits + draft_step_stride * s, draft_row_stride,
                                   n_layers, qs, k_prefix, v_prefix, kts, vts, kv_start, kv_tokens, kv_stride_t, kv_stride_h,
                                   max_prefix_len, sm_scale, out, target_logits + target_step_stride * s, target_row_stride,
-                                  target_tok, al, an, bt, stream);
+                                  target_tok, al, an, bt, stream, layered);
     if (r == TALON_OK)
       r = talon_commit(c, t, al, an, bt, kts, vts, k_prefix, v_prefix, kv_start, kv_limit, kv_tokens, kv_stride_t,
                        kv_stride_h, prefix_len, root_tok, counters, stream);
@@ -471,7 +508,8 @@ talon_status talon_timing_read(talon_ctx *c, void *stream, double *ms, int64_t *
   return TALON_OK;
 }
 
-// The launches of one step, in order, on `stream`.
+// The launches of one step, in order, on `stream`.  `layered`: one launch per layer even where the
+// rows of all node slots could be prepared in one pass.
 static talon_status step_enqueue(talon_ctx *c, const talon_tree *t, int32_t B, const int32_t *root_tok,
                                  const int32_t *prefix_len, const float *draft_logits, int64_t draft_row_stride,
                                  int32_t n_layers, const void *q, const void *k_prefix, const void *v_prefix,
@@ -479,18 +517,33 @@ static talon_status step_enqueue(talon_ctx *c, const talon_tree *t, int32_t B, c
                                  int64_t kv_stride_t, int64_t kv_stride_h, int32_t max_prefix_len, float sm_scale,
                                  void *out, const float *target_logits, int64_t target_row_stride,
                                  int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes, int32_t *bonus_tok,
-                                 void *stream) {
-  talon_status r = talon_reset(c, t, root_tok, prefix_len, B, stream);
-  for (int d = 0; r == TALON_OK && d < n_layers; ++d)
-    r = talon_expand_layer(c, t, draft_logits, draft_row_stride, c->p.budget, TALON_ROWS_BY_NODE, stream);
+                                 void *stream, bool layered) {
+  talon_status r = TALON_OK;
+  bool closed = false, accepted = false;
+  // (timed launches are reported per layer, so they take the layered sequence too)
+  if (!layered && c->step_rows && c->k_cap <= 32 && !(c->ev && !c->ev_paused) && n_layers > 0) {
+    r = check_reset(c, t, root_tok, prefix_len, B);
+    if (r == TALON_OK) r = check_rows(c, draft_logits, draft_row_stride);
+    if (r == TALON_OK) r = check_accept(c, t, target_logits, target_row_stride, accept_len, accept_nodes, bonus_tok);
+    if (r != TALON_OK) return r;
+    c->B = B;
+    r = talon::launch_grow_step(c, t, root_tok, prefix_len, draft_logits, draft_row_stride, n_layers, target_logits,
+                                target_row_stride, target_tok, accept_len, accept_nodes, bonus_tok, (cudaStream_t)stream,
+                                &accepted);
+    closed = true;
+  } else {
+    r = talon_reset(c, t, root_tok, prefix_len, B, stream);
+    for (int d = 0; r == TALON_OK && d < n_layers; ++d)
+      r = talon_expand_layer(c, t, draft_logits, draft_row_stride, c->p.budget, TALON_ROWS_BY_NODE, stream);
+  }
   // (no separate closing launch: the attention needs only sizes and mask rows, and the accept walk
   // writes positions and sentinel slots before it walks)
   if (r == TALON_OK)
     r = talon_tree_attention(c, t, q, k_prefix, v_prefix, k_tree, v_tree, kv_start, kv_tokens, kv_stride_t, kv_stride_h,
                              max_prefix_len, sm_scale, out, stream);
-  if (r == TALON_OK)
+  if (r == TALON_OK && !accepted)
     r = accept_checked(c, t, target_logits, target_row_stride, target_tok, accept_len, accept_nodes, bonus_tok,
-                       stream, true);
+                       stream, !closed);
   return r;
 }
 
@@ -514,15 +567,11 @@ talon_status talon_step(talon_ctx *c, const talon_tree *t, int32_t B, const int3
   // submission.  Not on the legacy default stream (it cannot be captured), not while the stream is
   // already being captured by the caller, and not while launches are being timed with events.
   const bool timing = c->ev && !c->ev_paused;
-  if (!c->step_graph || !t || st == nullptr || st == cudaStreamLegacy || timing) return step_enqueue(TALON_STEP_ARGS);
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return step_enqueue(TALON_STEP_ARGS);
-  }
+  if (!c->step_graph || !t || st == nullptr || st == cudaStreamLegacy || timing) return step_enqueue(TALON_STEP_ARGS, false);
+  if (being_captured(st)) return step_enqueue(TALON_STEP_ARGS, true);
   if (!c->graphs) {
     c->graphs = new (std::nothrow) talon::StepGraph[talon::STEP_GRAPH_SLOTS];
-    if (!c->graphs) return step_enqueue(TALON_STEP_ARGS);
+    if (!c->graphs) return step_enqueue(TALON_STEP_ARGS, false);
     std::memset(c->graphs, 0, sizeof(talon::StepGraph) * talon::STEP_GRAPH_SLOTS);
   }
   unsigned long long key[talon::STEP_GRAPH_WORDS];
@@ -553,17 +602,17 @@ talon_status talon_step(talon_ctx *c, const talon_tree *t, int32_t B, const int3
     std::memcpy(victim->args, key, sizeof(key));
     victim->used = true;
     victim->last_use = c->step_tick;
-    return step_enqueue(TALON_STEP_ARGS);
+    return step_enqueue(TALON_STEP_ARGS, false);
   }
   hit->last_use = c->step_tick;
   if (!hit->exec) {                // second sighting: capture
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
       cudaGetLastError();
       c->step_graph = 0;           // this stream or driver cannot capture: stop trying
-      return step_enqueue(TALON_STEP_ARGS);
+      return step_enqueue(TALON_STEP_ARGS, false);
     }
     const long long before = c->launches;
-    const talon_status r = step_enqueue(TALON_STEP_ARGS);
+    const talon_status r = step_enqueue(TALON_STEP_ARGS, false);
     cudaGraph_t graph = nullptr;
     const cudaError_t e = cudaStreamEndCapture(st, &graph);
     cudaGraphExec_t exec = nullptr;
@@ -579,7 +628,7 @@ talon_status talon_step(talon_ctx *c, const talon_tree *t, int32_t B, const int3
       hit->used = false;
       if (graph) cudaGraphDestroy(graph);
       if (r == TALON_OK) c->step_graph = 0;      // the capture itself failed: stop trying
-      return step_enqueue(TALON_STEP_ARGS);
+      return step_enqueue(TALON_STEP_ARGS, false);
     }
     cudaGraphDestroy(graph);
   }

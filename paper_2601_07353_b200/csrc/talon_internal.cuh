@@ -121,6 +121,13 @@ struct talon_ctx {
   unsigned int *d_row_count;         // [rows_cap]               chunks finished per row
   unsigned int *d_seq_count;         // [batch_max]              chunks finished per sequence (fused kernel)
   int fused_grid;                    // CTAs of the fused kernel at full width
+  // whole-step growth (grow_step.cu)
+  int row_grid;                      // CTAs of the row pass at full width
+  int32_t *d_growing, *d_depth_at;   // [batch_max] a sequence's tree still grows; layer it stopped at
+  unsigned int *d_row_bad;           // [batch_max * N] NaN in a target row (zero between calls)
+  double step_fuse_mb, step_round_mb;   // MB of logits up to which the target rows ride along / one round takes all rows
+  int step_rows;                     // 0: whole steps expand layer by layer too
+  int step_rounds;                   // rounds of a larger step
   int attn_cluster;                  // key ranges of the tensor-core attention merge inside a cluster (1) or in a second kernel (0)
   long long attn_cluster_min_rows;   // automatic mode: least rows x key ranges for the merge inside the cluster
   int attn_cluster_cap;              // more key ranges than eight are cut back to eight up to this many
@@ -215,6 +222,13 @@ talon_status launch_reset(talon_ctx *c, const talon_tree *t, const int32_t *root
                           const int32_t *prefix_len, int B, cudaStream_t st);
 talon_status launch_expand(talon_ctx *c, const talon_tree *t, const float *logits,
                            int64_t row_stride, int rows_per_seq, int layout, cudaStream_t st);
+// The draft phase of a whole step (reset, n_layers layers, closing pass) from the draft rows of all node
+// slots; k_cap <= 32.  *accepted: the target rows' arg-max and the walk are done as well.
+talon_status grow_step_setup(talon_ctx *c);
+talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len,
+                              const float *draft, int64_t draft_stride, int n_layers, const float *target,
+                              int64_t target_stride, int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes,
+                              int32_t *bonus_tok, cudaStream_t st, bool *accepted);
 talon_status launch_build(talon_ctx *c, const talon_tree *t, uint8_t *dense, cudaStream_t st);
 talon_status launch_prune(talon_ctx *c, const talon_tree *t, int keep, cudaStream_t st);
 talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, const void *kp,
