@@ -4,6 +4,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <type_traits>
 
 #include "talon_internal.cuh"
 
@@ -87,10 +88,12 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
   TALON_CUDA_OK(cudaGetDeviceCount(&n_dev));
   if (device < 0 || device >= n_dev) return TALON_ERR_INVALID_ARG;
   TALON_CUDA_OK(cudaSetDevice(device));
-  cudaDeviceProp prop;
-  TALON_CUDA_OK(cudaGetDeviceProperties(&prop, device));
-  if (prop.major < 10) {
-    std::fprintf(stderr, "talon: built for sm_100a, device reports sm_%d%d\n", prop.major, prop.minor);
+  int major = 0, minor = 0, sm_count = 0;
+  TALON_CUDA_OK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device));
+  TALON_CUDA_OK(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device));
+  TALON_CUDA_OK(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device));
+  if (major < 10) {
+    std::fprintf(stderr, "talon: built for sm_100a, device reports sm_%d%d\n", major, minor);
     return TALON_ERR_UNSUPPORTED;
   }
 
@@ -99,7 +102,7 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
   std::memset(c, 0, sizeof(*c));
   c->p = *p;
   c->device = device;
-  c->sm_count = prop.multiProcessorCount;
+  c->sm_count = sm_count;
   c->W = (p->budget + 63) / 64;
   int k = p->cand_topk == 0 ? p->budget - 1 : p->cand_topk;
   if (k > p->budget - 1) k = p->budget - 1;      // a parent never places more than N-1 children
@@ -131,11 +134,8 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     const char *ao = std::getenv("TALON_ARGMAX_OVERSPLIT");
     c->argmax_oversplit = ao ? std::atoi(ao) : 4;
     if (c->argmax_oversplit < 1) c->argmax_oversplit = 1;
-    const char *sf = std::getenv("TALON_STEP_FUSE_MB"), *sr = std::getenv("TALON_STEP_ROUND_MB"), *sn = std::getenv("TALON_STEP_ROUNDS");
-    c->step_fuse_mb = sf ? std::atof(sf) : 128.0;
-    c->step_round_mb = sr ? std::atof(sr) : 128.0;
-    c->step_rounds = sn ? std::atoi(sn) : 4;
-    if (c->step_rounds < 1) c->step_rounds = 1;
+    const char *sf = std::getenv("TALON_STEP_FIRST_ROWS");
+    c->step_first_rows = sf ? std::atoi(sf) : 0;
     const char *e = std::getenv("TALON_PDL");
     c->pdl = !e ? -1 : (e[0] == '1' ? 1 : 0);
     const char *rw = std::getenv("TALON_STEP_ROWS");
@@ -149,41 +149,42 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
   c->items_cap = c->exp_grid + c->rows_cap;
 
   const size_t nrow = (size_t)p->batch_max * p->budget;
-  bool ok = true;
-  auto alloc = [&](void **ptr, size_t bytes) {
-    if (ok && cudaMalloc(ptr, bytes ? bytes : 16) != cudaSuccess) ok = false;
-  };
-  alloc((void **)&c->d_status, sizeof(int));
-  alloc((void **)&c->d_prefix_len, sizeof(int32_t) * p->batch_max);
-  alloc((void **)&c->d_part_keys, sizeof(unsigned long long) * (size_t)c->items_cap * c->key_stride);
-  alloc((void **)&c->d_part_ms, sizeof(float2) * (size_t)c->items_cap);
-  alloc((void **)&c->d_row_keys, sizeof(unsigned long long) * (size_t)c->rows_cap * c->key_stride);
-  alloc((void **)&c->d_row_lse, sizeof(double) * (size_t)c->rows_cap);
-  alloc((void **)&c->d_row_score, sizeof(double) * (size_t)c->rows_cap * c->key_stride);
-  alloc((void **)&c->d_row_count, sizeof(unsigned int) * (size_t)c->rows_cap);
-  alloc((void **)&c->d_seq_count, sizeof(unsigned int) * (size_t)p->batch_max);
-  alloc((void **)&c->d_growing, sizeof(int32_t) * p->batch_max);
-  alloc((void **)&c->d_depth_at, sizeof(int32_t) * p->batch_max);
-  alloc((void **)&c->d_row_bad, sizeof(unsigned int) * nrow);
-  alloc((void **)&c->d_argmax, sizeof(unsigned long long) * nrow);
-  alloc((void **)&c->d_target_tok, sizeof(int32_t) * nrow);
-  alloc((void **)&c->d_walk_count, sizeof(unsigned int) * (size_t)p->batch_max);
-  alloc((void **)&c->d_samp_ms, sizeof(float2) * nrow * talon::EXP_MAX_SPLITS);
+  // One allocation holds the whole workspace (an allocation is a trip to the driver, tens to hundreds of
+  // microseconds, and a program may make a context per model or per request class); what has to start
+  // at zero comes first.
   c->attn_o_elems = talon::attention_workspace_elems(c, &c->attn_ml_elems);
-  alloc((void **)&c->d_attn_o, sizeof(float) * c->attn_o_elems);
-  alloc((void **)&c->d_attn_ml, sizeof(float2) * c->attn_ml_elems);
-  if (ok) {
-    ok = cudaMemset(c->d_status, 0, sizeof(int)) == cudaSuccess &&
-         cudaMemset(c->d_row_count, 0, sizeof(unsigned int) * (size_t)c->rows_cap) == cudaSuccess &&
-         cudaMemset(c->d_argmax, 0, sizeof(unsigned long long) * nrow) == cudaSuccess &&
-         cudaMemset(c->d_row_bad, 0, sizeof(unsigned int) * nrow) == cudaSuccess &&
-         cudaMemset(c->d_seq_count, 0, sizeof(unsigned int) * (size_t)p->batch_max) == cudaSuccess &&
-         cudaMemset(c->d_walk_count, 0, sizeof(unsigned int) * (size_t)p->batch_max) == cudaSuccess &&
-         cudaMemset(c->d_part_keys, 0, sizeof(unsigned long long) * (size_t)c->items_cap * c->key_stride) == cudaSuccess &&
-         talon::expand_setup(c) == TALON_OK && talon::attention_mma_setup() == TALON_OK &&
-         talon::attention_tc_setup() == TALON_OK &&
-         (c->k_cap > 32 || (talon::expand_fused_setup(c) == TALON_OK && talon::grow_step_setup(c) == TALON_OK));
+  const size_t items = c->items_cap, rows = c->rows_cap, ks = c->key_stride, bm = p->batch_max;
+  size_t zeroed = 0, total = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    total = 0;
+    auto take = [&](auto **ptr, size_t count) {
+      if (pass) *ptr = reinterpret_cast<std::remove_reference_t<decltype(*ptr)>>(static_cast<char *>(c->d_arena) + total);
+      total += (count * sizeof(**ptr) + 255) / 256 * 256;
+    };
+    take(&c->d_status, 1);
+    take(&c->d_row_count, rows);
+    take(&c->d_seq_count, bm);
+    take(&c->d_walk_count, bm);
+    take(&c->d_argmax, nrow);
+    take(&c->d_row_bad, nrow);
+    take(&c->d_part_keys, items * ks);
+    zeroed = total;
+    take(&c->d_prefix_len, bm);
+    take(&c->d_part_ms, items);
+    take(&c->d_row_keys, rows * ks);
+    take(&c->d_row_lse, rows);
+    take(&c->d_row_score, rows * ks);
+    take(&c->d_growing, bm);
+    take(&c->d_depth_at, bm);
+    take(&c->d_target_tok, nrow);
+    take(&c->d_samp_ms, nrow * talon::EXP_MAX_SPLITS);
+    take(&c->d_attn_o, c->attn_o_elems);
+    take(&c->d_attn_ml, c->attn_ml_elems);
+    if (pass == 0 && cudaMalloc(&c->d_arena, total) != cudaSuccess) break;
   }
+  const bool ok = c->d_arena && cudaMemset(c->d_arena, 0, zeroed) == cudaSuccess && talon::expand_setup(c) == TALON_OK &&
+                  talon::attention_mma_setup() == TALON_OK && talon::attention_tc_setup() == TALON_OK &&
+                  (c->k_cap > 32 || (talon::expand_fused_setup(c) == TALON_OK && talon::grow_step_setup(c) == TALON_OK));
   if (!ok) {
     std::fprintf(stderr, "talon: context creation failed: %s\n", cudaGetErrorString(cudaGetLastError()));
     talon_destroy(c);
@@ -196,10 +197,7 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
 talon_status talon_destroy(talon_ctx *c) {
   if (!c) return TALON_OK;
   cudaSetDevice(c->device);
-  cudaFree(c->d_status); cudaFree(c->d_prefix_len); cudaFree(c->d_part_keys); cudaFree(c->d_part_ms);
-  cudaFree(c->d_row_keys); cudaFree(c->d_row_lse); cudaFree(c->d_row_score); cudaFree(c->d_row_count); cudaFree(c->d_seq_count); cudaFree(c->d_argmax);
-  cudaFree(c->d_growing); cudaFree(c->d_depth_at); cudaFree(c->d_row_bad);
-  cudaFree(c->d_target_tok); cudaFree(c->d_walk_count); cudaFree(c->d_samp_ms); cudaFree(c->d_attn_o); cudaFree(c->d_attn_ml);
+  cudaFree(c->d_arena);
   free_stage(c->stage);
   talon_timing_enable(c, 0, 0u);
   if (c->graphs) {
@@ -272,11 +270,11 @@ talon_status talon_prune_tree(talon_ctx *c, const talon_tree *t, int32_t keep, v
   return talon::launch_prune(c, t, keep, (cudaStream_t)stream);
 }
 
-talon_status talon_tree_attention(talon_ctx *c, const talon_tree *t, const void *q, const void *k_prefix,
+static talon_status attention_checked(talon_ctx *c, const talon_tree *t, const void *q, const void *k_prefix,
                                   const void *v_prefix, const void *k_tree, const void *v_tree,
                                   const int64_t *kv_start, int64_t kv_tokens, int64_t kv_stride_t,
                                   int64_t kv_stride_h, int32_t max_prefix_len, float sm_scale, void *out,
-                                  void *stream) {
+                                  void *stream, const int32_t *early_prefix) {
   if (!c || !tree_complete(t) || !q || !k_tree || !v_tree || !kv_start || !out) return TALON_ERR_INVALID_ARG;
   if (c->B < 1 || max_prefix_len < 0 || kv_tokens < 0 || kv_tokens > 0x7FFFFFFFll) return TALON_ERR_INVALID_ARG;
   if (max_prefix_len > kv_tokens) return TALON_ERR_INVALID_ARG;
@@ -288,7 +286,16 @@ talon_status talon_tree_attention(talon_ctx *c, const talon_tree *t, const void 
   if (!(sm_scale == sm_scale)) return TALON_ERR_INVALID_ARG;
   return talon::launch_attention(c, t, q, k_prefix ? k_prefix : k_tree, v_prefix ? v_prefix : v_tree, k_tree,
                                  v_tree, kv_start, nullptr, 0, kv_tokens, kv_stride_t, kv_stride_h, max_prefix_len,
-                                 sm_scale, out, (cudaStream_t)stream);
+                                 sm_scale, out, (cudaStream_t)stream, early_prefix);
+}
+
+talon_status talon_tree_attention(talon_ctx *c, const talon_tree *t, const void *q, const void *k_prefix,
+                                  const void *v_prefix, const void *k_tree, const void *v_tree,
+                                  const int64_t *kv_start, int64_t kv_tokens, int64_t kv_stride_t,
+                                  int64_t kv_stride_h, int32_t max_prefix_len, float sm_scale, void *out,
+                                  void *stream) {
+  return attention_checked(c, t, q, k_prefix, v_prefix, k_tree, v_tree, kv_start, kv_tokens, kv_stride_t, kv_stride_h,
+                           max_prefix_len, sm_scale, out, stream, nullptr);
 }
 
 talon_status talon_tree_attention_paged(talon_ctx *c, const talon_tree *t, const void *q, const void *k_pages,
@@ -539,8 +546,8 @@ static talon_status step_enqueue(talon_ctx *c, const talon_tree *t, int32_t B, c
   // (no separate closing launch: the attention needs only sizes and mask rows, and the accept walk
   // writes positions and sentinel slots before it walks)
   if (r == TALON_OK)
-    r = talon_tree_attention(c, t, q, k_prefix, v_prefix, k_tree, v_tree, kv_start, kv_tokens, kv_stride_t, kv_stride_h,
-                             max_prefix_len, sm_scale, out, stream);
+    r = attention_checked(c, t, q, k_prefix, v_prefix, k_tree, v_tree, kv_start, kv_tokens, kv_stride_t, kv_stride_h,
+                          max_prefix_len, sm_scale, out, stream, closed ? prefix_len : nullptr);
   if (r == TALON_OK && !accepted)
     r = accept_checked(c, t, target_logits, target_row_stride, target_tok, accept_len, accept_nodes, bonus_tok,
                        stream, !closed);

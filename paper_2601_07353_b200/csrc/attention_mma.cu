@@ -347,7 +347,7 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
                               const void *kt, const void *vt, const int64_t *kv_start, const int32_t *block_table,
                               int bt_stride, int64_t kv_tokens,
                               int64_t stride_t, int64_t stride_h, int max_prefix_len, float sm_scale, void *out,
-                              cudaStream_t st) {
+                              cudaStream_t st, const int32_t *early_prefix) {
   AttnArgs a;
   a.q = (const __nv_bfloat16 *)q; a.kp = (const __nv_bfloat16 *)kp; a.vp = (const __nv_bfloat16 *)vp;
   a.kt = (const __nv_bfloat16 *)kt; a.vt = (const __nv_bfloat16 *)vt;
@@ -393,7 +393,7 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
     a.splits = sp;
     int merged = 0;
     talon_status r = launch_attention_tc(c, t, q, kp, vp, kt, vt, kv_start, block_table, bt_stride, stride_t, stride_h, kv_tokens,
-                                         max_prefix_len, sm_scale, out, sp, a.m_blocks, st, &merged);
+                                         max_prefix_len, sm_scale, out, sp, a.m_blocks, st, &merged, early_prefix);
     if (r != TALON_OK) return r;
     if (sp > 1 && !merged) {
       const int64_t rows = (int64_t)c->B * a.Hkv * a.g * a.N;

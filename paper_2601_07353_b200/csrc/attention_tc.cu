@@ -60,11 +60,12 @@ struct TcArgs {
   const int64_t *kv_start;
   const int32_t *block_table;  // paged prefix: [B, bt_stride] page numbers (null: contiguous blocks at kv_start)
   int bt_stride;
-  const int32_t *prefix_len, *n_nodes;
+  const int32_t *prefix_len, *n_nodes;   // prefix_len: the caller's array when early
   const unsigned long long *mask;
   int B, N, W, Hq, Hkv, g;
   float scale_log2;
   int splits, m_blocks;
+  int early;                   // launched beside the kernel that grows the trees (see the kernel)
   int cluster_merge;           // the key ranges of a (sequence, head, tile pair) form a cluster and merge in shared memory
   __nv_bfloat16 *out;
   float *part_o;
@@ -235,7 +236,11 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
   __shared__ uint32_t s_tmem_base;
   __shared__ int s_abort;
 
-  pdl_enter();
+  // `early`: the kernel before this one only grows the trees (grow_step.cu).  Everything about the
+  // prefix is complete then, so the CTA starts on its prefix tiles at once; the softmax warps wait for
+  // that kernel before they look at tree sizes and mask rows, and so before anything is written.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int mpair = blockIdx.x, split = blockIdx.y;
   const int bh = blockIdx.z, b = bh / a.Hkv, kvh = bh - b * a.Hkv;
@@ -249,10 +254,8 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
   unsigned char *gen_base = smem_dyn + (base - smem_u32(smem_dyn));      // generic pointer to `base`
   auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
 
-  const int n = a.n_nodes[b];
   const int L = a.prefix_len[b];
   const int rows_total = a.g * a.N;
-  const int rows_valid = a.g * n;
   int nmt = (rows_total - mpair * 2 * TC_MT + TC_MT - 1) / TC_MT;       // query tiles of this CTA with rows
   nmt = nmt > 2 ? 2 : nmt;
 
@@ -391,16 +394,26 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     const uint32_t t_lane = tmem + ((uint32_t)(quarter * 32) << 16);
     const uint32_t t_S = t_lane + 256 + 128 * i;
     const uint32_t t_O = t_lane + 128 * i;
-    const bool row_valid = R < rows_valid;
+    // tree size and this row's mask: known before the first tile, or (early) before the tree tile or the epilogue
+    int n = 0;
+    bool row_valid = false, have_tree = false;
     unsigned long long mrow[2] = {0ull, 0ull};
-    if (row_valid)
-      for (int w = 0; w < a.W; ++w) mrow[w] = a.mask[((int64_t)b * a.N + R / a.g) * a.W + w];
+    auto load_tree = [&]() {
+      if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+      n = __ldcg(a.n_nodes + b);
+      row_valid = R < a.g * n;
+      if (row_valid)
+        for (int w = 0; w < a.W; ++w) mrow[w] = __ldcg(a.mask + ((int64_t)b * a.N + R / a.g) * a.W + w);
+      have_tree = true;
+    };
+    if (!a.early) load_tree();
 
     float m_used = -CUDART_INF_F, l_run = 0.f;
     bool ok = (i < nmt) && nt > 0;
     for (int it = 0; it < nt && ok; ++it) {
       const int tg = t_begin + it;
       const bool tree_tile = tg >= nP;
+      if (tree_tile && !have_tree) load_tree();
       const int kvalid = tree_tile ? min(n - (tg - nP) * TC_BN, TC_BN) : min(L - tg * TC_BN, TC_BN);
       const int s = it % TC_STAGES;
       // keys beyond the valid range may hold anything: tile 0's warps clear their V rows so that
@@ -513,6 +526,8 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       tc_fence_before();
       mbar_arrive(bar(B_PFULL + i));
     }
+
+    if (!have_tree) load_tree();
 
     // ---- epilogue: O / l (or the partial result of this key range) ----
     // tcgen05.ld is a warp-wide instruction: every lane of a warp that holds any row takes part
@@ -707,7 +722,7 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
                                  const void *kt, const void *vt, const int64_t *kv_start, const int32_t *block_table,
                                  int bt_stride, int64_t stride_t,
                                  int64_t stride_h, int64_t kv_tokens, int max_prefix_len, float sm_scale, void *out,
-                                 int splits, int m_blocks, cudaStream_t st, int *merged_in_kernel) {
+                                 int splits, int m_blocks, cudaStream_t st, int *merged_in_kernel, const int32_t *early_prefix) {
   *merged_in_kernel = 0;
   const int N = c->p.budget, Hq = c->p.n_q_heads, Hkv = c->p.n_kv_heads, g = Hq / Hkv, B = c->B;
   CUtensorMap mq, mkp, mvp, mkt, mvt;
@@ -731,7 +746,8 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
   }
   TcArgs a;
   a.kv_start = kv_start; a.block_table = block_table; a.bt_stride = bt_stride;
-  a.prefix_len = c->d_prefix_len; a.n_nodes = t->n_nodes;
+  a.early = early_prefix != nullptr;
+  a.prefix_len = early_prefix ? early_prefix : c->d_prefix_len; a.n_nodes = t->n_nodes;
   a.mask = (const unsigned long long *)t->mask;
   a.B = B; a.N = N; a.W = c->W; a.Hq = Hq; a.Hkv = Hkv; a.g = g;
   a.scale_log2 = sm_scale * 1.4426950408889634f;
@@ -772,11 +788,11 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
       attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
       attr[1].val.programmaticStreamSerializationAllowed = 1;
       cfg.attrs = attr;
-      cfg.numAttrs = (c->pdl == 1 || (c->pdl < 0 && c->B <= PDL_AUTO_BATCH)) ? 2 : 1;
+      cfg.numAttrs = (c->pdl == 1 || (c->pdl < 0 && (c->B <= PDL_AUTO_BATCH || early_prefix))) ? 2 : 1;
       cudaLaunchKernelEx(&cfg, tree_attention_tc_kernel, mq, mkp, mvp, mkt, mvt, a);
       *merged_in_kernel = 1;
     } else {
-      launch_kernel(c, tree_attention_tc_kernel, grid, dim3(TC_THREADS), TC_SMEM, st, mq, mkp, mvp, mkt, mvt, a);
+      launch_kernel_pdl(c, early_prefix != nullptr, tree_attention_tc_kernel, grid, dim3(TC_THREADS), TC_SMEM, st, mq, mkp, mvp, mkt, mvt, a);
     }
   }
   if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;

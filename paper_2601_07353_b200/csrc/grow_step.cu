@@ -15,10 +15,9 @@
 //                     closes the tree; with the arg-max of the target rows at hand it walks the
 //                     accepted path too.
 //
-// Rows of slots that the tree turns out not to use, or not to expand, are read for nothing: cheap
-// while a step is a few MB, not when it is hundreds.  Large steps therefore go in rounds: a round
-// prepares the next rows of the sequences whose trees still grow, then the trees grow as far as those
-// rows carry them.
+// Rows of slots that the tree turns out not to use, or not to expand, are read for nothing.  Where that
+// could cost more than it saves (launch_grow_step has the rule) the step takes two rounds: the second
+// prepares the remaining rows of the sequences whose trees still grow.
 #include "expand_stream.cuh"
 
 namespace talon {
@@ -26,7 +25,7 @@ namespace talon {
 namespace {
 
 struct RowPassArgs {
-  const float *draft, *target;        // [B, N] rows; target null: draft rows only
+  const float *draft, *target;        // [B, N] rows
   int64_t draft_stride, target_stride;
   int B, N, V, k, key_stride, max_split;
   int r0, r1;                         // node slots of this round, per sequence
@@ -265,7 +264,6 @@ struct GrowArgs {
   double log_mu;
   int first;                    // round 0: start from the root
   int rows;                     // row lists of slots 0 .. rows-1 are there
-  int group;                    // lanes per row in the selection: k rounded up to a power of two
   const u64 *row_keys; const double *row_lp;
   int32_t *growing, *depth_at;  // [B] out: needs more rows; layer it stopped at
   unsigned int *row_count;      // [B * N] cleared (a row pass that timed out leaves counts behind)
@@ -275,66 +273,59 @@ struct GrowArgs {
   int32_t *target_tok, *accept_len, *accept_nodes, *bonus_tok;
 };
 
+constexpr double STEP_SPLIT_BYTES = 150e6;    // about 25 us at the copy bandwidth
 constexpr int GROW_THREADS = 256;
-constexpr int GROW_WARPS = GROW_THREADS / 32;
 
 struct GrowSmem {
-  u64 *key;            // [rows][k]
-  double *lp;          // [rows][k]
+  u64 *key;            // [k][pitch]  i-th best candidate of row r at i * pitch + r (lane = row: no bank conflicts)
+  double *lp;          // [k][pitch]
   double *score;       // [N]
   u64 *mask;           // [N][2]
   int *tok, *parent, *depth;   // [N]
-  int *off;            // [GROW_WARPS][MAX_BUDGET]  each warp's own copy of the rows' output offsets
-  int *cnt;            // [MAX_BUDGET]              candidates of a row still in
+  int *cnt;            // [MAX_BUDGET]  rows' candidates that survive the truncation; later the target's choices
 };
 
+__host__ __device__ inline int grow_pitch(int rows) { return rows | 1; }
 __host__ __device__ inline size_t grow_smem_bytes(int rows, int k, int N) {
-  return (size_t)rows * k * 16 + (size_t)N * (8 + 16 + 12) + GROW_WARPS * MAX_BUDGET * 4 + MAX_BUDGET * 4 + 32;
+  return (size_t)grow_pitch(rows) * k * 16 + (size_t)N * (8 + 16 + 12) + MAX_BUDGET * 4 + 32;
 }
 
-// Exclusive scan of cnt[0 .. F) into this warp's off[]; returns the total.
-__device__ __forceinline__ int scan_rows(const int *cnt, int *off, int F, int lane) {
-  int v[4], sum = 0;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) { const int jj = lane * 4 + i; v[i] = jj < F ? cnt[jj] : 0; sum += v[i]; }
-  int inc = sum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(FULL, inc, o);
-    if (lane >= o) inc += t;
-  }
-  int run = inc - sum;
-  *reinterpret_cast<int4 *>(off + lane * 4) = make_int4(run, run + v[0], run + v[0] + v[1], run + v[0] + v[1] + v[2]);
-  __syncwarp();
-  return __shfl_sync(FULL, inc, 31);
+// The largest value over the warp, in two reductions of half a key.
+__device__ __forceinline__ u64 warp_redux_max_u64(u64 v) {
+  const unsigned hi = __reduce_max_sync(FULL, (unsigned)(v >> 32));
+  const unsigned lo = __reduce_max_sync(FULL, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+  return ((u64)hi << 32) | lo;
 }
 
-// One CTA per sequence.  A layer is four short phases between barriers: the best candidate of the
-// frontier (the gate's anchor), how many candidates of each row pass (they are a prefix: lists are
-// sorted), the truncation by rank if more pass than the budget takes, the append.
+// One CTA per sequence.  A layer is a short serial chain (best candidate of the frontier, the gate,
+// how many candidates of each row pass, where each row's survivors go, append), so what counts is
+// latency: every warp computes the chain up to the offsets for itself, a lane per frontier row, without
+// a barrier; only the append is shared out over the warps, and one barrier ends the layer.  Row lists
+// are sorted, so the candidates of a row that pass are a prefix of its list.
+template <int NQ, int KMAX>  // frontier rows per lane; k rounded up to 8, 16 or 32
 __global__ void __launch_bounds__(GROW_THREADS)
 grow_kernel(GrowArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ u64 s_head[GROW_WARPS];
+  const int pitch = grow_pitch(a.rows);
   GrowSmem sm;
   {
     unsigned char *p = smem_raw;
-    sm.key = reinterpret_cast<u64 *>(p);       p += sizeof(u64) * a.rows * a.k;
-    sm.lp = reinterpret_cast<double *>(p);     p += sizeof(double) * a.rows * a.k;
+    sm.key = reinterpret_cast<u64 *>(p);       p += sizeof(u64) * pitch * a.k;
+    sm.lp = reinterpret_cast<double *>(p);     p += sizeof(double) * pitch * a.k;
     sm.mask = reinterpret_cast<u64 *>(p);      p += sizeof(u64) * 2 * a.N;
     sm.score = reinterpret_cast<double *>(p);  p += sizeof(double) * a.N;
-    p = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(p) + 15) & ~(uintptr_t)15);
-    sm.off = reinterpret_cast<int *>(p);       p += sizeof(int) * GROW_WARPS * MAX_BUDGET;
     sm.cnt = reinterpret_cast<int *>(p);       p += sizeof(int) * MAX_BUDGET;
     sm.tok = reinterpret_cast<int *>(p);       p += sizeof(int) * a.N;
     sm.parent = reinterpret_cast<int *>(p);    p += sizeof(int) * a.N;
     sm.depth = reinterpret_cast<int *>(p);
   }
-  pdl_enter();
+  // First the wait, then the trigger: the attention, when it is the next kernel, may start on the
+  // prefix while the trees grow, and what it reads for that has to be complete.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x, k = a.k, N = a.N;
   const size_t nb = (size_t)b * N;
-  int *off = sm.off + warp * MAX_BUDGET;
   int d = 0, lo = 0, hi = 1;
   if (!a.first) {
     if (!a.growing[b]) return;
@@ -345,12 +336,24 @@ grow_kernel(GrowArgs a) {
   const int n_start = hi;                              // nodes that global memory holds already (round 0: only the root, written below)
   const int L = a.prefix_len[b], root = a.root_tok[b];
   // everything the sequence needs: row lists of the slots that can still be expanded, and the nodes' scores and masks
-  for (int c = lo * k + tid; c < a.rows * k; c += GROW_THREADS) {
-    const int i = c / k;
-    const size_t at = (nb + i) * a.key_stride + (c - i * k);
-    sm.key[c] = __ldcg(a.row_keys + at);
-    sm.lp[c] = __ldcg(a.row_lp + at);
+  for (int c0 = lo * k + tid; c0 < a.rows * k; c0 += 4 * GROW_THREADS) {      // four entries per trip to L2
+    u64 key[4];
+    double lp[4];
+    int at[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int c = min(c0 + u * GROW_THREADS, a.rows * k - 1), i = c / k, pos = c - i * k;
+      at[u] = pos * pitch + i;
+      key[u] = __ldcg(a.row_keys + (nb + i) * a.key_stride + pos);
+      lp[u] = __ldcg(a.row_lp + (nb + i) * a.key_stride + pos);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { sm.key[at[u]] = key[u]; sm.lp[at[u]] = lp[u]; }
   }
+  // (the target's choices are needed only at the end: requested now, used then)
+  const bool mine = tid < N;
+  const u64 best_key = a.best && mine ? __ldcg(a.best + nb + tid) : 0ull;
+  const unsigned best_bad = a.best && mine ? __ldcg(a.row_bad + nb + tid) : 0u;
   for (int i = tid; i < N; i += GROW_THREADS) a.row_count[nb + i] = 0u;
   if (a.first) {
     if (tid == 0) {
@@ -370,9 +373,11 @@ grow_kernel(GrowArgs a) {
   }
   __syncthreads();
 
-  const int G = a.group, gl = lane & (G - 1), gbase = lane & ~(G - 1);     // lanes of one row
-  const unsigned gmask = (G == 32 ? FULL : ((1u << G) - 1u)) << gbase;
-  const int per_pass = GROW_THREADS / G, my_row = tid / G;
+  constexpr int G = KMAX;                               // lanes of one row in the append
+  const int gl = lane & (G - 1), gbase = lane & ~(G - 1);
+  const unsigned gmask = (G == 32 ? FULL : ((1u << (G & 31)) - 1u)) << gbase;
+  constexpr int per_pass = GROW_THREADS / G;
+  const int my_row = tid / G;
   bool paused = false;
   for (; d < a.n_layers; ++d) {
     const int F = hi - lo, n = hi;
@@ -380,93 +385,137 @@ grow_kernel(GrowArgs a) {
     if (hi > a.rows) { paused = true; break; }          // the frontier's rows are not all there yet
     const int R = N - n, ke = min(k, R);                // a parent can place at most R children
     // ---- the frontier's best candidate; rows without a softmax ----
-    int bad = 0;
+    double ps[NQ];                                      // log p of this lane's rows q * 32 + lane
     u64 head = 0ull;
-    if (tid < F) {
-      const double lp = sm.lp[(lo + tid) * k];
-      bad = lp != lp;
-      const double s = sm.score[lo + tid] + lp;
-      if (s > -CUDART_INF) head = f64_ord(s);
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int j = q * 32 + lane;
+      ps[q] = -CUDART_INF;
+      if (j < F) {
+        ps[q] = sm.score[lo + j];
+        const double lp = sm.lp[lo + j];
+        bad |= lp != lp;
+        const double s = ps[q] + lp;
+        if (s > -CUDART_INF) head = umax64(head, f64_ord(s));
+      }
     }
-    if (warp < MAX_BUDGET / 32) {
-      head = warp_max_u64(head);
-      if (lane == 0) s_head[warp] = head;
-    }
-    if (__syncthreads_or(bad)) {                        // this sequence adds nothing any more
-      if (tid == 0) atomicOr(a.status, STATUS_NONFINITE);
-      lo = hi;
+    if (__any_sync(FULL, bad)) {                        // this sequence adds nothing any more
+      if (tid == 0) {
+        atomicOr(a.status, STATUS_NONFINITE);
+        a.t.layer_off[b * a.lo_stride + d + 2] = n;
+      }
       ++d;
-      if (tid == 0) a.t.layer_off[b * a.lo_stride + d + 1] = n;
       break;
     }
     const bool init = d < a.init_layers;
-    double thr = -CUDART_INF;
-    const u64 anchor = umax64(umax64(s_head[0], s_head[1]), umax64(s_head[2], s_head[3]));
-    if (!init && anchor != 0ull) thr = a.log_mu + f64_unord(anchor);
-
-    // ---- eligible candidates of each row ----
-    for (int j = my_row; j < per_pass * ((F + per_pass - 1) / per_pass); j += per_pass) {
-      double s = -CUDART_INF;
-      if (j < F && gl < ke) s = sm.score[lo + j] + sm.lp[(lo + j) * k + gl];
-      const unsigned m = __ballot_sync(FULL, s > -CUDART_INF && s >= thr) & gmask;
-      if (gl == 0 && j < F) sm.cnt[j] = __popc(m);
+    double thr = -1.7976931348623157e308;                    // an impossible candidate (-inf) never passes
+    if (!init) {
+      head = warp_redux_max_u64(head);
+      if (head != 0ull) thr = a.log_mu + f64_unord(head);
     }
-    __syncthreads();
+    // ---- eligible candidates of each row, and the rows' output offsets ----
+    int cnt[NQ], off[NQ], total = 0;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      cnt[q] = 0;
+      if (q * 32 < F) {
+        const int r = lo + min(q * 32 + lane, F - 1);
+        double s[KMAX];                                 // (unconditional, so that the trips overlap)
+#pragma unroll
+        for (int i = 0; i < KMAX; ++i) s[i] = ps[q] + sm.lp[min(i, k - 1) * pitch + r];
+#pragma unroll
+        for (int i = 0; i < KMAX; ++i) cnt[q] += (i < ke && s[i] >= thr) ? 1 : 0;
+      }
+    }
+    auto scan = [&]() {
+      total = 0;
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        off[q] = total;
+        if (q * 32 >= F) continue;
+        int inc = cnt[q];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(FULL, inc, o);
+          if (lane >= o) inc += t;
+        }
+        off[q] = total + inc - cnt[q];
+        total += __shfl_sync(FULL, inc, 31);
+      }
+    };
+    scan();
+    // row j's value of a per-lane-row array (j / 32 is the same for the whole warp)
+    auto of_row = [&](const int (&v)[NQ], int j) {
+      int x = v[0];
+#pragma unroll
+      for (int q = 1; q < NQ; ++q) if ((j >> 5) == q) x = v[q];
+      return __shfl_sync(FULL, x, j & 31);
+    };
     const int want = init ? min(a.root_topk, R) : R;
-    int total = scan_rows(sm.cnt, off, F, lane);
     if (total > want) {
       // ---- budget truncation: rank by (score desc, parent asc, token asc) among the eligible; rows
       // are sorted that way already, so a rank is a sum of binary searches in the rows' prefixes ----
-      int keep[MAX_BUDGET / (GROW_THREADS / 32)];       // of this group's rows, one per pass (32 lanes a row at most)
-      int np = 0;
-      for (int j0 = 0; j0 < F; j0 += per_pass, ++np) {
-        const int j = j0 + my_row;
+      if (warp == 0)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) if (q * 32 + lane < F) sm.cnt[q * 32 + lane] = cnt[q];
+      __syncthreads();
+      int kept[16];                                     // of this group's row, per pass (at most 32 lanes a row, 128 rows)
+#pragma unroll
+      for (int np = 0; np < 16; ++np) {
+        const int j = np * per_pass + my_row;
+        if (np * per_pass >= F) break;
         bool sel = false;
         if (j < F && gl < sm.cnt[j]) {
-          const double s = sm.score[lo + j] + sm.lp[(lo + j) * k + gl];
+          const double s = sm.score[lo + j] + sm.lp[gl * pitch + lo + j];
           int rank = gl;
           for (int o = 0; o < F && rank < want; ++o) {
             int h = sm.cnt[o];
             if (o == j || h == 0) continue;
-            const double ps = sm.score[lo + o];
-            const double *lp = sm.lp + (lo + o) * k;
+            const double po = sm.score[lo + o];
             const bool before = o < j;
             int l = 0;
             while (l < h) {
               const int mid = (l + h) >> 1;
-              const double v = ps + lp[mid];
+              const double v = po + sm.lp[mid * pitch + lo + o];
               if (v > s || (v == s && before)) l = mid + 1; else h = mid;
             }
             rank += l;
           }
           sel = rank < want;
         }
-        const unsigned m = __ballot_sync(FULL, sel) & gmask;
-        keep[np & (MAX_BUDGET / (GROW_THREADS / 32) - 1)] = __popc(m);
+        kept[np] = __popc(__ballot_sync(FULL, sel) & gmask);
       }
       __syncthreads();
-      np = 0;
-      for (int j0 = 0; j0 < F; j0 += per_pass, ++np) {
-        const int j = j0 + my_row;
-        if (j < F && gl == 0) sm.cnt[j] = keep[np & (MAX_BUDGET / (GROW_THREADS / 32) - 1)];
+#pragma unroll
+      for (int np = 0; np < 16; ++np) {
+        const int j = np * per_pass + my_row;
+        if (np * per_pass >= F) break;
+        if (j < F && gl == 0) sm.cnt[j] = kept[np];
       }
       __syncthreads();
-      total = scan_rows(sm.cnt, off, F, lane);
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) cnt[q] = q * 32 + lane < F ? sm.cnt[q * 32 + lane] : 0;
+      scan();
     }
 
     // ---- append in storage order: (parent asc, token asc) ----
     for (int j0 = 0; j0 < F; j0 += per_pass) {
       const int j = j0 + my_row;
-      const int c = j < F ? sm.cnt[j] : 0;
-      const int tok = (gl < c) ? (int)key_tok(sm.key[(lo + j) * k + gl]) : 0x7FFFFFFF;
+      const int c0 = of_row(cnt, j), o0 = of_row(off, j);
+      const int c = j < F ? c0 : 0;
+      if (!__any_sync(FULL, c > 0)) continue;
+      const int par = lo + min(j, F - 1);
+      const int tok = (gl < c) ? (int)key_tok(sm.key[gl * pitch + par]) : 0x7FFFFFFF;
       int r = 0;
-      for (int i = 0; i < G; ++i) r += __shfl_sync(FULL, tok, gbase + i) < tok ? 1 : 0;
+#pragma unroll
+      for (int i = 0; i < KMAX; ++i) r += __shfl_sync(FULL, tok, gbase + i) < tok ? 1 : 0;      // unused lanes hold the largest
       if (gl < c) {
-        const int node = n + off[j] + r, par = lo + j;
+        const int node = n + o0 + r;
         sm.tok[node] = tok;
         sm.parent[node] = par;
         sm.depth[node] = d + 1;
-        sm.score[node] = sm.score[par] + sm.lp[par * k + gl];
+        sm.score[node] = sm.score[par] + sm.lp[gl * pitch + par];
         sm.mask[2 * node] = sm.mask[2 * par] | (node < 64 ? 1ull << node : 0ull);
         sm.mask[2 * node + 1] = sm.mask[2 * par + 1] | (node >= 64 ? 1ull << (node - 64) : 0ull);
       }
@@ -499,39 +548,31 @@ grow_kernel(GrowArgs a) {
   for (int i = d + 2 + tid; i < a.lo_stride; i += GROW_THREADS) a.t.layer_off[b * a.lo_stride + i] = n;
 
   if (!a.best) return;
-  // ---- greedy walk over the target's choices (Appendix B, temperature 0) ----
-  int *tgt = sm.cnt;                                    // [N]
+  // ---- greedy walk over the target's choices (Appendix B, temperature 0): every node that carries its
+  // parent's target token is that parent's next step (at most one: siblings have different tokens) ----
+  int *tgt = sm.cnt, *next = sm.depth;                  // [N] each (depths are written out)
   int bad = 0;
-  for (int i = tid; i < N; i += GROW_THREADS) {
-    const u64 key = __ldcg(a.best + nb + i);
-    a.best[nb + i] = 0ull;                              // leave the workspace clean
-    const int t = (i < n && key != 0ull) ? (int)key_tok(key) : -1;
-    tgt[i] = t;
-    a.target_tok[nb + i] = t;
-    if (a.row_bad[nb + i]) { bad |= i < n; a.row_bad[nb + i] = 0u; }
+  int t = -1;
+  __syncthreads();
+  if (mine) {
+    if (tid < n && best_key != 0ull) t = (int)key_tok(best_key);
+    tgt[tid] = t;
+    next[tid] = -1;
+    a.target_tok[nb + tid] = t;
+    a.best[nb + tid] = 0ull;                            // leave the workspace clean
+    if (best_bad) { bad = tid < n; a.row_bad[nb + tid] = 0u; }
   }
   if (__syncthreads_or(bad) && tid == 0) atomicOr(a.status, STATUS_NONFINITE);
-  if (warp != 0) return;
-  int cur = 0, len = 0;
-  int32_t *path = a.accept_nodes + (size_t)b * (a.max_depth + 1);
-  if (lane == 0) path[0] = 0;
-  for (int step = 0; step < a.max_depth; ++step) {
-    const int want = tgt[cur];
-    int found = -1;
-    for (int c0 = (cur + 1) & ~31; c0 < n; c0 += 32) {   // a child comes after its parent
-      const int c = c0 + lane;
-      const unsigned m = __ballot_sync(FULL, c < n && sm.parent[c] == cur && sm.tok[c] == want);
-      if (m) { found = c0 + __ffs(m) - 1; break; }
-    }
-    if (found < 0) break;
-    cur = found;
-    ++len;
-    if (lane == 0) path[len] = cur;
-  }
-  for (int i = len + 1 + lane; i <= a.max_depth; i += 32) path[i] = -1;
-  if (lane == 0) {
+  if (tid > 0 && tid < n && sm.tok[tid] == tgt[sm.parent[tid]]) next[sm.parent[tid]] = tid;
+  __syncthreads();
+  if (tid == 0) {
+    int32_t *path = a.accept_nodes + (size_t)b * (a.max_depth + 1);
+    int cur = 0, len = 0;
+    path[0] = 0;
+    for (int c = next[0]; c >= 0 && len < a.max_depth; c = next[c]) { cur = c; path[++len] = c; }
     a.accept_len[b] = len;
     a.bonus_tok[b] = tgt[cur];
+    for (int i = len + 1; i <= a.max_depth; ++i) path[i] = -1;
   }
 }
 
@@ -543,9 +584,18 @@ static size_t row_pass_smem(const talon_ctx *c, bool scan) {
          (scan ? sizeof(int) * (MAX_BATCH + 1) : 0);
 }
 
+template <int NQ>
+static void (*grow_kernel_k(int k))(GrowArgs) {
+  return k <= 8 ? grow_kernel<NQ, 8> : (k <= 16 ? grow_kernel<NQ, 16> : grow_kernel<NQ, 32>);
+}
+static void (*grow_kernel_for(const talon_ctx *c))(GrowArgs) {
+  const int rows = c->p.budget - 1;          // a frontier is never wider
+  return rows <= 32 ? grow_kernel_k<1>(c->k_cap) : (rows <= 64 ? grow_kernel_k<2>(c->k_cap) : grow_kernel_k<4>(c->k_cap));
+}
+
 talon_status grow_step_setup(talon_ctx *c) {
   if (cudaFuncSetAttribute(row_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_pass_smem(c, true)) != cudaSuccess ||
-      cudaFuncSetAttribute(grow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaFuncSetAttribute(grow_kernel_for(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)grow_smem_bytes(c->p.budget, c->k_cap, c->p.budget)) != cudaSuccess)
     return TALON_ERR_CUDA;
   int per_sm = 0;
@@ -579,14 +629,19 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
   const int B = c->B, N = p.budget, k = c->k_cap;
   int expandable, nodes;
   step_bounds(c, n_layers, &expandable, &nodes);
+  // One round with the target rows alongside is the quickest way even where a part of the rows is read
+  // for nothing (the pass then runs at the copy bandwidth; a round of its own costs about 20 us: pass
+  // start-up, hand-off, growth).  A tree of few layers cannot get near a large budget, though: on
+  // confident rows a layer adds one node, on flat ones K, seldom more.  Where the slots beyond
+  // 1 + 7/8 K D would cost more to read than a second round, the first round stops there, the second
+  // takes the rest for the trees that do go on, and the target rows wait for the trees' sizes.
   const double row_bytes = 4.0 * p.vocab * B;           // of one slot of every sequence
-  const bool with_target = target && row_bytes * (expandable + nodes) <= c->step_fuse_mb * 1e6;
+  int first = 1 + p.root_topk * n_layers * 7 / 8;
+  if (c->step_first_rows > 0) first = c->step_first_rows;
+  else if (row_bytes * 2.0 * (expandable - first) < STEP_SPLIT_BYTES) first = expandable;
+  if (first > expandable) first = expandable;
+  const bool with_target = first == expandable;
   *accepted = with_target;
-  int rounds = 1;
-  if (!with_target && row_bytes * expandable > c->step_round_mb * 1e6) {
-    rounds = c->step_rounds;
-    if (rounds > expandable) rounds = expandable;
-  }
   RowPassArgs ra;
   ra.draft = draft; ra.draft_stride = draft_stride;
   ra.target = with_target ? target : nullptr; ra.target_stride = target_stride;
@@ -599,8 +654,6 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
   ga.lo_stride = p.max_depth + 2; ga.B = B; ga.N = N; ga.W = c->W; ga.k = k; ga.key_stride = c->key_stride;
   ga.n_layers = n_layers; ga.max_depth = p.max_depth; ga.root_topk = p.root_topk; ga.init_layers = p.init_layers;
   ga.log_mu = c->log_mu;
-  ga.group = 1;
-  while (ga.group < k) ga.group *= 2;
   ga.row_keys = c->d_row_keys; ga.row_lp = c->d_row_score; ga.growing = c->d_growing; ga.depth_at = c->d_depth_at;
   ga.row_count = c->d_row_count; ga.status = c->d_status;
   ga.best = with_target ? c->d_argmax : nullptr; ga.row_bad = c->d_row_bad;
@@ -608,8 +661,8 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
   ga.accept_len = accept_len; ga.accept_nodes = accept_nodes; ga.bonus_tok = bonus_tok;
 
   int done = 0;
-  for (int r = 0; r < rounds; ++r) {
-    const int upto = (int)((long long)expandable * (r + 1) / rounds);
+  for (int r = 0; done < expandable; ++r) {
+    const int upto = r == 0 ? first : expandable;
     ra.r0 = done; ra.r1 = upto; ra.t1 = with_target ? nodes : done;
     ra.growing = r ? c->d_growing : nullptr;
     ra.clear_status = r == 0;
@@ -651,7 +704,7 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
     ga.first = r == 0; ga.rows = upto;
     {
       LaunchTimer lt(c, TALON_K_SELECT, st);
-      launch_kernel_pdl(c, true, grow_kernel, dim3(B), dim3(GROW_THREADS), grow_smem_bytes(upto, k, N), st, ga);
+      launch_kernel_pdl(c, true, grow_kernel_for(c), dim3(B), dim3(GROW_THREADS), grow_smem_bytes(upto, k, N), st, ga);
     }
     if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
     c->launches += 2;

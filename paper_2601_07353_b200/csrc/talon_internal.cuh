@@ -107,6 +107,7 @@ struct talon_ctx {
   int64_t launches;
   double log_mu;
 
+  void *d_arena;                  // the one allocation behind the pointers below
   int *d_status;
   int32_t *d_prefix_len;          // [batch_max]
   // expansion workspace
@@ -125,9 +126,8 @@ struct talon_ctx {
   int row_grid;                      // CTAs of the row pass at full width
   int32_t *d_growing, *d_depth_at;   // [batch_max] a sequence's tree still grows; layer it stopped at
   unsigned int *d_row_bad;           // [batch_max * N] NaN in a target row (zero between calls)
-  double step_fuse_mb, step_round_mb;   // MB of logits up to which the target rows ride along / one round takes all rows
   int step_rows;                     // 0: whole steps expand layer by layer too
-  int step_rounds;                   // rounds of a larger step
+  int step_first_rows;               // > 0: slots per sequence the first round of a step prepares (for experiments)
   int attn_cluster;                  // key ranges of the tensor-core attention merge inside a cluster (1) or in a second kernel (0)
   long long attn_cluster_min_rows;   // automatic mode: least rows x key ranges for the merge inside the cluster
   int attn_cluster_cap;              // more key ranges than eight are cut back to eight up to this many
@@ -217,7 +217,8 @@ struct LaunchTimer {
   }
 };
 
-// launchers implemented in the .cu files (all asynchronous on `st`)
+// launchers implemented in the .cu files (all asynchronous on `st`).  launch_attention's early_prefix: the
+// kernel launched just before is grow_kernel, and this array holds the prefix lengths it copies
 talon_status launch_reset(talon_ctx *c, const talon_tree *t, const int32_t *root_tok,
                           const int32_t *prefix_len, int B, cudaStream_t st);
 talon_status launch_expand(talon_ctx *c, const talon_tree *t, const float *logits,
@@ -235,12 +236,14 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
                               const void *vp, const void *kt, const void *vt,
                               const int64_t *kv_start, const int32_t *block_table, int bt_stride, int64_t kv_tokens,
                               int64_t stride_t, int64_t stride_h,
-                              int max_prefix_len, float sm_scale, void *out, cudaStream_t st);
+                              int max_prefix_len, float sm_scale, void *out, cudaStream_t st,
+                              const int32_t *early_prefix = nullptr);
 bool attention_tc_supported(const talon_ctx *c, int64_t stride_t, int64_t stride_h, float sm_scale);
 talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *q, const void *kp, const void *vp,
                                  const void *kt, const void *vt, const int64_t *kv_start, const int32_t *block_table,
                                  int bt_stride, int64_t stride_t, int64_t stride_h, int64_t kv_tokens, int max_prefix_len, float sm_scale, void *out,
-                                 int splits, int m_blocks, cudaStream_t st, int *merged_in_kernel);
+                                 int splits, int m_blocks, cudaStream_t st, int *merged_in_kernel,
+                                 const int32_t *early_prefix);
 talon_status launch_accept(talon_ctx *c, const talon_tree *t, const float *target_logits,
                            int64_t row_stride, int32_t *target_tok, int32_t *accept_len,
                            int32_t *accept_nodes, int32_t *bonus_tok, cudaStream_t st, bool close_tree = false);
