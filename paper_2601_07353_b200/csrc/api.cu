@@ -9,7 +9,6 @@
 #include "talon_internal.cuh"
 
 namespace talon {
-talon_status expand_setup(talon_ctx *c);
 talon_status attention_mma_setup();
 talon_status attention_tc_setup();
 }  // namespace talon
@@ -109,7 +108,6 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
   if (k > p->vocab) k = p->vocab;
   if (k < 1) k = 1;
   c->k_cap = k;
-  c->k_slots = k <= 32 ? 1 : (k <= 64 ? 2 : 4);
   c->key_stride = (k + 3) & ~3;
   c->log_mu = std::log(p->mu);
   {
@@ -172,7 +170,6 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     take(&c->d_prefix_len, bm);
     take(&c->d_part_ms, items);
     take(&c->d_row_keys, rows * ks);
-    take(&c->d_row_lse, rows);
     take(&c->d_row_score, rows * ks);
     take(&c->d_growing, bm);
     take(&c->d_depth_at, bm);
@@ -182,9 +179,9 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     take(&c->d_attn_ml, c->attn_ml_elems);
     if (pass == 0 && cudaMalloc(&c->d_arena, total) != cudaSuccess) break;
   }
-  const bool ok = c->d_arena && cudaMemset(c->d_arena, 0, zeroed) == cudaSuccess && talon::expand_setup(c) == TALON_OK &&
+  const bool ok = c->d_arena && cudaMemset(c->d_arena, 0, zeroed) == cudaSuccess && 
                   talon::attention_mma_setup() == TALON_OK && talon::attention_tc_setup() == TALON_OK &&
-                  (c->k_cap > 32 || (talon::expand_fused_setup(c) == TALON_OK && talon::grow_step_setup(c) == TALON_OK));
+                  talon::expand_fused_setup(c) == TALON_OK && (c->k_cap > 32 || talon::grow_step_setup(c) == TALON_OK);
   if (!ok) {
     std::fprintf(stderr, "talon: context creation failed: %s\n", cudaGetErrorString(cudaGetLastError()));
     talon_destroy(c);

@@ -1,5 +1,5 @@
 // Adaptive draft-tree expansion (Algorithm 2 of the paper; Eq. 2-5) as ONE kernel per layer,
-// for per-parent candidate caps k <= 32 (the usual case: the paper's K is 10).
+// for every per-parent candidate cap k (lists of up to 32 keys a row, the paper's K is 10, and wide ones).
 //
 // Streaming phase: expand_stream.cuh.  The frontier's fp32 logit rows are cut into equal chunks, one
 // CTA per chunk at a time; a chunk leaves its k best keys and its share of the normaliser.
@@ -26,7 +26,7 @@ struct FusedArgs {
   int rows_per_seq, layout;
   talon_tree t;
   int lo_stride;
-  int B, N, W, V, d, k, key_stride, max_split, base_offset;
+  int B, N, W, V, d, k, key_stride, max_split, base_offset, pool_cap;
   int root_topk, init_layers;
   double log_mu;
   u64 *part_keys;          // [items, key_stride]  per-chunk top-k, descending
@@ -137,13 +137,12 @@ struct TailSmem {
 
 // Gate, budget truncation and append for one sequence, from the pooled candidates in shared
 // memory (sm.row_keys / sm.score: F rows of k, each row descending; sm.row_mask: the parents'
-// mask rows).  n is the tree's size before the layer.
-__device__ void select_and_append(const FusedArgs &a, const TailSmem &sm, int b, int lo, int F, int n,
+// mask rows).  n is the tree's size before the layer, k the pitch of the rows.
+__device__ void select_and_append(const FusedArgs &a, const TailSmem &sm, int b, int lo, int F, int n, int k,
                                   u64 *s_anchor, int *s_cnt) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int k = a.k;
   const int R = a.N - n;
-  const int ke = min(k, R);                 // a parent can place at most R children
+  const int ke = min(a.k, R);               // a parent can place at most R children
   const size_t nb = (size_t)b * a.N;
   const int C = F * k;
 
@@ -177,7 +176,7 @@ __device__ void select_and_append(const FusedArgs &a, const TailSmem &sm, int b,
       const int j = c / k, i = c - j * k;
       const double s = sm.score[c];
       int rank = i;
-      for (int o = 0; o < F; ++o) {
+      for (int o = 0; o < F && rank < want; ++o) {
         if (o == j) continue;
         const double *sc = sm.score + o * k;
         const bool before = o < j;
@@ -241,11 +240,14 @@ __device__ void select_and_append(const FusedArgs &a, const TailSmem &sm, int b,
   }
 }
 
-__global__ void __launch_bounds__(EXP_THREADS, 3)
+// WIDE: k above 32 (see expand_stream.cuh); a row is then merged by the whole CTA that completes it,
+// whatever the width of the frontier.
+template <bool WIDE>
+__global__ void __launch_bounds__(EXP_THREADS, WIDE ? 2 : 3)
 expand_fused_kernel(FusedArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ u64 s_buf[EXP_WARPS][XS_BUF];          // per-warp buffers of keys that reached the threshold
-  __shared__ u64 s_pool[XS_POOL];                   // the chunk's candidates, all warps
+  __shared__ u64 s_buf[EXP_WARPS][ListSize<WIDE>::BUF];          // per-warp buffers of keys that reached the threshold
+  __shared__ u64 s_pool[ListSize<WIDE>::POOL];                   // the chunk's candidates, all warps
   __shared__ int s_warp[EXP_WARPS];
   __shared__ float s_m[EXP_WARPS], s_s[EXP_WARPS];
   __shared__ __align__(8) u64 s_bar[EXP_WARPS][XS_RING];   // "tile landed" barriers, per warp
@@ -329,12 +331,12 @@ expand_fused_kernel(FusedArgs a) {
     const int lo = rl.node - rl.j;               // first frontier node of the sequence
     const int n_before = lo + rl.F;              // the tree's size before this layer
     const int ke = min(k, a.N - n_before);       // a parent can place at most N - |T| children
-    if (!stream_chunk(sh, rowp, start, end, k, ke, gated, ln_mu, (size_t)item, res, wt)) return;
+    if (!stream_chunk<WIDE>(sh, rowp, start, end, k, ke, gated, ln_mu, (size_t)item, res, wt)) return;
 
     // ---- hand-off.  The barrier orders this CTA's writes before thread 0's device-scope
     // release; the last arrival acquires.  Narrow frontiers count chunks per sequence, wide ones
     // chunks per row and then rows per sequence. ----
-    const bool two_level = rl.F > XS_TWO_LEVEL;
+    const bool two_level = WIDE || rl.F > XS_TWO_LEVEL;
     __syncthreads();
     chunk_clear(sh);
     if (tid == 0) {
@@ -354,11 +356,15 @@ expand_fused_kernel(FusedArgs a) {
 
     TailSmem sm;
     const int rows_max = a.N - 1;
+    // pitch of the pooled rows; WIDE rows are packed at the ke children a parent can still place, which
+    // bounds the pool by rows x remaining budget
+    const int kp = WIDE ? ke : k;
+    const int pool_cap = WIDE ? a.pool_cap : rows_max * k;
     {
       unsigned char *p = smem_raw;
-      sm.stage = reinterpret_cast<u64 *>(p);            p += sizeof(u64) * EXP_WARPS * stage_words(k);
-      sm.row_keys = reinterpret_cast<u64 *>(p);         p += sizeof(u64) * rows_max * k;
-      sm.score = reinterpret_cast<double *>(p);         p += sizeof(double) * rows_max * k;
+      sm.stage = reinterpret_cast<u64 *>(p);            p += WIDE ? 0 : sizeof(u64) * EXP_WARPS * stage_words(k);
+      sm.row_keys = reinterpret_cast<u64 *>(p);         p += sizeof(u64) * pool_cap;
+      sm.score = reinterpret_cast<double *>(p);         p += sizeof(double) * pool_cap;
       sm.row_mask = reinterpret_cast<u64 *>(p);         p += sizeof(u64) * rows_max * a.W;
       sm.row_cnt = reinterpret_cast<int *>(p);          p += sizeof(int) * rows_max;
       sm.row_off = reinterpret_cast<int *>(p);          p += sizeof(int) * rows_max;
@@ -368,19 +374,28 @@ expand_fused_kernel(FusedArgs a) {
     if (two_level) {
       // ---- this CTA finished a row of a wide frontier: one warp merges it, publishes the result
       // and counts the row; the CTA that counts the sequence's last row goes on ----
-      if (warp == 0) {
-        u64 key; double sc;
+      if (WIDE) {
         int item0, S;
         row_chunks(g, row, item0, S);
-        const double ps = a.t.score[nb + rl.node];
-        const bool finite = merge_row(res, (size_t)item0, S, k, ke, ps, sm.stage, key, sc);
-        if (!finite) {
-          sc = lane == 0 ? CUDART_NAN : -CUDART_INF;
-          if (lane == 0) atomicOr(a.status, STATUS_NONFINITE);
-        }
-        if (lane < k) {
-          a.row_keys[(size_t)row * a.key_stride + lane] = key;
-          a.row_score[(size_t)row * a.key_stride + lane] = sc;
+        merge_row_wide(res, (size_t)item0, S, k, ke, a.t.score[nb + rl.node], reinterpret_cast<u64 *>(smem_raw),
+                       a.row_keys + (size_t)row * a.key_stride, a.row_score + (size_t)row * a.key_stride, a.status);
+        __syncthreads();
+      }
+      if (warp == 0) {
+        if (!WIDE) {
+          u64 key; double sc;
+          int item0, S;
+          row_chunks(g, row, item0, S);
+          const double ps = a.t.score[nb + rl.node];
+          const bool finite = merge_row(res, (size_t)item0, S, k, ke, ps, sm.stage, key, sc);
+          if (!finite) {
+            sc = lane == 0 ? CUDART_NAN : -CUDART_INF;
+            if (lane == 0) atomicOr(a.status, STATUS_NONFINITE);
+          }
+          if (lane < k) {
+            a.row_keys[(size_t)row * a.key_stride + lane] = key;
+            a.row_score[(size_t)row * a.key_stride + lane] = sc;
+          }
         }
         __syncwarp();
         if (lane == 0) {
@@ -390,17 +405,18 @@ expand_fused_kernel(FusedArgs a) {
           if (s_last_seq) c.store(0u, cuda::memory_order_relaxed);
         }
       }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the merge wrote where copies will land
       __syncthreads();
       if (!s_last_seq) continue;
       // ---- collect the sequence's row results and the parents' mask rows: four loads per thread
       // go to registers before the first store, so that they share one trip to L2 ----
-      const int C = rl.F * k;
+      const int C = rl.F * kp;
       for (int c0 = 0; c0 < C; c0 += 4 * EXP_THREADS) {
         u64 key[4]; double sc[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int c = c0 + u * EXP_THREADS + tid;
-          const int j = c / k, i = c - j * k;
+          const int j = c / kp, i = c - j * kp;
           key[u] = c < C ? __ldcg(a.row_keys + (size_t)(rl.row0 + j) * a.key_stride + i) : 0ull;
           sc[u] = c < C ? __ldcg(a.row_score + (size_t)(rl.row0 + j) * a.key_stride + i) : -CUDART_INF;
         }
@@ -415,14 +431,14 @@ expand_fused_kernel(FusedArgs a) {
           else {
             sm.score[c] = sc[u];
             // rows are sorted: heads carry the maxima
-            if (c % k == 0 && sc[u] > -CUDART_INF) atomicMax(&s_anchor, f64_ord(sc[u]));
+            if (c % kp == 0 && sc[u] > -CUDART_INF) atomicMax(&s_anchor, f64_ord(sc[u]));
           }
         }
         if (mi < rl.F * a.W) sm.row_mask[mi] = mword;
       }
       for (int mi = (C + 4 * EXP_THREADS - 1) / (4 * EXP_THREADS) * EXP_THREADS + tid; mi < rl.F * a.W; mi += EXP_THREADS)
         sm.row_mask[mi] = a.t.mask[(nb + lo) * a.W + mi];
-    } else {
+    } else if (!WIDE) {
       // ---- this CTA finished the sequence: one warp per row ----
       for (int j = warp; j < rl.F; j += EXP_WARPS) {
         u64 key; double sc;
@@ -444,34 +460,55 @@ expand_fused_kernel(FusedArgs a) {
     if (s_bad) {             // a frontier row was not finite: this sequence adds nothing
       if (tid == 0) a.t.layer_off[rl.b * a.lo_stride + a.d + 2] = n_before;
     } else {
-      select_and_append(a, sm, rl.b, lo, rl.F, n_before, &s_anchor, &s_ecnt);
+      select_and_append(a, sm, rl.b, lo, rl.F, n_before, kp, &s_anchor, &s_ecnt);
     }
-    __syncthreads();     // the next chunk's bulk copies land in the memory the selection phase just used
+    // the next chunk's bulk copies land in the memory the selection phase just used
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
     if (tid == 0) { s_anchor = 0ull; s_ecnt = 0; s_bad = 0; }
   }
 }
 
+// Largest pool of a layer: F rows of min(k, N - 1 - F) candidates (the tree holds F + 1 nodes at least;
+// the root's layer: one row of up to N - 1).
+int pool_capacity(const talon_ctx *c) {
+  int best = 1;
+  for (int f = 1; f <= c->p.budget - 1; ++f) {
+    const int r = f == 1 ? c->p.budget - 1 : c->p.budget - 1 - f;
+    const int ke = c->k_cap < r ? c->k_cap : r;
+    if (f * ke > best) best = f * ke;
+  }
+  return best;
+}
+
 size_t fused_smem_bytes(const talon_ctx *c) {
   const size_t rows = c->p.budget - 1, k = c->k_cap, W = c->W;
-  const size_t tail = sizeof(u64) * EXP_WARPS * (FX_MAX_SPLITS * k + FX_SURV + k) + rows * k * (8 + 8 + 1) +
-                      rows * (8 * W + 4 + 4) + 16;
-  const size_t ring = sizeof(float) * EXP_WARPS * XS_RING * XS_WTILE;       // the two phases share the space
-  return ((tail > ring ? tail : ring) + 15) & ~(size_t)15;
+  const bool wide = c->k_cap > 32;
+  const size_t pool = wide ? pool_capacity(c) : rows * k;
+  const size_t tail = (wide ? 0 : sizeof(u64) * EXP_WARPS * stage_words(k)) + pool * (8 + 8 + 1) + rows * (8 * W + 4 + 4) + 16;
+  size_t bytes = sizeof(float) * EXP_WARPS * XS_RING * XS_WTILE;            // the two phases share the space
+  if (bytes < tail) bytes = tail;
+  if (wide && bytes < sizeof(u64) * WIDE_STAGE_WORDS) bytes = sizeof(u64) * WIDE_STAGE_WORDS;
+  return (bytes + 15) & ~(size_t)15;
 }
 
 // batches above 32 sequences keep the frontier bases in dynamic shared memory behind that
 size_t fused_base_bytes(int B) { return B > 32 ? sizeof(int) * (MAX_BATCH + 1) : 0; }
 
+void (*fused_kernel_for(const talon_ctx *c))(FusedArgs) {
+  return c->k_cap > 32 ? expand_fused_kernel<true> : expand_fused_kernel<false>;
+}
+
 }  // namespace
 
 talon_status expand_fused_setup(talon_ctx *c) {
   const size_t bytes = fused_smem_bytes(c);
-  if (cudaFuncSetAttribute(expand_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute(fused_kernel_for(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(bytes + fused_base_bytes(c->p.batch_max))) !=
       cudaSuccess)
     return TALON_ERR_CUDA;
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expand_fused_kernel, EXP_THREADS, bytes) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_kernel_for(c), EXP_THREADS, bytes) !=
       cudaSuccess || per_sm < 1)
     return TALON_ERR_CUDA;
   if (per_sm > EXP_CTAS_PER_SM) per_sm = EXP_CTAS_PER_SM;
@@ -487,6 +524,7 @@ talon_status launch_expand_fused(talon_ctx *c, const talon_tree *t, const float 
   a.B = c->B; a.N = c->p.budget; a.W = c->W; a.V = c->p.vocab; a.d = c->layers_run; a.k = c->k_cap;
   a.key_stride = c->key_stride;
   a.max_split = c->expand_max_split;
+  a.pool_cap = pool_capacity(c);
   long long max_items = (long long)rows_bound * FX_MAX_SPLITS;
   int grid = c->fused_grid;
   if (max_items < grid) grid = (int)max_items;
@@ -497,7 +535,7 @@ talon_status launch_expand_fused(talon_ctx *c, const talon_tree *t, const float 
   {
     LaunchTimer lt(c, TALON_K_EXPAND_ROWS, st);
     a.base_offset = (int)fused_smem_bytes(c);
-    launch_kernel_pdl(c, true, expand_fused_kernel, dim3(grid), dim3(EXP_THREADS), fused_smem_bytes(c) + fused_base_bytes(c->B), st, a);
+    launch_kernel_pdl(c, true, fused_kernel_for(c), dim3(grid), dim3(EXP_THREADS), fused_smem_bytes(c) + fused_base_bytes(c->B), st, a);
   }
   if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
   c->launches += 1;

@@ -36,10 +36,15 @@ typedef unsigned long long u64;
 
 constexpr int XS_WTILE = 512;                 // floats a warp takes per step: 16 per lane, one 2 KB copy
 constexpr int XS_RING = 3;                    // copies in flight per warp
-constexpr int XS_BUF = FX_QCAP;               // keys a warp's candidate buffer holds
-constexpr int XS_POOL = 384;                  // keys the CTA pool holds
+// Two variants: lists of up to 32 keys a row (the paper's K is 10), and WIDE ones of up to 128 (the
+// whole-vocabulary pool keeps N - 1 per parent).
+template <bool WIDE> struct ListSize {
+  static constexpr int BUF = WIDE ? 256 : 128;      // keys a warp's candidate buffer holds
+  static constexpr int POOL = WIDE ? 1024 : 384;    // keys the CTA pool holds
+  static constexpr int KMAX = WIDE ? 128 : 32;
+  static_assert(BUF >= KMAX + 32 && POOL >= EXP_WARPS * KMAX, "buffers must hold a cut-back list plus one ballot");
+};
 static_assert(XS_WTILE * EXP_WARPS == EXP_TILE, "a CTA step is eight warp tiles");
-static_assert(XS_BUF >= 64 && XS_POOL >= EXP_WARPS * 32, "buffers must hold a cut-back list plus one ballot");
 
 // 2^x on the special-function unit (relative error about 2^-22, results below 2^-126 flush to 0)
 __device__ __forceinline__ float fast_exp2(float x) {
@@ -257,9 +262,39 @@ __device__ __noinline__ CutBack cut_back_impl(u64 *buf, int ke, int n, float thr
   __syncwarp();
   return r;
 }
-__device__ __forceinline__ void cut_back(u64 *buf, int ke, WarpStream &w, int lane) {
-  (void)lane;
-  const CutBack r = cut_back_impl(buf, ke, w.cnt, w.thr_f, w.thr_key);
+// The same for lists beyond one key per lane: ranked by counting (rare: the buffer holds twice the list).
+__device__ __noinline__ CutBack cut_back_wide_impl(u64 *buf, int ke, int n, float thr_f, u64 thr_key) {
+  constexpr int PER = ListSize<true>::BUF / 32;
+  const int lane = threadIdx.x & 31;
+  u64 own[PER];
+  int rank[PER];
+#pragma unroll
+  for (int u = 0; u < PER; ++u) { own[u] = u * 32 + lane < n ? buf[u * 32 + lane] : 0ull; rank[u] = 0; }
+  for (int o = 0; o < n; ++o) {
+    const u64 key = buf[o];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) rank[u] += key > own[u] ? 1 : 0;
+  }
+  __syncwarp();
+  CutBack r;
+  r.cnt = 0; r.thr_key = thr_key; r.thr_f = thr_f;
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    const bool keep = own[u] != 0ull && rank[u] < ke;
+    if (keep) buf[rank[u]] = own[u];
+    r.cnt += __popc(__ballot_sync(FULL, keep));
+  }
+  __syncwarp();
+  if (r.cnt == ke) {
+    r.thr_key = buf[ke - 1];
+    r.thr_f = fmaxf(thr_f, key_logit(r.thr_key));
+  }
+  return r;
+}
+template <bool WIDE>
+__device__ __forceinline__ void cut_back(u64 *buf, int ke, WarpStream &w) {
+  const CutBack r = WIDE ? cut_back_wide_impl(buf, ke, w.cnt, w.thr_f, w.thr_key)
+                         : cut_back_impl(buf, ke, w.cnt, w.thr_f, w.thr_key);
   w.cnt = r.cnt; w.thr_key = r.thr_key; w.thr_f = r.thr_f;
 }
 
@@ -306,11 +341,37 @@ __device__ __forceinline__ void refresh_threshold(WarpStream &w, int ke, int sha
   w.thr_f = fmaxf(w.thr_f, cand);
 }
 
+// WIDE lists: a row's k-th largest needs more elements than a warp has lanes, so the bound is the
+// smallest of the `active` warps' (share_pos + 1)-th largest lane maxima alone; publish, barrier (the
+// caller's, where all warps can meet), then read.
+__device__ __forceinline__ void publish_maxima(const WarpStream &w, int share_pos, float *s_wtop, float *s_wmax, int lane, int warp) {
+  const float sorted = warp_sort_desc_f32(w.m_t, lane);
+  const float mine = __shfl_sync(FULL, sorted, share_pos & 31), wmax = __shfl_sync(FULL, sorted, 0);
+  if (lane == 0) { s_wtop[warp] = share_pos < 32 ? mine : -CUDART_INF_F; s_wmax[warp] = wmax; }
+  __syncwarp();
+}
+__device__ __forceinline__ void read_threshold(WarpStream &w, int active, bool gated, float ln_mu, const float *s_wtop,
+                                               const float *s_wmax, int lane) {
+  float omin = lane < active ? s_wtop[lane] : CUDART_INF_F;
+  float omax = lane < active ? s_wmax[lane] : -CUDART_INF_F;
+#pragma unroll
+  for (int o = 4; o; o >>= 1) {
+    omin = fminf(omin, __shfl_xor_sync(FULL, omin, o));
+    omax = fmaxf(omax, __shfl_xor_sync(FULL, omax, o));
+  }
+  omin = __shfl_sync(FULL, omin, 0);
+  omax = __shfl_sync(FULL, omax, 0);
+  if (active > 0) w.thr_f = fmaxf(w.thr_f, omin);
+  if (gated && omax > -CUDART_INF_F) w.thr_f = fmaxf(w.thr_f, omax + ln_mu - (1e-4f + 1e-6f * fabsf(omax)));
+}
+
 // Appends the elements of one tile that reach the threshold to the warp's buffer.  `slot` is the
 // warp's copy of the tile in shared memory (still intact: it is refilled after this call), tok_tile
 // the token id of its first element; lane l holds elements (i / 4) * 128 + l * 4 + i % 4 of it in v.
+template <bool WIDE>
 __device__ __forceinline__ void collect_tile(const float *slot, const float (&v)[16], int tok_tile, int ke, u64 *buf,
                                              WarpStream &w, int lane) {
+  constexpr int BUF = ListSize<WIDE>::BUF;
   unsigned mm = 0u;
 #pragma unroll
   for (int i = 0; i < 16; ++i)
@@ -323,7 +384,7 @@ __device__ __forceinline__ void collect_tile(const float *slot, const float (&v)
     if (lane >= o) inc += t;
   }
   const int total = __shfl_sync(FULL, inc, 31);
-  if (w.cnt + total <= XS_BUF) {
+  if (w.cnt + total <= BUF) {
     // the usual case: a handful of elements in a few lanes; each lane fetches its own from the
     // slot.  After a cut-back only keys above the buffer's k-th count: the others leave an empty
     // slot (key 0), which every reader of the buffer skips.
@@ -337,13 +398,13 @@ __device__ __forceinline__ void collect_tile(const float *slot, const float (&v)
     }
     w.cnt += total;
     __syncwarp();
-    if (w.cnt > XS_BUF - 32) cut_back(buf, ke, w, lane);
+    if (w.cnt > BUF - 32) cut_back<WIDE>(buf, ke, w);
     return;
   }
   // More than the buffer holds (equal logits, a sorted row, a cold threshold): cut the buffer
   // back, then take the tile one register slot at a time, cutting back whenever a ballot's worth
   // might not fit.
-  cut_back(buf, ke, w, lane);
+  cut_back<WIDE>(buf, ke, w);
 #pragma unroll 1
   for (int i = 0; i < 16; ++i) {
     const int e = (i >> 2) * 128 + lane * 4 + (i & 3);
@@ -352,8 +413,8 @@ __device__ __forceinline__ void collect_tile(const float *slot, const float (&v)
     bool ok = ((mm >> i) & 1u) && x >= w.thr_f && key > w.thr_key;
     unsigned mk = __ballot_sync(FULL, ok);
     if (mk == 0u) continue;
-    if (w.cnt + __popc(mk) > XS_BUF) {
-      cut_back(buf, ke, w, lane);
+    if (w.cnt + __popc(mk) > BUF) {
+      cut_back<WIDE>(buf, ke, w);
       ok = ok && x >= w.thr_f && key > w.thr_key;
       mk = __ballot_sync(FULL, ok);
     }
@@ -370,8 +431,8 @@ __device__ __forceinline__ void collect_tile(const float *slot, const float (&v)
 struct ChunkShared {
   float *ring;             // [XS_RING][XS_WTILE]
   u64 *bar;                // [XS_RING]              "tile landed" barriers
-  u64 *buf;                // [XS_BUF]               keys that reached the threshold
-  u64 *pool;               // [XS_POOL]              the chunk's candidates, all warps
+  u64 *buf;                // [BUF]                  keys that reached the threshold
+  u64 *pool;               // [POOL]                 the chunk's candidates, all warps
   float *m, *s;            // [EXP_WARPS]            each warp's maximum and sum of exponentials
   float *wtop, *wmax;      // [EXP_WARPS]            each warp's ceil(k/8)-th largest and largest lane maximum
   int *pool_n, *abort_flag;
@@ -387,10 +448,11 @@ struct ChunkOut {
 // k) and (max, sum) at index `item`; all threads of the CTA.  wt counts the tiles this warp has taken
 // from its ring since the kernel began.  sh.pool_n, sh.wtop and sh.wmax have to be as chunk_clear()
 // leaves them.  Returns false, for the whole CTA, when a copy did not land in time.
+template <bool WIDE>
 __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float *rowp, int start, int end, int k, int ke,
                                              bool gated, float ln_mu, size_t item, const ChunkOut &res, unsigned &wt) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int share_pos = (ke + EXP_WARPS - 1) / EXP_WARPS - 1;
+  constexpr int POOL = ListSize<WIDE>::POOL;
 
   // ---- this warp's slice of the chunk ----
   // (a short chunk goes to fewer warps, a full tile each: thresholds need elements to work with)
@@ -398,6 +460,9 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
   const int ws = start + warp * wlen;
   const int we = min(end, ws + wlen);
   const int nt = ws < we ? (we - ws + XS_WTILE - 1) / XS_WTILE : 0;
+  // warps with a slice; each publishes so many lane maxima that all together cover ke elements
+  const int active = WIDE ? max(min((end - start + wlen - 1) / wlen, EXP_WARPS), 0) : EXP_WARPS;
+  const int share_pos = (ke + active - 1) / max(active, 1) - 1;
   auto issue = [&](int t, unsigned slot_index) {
     const int base = ws + t * XS_WTILE;
     const int n = min(XS_WTILE, we - base);
@@ -463,9 +528,15 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
     }
     refreshed = (t & (t + 1)) == 0 || t == 2;  // after tiles 1, 2, 3, 4, 8, 16, ... of the slice
     // (the first tile has nothing but its own lane maxima to go by: their exact ke-th largest)
-    if (refreshed) refresh_threshold(w, ke, share_pos, gated, ln_mu, sh.wtop, sh.wmax, lane, warp, t == 0);
+    if (WIDE) {
+      if (refreshed) {
+        publish_maxima(w, share_pos, sh.wtop, sh.wmax, lane, warp);
+        if (t == 0) __syncthreads();           // before it there is no threshold at all
+        read_threshold(w, active, gated, ln_mu, sh.wtop, sh.wmax, lane);
+      }
+    } else if (refreshed) refresh_threshold(w, ke, share_pos, gated, ln_mu, sh.wtop, sh.wmax, lane, warp, t == 0);
     if (__ballot_sync(FULL, bm >= w.thr_f) != 0u) {
-      collect_tile(sh.ring + sl * XS_WTILE, v, base, ke, sh.buf, w, lane);
+      collect_tile<WIDE>(sh.ring + sl * XS_WTILE, v, base, ke, sh.buf, w, lane);
       __syncwarp();
     }
     // Every lane's loads from the slot have delivered their data (the vote needs every lane's
@@ -473,19 +544,24 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
     // tile XS_RING ahead.
     if (lane == 0 && t + XS_RING < nt) issue(t + XS_RING, wt - 1 + XS_RING);
   }
-  if (nt > 4 && !refreshed) refresh_threshold(w, ke, share_pos, gated, ln_mu, sh.wtop, sh.wmax, lane, warp, false);
+  if (WIDE) {
+    if (nt > 0) publish_maxima(w, share_pos, sh.wtop, sh.wmax, lane, warp);
+    else __syncthreads();                      // the others' barrier after their first tile
+    __syncthreads();
+    read_threshold(w, active, gated, ln_mu, sh.wtop, sh.wmax, lane);
+  } else if (nt > 4 && !refreshed) refresh_threshold(w, ke, share_pos, gated, ln_mu, sh.wtop, sh.wmax, lane, warp, false);
 
   // ---- the warp's survivors -> the CTA pool; its normaliser -> shared memory ----
   {
     // a warp that could not build a threshold (a short slice) brings its ke best keys only, so
     // that eight warps never overflow the pool
-    if (w.cnt > XS_POOL / EXP_WARPS) cut_back(sh.buf, ke, w, lane);
+    if (w.cnt > POOL / EXP_WARPS) cut_back<WIDE>(sh.buf, ke, w);
     const int n = w.cnt;
     for (int i = lane; i < n; i += 32) {
       const u64 key = sh.buf[i];
       if (key != 0ull && key_logit(key) >= w.thr_f) {
         const int pos = atomicAdd(sh.pool_n, 1);
-        if (pos < XS_POOL) sh.pool[pos] = key;
+        if (pos < POOL) sh.pool[pos] = key;
       }
     }
     float wm = w.m_t;
@@ -499,17 +575,17 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
   }
   __syncthreads();
   if (*sh.abort_flag) return false;
-  if (*sh.pool_n > XS_POOL) {
+  if (*sh.pool_n > POOL) {
     // the pool cannot hold every survivor (equal logits): each warp brings its ke best only
     __syncthreads();
     if (tid == 0) *sh.pool_n = 0;
     __syncthreads();
-    cut_back(sh.buf, ke, w, lane);
+    cut_back<WIDE>(sh.buf, ke, w);
     const int n = w.cnt;
     int pos = 0;
     if (lane == 0) pos = atomicAdd(sh.pool_n, n);
     pos = __shfl_sync(FULL, pos, 0);
-    if (lane < n) sh.pool[pos + lane] = sh.buf[lane];
+    for (int i = lane; i < n; i += 32) sh.pool[pos + i] = sh.buf[i];
     __syncthreads();
   }
 
@@ -655,6 +731,78 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
   }
   __syncwarp();
   return finite;
+}
+
+// The same for WIDE lists, by the whole CTA: the row's k best keys and scores go straight to
+// key_out / score_out [k] (slot 0 of score_out NaN when the row has no softmax).  st: WIDE_STAGE_WORDS
+// words of shared memory.
+constexpr int WIDE_STAGE_WORDS = 2 * FX_MAX_SPLITS * 128 + 4;
+__device__ __forceinline__ void merge_row_wide(const ChunkOut &res, size_t item0, int S, int k, int ke, double ps, u64 *st,
+                                               u64 *key_out, double *score_out, int *status) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ks = res.key_stride, total = S * ke;
+  u64 *sv = st + FX_MAX_SPLITS * 128;
+  double *s_lse = reinterpret_cast<double *>(sv + FX_MAX_SPLITS * 128);
+  int *s_n = reinterpret_cast<int *>(s_lse + 1);
+  u64 *s_tau = reinterpret_cast<u64 *>(s_lse + 2);
+  for (int i = tid; i < total; i += EXP_THREADS) {
+    const int c = i / ke;
+    st[i] = __ldcg(res.part_keys + (item0 + c) * ks + (i - c * ke));
+  }
+  if (warp == EXP_WARPS - 1) {
+    const float2 ms = lane < S ? __ldcg(res.part_ms + item0 + lane) : make_float2(-CUDART_INF_F, 0.f);
+    float mx = ms.x;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
+    double t = 0.0;
+    if (ms.y != ms.y) t = (double)ms.y;                                 // NaN or +inf logit in the chunk
+    else if (ms.x > -CUDART_INF_F) t = (double)ms.y * (double)exp2f((ms.x - mx) * LOG2E_F);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+    const bool finite = (t > 0.0) && (t < CUDART_INF) && (mx < CUDART_INF_F) && (mx > -CUDART_INF_F);
+    if (lane == 0) {
+      *s_lse = finite ? (double)mx + log(t) : CUDART_NAN;
+      *s_n = 0;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    // Lower bounds of the row's ke-th best key: S chunks hold ceil(ke / S) keys each at least as large
+    // as the smallest of their ceil(ke / S)-th keys; one chunk alone holds ke at least its ke-th.
+    const int p = (ke + S - 1) / S - 1;
+    u64 low = lane < S ? st[lane * ke + p] : ~0ull, own = lane < S ? st[lane * ke + ke - 1] : 0ull;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) { low = umin64(low, shfl_xor_u64(low, o)); own = umax64(own, shfl_xor_u64(own, o)); }
+    if (lane == 0) *s_tau = umax64(low, own);
+  }
+  __syncthreads();
+  const u64 tau = *s_tau;
+  for (int i = tid; i < total; i += EXP_THREADS) {
+    const u64 key = st[i];
+    if (key != 0ull && key >= tau) sv[atomicAdd(s_n, 1)] = key;
+  }
+  __syncthreads();
+  const int ns = *s_n;
+  const double lse = *s_lse;
+  for (int c0 = 0; c0 < ns; c0 += EXP_THREADS / 4) {                     // four lanes count a key's betters
+    const int ci = c0 + (tid >> 2), q = tid & 3;
+    const u64 key = ci < ns ? sv[ci] : 0ull;
+    int r = 0;
+#pragma unroll 4
+    for (int o = q; o < ns; o += 4) r += (sv[o] > key) ? 1 : 0;
+    r += __shfl_xor_sync(FULL, r, 1);
+    r += __shfl_xor_sync(FULL, r, 2);
+    if (q == 0 && ci < ns && r < ke) {
+      const double s = ps + ((double)key_logit(key) - lse);
+      key_out[r] = key;
+      score_out[r] = lse != lse ? (r == 0 ? CUDART_NAN : -CUDART_INF) : (s == s && s > -CUDART_INF ? s : -CUDART_INF);
+    }
+  }
+  for (int r = min(ns, ke) + tid; r < k; r += EXP_THREADS) {
+    key_out[r] = 0ull;
+    score_out[r] = (r == 0 && lse != lse) ? CUDART_NAN : -CUDART_INF;
+  }
+  if (tid == 0 && lse != lse) atomicOr(status, STATUS_NONFINITE);
 }
 
 }  // namespace

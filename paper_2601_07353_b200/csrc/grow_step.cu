@@ -152,8 +152,8 @@ __device__ __forceinline__ void argmax_chunk(const float *rowp, int start, int e
 __global__ void __launch_bounds__(EXP_THREADS, 3)
 row_pass_kernel(RowPassArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ u64 s_buf[EXP_WARPS][XS_BUF];
-  __shared__ u64 s_pool[XS_POOL];
+  __shared__ u64 s_buf[EXP_WARPS][ListSize<false>::BUF];
+  __shared__ u64 s_pool[ListSize<false>::POOL];
   __shared__ float s_m[EXP_WARPS], s_s[EXP_WARPS], s_wtop[EXP_WARPS], s_wmax[EXP_WARPS];
   __shared__ __align__(8) u64 s_bar[EXP_WARPS][XS_RING];
   __shared__ int s_warp[EXP_WARPS];
@@ -222,7 +222,7 @@ row_pass_kernel(RowPassArgs a) {
     // a node below the root is gated when every layer but the first is; deeper Top-K layers are not told apart here
     const bool gated = a.init_layers == 0 || (a.init_layers == 1 && node > 0);
     const int item = cta + row;
-    if (!stream_chunk(sh, a.draft + (int64_t)slot * a.draft_stride, start, end, k, k, gated, ln_mu, (size_t)item, res, wt)) return;
+    if (!stream_chunk<false>(sh, a.draft + (int64_t)slot * a.draft_stride, start, end, k, k, gated, ln_mu, (size_t)item, res, wt)) return;
 
     // the barrier orders this CTA's chunk results before thread 0's device-scope release; whoever
     // brings the row's last elements acquires and merges the row

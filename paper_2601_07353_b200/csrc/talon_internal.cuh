@@ -26,7 +26,6 @@ constexpr int MAX_BUDGET = 128;
 constexpr int MAX_BATCH = 1024;
 constexpr int SEL_THREADS = 512;
 // fused expansion kernel (k <= 32)
-constexpr int FX_QCAP = 128;               // keys a warp's candidate buffer can hold
 constexpr int FX_SURV = 64;                // keys of a row that may pass the merge bound before the slow path
 constexpr int FX_MAX_SPLITS = 16;          // chunks per row, at most (one lane per chunk in the merge)
 
@@ -100,7 +99,6 @@ struct talon_ctx {
   int sm_count;
   int W;                  // mask words per node
   int k_cap;              // per-parent candidate cap actually used (cand_topk or N-1)
-  int k_slots;            // ceil(k_cap / 32): list registers per lane
   int key_stride;         // keys stored per row / per item (k_cap rounded up to 4)
   int B;                  // batch of the current reset
   int layers_run;         // expand calls since reset
@@ -117,7 +115,6 @@ struct talon_ctx {
   unsigned long long *d_part_keys;   // [items_cap, key_stride]  per-chunk top-k
   float2 *d_part_ms;                 // [items_cap]              per-chunk (max, sum exp)
   unsigned long long *d_row_keys;    // [rows_cap, key_stride]   per-row top-k
-  double *d_row_lse;                 // [rows_cap]               per-row log-sum-exp
   double *d_row_score;               // [rows_cap, key_stride]   per-row candidate scores (fused kernel, wide frontiers)
   unsigned int *d_row_count;         // [rows_cap]               chunks finished per row
   unsigned int *d_seq_count;         // [batch_max]              chunks finished per sequence (fused kernel)
