@@ -242,9 +242,10 @@ __device__ void select_and_append(const FusedArgs &a, const TailSmem &sm, int b,
 
 // WIDE: k above 32 (see expand_stream.cuh); a row is then merged by the whole CTA that completes it,
 // whatever the width of the frontier.
-template <bool WIDE>
-__global__ void __launch_bounds__(EXP_THREADS, WIDE ? 2 : 3)
+template <int KMAX>          // k rounded up to 8, 16, 32 or 128 (WIDE)
+__global__ void __launch_bounds__(EXP_THREADS, KMAX > 32 ? 2 : 3)
 expand_fused_kernel(FusedArgs a) {
+  constexpr bool WIDE = KMAX > 32;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ u64 s_buf[EXP_WARPS][ListSize<WIDE>::BUF];          // per-warp buffers of keys that reached the threshold
   __shared__ u64 s_pool[ListSize<WIDE>::POOL];                   // the chunk's candidates, all warps
@@ -287,12 +288,12 @@ expand_fused_kernel(FusedArgs a) {
     }
     int inc = fr.f_l;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
+    for (int o = 1; o < a.B; o <<= 1) {
       const int t = __shfl_up_sync(FULL, inc, o);
       if (lane >= o) inc += t;
     }
     fr.base_l = inc - fr.f_l;
-    fr.total = __shfl_sync(FULL, inc, 31);
+    fr.total = __shfl_sync(FULL, inc, a.B - 1);
   } else {
     frontier_bases(a, s_base, s_warp);
     fr.total = s_base[a.B];
@@ -359,7 +360,9 @@ expand_fused_kernel(FusedArgs a) {
     // pitch of the pooled rows; WIDE rows are packed at the ke children a parent can still place, which
     // bounds the pool by rows x remaining budget
     const int kp = WIDE ? ke : k;
-    const int pool_cap = WIDE ? a.pool_cap : rows_max * k;
+    // (the others lie candidate by candidate, a row per lane)
+    const int pitch = rows_max | 1;
+    const int pool_cap = WIDE ? a.pool_cap : pitch * k;
     {
       unsigned char *p = smem_raw;
       sm.stage = reinterpret_cast<u64 *>(p);            p += WIDE ? 0 : sizeof(u64) * EXP_WARPS * stage_words(k);
@@ -387,7 +390,7 @@ expand_fused_kernel(FusedArgs a) {
           int item0, S;
           row_chunks(g, row, item0, S);
           const double ps = a.t.score[nb + rl.node];
-          const bool finite = merge_row(res, (size_t)item0, S, k, ke, ps, sm.stage, key, sc);
+          const bool finite = merge_row<KMAX>(res, (size_t)item0, S, k, ke, ps, sm.stage, key, sc);
           if (!finite) {
             sc = lane == 0 ? CUDART_NAN : -CUDART_INF;
             if (lane == 0) atomicOr(a.status, STATUS_NONFINITE);
@@ -426,12 +429,13 @@ expand_fused_kernel(FusedArgs a) {
         for (int u = 0; u < 4; ++u) {
           const int c = c0 + u * EXP_THREADS + tid;
           if (c >= C) continue;
-          sm.row_keys[c] = key[u];
-          if (sc[u] != sc[u]) { s_bad = 1; sm.score[c] = -CUDART_INF; }
+          const int at = WIDE ? c : (c % kp) * pitch + c / kp;
+          sm.row_keys[at] = key[u];
+          if (sc[u] != sc[u]) { s_bad = 1; sm.score[at] = -CUDART_INF; }
           else {
-            sm.score[c] = sc[u];
+            sm.score[at] = sc[u];
             // rows are sorted: heads carry the maxima
-            if (c % kp == 0 && sc[u] > -CUDART_INF) atomicMax(&s_anchor, f64_ord(sc[u]));
+            if (WIDE && c % kp == 0 && sc[u] > -CUDART_INF) atomicMax(&s_anchor, f64_ord(sc[u]));
           }
         }
         if (mi < rl.F * a.W) sm.row_mask[mi] = mword;
@@ -446,21 +450,46 @@ expand_fused_kernel(FusedArgs a) {
         row_chunks(g, rl.row0 + j, item0, S);
         const double ps = a.t.score[nb + lo + j];
         const u64 pmask = lane < a.W ? a.t.mask[(nb + lo + j) * a.W + lane] : 0ull;     // the parent's ancestor-mask row
-        const bool finite = merge_row(res, (size_t)item0, S, k, ke, ps, sm.stage + warp * stage_words(k), key, sc);
+        const bool finite = merge_row<KMAX>(res, (size_t)item0, S, k, ke, ps, sm.stage + warp * stage_words(k), key, sc);
         if (!finite && lane == 0) { s_bad = 1; atomicOr(a.status, STATUS_NONFINITE); }
         if (lane < k) {
-          sm.row_keys[j * k + lane] = key;
-          sm.score[j * k + lane] = sc;
+          sm.row_keys[lane * pitch + j] = key;
+          sm.score[lane * pitch + j] = sc;
         }
         if (lane < a.W) sm.row_mask[j * a.W + lane] = pmask;
-        if (lane == 0 && sc > -CUDART_INF) atomicMax(&s_anchor, f64_ord(sc));
       }
     }
     __syncthreads();
     if (s_bad) {             // a frontier row was not finite: this sequence adds nothing
       if (tid == 0) a.t.layer_off[rl.b * a.lo_stride + a.d + 2] = n_before;
     } else {
-      select_and_append(a, sm, rl.b, lo, rl.F, n_before, kp, &s_anchor, &s_ecnt);
+      if (WIDE) {
+        select_and_append(a, sm, rl.b, lo, rl.F, n_before, kp, &s_anchor, &s_ecnt);
+      } else {
+        auto append = [&](int slot, int j, int, int tok, double score) {
+          const int node = n_before + slot;
+          a.t.token[nb + node] = tok;
+          a.t.parent[nb + node] = lo + j;
+          a.t.depth[nb + node] = a.d + 1;
+          a.t.score[nb + node] = score;
+          for (int w = 0; w < a.W; ++w) {
+            u64 m = sm.row_mask[j * a.W + w];
+            if ((node >> 6) == w) m |= 1ull << (node & 63);
+            a.t.mask[(nb + node) * a.W + w] = m;
+          }
+        };
+        auto score = [&](int j, int i) { return sm.score[i * pitch + j]; };
+        auto tok = [&](int j, int i) { return (int)key_tok(sm.row_keys[i * pitch + j]); };
+        const bool init = !gated;
+        const int R = a.N - n_before, want = init ? min(a.root_topk, R) : R;
+        constexpr int KN = WIDE ? 32 : KMAX;
+        const int total = rl.F <= 32 ? layer_select<1, KN, EXP_THREADS>(rl.F, k, ke, want, init, a.log_mu, sm.row_cnt, score, tok, append)
+                                     : layer_select<4, KN, EXP_THREADS>(rl.F, k, ke, want, init, a.log_mu, sm.row_cnt, score, tok, append);
+        if (tid == 0) {
+          a.t.n_nodes[rl.b] = n_before + total;
+          a.t.layer_off[rl.b * a.lo_stride + a.d + 2] = n_before + total;
+        }
+      }
     }
     // the next chunk's bulk copies land in the memory the selection phase just used
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -484,7 +513,7 @@ int pool_capacity(const talon_ctx *c) {
 size_t fused_smem_bytes(const talon_ctx *c) {
   const size_t rows = c->p.budget - 1, k = c->k_cap, W = c->W;
   const bool wide = c->k_cap > 32;
-  const size_t pool = wide ? pool_capacity(c) : rows * k;
+  const size_t pool = wide ? pool_capacity(c) : (rows | 1) * k;
   const size_t tail = (wide ? 0 : sizeof(u64) * EXP_WARPS * stage_words(k)) + pool * (8 + 8 + 1) + rows * (8 * W + 4 + 4) + 16;
   size_t bytes = sizeof(float) * EXP_WARPS * XS_RING * XS_WTILE;            // the two phases share the space
   if (bytes < tail) bytes = tail;
@@ -496,7 +525,8 @@ size_t fused_smem_bytes(const talon_ctx *c) {
 size_t fused_base_bytes(int B) { return B > 32 ? sizeof(int) * (MAX_BATCH + 1) : 0; }
 
 void (*fused_kernel_for(const talon_ctx *c))(FusedArgs) {
-  return c->k_cap > 32 ? expand_fused_kernel<true> : expand_fused_kernel<false>;
+  return c->k_cap <= 8 ? expand_fused_kernel<8>
+                       : (c->k_cap <= 16 ? expand_fused_kernel<16> : (c->k_cap <= 32 ? expand_fused_kernel<32> : expand_fused_kernel<128>));
 }
 
 }  // namespace

@@ -36,8 +36,9 @@ typedef unsigned long long u64;
 
 constexpr int XS_WTILE = 512;                 // floats a warp takes per step: 16 per lane, one 2 KB copy
 constexpr int XS_RING = 3;                    // copies in flight per warp
-// Two variants: lists of up to 32 keys a row (the paper's K is 10), and WIDE ones of up to 128 (the
-// whole-vocabulary pool keeps N - 1 per parent).
+// List variants: up to 8, 16 or 32 keys a row (the paper's K is 10; kernels are instantiated per bound,
+// the first two merge a row in registers), and WIDE ones of up to 128 (the whole-vocabulary pool keeps
+// N - 1 per parent).
 template <bool WIDE> struct ListSize {
   static constexpr int BUF = WIDE ? 256 : 128;      // keys a warp's candidate buffer holds
   static constexpr int POOL = WIDE ? 1024 : 384;    // keys the CTA pool holds
@@ -461,7 +462,7 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
   const int we = min(end, ws + wlen);
   const int nt = ws < we ? (we - ws + XS_WTILE - 1) / XS_WTILE : 0;
   // warps with a slice; each publishes so many lane maxima that all together cover ke elements
-  const int active = WIDE ? max(min((end - start + wlen - 1) / wlen, EXP_WARPS), 0) : EXP_WARPS;
+  const int active = max(min((end - start + wlen - 1) / wlen, EXP_WARPS), 0);
   const int share_pos = (ke + active - 1) / max(active, 1) - 1;
   auto issue = [&](int t, unsigned slot_index) {
     const int base = ws + t * XS_WTILE;
@@ -473,120 +474,230 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
   };
   if (lane == 0)
     for (int t = 0; t < nt && t < XS_RING; ++t) issue(t, wt + t);
-  WarpStream w;
-  w.m_t = -CUDART_INF_F; w.s_t = 0.f;
-  w.thr_f = -CUDART_MAX_NORMAL_F;              // -inf never competes (probability zero)
-  w.thr_key = 0ull;
-  w.cnt = 0;
-  bool refreshed = false;
-  for (int t = 0; t < nt; ++t) {
-    const int base = ws + t * XS_WTILE;
-    const unsigned sl = wt % XS_RING;
-    if (!ring_wait(smem_addr(sh.bar + sl), (wt / XS_RING) & 1u)) {
-      // The copy did not land in time: the launch is reported as timed out (the tree arrays are
-      // undefined from here on) and the CTA leaves at the end of this chunk.  The copy gets one
-      // more bounded wait so that it does not land in memory the CTA has already given back.
-      if (lane == 0) { atomicOr(res.status, STATUS_TIMEOUT); *sh.abort_flag = 1; }
-      ring_wait(smem_addr(sh.bar + sl), (wt / XS_RING) & 1u);
-    }
-    float v[16];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const float4 x = *reinterpret_cast<const float4 *>(sh.ring + sl * XS_WTILE + u * 128 + lane * 4);
-      v[4 * u + 0] = x.x; v[4 * u + 1] = x.y; v[4 * u + 2] = x.z; v[4 * u + 3] = x.w;
-    }
-    if (base + XS_WTILE > we) {             // the slice's last, partial tile: nothing past `we` counts
-#pragma unroll
-      for (int i = 0; i < 16; ++i)
-        if (base + (i >> 2) * 128 + lane * 4 + (i & 3) >= we) v[i] = -CUDART_INF_F;
-    }
-    ++wt;
-    float bm = max3(max3(v[0], v[1], v[2]), max3(v[3], v[4], v[5]), max3(v[6], v[7], v[8]));
-    bm = max3(bm, max3(v[9], v[10], v[11]), max3(v[12], v[13], v[14]));
-    bm = fmaxf(bm, v[15]);
-    // running softmax normaliser of this lane's elements
-    if (bm > w.m_t) {
-      w.s_t *= fast_exp2((w.m_t - bm) * LOG2E_F);
-      w.m_t = bm;
-    }
-    if (w.m_t > -CUDART_INF_F) {
-      // exp(v - m) = 2^(v * log2e - m * log2e); an infinite m (a +inf logit) must give NaN
-      const float c = -w.m_t * LOG2E_F;
-      const u64 c2 = pack_f32x2(c, c), l2 = pack_f32x2(LOG2E_F, LOG2E_F);
-      u64 acc0 = 0ull, acc1 = 0ull;              // two pairs of +0.0f
-#pragma unroll
-      for (int i = 0; i < 16; i += 4) {
-        float x0, x1, x2, x3;
-        unpack_f32x2(fma_f32x2(pack_f32x2(v[i], v[i + 1]), l2, c2), x0, x1);
-        unpack_f32x2(fma_f32x2(pack_f32x2(v[i + 2], v[i + 3]), l2, c2), x2, x3);
-        acc0 = add_f32x2(acc0, pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
-        acc1 = add_f32x2(acc1, pack_f32x2(fast_exp2(x2), fast_exp2(x3)));
-      }
-      float s0, s1;
-      unpack_f32x2(add_f32x2(acc0, acc1), s0, s1);
-      w.s_t += s0 + s1;
-    }
-    refreshed = (t & (t + 1)) == 0 || t == 2;  // after tiles 1, 2, 3, 4, 8, 16, ... of the slice
-    // (the first tile has nothing but its own lane maxima to go by: their exact ke-th largest)
-    if (WIDE) {
-      if (refreshed) {
-        publish_maxima(w, share_pos, sh.wtop, sh.wmax, lane, warp);
-        if (t == 0) __syncthreads();           // before it there is no threshold at all
-        read_threshold(w, active, gated, ln_mu, sh.wtop, sh.wmax, lane);
-      }
-    } else if (refreshed) refresh_threshold(w, ke, share_pos, gated, ln_mu, sh.wtop, sh.wmax, lane, warp, t == 0);
-    if (__ballot_sync(FULL, bm >= w.thr_f) != 0u) {
-      collect_tile<WIDE>(sh.ring + sl * XS_WTILE, v, base, ke, sh.buf, w, lane);
-      __syncwarp();
-    }
-    // Every lane's loads from the slot have delivered their data (the vote needs every lane's
-    // maximum, and what the collection read has gone into the buffer): the slot can take the
-    // tile XS_RING ahead.
-    if (lane == 0 && t + XS_RING < nt) issue(t + XS_RING, wt - 1 + XS_RING);
-  }
-  if (WIDE) {
-    if (nt > 0) publish_maxima(w, share_pos, sh.wtop, sh.wmax, lane, warp);
-    else __syncthreads();                      // the others' barrier after their first tile
-    __syncthreads();
-    read_threshold(w, active, gated, ln_mu, sh.wtop, sh.wmax, lane);
-  } else if (nt > 4 && !refreshed) refresh_threshold(w, ke, share_pos, gated, ln_mu, sh.wtop, sh.wmax, lane, warp, false);
 
-  // ---- the warp's survivors -> the CTA pool; its normaliser -> shared memory ----
-  {
-    // a warp that could not build a threshold (a short slice) brings its ke best keys only, so
-    // that eight warps never overflow the pool
-    if (w.cnt > POOL / EXP_WARPS) cut_back<WIDE>(sh.buf, ke, w);
-    const int n = w.cnt;
-    for (int i = lane; i < n; i += 32) {
-      const u64 key = sh.buf[i];
-      if (key != 0ull && key_logit(key) >= w.thr_f) {
-        const int pos = atomicAdd(sh.pool_n, 1);
-        if (pos < POOL) sh.pool[pos] = key;
+  // ---- short slices: everything is in the ring at once ----
+  // No running maximum and no threshold that has to be raised from tile to tile (those steps, not the
+  // bytes, were most of a short chunk's time: 3.5 us of it at 8552 elements, 1.3 us this way): the lane
+  // maxima give one bound for the whole chunk, and what reaches it goes straight to the CTA pool.
+  bool resident = wlen <= XS_RING * XS_WTILE;              // (the same for all warps)
+  if (resident) {
+    auto element = [&](int t, int u, float (&x)[4]) {      // four elements of this lane; -inf past the slice
+      const unsigned sl = (wt + t) % XS_RING;
+      const float4 y = *reinterpret_cast<const float4 *>(sh.ring + sl * XS_WTILE + u * 128 + lane * 4);
+      x[0] = y.x; x[1] = y.y; x[2] = y.z; x[3] = y.w;
+      if (t == nt - 1) {
+        const int at = ws + t * XS_WTILE + u * 128 + lane * 4;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) if (at + e >= we) x[e] = -CUDART_INF_F;
+      }
+    };
+    float mt = -CUDART_INF_F, st = 0.f;
+#pragma unroll 1
+    for (int t = 0; t < nt; ++t) {
+      if (!ring_wait(smem_addr(sh.bar + (wt + t) % XS_RING), ((wt + t) / XS_RING) & 1u)) {
+        if (lane == 0) { atomicOr(res.status, STATUS_TIMEOUT); *sh.abort_flag = 1; }
+        ring_wait(smem_addr(sh.bar + (wt + t) % XS_RING), ((wt + t) / XS_RING) & 1u);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float x[4];
+        element(t, u, x);
+        mt = max3(max3(mt, x[0], x[1]), x[2], x[3]);
       }
     }
-    float wm = w.m_t;
+    // the warp's largest lane maximum and its (share_pos + 1)-th largest
+    float wmax;
+    {
+      unsigned o = f32_ord(mt), top = __reduce_max_sync(FULL, o);
+      wmax = f32_unord(top);
+      float mine = wmax;
+      if (share_pos < 4) {
+        for (int i = 0; i < share_pos; ++i) {
+          if (lane == __ffs(__ballot_sync(FULL, o == top)) - 1) o = 0u;
+          top = __reduce_max_sync(FULL, o);
+        }
+        mine = f32_unord(top);
+      } else {
+        mine = __shfl_sync(FULL, warp_sort_desc_f32(mt, lane), share_pos & 31);
+        if (share_pos > 31) mine = -CUDART_INF_F;
+      }
+      if (lane == 0) { sh.wtop[warp] = mine; sh.wmax[warp] = wmax; }
+    }
+    if (mt > -CUDART_INF_F) {
+      const float c = -mt * LOG2E_F;
+      const u64 c2 = pack_f32x2(c, c), l2 = pack_f32x2(LOG2E_F, LOG2E_F);
+#pragma unroll 1
+      for (int t = 0; t < nt; ++t) {
+        u64 acc0 = 0ull, acc1 = 0ull;                      // two pairs of +0.0f
 #pragma unroll
-    for (int o = 16; o; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(FULL, wm, o));
+        for (int u = 0; u < 4; ++u) {
+          float x[4], x0, x1, x2, x3;
+          element(t, u, x);
+          unpack_f32x2(fma_f32x2(pack_f32x2(x[0], x[1]), l2, c2), x0, x1);
+          unpack_f32x2(fma_f32x2(pack_f32x2(x[2], x[3]), l2, c2), x2, x3);
+          acc0 = add_f32x2(acc0, pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
+          acc1 = add_f32x2(acc1, pack_f32x2(fast_exp2(x2), fast_exp2(x3)));
+        }
+        float s0, s1;
+        unpack_f32x2(add_f32x2(acc0, acc1), s0, s1);
+        st += s0 + s1;
+      }
+    }
+    __syncthreads();
+    if (*sh.abort_flag) return false;
+    const float omin = f32_unord(__reduce_min_sync(FULL, lane < active ? f32_ord(sh.wtop[lane]) : 0xFFFFFFFFu));
+    const float omax = f32_unord(__reduce_max_sync(FULL, lane < active ? f32_ord(sh.wmax[lane]) : 0u));
+    float thr = -CUDART_MAX_NORMAL_F;                      // -inf never competes (probability zero)
+    if (active > 0) thr = fmaxf(thr, omin);
+    // (slack: fp32 rounding of the sum and of ln(mu), and the 1e-5 band around the gate)
+    if (gated && omax > -CUDART_INF_F) thr = fmaxf(thr, omax + ln_mu - (1e-4f + 1e-6f * fabsf(omax)));
+    if (mt >= thr) {
+#pragma unroll 1
+      for (int t = 0; t < nt; ++t)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          float x[4];
+          element(t, u, x);
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (x[e] >= thr) {
+              const int at = atomicAdd(sh.pool_n, 1);
+              if (at < POOL) sh.pool[at] = cand_key(x[e], (uint32_t)(ws + t * XS_WTILE + u * 128 + lane * 4 + e));
+            }
+        }
+    }
     // lane partial rescaled to the warp maximum; a NaN partial (NaN or +inf logit) propagates
-    float wsum = (w.m_t > -CUDART_INF_F || w.s_t != w.s_t) ? w.s_t * exp2f((w.m_t - wm) * LOG2E_F) : 0.f;
+    float wsum = (mt > -CUDART_INF_F || st != st) ? st * exp2f((mt - wmax) * LOG2E_F) : 0.f;
 #pragma unroll
     for (int o = 16; o; o >>= 1) wsum += __shfl_xor_sync(FULL, wsum, o);
-    if (lane == 0) { sh.m[warp] = wm; sh.s[warp] = wsum; }
+    if (lane == 0) { sh.m[warp] = wmax; sh.s[warp] = wsum; }
+    __syncthreads();
+    if (*sh.pool_n > POOL) {
+      // too many at the bound (equal logits, a sorted row): the general way over the tiles in the ring
+      __syncthreads();
+      if (tid == 0) *sh.pool_n = 0;
+      __syncthreads();
+      resident = false;
+    } else {
+      wt += (unsigned)nt;
+    }
   }
-  __syncthreads();
-  if (*sh.abort_flag) return false;
-  if (*sh.pool_n > POOL) {
-    // the pool cannot hold every survivor (equal logits): each warp brings its ke best only
+  if (!resident) {
+    WarpStream w;
+    w.m_t = -CUDART_INF_F; w.s_t = 0.f;
+    w.thr_f = -CUDART_MAX_NORMAL_F;              // -inf never competes (probability zero)
+    w.thr_key = 0ull;
+    w.cnt = 0;
+    bool refreshed = false;
+    for (int t = 0; t < nt; ++t) {
+      const int base = ws + t * XS_WTILE;
+      const unsigned sl = wt % XS_RING;
+      if (!ring_wait(smem_addr(sh.bar + sl), (wt / XS_RING) & 1u)) {
+        // The copy did not land in time: the launch is reported as timed out (the tree arrays are
+        // undefined from here on) and the CTA leaves at the end of this chunk.  The copy gets one
+        // more bounded wait so that it does not land in memory the CTA has already given back.
+        if (lane == 0) { atomicOr(res.status, STATUS_TIMEOUT); *sh.abort_flag = 1; }
+        ring_wait(smem_addr(sh.bar + sl), (wt / XS_RING) & 1u);
+      }
+      float v[16];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 x = *reinterpret_cast<const float4 *>(sh.ring + sl * XS_WTILE + u * 128 + lane * 4);
+        v[4 * u + 0] = x.x; v[4 * u + 1] = x.y; v[4 * u + 2] = x.z; v[4 * u + 3] = x.w;
+      }
+      if (base + XS_WTILE > we) {             // the slice's last, partial tile: nothing past `we` counts
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if (base + (i >> 2) * 128 + lane * 4 + (i & 3) >= we) v[i] = -CUDART_INF_F;
+      }
+      ++wt;
+      float bm = max3(max3(v[0], v[1], v[2]), max3(v[3], v[4], v[5]), max3(v[6], v[7], v[8]));
+      bm = max3(bm, max3(v[9], v[10], v[11]), max3(v[12], v[13], v[14]));
+      bm = fmaxf(bm, v[15]);
+      // running softmax normaliser of this lane's elements
+      if (bm > w.m_t) {
+        w.s_t *= fast_exp2((w.m_t - bm) * LOG2E_F);
+        w.m_t = bm;
+      }
+      if (w.m_t > -CUDART_INF_F) {
+        // exp(v - m) = 2^(v * log2e - m * log2e); an infinite m (a +inf logit) must give NaN
+        const float c = -w.m_t * LOG2E_F;
+        const u64 c2 = pack_f32x2(c, c), l2 = pack_f32x2(LOG2E_F, LOG2E_F);
+        u64 acc0 = 0ull, acc1 = 0ull;              // two pairs of +0.0f
+#pragma unroll
+        for (int i = 0; i < 16; i += 4) {
+          float x0, x1, x2, x3;
+          unpack_f32x2(fma_f32x2(pack_f32x2(v[i], v[i + 1]), l2, c2), x0, x1);
+          unpack_f32x2(fma_f32x2(pack_f32x2(v[i + 2], v[i + 3]), l2, c2), x2, x3);
+          acc0 = add_f32x2(acc0, pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
+          acc1 = add_f32x2(acc1, pack_f32x2(fast_exp2(x2), fast_exp2(x3)));
+        }
+        float s0, s1;
+        unpack_f32x2(add_f32x2(acc0, acc1), s0, s1);
+        w.s_t += s0 + s1;
+      }
+      refreshed = (t & (t + 1)) == 0 || t == 2;  // after tiles 1, 2, 3, 4, 8, 16, ... of the slice
+      // (the first tile has nothing but its own lane maxima to go by: their exact ke-th largest)
+      if (WIDE) {
+        if (refreshed) {
+          publish_maxima(w, share_pos, sh.wtop, sh.wmax, lane, warp);
+          if (t == 0) __syncthreads();           // before it there is no threshold at all
+          read_threshold(w, active, gated, ln_mu, sh.wtop, sh.wmax, lane);
+        }
+      } else if (refreshed) refresh_threshold(w, ke, share_pos, gated, ln_mu, sh.wtop, sh.wmax, lane, warp, t == 0);
+      if (__ballot_sync(FULL, bm >= w.thr_f) != 0u) {
+        collect_tile<WIDE>(sh.ring + sl * XS_WTILE, v, base, ke, sh.buf, w, lane);
+        __syncwarp();
+      }
+      // Every lane's loads from the slot have delivered their data (the vote needs every lane's
+      // maximum, and what the collection read has gone into the buffer): the slot can take the
+      // tile XS_RING ahead.
+      if (lane == 0 && t + XS_RING < nt) issue(t + XS_RING, wt - 1 + XS_RING);
+    }
+    if (WIDE) {
+      if (nt > 0) publish_maxima(w, share_pos, sh.wtop, sh.wmax, lane, warp);
+      else __syncthreads();                      // the others' barrier after their first tile
+      __syncthreads();
+      read_threshold(w, active, gated, ln_mu, sh.wtop, sh.wmax, lane);
+    } else if (nt > 4 && !refreshed) refresh_threshold(w, ke, share_pos, gated, ln_mu, sh.wtop, sh.wmax, lane, warp, false);
+
+    // ---- the warp's survivors -> the CTA pool; its normaliser -> shared memory ----
+    {
+      // a warp that could not build a threshold (a short slice) brings its ke best keys only, so
+      // that eight warps never overflow the pool
+      if (w.cnt > POOL / EXP_WARPS) cut_back<WIDE>(sh.buf, ke, w);
+      const int n = w.cnt;
+      for (int i = lane; i < n; i += 32) {
+        const u64 key = sh.buf[i];
+        if (key != 0ull && key_logit(key) >= w.thr_f) {
+          const int pos = atomicAdd(sh.pool_n, 1);
+          if (pos < POOL) sh.pool[pos] = key;
+        }
+      }
+      float wm = w.m_t;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(FULL, wm, o));
+      // lane partial rescaled to the warp maximum; a NaN partial (NaN or +inf logit) propagates
+      float wsum = (w.m_t > -CUDART_INF_F || w.s_t != w.s_t) ? w.s_t * exp2f((w.m_t - wm) * LOG2E_F) : 0.f;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) wsum += __shfl_xor_sync(FULL, wsum, o);
+      if (lane == 0) { sh.m[warp] = wm; sh.s[warp] = wsum; }
+    }
     __syncthreads();
-    if (tid == 0) *sh.pool_n = 0;
-    __syncthreads();
-    cut_back<WIDE>(sh.buf, ke, w);
-    const int n = w.cnt;
-    int pos = 0;
-    if (lane == 0) pos = atomicAdd(sh.pool_n, n);
-    pos = __shfl_sync(FULL, pos, 0);
-    for (int i = lane; i < n; i += 32) sh.pool[pos + i] = sh.buf[i];
-    __syncthreads();
+    if (*sh.abort_flag) return false;
+    if (*sh.pool_n > POOL) {
+      // the pool cannot hold every survivor (equal logits): each warp brings its ke best only
+      __syncthreads();
+      if (tid == 0) *sh.pool_n = 0;
+      __syncthreads();
+      cut_back<WIDE>(sh.buf, ke, w);
+      const int n = w.cnt;
+      int pos = 0;
+      if (lane == 0) pos = atomicAdd(sh.pool_n, n);
+      pos = __shfl_sync(FULL, pos, 0);
+      for (int i = lane; i < n; i += 32) sh.pool[pos + i] = sh.buf[i];
+      __syncthreads();
+    }
   }
 
   // ---- the chunk's ke best keys: four lanes count each candidate's betters (keys are unique) ----
@@ -628,11 +739,55 @@ __device__ __forceinline__ void chunk_clear(const ChunkShared &sh) {
 
 __host__ __device__ inline int stage_words(int k) { return FX_MAX_SPLITS * k + FX_SURV + k; }
 
-// One warp merges the S chunk results of a row, st: its stage_words(k) words of shared memory.
+// The largest value over the warp, in two reductions of half a key.
+__device__ __forceinline__ u64 warp_redux_max_u64(u64 v) {
+  const unsigned hi = __reduce_max_sync(FULL, (unsigned)(v >> 32));
+  const unsigned lo = __reduce_max_sync(FULL, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+  return ((u64)hi << 32) | lo;
+}
+
+// Two lists, each descending over groups of K lanes (a here, b already reversed): their K largest.
+template <int K>
+__device__ __forceinline__ u64 merge_groups(u64 a, u64 b_rev, int lane) {
+  u64 x = umax64(a, b_rev);                       // bitonic, and holds the K largest
+#pragma unroll
+  for (int j = K / 2; j > 0; j >>= 1) {
+    const u64 o = shfl_xor_u64(x, j);
+    x = ((lane & j) == 0) ? umax64(x, o) : umin64(x, o);
+  }
+  return x;
+}
+
+// The k <= K best of S descending lists of k keys, K = 8 or 16, in lanes 0 .. K-1 descending: 16 lists
+// lie K lanes each in K / 2 registers and are merged pairwise, first register with register, then
+// lane group with lane group.  A dozen dependent shuffles, no shared memory, no data-dependent loop
+// (collecting the survivors of a bound and ranking them took 2.5 us at 15 lists of 8, this 1 us).
+template <int K>
+__device__ __forceinline__ u64 merge_lists(const u64 *lists, int stride, int S, int k, int lane) {
+  constexpr int PER = 32 / K;                     // lists per register
+  constexpr int NR = FX_MAX_SPLITS / PER;
+  u64 r[NR];
+  const int sub = lane / K, pos = lane & (K - 1);
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    const int c = i * PER + sub;
+    r[i] = (c < S && pos < k) ? __ldcg(lists + (size_t)c * stride + pos) : 0ull;
+  }
+#pragma unroll
+  for (int n = NR / 2; n > 0; n >>= 1)
+#pragma unroll
+    for (int i = 0; i < n; ++i) r[i] = merge_groups<K>(r[i], shfl_xor_u64(r[i + n], K - 1), lane);
+#pragma unroll
+  for (int g = K; g < 32; g <<= 1) r[0] = merge_groups<K>(r[0], shfl_xor_u64(r[0], g | (K - 1)), lane);
+  return r[0];
+}
+
+// One warp merges the S chunk results of a row, st: its stage_words(k) words of shared memory (KMAX 32).
 // Afterwards lane i < k holds the row's i-th best key and the score ps + (z - lse), with ps the
 // log-probability of the row's node (Eq. 2-3; -inf for an empty slot or one past the ke children the
 // budget still allows).  Returns false, for the whole warp, when the row's normaliser is not a
 // positive finite number (a NaN or +inf logit, a row of -inf only).
+template <int KMAX>
 __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int S, int k, int ke, double ps, u64 *st,
                                           u64 &out_key, double &out_score) {
   const int lane = threadIdx.x & 31;
@@ -643,7 +798,10 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
   // load cannot pass a store through a pointer the compiler cannot tell apart): one trip to L2
   // for the row, not one per load.
   const float2 ms = (lane < S) ? __ldcg(res.part_ms + item0 + lane) : make_float2(-CUDART_INF_F, 0.f);
-  if (S == 1) {
+  u64 own = 0ull;                                // KMAX 8 and 16: this lane's key of the merged list
+  if (KMAX <= 16) {
+    own = merge_lists<KMAX <= 16 ? KMAX : 16>(res.part_keys + item0 * ks, ks, S, k, lane);
+  } else if (S == 1) {
     const u64 key = lane < k ? __ldcg(res.part_keys + item0 * ks + lane) : 0ull;
     if (lane < k) rk[lane] = key;
   } else {
@@ -674,7 +832,7 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
   t = __shfl_sync(FULL, t, 0);
   const bool finite = (t > 0.0) && (t < CUDART_INF) && (mx < CUDART_INF_F) && (mx > -CUDART_INF_F);
 
-  if (S > 1) {
+  if (KMAX > 16 && S > 1) {
     if (lane < k) rk[lane] = 0ull;
     __syncwarp();
     // Two lower bounds of the row's ke-th best key (chunk lists hold ke keys at most): the best
@@ -723,7 +881,7 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
     }
   }
   __syncwarp();
-  out_key = lane < k ? rk[lane] : 0ull;
+  out_key = lane < k ? (KMAX <= 16 ? own : rk[lane]) : 0ull;
   out_score = -CUDART_INF;
   if (finite && lane < ke && out_key != 0ull) {
     const double s = ps + ((double)key_logit(out_key) - ((double)mx + log(t)));
@@ -803,6 +961,139 @@ __device__ __forceinline__ void merge_row_wide(const ChunkOut &res, size_t item0
     score_out[r] = (r == 0 && lse != lse) ? CUDART_NAN : -CUDART_INF;
   }
   if (tid == 0 && lse != lse) atomicOr(status, STATUS_NONFINITE);
+}
+
+// ---------------------------------------------------------------------------------------
+// Selection of one layer (Eq. 4, Eq. 5, truncation to the budget)
+// ---------------------------------------------------------------------------------------
+// Called by all THREADS threads of a CTA.  A frontier of F rows (32 NQ at most), row j's candidates
+// sorted by score: score(j, i) for i < k (-inf: none), tok(j, i) its token.  At most `want` candidates
+// are taken, the best ones, after the gate p(u) >= mu * max p when not `init`; append(slot, j, i, tok,
+// score) is called for each, slot counting them in storage order (parent asc, token asc).  Returns how
+// many; s_cnt: MAX_BUDGET ints of shared memory.  The caller puts a barrier behind it.
+//
+// The chain (best candidate, gate, how many candidates of each row pass, where each row's survivors go,
+// append) is short and serial, so what counts is latency: every warp computes it up to the offsets for
+// itself, a lane per row, without a barrier; only the append is shared out over the warps.  Rows are
+// sorted, so the candidates of a row that pass are a prefix.
+template <int NQ, int KMAX, int THREADS, class Score, class Tok, class Append>
+__device__ __forceinline__ int layer_select(int F, int k, int ke, int want, bool init, double log_mu, int *s_cnt, Score score,
+                                            Tok tok, Append append) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int G = KMAX;                               // lanes of one row in the append
+  const int gl = lane & (G - 1), gbase = lane & ~(G - 1);
+  const unsigned gmask = (G == 32 ? FULL : ((1u << (G & 31)) - 1u)) << gbase;
+  constexpr int per_pass = THREADS / G;
+  constexpr int PASSES = 32 * NQ / per_pass > 0 ? 32 * NQ / per_pass : 1;
+  const int my_row = tid / G;
+
+  double thr = -1.7976931348623157e308;                 // an impossible candidate (-inf) never passes
+  if (!init) {
+    u64 head = 0ull;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int j = q * 32 + lane;
+      if (j < F) {
+        const double s = score(j, 0);
+        if (s > -CUDART_INF) head = umax64(head, f64_ord(s));
+      }
+    }
+    head = warp_redux_max_u64(head);
+    if (head != 0ull) thr = log_mu + f64_unord(head);
+  }
+  // ---- eligible candidates of each row, and the rows' output offsets ----
+  int cnt[NQ], off[NQ], total = 0;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    cnt[q] = 0;
+    if (q * 32 < F) {
+      const int r = min(q * 32 + lane, F - 1);
+      double s[KMAX];                                   // (unconditional, so that the trips overlap)
+#pragma unroll
+      for (int i = 0; i < KMAX; ++i) s[i] = score(r, min(i, k - 1));
+#pragma unroll
+      for (int i = 0; i < KMAX; ++i) cnt[q] += (i < ke && s[i] >= thr) ? 1 : 0;
+      if (q * 32 + lane >= F) cnt[q] = 0;
+    }
+  }
+  auto scan = [&]() {
+    total = 0;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      off[q] = total;
+      if (q * 32 >= F) continue;
+      int inc = cnt[q];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += t;
+      }
+      off[q] = total + inc - cnt[q];
+      total += __shfl_sync(FULL, inc, 31);
+    }
+  };
+  scan();
+  // row j's value of a per-lane-row array (j / 32 is the same for the whole warp)
+  auto of_row = [&](const int (&v)[NQ], int j) {
+    int x = v[0];
+#pragma unroll
+    for (int q = 1; q < NQ; ++q) if ((j >> 5) == q) x = v[q];
+    return __shfl_sync(FULL, x, j & 31);
+  };
+  if (total > want) {
+    // ---- truncation: rank by (score desc, parent asc, token asc) among the eligible; rows are sorted
+    // that way already, so a rank is a sum of binary searches in the rows' prefixes ----
+    if (warp == 0)
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) if (q * 32 + lane < F) s_cnt[q * 32 + lane] = cnt[q];
+    __syncthreads();
+    int kept[PASSES];                                   // of this group's row, per pass
+#pragma unroll
+    for (int np = 0; np < PASSES; ++np) {
+      const int j = np * per_pass + my_row;
+      kept[np] = 0;
+      if (np * per_pass >= F) continue;
+      bool sel = false;
+      if (j < F && gl < s_cnt[j]) {
+        const double s = score(j, gl);
+        int rank = gl;
+        for (int o = 0; o < F && rank < want; ++o) {
+          int l = 0, h = o == j ? 0 : s_cnt[o];
+          while (l < h) {
+            const int mid = (l + h) >> 1;
+            const double v = score(o, mid);
+            if (v > s || (v == s && o < j)) l = mid + 1; else h = mid;
+          }
+          rank += l;
+        }
+        sel = rank < want;
+      }
+      kept[np] = __popc(__ballot_sync(FULL, sel) & gmask);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int np = 0; np < PASSES; ++np) {
+      const int j = np * per_pass + my_row;
+      if (j < F && gl == 0) s_cnt[j] = kept[np];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) cnt[q] = q * 32 + lane < F ? s_cnt[q * 32 + lane] : 0;
+    scan();
+  }
+  // ---- append ----
+  for (int j0 = 0; j0 < F; j0 += per_pass) {
+    const int j = j0 + my_row;
+    const int c0 = of_row(cnt, j), o0 = of_row(off, j);
+    const int c = j < F ? c0 : 0;
+    if (!__any_sync(FULL, c > 0)) continue;
+    const int t = (gl < c) ? tok(j, gl) : 0x7FFFFFFF;
+    int r = 0;
+#pragma unroll
+    for (int i = 0; i < KMAX; ++i) r += __shfl_sync(FULL, t, gbase + i) < t ? 1 : 0;      // unused lanes hold the largest
+    if (gl < c) append(o0 + r, j, gl, t, score(j, gl));
+  }
+  return total;
 }
 
 }  // namespace

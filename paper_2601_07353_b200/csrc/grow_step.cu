@@ -149,6 +149,7 @@ __device__ __forceinline__ void argmax_chunk(const float *rowp, int start, int e
   __syncthreads();
 }
 
+template <int KMAX>          // k rounded up to 8, 16 or 32
 __global__ void __launch_bounds__(EXP_THREADS, 3)
 row_pass_kernel(RowPassArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -242,7 +243,7 @@ row_pass_kernel(RowPassArgs a) {
       u64 key; double lp;
       int item0, S;
       row_chunks(g, row, item0, S);
-      const bool finite = merge_row(res, (size_t)item0, S, k, k, 0.0, stage, key, lp);
+      const bool finite = merge_row<KMAX>(res, (size_t)item0, S, k, k, 0.0, stage, key, lp);
       if (!finite) lp = lane == 0 ? CUDART_NAN : -CUDART_INF;
       if (lane < k) {
         a.row_keys[slot * a.key_stride + lane] = key;
@@ -290,18 +291,7 @@ __host__ __device__ inline size_t grow_smem_bytes(int rows, int k, int N) {
   return (size_t)grow_pitch(rows) * k * 16 + (size_t)N * (8 + 16 + 12) + MAX_BUDGET * 4 + 32;
 }
 
-// The largest value over the warp, in two reductions of half a key.
-__device__ __forceinline__ u64 warp_redux_max_u64(u64 v) {
-  const unsigned hi = __reduce_max_sync(FULL, (unsigned)(v >> 32));
-  const unsigned lo = __reduce_max_sync(FULL, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
-  return ((u64)hi << 32) | lo;
-}
-
-// One CTA per sequence.  A layer is a short serial chain (best candidate of the frontier, the gate,
-// how many candidates of each row pass, where each row's survivors go, append), so what counts is
-// latency: every warp computes the chain up to the offsets for itself, a lane per frontier row, without
-// a barrier; only the append is shared out over the warps, and one barrier ends the layer.  Row lists
-// are sorted, so the candidates of a row that pass are a prefix of its list.
+// One CTA per sequence, a layer per turn of the loop (layer_select), one barrier each.
 template <int NQ, int KMAX>  // frontier rows per lane; k rounded up to 8, 16 or 32
 __global__ void __launch_bounds__(GROW_THREADS)
 grow_kernel(GrowArgs a) {
@@ -373,33 +363,19 @@ grow_kernel(GrowArgs a) {
   }
   __syncthreads();
 
-  constexpr int G = KMAX;                               // lanes of one row in the append
-  const int gl = lane & (G - 1), gbase = lane & ~(G - 1);
-  const unsigned gmask = (G == 32 ? FULL : ((1u << (G & 31)) - 1u)) << gbase;
-  constexpr int per_pass = GROW_THREADS / G;
-  const int my_row = tid / G;
   bool paused = false;
   for (; d < a.n_layers; ++d) {
     const int F = hi - lo, n = hi;
     if (F <= 0 || n >= N) break;
     if (hi > a.rows) { paused = true; break; }          // the frontier's rows are not all there yet
     const int R = N - n, ke = min(k, R);                // a parent can place at most R children
-    // ---- the frontier's best candidate; rows without a softmax ----
-    double ps[NQ];                                      // log p of this lane's rows q * 32 + lane
-    u64 head = 0ull;
-    bool bad = false;
+    bool bad = false;                                   // rows without a softmax
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      const int j = q * 32 + lane;
-      ps[q] = -CUDART_INF;
-      if (j < F) {
-        ps[q] = sm.score[lo + j];
-        const double lp = sm.lp[lo + j];
+    for (int q = 0; q < NQ; ++q)
+      if (q * 32 + lane < F) {
+        const double lp = sm.lp[lo + q * 32 + lane];
         bad |= lp != lp;
-        const double s = ps[q] + lp;
-        if (s > -CUDART_INF) head = umax64(head, f64_ord(s));
       }
-    }
     if (__any_sync(FULL, bad)) {                        // this sequence adds nothing any more
       if (tid == 0) {
         atomicOr(a.status, STATUS_NONFINITE);
@@ -409,117 +385,19 @@ grow_kernel(GrowArgs a) {
       break;
     }
     const bool init = d < a.init_layers;
-    double thr = -1.7976931348623157e308;                    // an impossible candidate (-inf) never passes
-    if (!init) {
-      head = warp_redux_max_u64(head);
-      if (head != 0ull) thr = a.log_mu + f64_unord(head);
-    }
-    // ---- eligible candidates of each row, and the rows' output offsets ----
-    int cnt[NQ], off[NQ], total = 0;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      cnt[q] = 0;
-      if (q * 32 < F) {
-        const int r = lo + min(q * 32 + lane, F - 1);
-        double s[KMAX];                                 // (unconditional, so that the trips overlap)
-#pragma unroll
-        for (int i = 0; i < KMAX; ++i) s[i] = ps[q] + sm.lp[min(i, k - 1) * pitch + r];
-#pragma unroll
-        for (int i = 0; i < KMAX; ++i) cnt[q] += (i < ke && s[i] >= thr) ? 1 : 0;
-      }
-    }
-    auto scan = [&]() {
-      total = 0;
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        off[q] = total;
-        if (q * 32 >= F) continue;
-        int inc = cnt[q];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int t = __shfl_up_sync(FULL, inc, o);
-          if (lane >= o) inc += t;
-        }
-        off[q] = total + inc - cnt[q];
-        total += __shfl_sync(FULL, inc, 31);
-      }
-    };
-    scan();
-    // row j's value of a per-lane-row array (j / 32 is the same for the whole warp)
-    auto of_row = [&](const int (&v)[NQ], int j) {
-      int x = v[0];
-#pragma unroll
-      for (int q = 1; q < NQ; ++q) if ((j >> 5) == q) x = v[q];
-      return __shfl_sync(FULL, x, j & 31);
-    };
-    const int want = init ? min(a.root_topk, R) : R;
-    if (total > want) {
-      // ---- budget truncation: rank by (score desc, parent asc, token asc) among the eligible; rows
-      // are sorted that way already, so a rank is a sum of binary searches in the rows' prefixes ----
-      if (warp == 0)
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) if (q * 32 + lane < F) sm.cnt[q * 32 + lane] = cnt[q];
-      __syncthreads();
-      int kept[16];                                     // of this group's row, per pass (at most 32 lanes a row, 128 rows)
-#pragma unroll
-      for (int np = 0; np < 16; ++np) {
-        const int j = np * per_pass + my_row;
-        if (np * per_pass >= F) break;
-        bool sel = false;
-        if (j < F && gl < sm.cnt[j]) {
-          const double s = sm.score[lo + j] + sm.lp[gl * pitch + lo + j];
-          int rank = gl;
-          for (int o = 0; o < F && rank < want; ++o) {
-            int h = sm.cnt[o];
-            if (o == j || h == 0) continue;
-            const double po = sm.score[lo + o];
-            const bool before = o < j;
-            int l = 0;
-            while (l < h) {
-              const int mid = (l + h) >> 1;
-              const double v = po + sm.lp[mid * pitch + lo + o];
-              if (v > s || (v == s && before)) l = mid + 1; else h = mid;
-            }
-            rank += l;
-          }
-          sel = rank < want;
-        }
-        kept[np] = __popc(__ballot_sync(FULL, sel) & gmask);
-      }
-      __syncthreads();
-#pragma unroll
-      for (int np = 0; np < 16; ++np) {
-        const int j = np * per_pass + my_row;
-        if (np * per_pass >= F) break;
-        if (j < F && gl == 0) sm.cnt[j] = kept[np];
-      }
-      __syncthreads();
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) cnt[q] = q * 32 + lane < F ? sm.cnt[q * 32 + lane] : 0;
-      scan();
-    }
-
-    // ---- append in storage order: (parent asc, token asc) ----
-    for (int j0 = 0; j0 < F; j0 += per_pass) {
-      const int j = j0 + my_row;
-      const int c0 = of_row(cnt, j), o0 = of_row(off, j);
-      const int c = j < F ? c0 : 0;
-      if (!__any_sync(FULL, c > 0)) continue;
-      const int par = lo + min(j, F - 1);
-      const int tok = (gl < c) ? (int)key_tok(sm.key[gl * pitch + par]) : 0x7FFFFFFF;
-      int r = 0;
-#pragma unroll
-      for (int i = 0; i < KMAX; ++i) r += __shfl_sync(FULL, tok, gbase + i) < tok ? 1 : 0;      // unused lanes hold the largest
-      if (gl < c) {
-        const int node = n + o0 + r;
-        sm.tok[node] = tok;
-        sm.parent[node] = par;
-        sm.depth[node] = d + 1;
-        sm.score[node] = sm.score[par] + sm.lp[gl * pitch + par];
-        sm.mask[2 * node] = sm.mask[2 * par] | (node < 64 ? 1ull << node : 0ull);
-        sm.mask[2 * node + 1] = sm.mask[2 * par + 1] | (node >= 64 ? 1ull << (node - 64) : 0ull);
-      }
-    }
+    const int total = layer_select<NQ, KMAX, GROW_THREADS>(
+        F, k, ke, init ? min(a.root_topk, R) : R, init, a.log_mu, sm.cnt,
+        [&](int j, int i) { return sm.score[lo + j] + sm.lp[i * pitch + lo + j]; },
+        [&](int j, int i) { return (int)key_tok(sm.key[i * pitch + lo + j]); },
+        [&](int slot, int j, int i, int tok, double score) {
+          const int node = n + slot, par = lo + j;
+          sm.tok[node] = tok;
+          sm.parent[node] = par;
+          sm.depth[node] = d + 1;
+          sm.score[node] = score;
+          sm.mask[2 * node] = sm.mask[2 * par] | (node < 64 ? 1ull << node : 0ull);
+          sm.mask[2 * node + 1] = sm.mask[2 * par + 1] | (node >= 64 ? 1ull << (node - 64) : 0ull);
+        });
     lo = hi;
     hi = n + total;
     if (tid == 0) a.t.layer_off[b * a.lo_stride + d + 2] = hi;
@@ -593,13 +471,17 @@ static void (*grow_kernel_for(const talon_ctx *c))(GrowArgs) {
   return rows <= 32 ? grow_kernel_k<1>(c->k_cap) : (rows <= 64 ? grow_kernel_k<2>(c->k_cap) : grow_kernel_k<4>(c->k_cap));
 }
 
+static void (*row_pass_for(const talon_ctx *c))(RowPassArgs) {
+  return c->k_cap <= 8 ? row_pass_kernel<8> : (c->k_cap <= 16 ? row_pass_kernel<16> : row_pass_kernel<32>);
+}
+
 talon_status grow_step_setup(talon_ctx *c) {
-  if (cudaFuncSetAttribute(row_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_pass_smem(c, true)) != cudaSuccess ||
+  if (cudaFuncSetAttribute(row_pass_for(c), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_pass_smem(c, true)) != cudaSuccess ||
       cudaFuncSetAttribute(grow_kernel_for(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)grow_smem_bytes(c->p.budget, c->k_cap, c->p.budget)) != cudaSuccess)
     return TALON_ERR_CUDA;
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, row_pass_kernel, EXP_THREADS, row_pass_smem(c, false)) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, row_pass_for(c), EXP_THREADS, row_pass_smem(c, false)) != cudaSuccess ||
       per_sm < 1)
     return TALON_ERR_CUDA;
   if (per_sm > EXP_CTAS_PER_SM) per_sm = EXP_CTAS_PER_SM;
@@ -698,7 +580,7 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
     if (grid < 1) grid = 1;
     {
       LaunchTimer lt(c, TALON_K_EXPAND_ROWS, st);
-      launch_kernel(c, row_pass_kernel, dim3(grid), dim3(EXP_THREADS), row_pass_smem(c, r > 0 && B > 32), st, ra);
+      launch_kernel(c, row_pass_for(c), dim3(grid), dim3(EXP_THREADS), row_pass_smem(c, r > 0 && B > 32), st, ra);
     }
     if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
     ga.first = r == 0; ga.rows = upto;
