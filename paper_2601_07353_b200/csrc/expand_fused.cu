@@ -29,6 +29,7 @@ struct FusedArgs {
   int B, N, W, V, d, k, key_stride, max_split, base_offset, pool_cap;
   int root_topk, init_layers;
   double log_mu;
+  SpanTable spans;
   u64 *part_keys;          // [items, key_stride]  per-chunk top-k, descending
   float2 *part_ms;         // [items]              per-chunk (max, sum of exp)
   u64 *row_keys;           // [rows, key_stride]   per-row top-k (wide frontiers)
@@ -302,7 +303,7 @@ expand_fused_kernel(FusedArgs a) {
         if (s_base[b + 1] == s_base[b])
           a.t.layer_off[b * a.lo_stride + a.d + 2] = a.t.layer_off[b * a.lo_stride + a.d + 1];
   }
-  const SpanGeom g = span_geom(fr.total, a.V, (int)gridDim.x, a.max_split);
+  const SpanGeom g = span_geom(fr.total, a.V, (int)gridDim.x, a.max_split, a.spans);
   const unsigned long long line_end = (unsigned long long)fr.total * g.pitch;
   const bool gated = a.d >= a.init_layers;
   const float ln_mu = (float)a.log_mu;
@@ -314,7 +315,7 @@ expand_fused_kernel(FusedArgs a) {
 
   unsigned long long pos = (unsigned long long)blockIdx.x * g.span;
   const unsigned long long span_end = min(line_end, pos + g.span);
-  int row = pos < span_end ? (int)div_u64(pos, g.pitch) : 0;
+  int row = pos < span_end ? (g.per_row ? (int)div_small(blockIdx.x, g.per_row) : (int)div_u64(pos, g.pitch)) : 0;
   int start = pos < span_end ? (int)(pos - (unsigned long long)row * g.pitch) : 0;
   for (; pos < span_end; ++row, start = 0) {
     // ---- one chunk: elements [start, start + len) of packed row `row` ----
@@ -555,6 +556,7 @@ talon_status launch_expand_fused(talon_ctx *c, const talon_tree *t, const float 
   a.key_stride = c->key_stride;
   a.max_split = c->expand_max_split;
   a.pool_cap = pool_capacity(c);
+  a.spans = span_table(c->p.vocab);
   long long max_items = (long long)rows_bound * FX_MAX_SPLITS;
   int grid = c->fused_grid;
   if (max_items < grid) grid = (int)max_items;

@@ -199,13 +199,32 @@ __device__ inline unsigned div_u64(unsigned long long a, unsigned b) {
   return a <= 0xFFFFFFFFull ? (unsigned)a / b : (unsigned)(a / b);
 }
 
-__device__ inline SpanGeom span_geom(int total_rows, int vocab, int grid, int max_split) {
+// (An integer division is a chain of some 60 clocks on the way to the first byte: the spans of whole-row
+// fractions come from the host, and small quotients by way of a float, exact for operands below 2^16.)
+struct SpanTable { unsigned of[FX_MAX_SPLITS]; };      // [S]: elements of a chunk when a row is cut into S
+inline SpanTable span_table(int vocab) {
+  SpanTable t = {};
+  const unsigned vp = ((unsigned)vocab + 3u) & ~3u;
+  for (unsigned S = 1; S < FX_MAX_SPLITS; ++S) t.of[S] = ((vp + S - 1u) / S + 3u) & ~3u;
+  return t;
+}
+__device__ inline unsigned div_small(unsigned a, unsigned b) { return (unsigned)__fdividef((float)a + 0.5f, (float)b); }
+
+// ceil(a / b) for quotients up to 16 of larger numbers
+__device__ inline int div_up_small(int a, int b) {
+  int q = 0;
+#pragma unroll
+  for (int i = 0; i < EXP_WARPS; ++i) q += a > i * b ? 1 : 0;
+  return q;
+}
+
+__device__ inline SpanGeom span_geom(int total_rows, int vocab, int grid, int max_split, const SpanTable &table) {
   SpanGeom g;
   const unsigned vp = ((unsigned)vocab + 3u) & ~3u;
-  const unsigned per_row = total_rows > 0 ? (unsigned)grid / (unsigned)total_rows : 1u;
+  const unsigned per_row = total_rows > 0 ? (total_rows < grid ? div_small((unsigned)grid, (unsigned)total_rows) : (total_rows == grid ? 1u : 0u)) : 1u;
   if (per_row >= 2u) {
     const unsigned S = max(1u, min(min(per_row, (unsigned)max_split), vp / 4096u));
-    g.span = ((vp + S - 1u) / S + 3u) & ~3u;
+    g.span = table.of[S];
     g.pitch = S * g.span;
     g.per_row = S;
   } else {
@@ -461,9 +480,6 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
   const int ws = start + warp * wlen;
   const int we = min(end, ws + wlen);
   const int nt = ws < we ? (we - ws + XS_WTILE - 1) / XS_WTILE : 0;
-  // warps with a slice; each publishes so many lane maxima that all together cover ke elements
-  const int active = max(min((end - start + wlen - 1) / wlen, EXP_WARPS), 0);
-  const int share_pos = (ke + active - 1) / max(active, 1) - 1;
   auto issue = [&](int t, unsigned slot_index) {
     const int base = ws + t * XS_WTILE;
     const int n = min(XS_WTILE, we - base);
@@ -474,6 +490,9 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
   };
   if (lane == 0)
     for (int t = 0; t < nt && t < XS_RING; ++t) issue(t, wt + t);
+  // warps with a slice; each publishes so many lane maxima that all together cover ke elements
+  const int active = max(0, min((int)div_up_small(end - start, wlen), EXP_WARPS));
+  const int share_pos = (int)div_small((unsigned)(ke + active - 1), (unsigned)max(active, 1)) - 1;
 
   // ---- short slices: everything is in the ring at once ----
   // No running maximum and no threshold that has to be raised from tile to tile (those steps, not the
@@ -481,28 +500,49 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
   // maxima give one bound for the whole chunk, and what reaches it goes straight to the CTA pool.
   bool resident = wlen <= XS_RING * XS_WTILE;              // (the same for all warps)
   if (resident) {
-    auto element = [&](int t, int u, float (&x)[4]) {      // four elements of this lane; -inf past the slice
-      const unsigned sl = (wt + t) % XS_RING;
-      const float4 y = *reinterpret_cast<const float4 *>(sh.ring + sl * XS_WTILE + u * 128 + lane * 4);
-      x[0] = y.x; x[1] = y.y; x[2] = y.z; x[3] = y.w;
-      if (t == nt - 1) {
-        const int at = ws + t * XS_WTILE + u * 128 + lane * 4;
+    auto tile = [&](int t) { return sh.ring + ((wt + t) % XS_RING) * XS_WTILE; };
+    float mt = -CUDART_INF_F, st = 0.f, bm[XS_RING];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) if (at + e >= we) x[e] = -CUDART_INF_F;
-      }
-    };
-    float mt = -CUDART_INF_F, st = 0.f;
-#pragma unroll 1
-    for (int t = 0; t < nt; ++t) {
+    for (int t = 0; t < XS_RING; ++t) {
+      bm[t] = -CUDART_INF_F;
+      if (t >= nt) continue;
       if (!ring_wait(smem_addr(sh.bar + (wt + t) % XS_RING), ((wt + t) / XS_RING) & 1u)) {
         if (lane == 0) { atomicOr(res.status, STATUS_TIMEOUT); *sh.abort_flag = 1; }
         ring_wait(smem_addr(sh.bar + (wt + t) % XS_RING), ((wt + t) / XS_RING) & 1u);
       }
+      float *slot = tile(t);
+      if (t == nt - 1) {                                   // what the last copy left untouched must not count
+        for (int e = we - ws - t * XS_WTILE + lane; e < XS_WTILE; e += 32) slot[e] = -CUDART_INF_F;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+      }
+      float v[16];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        float x[4];
-        element(t, u, x);
-        mt = max3(max3(mt, x[0], x[1]), x[2], x[3]);
+        const float4 y = *reinterpret_cast<const float4 *>(slot + u * 128 + lane * 4);
+        v[4 * u] = y.x; v[4 * u + 1] = y.y; v[4 * u + 2] = y.z; v[4 * u + 3] = y.w;
+      }
+      float m = max3(max3(v[0], v[1], v[2]), max3(v[3], v[4], v[5]), max3(v[6], v[7], v[8]));
+      bm[t] = fmaxf(max3(m, max3(v[9], v[10], v[11]), max3(v[12], v[13], v[14])), v[15]);
+      if (bm[t] > mt) {
+        st *= fast_exp2((mt - bm[t]) * LOG2E_F);
+        mt = bm[t];
+      }
+      if (mt > -CUDART_INF_F) {
+        const float c = -mt * LOG2E_F;
+        const u64 c2 = pack_f32x2(c, c), l2 = pack_f32x2(LOG2E_F, LOG2E_F);
+        u64 acc0 = 0ull, acc1 = 0ull;                      // two pairs of +0.0f
+#pragma unroll
+        for (int i = 0; i < 16; i += 4) {
+          float x0, x1, x2, x3;
+          unpack_f32x2(fma_f32x2(pack_f32x2(v[i], v[i + 1]), l2, c2), x0, x1);
+          unpack_f32x2(fma_f32x2(pack_f32x2(v[i + 2], v[i + 3]), l2, c2), x2, x3);
+          acc0 = add_f32x2(acc0, pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
+          acc1 = add_f32x2(acc1, pack_f32x2(fast_exp2(x2), fast_exp2(x3)));
+        }
+        float s0, s1;
+        unpack_f32x2(add_f32x2(acc0, acc1), s0, s1);
+        st += s0 + s1;
       }
     }
     // the warp's largest lane maximum and its (share_pos + 1)-th largest
@@ -523,26 +563,6 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
       }
       if (lane == 0) { sh.wtop[warp] = mine; sh.wmax[warp] = wmax; }
     }
-    if (mt > -CUDART_INF_F) {
-      const float c = -mt * LOG2E_F;
-      const u64 c2 = pack_f32x2(c, c), l2 = pack_f32x2(LOG2E_F, LOG2E_F);
-#pragma unroll 1
-      for (int t = 0; t < nt; ++t) {
-        u64 acc0 = 0ull, acc1 = 0ull;                      // two pairs of +0.0f
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          float x[4], x0, x1, x2, x3;
-          element(t, u, x);
-          unpack_f32x2(fma_f32x2(pack_f32x2(x[0], x[1]), l2, c2), x0, x1);
-          unpack_f32x2(fma_f32x2(pack_f32x2(x[2], x[3]), l2, c2), x2, x3);
-          acc0 = add_f32x2(acc0, pack_f32x2(fast_exp2(x0), fast_exp2(x1)));
-          acc1 = add_f32x2(acc1, pack_f32x2(fast_exp2(x2), fast_exp2(x3)));
-        }
-        float s0, s1;
-        unpack_f32x2(add_f32x2(acc0, acc1), s0, s1);
-        st += s0 + s1;
-      }
-    }
     __syncthreads();
     if (*sh.abort_flag) return false;
     const float omin = f32_unord(__reduce_min_sync(FULL, lane < active ? f32_ord(sh.wtop[lane]) : 0xFFFFFFFFu));
@@ -551,20 +571,27 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
     if (active > 0) thr = fmaxf(thr, omin);
     // (slack: fp32 rounding of the sum and of ln(mu), and the 1e-5 band around the gate)
     if (gated && omax > -CUDART_INF_F) thr = fmaxf(thr, omax + ln_mu - (1e-4f + 1e-6f * fabsf(omax)));
-    if (mt >= thr) {
-#pragma unroll 1
-      for (int t = 0; t < nt; ++t)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          float x[4];
-          element(t, u, x);
+    for (int t = 0; t < XS_RING; ++t) {
+      if (!__any_sync(FULL, bm[t] >= thr)) continue;       // (bm is -inf past the slice)
+      const float *slot = tile(t);
+      unsigned mm = 0u;
 #pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (x[e] >= thr) {
-              const int at = atomicAdd(sh.pool_n, 1);
-              if (at < POOL) sh.pool[at] = cand_key(x[e], (uint32_t)(ws + t * XS_WTILE + u * 128 + lane * 4 + e));
-            }
-        }
+      for (int u = 0; u < 4; ++u) {
+        const float4 y = *reinterpret_cast<const float4 *>(slot + u * 128 + lane * 4);
+        mm |= (y.x >= thr ? 1u << (4 * u) : 0u) | (y.y >= thr ? 2u << (4 * u) : 0u) | (y.z >= thr ? 4u << (4 * u) : 0u) |
+              (y.w >= thr ? 8u << (4 * u) : 0u);
+      }
+      if (mm) {
+        int at = atomicAdd(sh.pool_n, __popc(mm));
+        do {
+          const int i = __ffs(mm) - 1, e = (i >> 2) * 128 + lane * 4 + (i & 3);
+          if (at < POOL) sh.pool[at] = cand_key(slot[e], (uint32_t)(ws + t * XS_WTILE + e));
+          ++at;
+          mm &= mm - 1u;
+        } while (mm);
+      }
+      __syncwarp();
     }
     // lane partial rescaled to the warp maximum; a NaN partial (NaN or +inf logit) propagates
     float wsum = (mt > -CUDART_INF_F || st != st) ? st * exp2f((mt - wmax) * LOG2E_F) : 0.f;

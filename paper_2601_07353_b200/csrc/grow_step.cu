@@ -33,6 +33,7 @@ struct RowPassArgs {
   int draft_ctas;                     // CTAs 0 .. draft_ctas-1 take draft rows, the others target rows
   int init_layers;
   double log_mu;
+  SpanTable spans;
   const int32_t *growing;             // [B] nonzero: this sequence still needs rows; null: all do
   u64 *part_keys; float2 *part_ms;
   u64 *row_keys; double *row_lp;      // [B * N, key_stride]; row_lp slot 0 NaN: row without a softmax
@@ -198,14 +199,14 @@ row_pass_kernel(RowPassArgs a) {
   __syncthreads();
 
   const int cta = is_draft ? (int)blockIdx.x : (int)blockIdx.x - a.draft_ctas;
-  const SpanGeom g = span_geom(q.total, a.V, is_draft ? a.draft_ctas : (int)gridDim.x - a.draft_ctas, a.max_split);
+  const SpanGeom g = span_geom(q.total, a.V, is_draft ? a.draft_ctas : (int)gridDim.x - a.draft_ctas, a.max_split, a.spans);
   const unsigned long long line_end = (unsigned long long)q.total * g.pitch;
   const float ln_mu = (float)a.log_mu;
   unsigned wt = 0;
 
   unsigned long long pos = (unsigned long long)cta * g.span;
   const unsigned long long span_end = min(line_end, pos + g.span);
-  int row = pos < span_end ? (int)div_u64(pos, g.pitch) : 0;
+  int row = pos < span_end ? (g.per_row ? (int)div_small((unsigned)cta, g.per_row) : (int)div_u64(pos, g.pitch)) : 0;
   int start = pos < span_end ? (int)(pos - (unsigned long long)row * g.pitch) : 0;
   for (; pos < span_end; ++row, start = 0) {
     const int len = (int)min((unsigned long long)(g.pitch - (unsigned)start), span_end - pos);
@@ -528,7 +529,7 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
   ra.draft = draft; ra.draft_stride = draft_stride;
   ra.target = with_target ? target : nullptr; ra.target_stride = target_stride;
   ra.B = B; ra.N = N; ra.V = p.vocab; ra.k = k; ra.key_stride = c->key_stride; ra.max_split = c->expand_max_split;
-  ra.init_layers = p.init_layers; ra.log_mu = c->log_mu;
+  ra.init_layers = p.init_layers; ra.log_mu = c->log_mu; ra.spans = span_table(p.vocab);
   ra.part_keys = c->d_part_keys; ra.part_ms = c->d_part_ms; ra.row_keys = c->d_row_keys; ra.row_lp = c->d_row_score;
   ra.row_count = c->d_row_count; ra.best = c->d_argmax; ra.row_bad = c->d_row_bad; ra.status = c->d_status;
   GrowArgs ga;

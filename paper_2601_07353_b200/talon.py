@@ -38,7 +38,7 @@ class TalonTreeStruct(C.Structure):
 
 
 _vp, _i32, _i64, _f32 = C.c_void_p, C.c_int32, C.c_int64, C.c_float
-_TP = C.POINTER(TalonTreeStruct)
+_TP = C.c_void_p                         # const talon_tree *, passed as an address
 _lib.talon_create.argtypes = [C.POINTER(_vp), C.POINTER(TalonParams), C.c_int]
 _lib.talon_destroy.argtypes = [_vp]
 _lib.talon_reset.argtypes = [_vp, _TP, _vp, _vp, _i32, _vp]
@@ -102,12 +102,19 @@ def _check(code: int, where: str):
         raise TalonError(code, where)
 
 
+# A step of separate calls is a dozen library entries of about 8 us of GPU work each, so what a call
+# costs on the host shows: addresses go as plain integers, the stream handle is read without making a
+# Stream object, and a tree's struct is kept (see Tree.address).
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(device) -> C.c_void_p:
-    return C.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+_raw_stream = torch._C._cuda_getCurrentRawStream if hasattr(torch._C, "_cuda_getCurrentRawStream") else (
+    lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
+def _stream(device) -> int:
+    return _raw_stream(device.index)
 
 
 def loop_metrics(counters: torch.Tensor, cost_ratio: float) -> dict:
@@ -149,6 +156,25 @@ class Tree:
         return TalonTreeStruct(*(t.data_ptr() for t in (self.n_nodes, self.token, self.parent, self.depth,
                                                           self.position, self.layer_off, self.score, self.mask)))
 
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        object.__setattr__(self, "_kept", None)          # another array: the struct is made anew
+
+    def address(self) -> int:
+        """Address of a ``talon_tree`` for this tree.  The struct is kept between calls and made anew when
+        an array was replaced or its memory moved."""
+        kept = self._kept
+        if kept is not None:
+            readers, ptrs, _, address = kept
+            if [f() for f in readers] == ptrs:
+                return address
+        readers = [t.data_ptr for t in (self.n_nodes, self.token, self.parent, self.depth, self.position, self.layer_off,
+                                        self.score, self.mask)]
+        ptrs = [f() for f in readers]
+        struct = TalonTreeStruct(*ptrs)
+        object.__setattr__(self, "_kept", (readers, ptrs, struct, C.addressof(struct)))
+        return self._kept[3]
+
 
 class Talon:
     """One library context (``talon_ctx``) on one CUDA device; methods mirror the C calls."""
@@ -186,89 +212,78 @@ class Talon:
 
     def reset(self, tree: Tree, root_tok: torch.Tensor, prefix_len: torch.Tensor):
         B = root_tok.shape[0]
-        ts = tree.struct()
-        _check(_lib.talon_reset(self._ctx, C.byref(ts), _ptr(root_tok), _ptr(prefix_len), B,
+        _check(_lib.talon_reset(self._ctx, tree.address(), _ptr(root_tok), _ptr(prefix_len), B,
                                 _stream(self.device)), "talon_reset")
 
     def expand_layer(self, tree: Tree, logits: torch.Tensor, rows_per_seq: Optional[int] = None,
                      layout: int = ROWS_BY_NODE, row_stride: Optional[int] = None):
-        ts = tree.struct()
         if row_stride is None:
             row_stride = logits.stride(-2)
         if rows_per_seq is None:
             rows_per_seq = logits.shape[-2]
-        _check(_lib.talon_expand_layer(self._ctx, C.byref(ts), _ptr(logits), row_stride, rows_per_seq, layout,
+        _check(_lib.talon_expand_layer(self._ctx, tree.address(), _ptr(logits), row_stride, rows_per_seq, layout,
                                        _stream(self.device)), "talon_expand_layer")
 
     def layers_run(self) -> int:
         return _lib.talon_layers_run(self._ctx)
 
     def build_tree(self, tree: Tree, dense_mask: Optional[torch.Tensor] = None):
-        ts = tree.struct()
-        _check(_lib.talon_build_tree(self._ctx, C.byref(ts), _ptr(dense_mask), _stream(self.device)),
+        _check(_lib.talon_build_tree(self._ctx, tree.address(), _ptr(dense_mask), _stream(self.device)),
                "talon_build_tree")
 
     def prune_tree(self, tree: Tree, keep: int):
         """``talon_prune_tree``: the final Top-N step of the static construction (Algorithm 1)."""
-        ts = tree.struct()
-        _check(_lib.talon_prune_tree(self._ctx, C.byref(ts), int(keep), _stream(self.device)), "talon_prune_tree")
+        _check(_lib.talon_prune_tree(self._ctx, tree.address(), int(keep), _stream(self.device)), "talon_prune_tree")
 
     def tree_attention(self, tree: Tree, q, k_prefix, v_prefix, k_tree, v_tree, kv_start, kv_tokens, kv_stride_t,
                        kv_stride_h, max_prefix_len, sm_scale, out):
-        ts = tree.struct()
-        _check(_lib.talon_tree_attention(self._ctx, C.byref(ts), _ptr(q), _ptr(k_prefix), _ptr(v_prefix),
+        _check(_lib.talon_tree_attention(self._ctx, tree.address(), _ptr(q), _ptr(k_prefix), _ptr(v_prefix),
                                          _ptr(k_tree), _ptr(v_tree), _ptr(kv_start), kv_tokens, kv_stride_t, kv_stride_h,
                                          max_prefix_len, sm_scale, _ptr(out), _stream(self.device)),
                "talon_tree_attention")
 
     def accept(self, tree: Tree, target_logits, accept_len, accept_nodes, bonus_tok, target_tok=None,
                row_stride: Optional[int] = None):
-        ts = tree.struct()
         if row_stride is None:
             row_stride = target_logits.stride(-2)
-        _check(_lib.talon_accept(self._ctx, C.byref(ts), _ptr(target_logits), row_stride, _ptr(target_tok),
+        _check(_lib.talon_accept(self._ctx, tree.address(), _ptr(target_logits), row_stride, _ptr(target_tok),
                                  _ptr(accept_len), _ptr(accept_nodes), _ptr(bonus_tok), _stream(self.device)),
                "talon_accept")
 
     def close_and_accept(self, tree: Tree, target_logits, accept_len, accept_nodes, bonus_tok, target_tok=None,
                          row_stride: Optional[int] = None):
-        ts = tree.struct()
         if row_stride is None:
             row_stride = target_logits.stride(-2)
-        _check(_lib.talon_close_and_accept(self._ctx, C.byref(ts), _ptr(target_logits), row_stride, _ptr(target_tok),
+        _check(_lib.talon_close_and_accept(self._ctx, tree.address(), _ptr(target_logits), row_stride, _ptr(target_tok),
                                            _ptr(accept_len), _ptr(accept_nodes), _ptr(bonus_tok), _stream(self.device)),
                "talon_close_and_accept")
 
     def accept_sample(self, tree: Tree, target_logits, temperature: float, u_accept, u_sample, accept_len,
                       accept_nodes, out_tok, row_stride: Optional[int] = None):
-        ts = tree.struct()
         if row_stride is None:
             row_stride = target_logits.stride(-2)
         assert u_accept.dtype == torch.float64 and u_sample.dtype == torch.float64
-        _check(_lib.talon_accept_sample(self._ctx, C.byref(ts), _ptr(target_logits), row_stride, float(temperature),
+        _check(_lib.talon_accept_sample(self._ctx, tree.address(), _ptr(target_logits), row_stride, float(temperature),
                                         _ptr(u_accept), _ptr(u_sample), _ptr(accept_len), _ptr(accept_nodes),
                                         _ptr(out_tok), _stream(self.device)), "talon_accept_sample")
 
     def commit(self, tree: Tree, accept_len, accept_nodes, next_tok, k_tree, v_tree, k_prefix, v_prefix, kv_start,
                kv_limit, kv_tokens, kv_stride_t, kv_stride_h, prefix_len, root_tok, counters=None):
-        ts = tree.struct()
-        _check(_lib.talon_commit(self._ctx, C.byref(ts), _ptr(accept_len), _ptr(accept_nodes), _ptr(next_tok),
+        _check(_lib.talon_commit(self._ctx, tree.address(), _ptr(accept_len), _ptr(accept_nodes), _ptr(next_tok),
                                  _ptr(k_tree), _ptr(v_tree), _ptr(k_prefix), _ptr(v_prefix), _ptr(kv_start),
                                  _ptr(kv_limit), kv_tokens, kv_stride_t, kv_stride_h, _ptr(prefix_len), _ptr(root_tok),
                                  _ptr(counters), _stream(self.device)), "talon_commit")
 
     def tree_attention_paged(self, tree: Tree, q, k_pages, v_pages, k_tree, v_tree, block_table, n_pages, kv_stride_t,
                              kv_stride_h, max_prefix_len, sm_scale, out):
-        ts = tree.struct()
-        _check(_lib.talon_tree_attention_paged(self._ctx, C.byref(ts), _ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(k_tree),
+        _check(_lib.talon_tree_attention_paged(self._ctx, tree.address(), _ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(k_tree),
                                                _ptr(v_tree), _ptr(block_table), block_table.stride(0), n_pages, kv_stride_t,
                                                kv_stride_h, max_prefix_len, sm_scale, _ptr(out), _stream(self.device)),
                "talon_tree_attention_paged")
 
     def commit_paged(self, tree: Tree, accept_len, accept_nodes, next_tok, k_tree, v_tree, k_pages, v_pages, block_table,
                      n_blocks, n_pages, kv_stride_t, kv_stride_h, prefix_len, root_tok, counters=None):
-        ts = tree.struct()
-        _check(_lib.talon_commit_paged(self._ctx, C.byref(ts), _ptr(accept_len), _ptr(accept_nodes), _ptr(next_tok),
+        _check(_lib.talon_commit_paged(self._ctx, tree.address(), _ptr(accept_len), _ptr(accept_nodes), _ptr(next_tok),
                                        _ptr(k_tree), _ptr(v_tree), _ptr(k_pages), _ptr(v_pages), _ptr(block_table),
                                        block_table.stride(0), _ptr(n_blocks), n_pages, kv_stride_t, kv_stride_h,
                                        _ptr(prefix_len), _ptr(root_tok), _ptr(counters), _stream(self.device)),
@@ -280,9 +295,8 @@ class Talon:
         """``talon_loop``: ``n_steps`` draft-and-verify steps with the commit between them.  ``draft`` and
         ``target`` are [S, B, N, V]; ``q``, ``k_tree``, ``v_tree`` [S, B, N, H, Dh]; with ``keep_results`` the
         result arrays are [S, B(, D_max + 1)], else the last step's."""
-        ts = tree.struct()
         B = root_tok.shape[0]
-        _check(_lib.talon_loop(self._ctx, C.byref(ts), B, n_steps, _ptr(root_tok), _ptr(prefix_len), _ptr(draft),
+        _check(_lib.talon_loop(self._ctx, tree.address(), B, n_steps, _ptr(root_tok), _ptr(prefix_len), _ptr(draft),
                                draft.stride(-2), draft.stride(0), n_layers, _ptr(q), q.stride(0), _ptr(k_prefix),
                                _ptr(v_prefix), _ptr(k_tree), _ptr(v_tree), k_tree.stride(0), _ptr(kv_start), _ptr(kv_limit),
                                kv_tokens, kv_stride_t, kv_stride_h, max_prefix_len, sm_scale, _ptr(out), _ptr(target),
@@ -300,8 +314,7 @@ class Talon:
              kv_start, kv_tokens, kv_stride_t, kv_stride_h, max_prefix_len, sm_scale, out, target_logits, target_tok,
              accept_len, accept_nodes, bonus_tok):
         """``talon_step``: the whole draft-and-verify step on device-resident inputs, one library call."""
-        ts = tree.struct()
-        _check(_lib.talon_step(self._ctx, C.byref(ts), root_tok.shape[0], _ptr(root_tok), _ptr(prefix_len),
+        _check(_lib.talon_step(self._ctx, tree.address(), root_tok.shape[0], _ptr(root_tok), _ptr(prefix_len),
                                _ptr(draft_logits), draft_logits.stride(-2), n_layers, _ptr(q), _ptr(k_prefix),
                                _ptr(v_prefix), _ptr(k_tree), _ptr(v_tree), _ptr(kv_start), kv_tokens, kv_stride_t,
                                kv_stride_h, max_prefix_len, sm_scale, _ptr(out), _ptr(target_logits), target_logits.stride(-2),
