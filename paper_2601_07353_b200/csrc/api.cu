@@ -117,9 +117,8 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     c->attn_min_tiles = mt ? std::atoi(mt) : 2;
     if (c->attn_min_tiles < 1) c->attn_min_tiles = 1;
     const char *ms = std::getenv("TALON_EXPAND_MAX_SPLIT");
-    c->expand_max_split = ms ? std::atoi(ms) : talon::FX_MAX_SPLITS - 1;
+    c->expand_max_split = ms ? std::atoi(ms) : talon::FX_MAX_SPLITS;
     if (c->expand_max_split < 1) c->expand_max_split = 1;
-    if (c->expand_max_split > talon::FX_MAX_SPLITS - 1) c->expand_max_split = talon::FX_MAX_SPLITS - 1;
     const char *ac = std::getenv("TALON_ATTN_CLUSTER");
     c->attn_cluster = ac ? std::atoi(ac) : 1;
     for (int i = 0; i < 9; ++i) c->attn_cluster_ok[i] = -1;

@@ -26,7 +26,7 @@ struct FusedArgs {
   int rows_per_seq, layout;
   talon_tree t;
   int lo_stride;
-  int B, N, W, V, d, k, key_stride, max_split, base_offset, pool_cap;
+  int B, N, W, V, d, k, key_stride, base_offset, pool_cap;
   int root_topk, init_layers;
   double log_mu;
   SpanTable spans;
@@ -128,7 +128,7 @@ __device__ inline RowLoc locate_row(const FusedArgs &a, const Frontier &fr, int 
 // ---------------------------------------------------------------------------------------
 // Shared-memory carve-up of the selection phase (it reuses the streaming ring).
 struct TailSmem {
-  u64 *stage;        // [EXP_WARPS][FX_MAX_SPLITS k + FX_SURV + k]  chunk lists of the row a warp is merging, survivors, result
+  u64 *stage;        // [EXP_WARPS][stage_words(k)]  chunk lists of the row a warp is merging, survivors, result
   u64 *row_keys;     // [N-1][k]               per-row top-k keys, descending
   double *score;     // [N-1][k]               log p(u) of each pooled candidate
   u64 *row_mask;     // [N-1][W]               ancestor mask of the row's parent
@@ -303,7 +303,7 @@ expand_fused_kernel(FusedArgs a) {
         if (s_base[b + 1] == s_base[b])
           a.t.layer_off[b * a.lo_stride + a.d + 2] = a.t.layer_off[b * a.lo_stride + a.d + 1];
   }
-  const SpanGeom g = span_geom(fr.total, a.V, (int)gridDim.x, a.max_split, a.spans);
+  const SpanGeom g = span_geom(fr.total, a.V, (int)gridDim.x, a.spans);
   const unsigned long long line_end = (unsigned long long)fr.total * g.pitch;
   const bool gated = a.d >= a.init_layers;
   const float ln_mu = (float)a.log_mu;
@@ -554,9 +554,8 @@ talon_status launch_expand_fused(talon_ctx *c, const talon_tree *t, const float 
   a.t = *t; a.lo_stride = c->p.max_depth + 2;
   a.B = c->B; a.N = c->p.budget; a.W = c->W; a.V = c->p.vocab; a.d = c->layers_run; a.k = c->k_cap;
   a.key_stride = c->key_stride;
-  a.max_split = c->expand_max_split;
   a.pool_cap = pool_capacity(c);
-  a.spans = span_table(c->p.vocab);
+  a.spans = span_table(c->p.vocab, c->k_cap, c->expand_max_split);
   long long max_items = (long long)rows_bound * FX_MAX_SPLITS;
   int grid = c->fused_grid;
   if (max_items < grid) grid = (int)max_items;

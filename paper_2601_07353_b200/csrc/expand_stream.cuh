@@ -92,17 +92,20 @@ __device__ inline void ring_issue(uint32_t dst, const float *src, uint32_t bytes
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 // Waits for the phase of `bar` with the given parity, for about two seconds at most.
+__device__ inline bool ring_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  // the hint lets the hardware park the thread until the phase completes (or ~20 us pass)
+  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.b32 %0, 1, 0, p;\n}"
+               : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
+  return ok != 0;
+}
 __device__ inline bool ring_wait(uint32_t bar, uint32_t parity) {
+  if (ring_try(bar, parity)) return true;
   const long long t0 = clock64();
   for (;;) {
 #pragma unroll 1
-    for (int i = 0; i < 64; ++i) {
-      uint32_t ok;
-      // the hint lets the hardware park the thread until the phase completes (or ~20 us pass)
-      asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.b32 %0, 1, 0, p;\n}"
-                   : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
-      if (ok) return true;
-    }
+    for (int i = 0; i < 64; ++i)
+      if (ring_try(bar, parity)) return true;
     if (clock64() - t0 > 4000000000ll) return false;
   }
 }
@@ -181,8 +184,8 @@ __device__ inline double f64_unord(u64 o) {
 // and the CTAs of the grid take consecutive spans of `span` elements of that line (both multiples
 // of four: rows are 16-byte aligned).
 //   * Few rows (the grid holds at least two CTAs per row): a row is cut into S equal chunks, one
-//     CTA each, S as large as the grid allows (at most FX_MAX_SPLITS - 1, at least 4096 elements
-//     per chunk); pitch = S * span, so no span crosses a row.
+//     CTA each, S as large as the grid allows, down to chunks of one CTA step (4096 elements: a tile
+//     per warp); pitch = S * span, so no span crosses a row.
 //   * Many rows: pitch is the row length and every CTA takes the same share of the whole line, so
 //     every CTA (and every SM) streams the same number of bytes whatever the number of rows; a span
 //     that crosses a row boundary is worked off as one chunk per row it touches.
@@ -201,11 +204,22 @@ __device__ inline unsigned div_u64(unsigned long long a, unsigned b) {
 
 // (An integer division is a chain of some 60 clocks on the way to the first byte: the spans of whole-row
 // fractions come from the host, and small quotients by way of a float, exact for operands below 2^16.)
-struct SpanTable { unsigned of[FX_MAX_SPLITS]; };      // [S]: elements of a chunk when a row is cut into S
-inline SpanTable span_table(int vocab) {
+struct SpanTable {
+  unsigned of[FX_MAX_SPLITS + 1];      // [S]: elements of a chunk when a row is cut into S
+  unsigned line_min;                   // least span of the shared line
+  unsigned most;                       // most chunks of a whole row
+};
+inline SpanTable span_table(int vocab, int k, int max_split) {
   SpanTable t = {};
-  const unsigned vp = ((unsigned)vocab + 3u) & ~3u;
-  for (unsigned S = 1; S < FX_MAX_SPLITS; ++S) t.of[S] = ((vp + S - 1u) / S + 3u) & ~3u;
+  const unsigned vp = ((unsigned)vocab + 3u) & ~3u, lists = k <= 16 ? FX_MAX_SPLITS : FX_LONG_SPLITS;
+  for (unsigned S = 1; S <= FX_MAX_SPLITS; ++S) t.of[S] = ((vp + S - 1u) / S + 3u) & ~3u;
+  // a row touches one span more than it has span lengths
+  t.line_min = ((vp + lists - 2u) / (lists - 1u) + 3u) & ~3u;
+  if (t.line_min < (unsigned)EXP_TILE) t.line_min = EXP_TILE;
+  // chunks of at most a CTA step (eight warp tiles): a finer cut leaves warps without work
+  t.most = (vp + EXP_TILE - 1u) / EXP_TILE;
+  if (t.most > (unsigned)max_split) t.most = max_split;
+  if (t.most > lists) t.most = lists;
   return t;
 }
 __device__ inline unsigned div_small(unsigned a, unsigned b) { return (unsigned)__fdividef((float)a + 0.5f, (float)b); }
@@ -218,20 +232,19 @@ __device__ inline int div_up_small(int a, int b) {
   return q;
 }
 
-__device__ inline SpanGeom span_geom(int total_rows, int vocab, int grid, int max_split, const SpanTable &table) {
+__device__ inline SpanGeom span_geom(int total_rows, int vocab, int grid, const SpanTable &table) {
   SpanGeom g;
   const unsigned vp = ((unsigned)vocab + 3u) & ~3u;
   const unsigned per_row = total_rows > 0 ? (total_rows < grid ? div_small((unsigned)grid, (unsigned)total_rows) : (total_rows == grid ? 1u : 0u)) : 1u;
   if (per_row >= 2u) {
-    const unsigned S = max(1u, min(min(per_row, (unsigned)max_split), vp / 4096u));
+    const unsigned S = min(per_row, table.most);
     g.span = table.of[S];
     g.pitch = S * g.span;
     g.per_row = S;
   } else {
     const unsigned long long line = (unsigned long long)total_rows * vp;
     const unsigned span = (div_u64(line + grid - 1, (unsigned)grid) + 3u) & ~3u;
-    const unsigned span_min = max(4096u, ((vp + FX_MAX_SPLITS - 2) / (FX_MAX_SPLITS - 1) + 3u) & ~3u);
-    g.span = max(span, span_min);
+    g.span = max(span, table.line_min);
     g.pitch = vp;
     g.per_row = 0u;
   }
@@ -501,11 +514,12 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
   bool resident = wlen <= XS_RING * XS_WTILE;              // (the same for all warps)
   if (resident) {
     auto tile = [&](int t) { return sh.ring + ((wt + t) % XS_RING) * XS_WTILE; };
-    float mt = -CUDART_INF_F, st = 0.f, bm[XS_RING];
-#pragma unroll
-    for (int t = 0; t < XS_RING; ++t) {
-      bm[t] = -CUDART_INF_F;
-      if (t >= nt) continue;
+    // (the loops over tiles stay loops: a layer's launch finds its code cold, and fetching three copies
+    // of the body cost more than running one three times)
+    float mt = -CUDART_INF_F, st = 0.f, bm0 = -CUDART_INF_F, bm1 = -CUDART_INF_F, bm2 = -CUDART_INF_F;
+    static_assert(XS_RING == 3, "one maximum per slot");
+#pragma unroll 1
+    for (int t = 0; t < nt; ++t) {
       if (!ring_wait(smem_addr(sh.bar + (wt + t) % XS_RING), ((wt + t) / XS_RING) & 1u)) {
         if (lane == 0) { atomicOr(res.status, STATUS_TIMEOUT); *sh.abort_flag = 1; }
         ring_wait(smem_addr(sh.bar + (wt + t) % XS_RING), ((wt + t) / XS_RING) & 1u);
@@ -523,10 +537,11 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
         v[4 * u] = y.x; v[4 * u + 1] = y.y; v[4 * u + 2] = y.z; v[4 * u + 3] = y.w;
       }
       float m = max3(max3(v[0], v[1], v[2]), max3(v[3], v[4], v[5]), max3(v[6], v[7], v[8]));
-      bm[t] = fmaxf(max3(m, max3(v[9], v[10], v[11]), max3(v[12], v[13], v[14])), v[15]);
-      if (bm[t] > mt) {
-        st *= fast_exp2((mt - bm[t]) * LOG2E_F);
-        mt = bm[t];
+      m = fmaxf(max3(m, max3(v[9], v[10], v[11]), max3(v[12], v[13], v[14])), v[15]);
+      bm2 = t == 2 ? m : bm2; bm1 = t == 1 ? m : bm1; bm0 = t == 0 ? m : bm0;
+      if (m > mt) {
+        st *= fast_exp2((mt - m) * LOG2E_F);
+        mt = m;
       }
       if (mt > -CUDART_INF_F) {
         const float c = -mt * LOG2E_F;
@@ -563,6 +578,11 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
       }
       if (lane == 0) { sh.wtop[warp] = mine; sh.wmax[warp] = wmax; }
     }
+    // lane partial rescaled to the warp maximum; a NaN partial (NaN or +inf logit) propagates
+    float wsum = (mt > -CUDART_INF_F || st != st) ? st * exp2f((mt - wmax) * LOG2E_F) : 0.f;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) wsum += __shfl_xor_sync(FULL, wsum, o);
+    if (lane == 0) { sh.m[warp] = wmax; sh.s[warp] = wsum; }
     __syncthreads();
     if (*sh.abort_flag) return false;
     const float omin = f32_unord(__reduce_min_sync(FULL, lane < active ? f32_ord(sh.wtop[lane]) : 0xFFFFFFFFu));
@@ -571,9 +591,9 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
     if (active > 0) thr = fmaxf(thr, omin);
     // (slack: fp32 rounding of the sum and of ln(mu), and the 1e-5 band around the gate)
     if (gated && omax > -CUDART_INF_F) thr = fmaxf(thr, omax + ln_mu - (1e-4f + 1e-6f * fabsf(omax)));
-#pragma unroll
-    for (int t = 0; t < XS_RING; ++t) {
-      if (!__any_sync(FULL, bm[t] >= thr)) continue;       // (bm is -inf past the slice)
+#pragma unroll 1
+    for (int t = 0; t < nt; ++t) {
+      if (!__any_sync(FULL, (t == 0 ? bm0 : (t == 1 ? bm1 : bm2)) >= thr)) continue;
       const float *slot = tile(t);
       unsigned mm = 0u;
 #pragma unroll
@@ -593,11 +613,6 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
       }
       __syncwarp();
     }
-    // lane partial rescaled to the warp maximum; a NaN partial (NaN or +inf logit) propagates
-    float wsum = (mt > -CUDART_INF_F || st != st) ? st * exp2f((mt - wmax) * LOG2E_F) : 0.f;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) wsum += __shfl_xor_sync(FULL, wsum, o);
-    if (lane == 0) { sh.m[warp] = wmax; sh.s[warp] = wsum; }
     __syncthreads();
     if (*sh.pool_n > POOL) {
       // too many at the bound (equal logits, a sorted row): the general way over the tiles in the ring
@@ -764,7 +779,7 @@ __device__ __forceinline__ void chunk_clear(const ChunkShared &sh) {
   if (threadIdx.x == 0) *sh.pool_n = 0;
 }
 
-__host__ __device__ inline int stage_words(int k) { return FX_MAX_SPLITS * k + FX_SURV + k; }
+__host__ __device__ inline int stage_words(int k) { return FX_LONG_SPLITS * k + FX_SURV + k; }
 
 // The largest value over the warp, in two reductions of half a key.
 __device__ __forceinline__ u64 warp_redux_max_u64(u64 v) {
@@ -785,14 +800,14 @@ __device__ __forceinline__ u64 merge_groups(u64 a, u64 b_rev, int lane) {
   return x;
 }
 
-// The k <= K best of S descending lists of k keys, K = 8 or 16, in lanes 0 .. K-1 descending: 16 lists
-// lie K lanes each in K / 2 registers and are merged pairwise, first register with register, then
+// The k <= K best of S <= LISTS descending lists of k keys, K = 8 or 16, in lanes 0 .. K-1 descending:
+// the lists lie K lanes each in LISTS K / 32 registers and are merged pairwise, first register with register, then
 // lane group with lane group.  A dozen dependent shuffles, no shared memory, no data-dependent loop
 // (collecting the survivors of a bound and ranking them took 2.5 us at 15 lists of 8, this 1 us).
-template <int K>
+template <int K, int LISTS>
 __device__ __forceinline__ u64 merge_lists(const u64 *lists, int stride, int S, int k, int lane) {
   constexpr int PER = 32 / K;                     // lists per register
-  constexpr int NR = FX_MAX_SPLITS / PER;
+  constexpr int NR = LISTS / PER;
   u64 r[NR];
   const int sub = lane / K, pos = lane & (K - 1);
 #pragma unroll
@@ -819,7 +834,7 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
                                           u64 &out_key, double &out_score) {
   const int lane = threadIdx.x & 31;
   const int ks = res.key_stride;
-  u64 *sv = st + FX_MAX_SPLITS * k;              // keys that reach the bound
+  u64 *sv = st + FX_LONG_SPLITS * k;              // keys that reach the bound
   u64 *rk = sv + FX_SURV;                        // the row's k best keys
   // Everything the row needs from global memory (ps among it) goes to registers before the first store (a
   // load cannot pass a store through a pointer the compiler cannot tell apart): one trip to L2
@@ -827,7 +842,9 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
   const float2 ms = (lane < S) ? __ldcg(res.part_ms + item0 + lane) : make_float2(-CUDART_INF_F, 0.f);
   u64 own = 0ull;                                // KMAX 8 and 16: this lane's key of the merged list
   if (KMAX <= 16) {
-    own = merge_lists<KMAX <= 16 ? KMAX : 16>(res.part_keys + item0 * ks, ks, S, k, lane);
+    constexpr int K = KMAX <= 16 ? KMAX : 16;
+    const u64 *lists = res.part_keys + item0 * ks;
+    own = S <= 16 ? merge_lists<K, 16>(lists, ks, S, k, lane) : merge_lists<K, FX_MAX_SPLITS>(lists, ks, S, k, lane);
   } else if (S == 1) {
     const u64 key = lane < k ? __ldcg(res.part_keys + item0 * ks + lane) : 0ull;
     if (lane < k) rk[lane] = key;
@@ -841,22 +858,19 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int i = i0 + 2 * u;
-        if (lane < S && i < k) st[i * FX_MAX_SPLITS + lane] = x[u].x;
-        if (lane < S && i + 1 < k) st[(i + 1) * FX_MAX_SPLITS + lane] = x[u].y;
+        if (lane < S && i < k) st[i * FX_LONG_SPLITS + lane] = x[u].x;
+        if (lane < S && i + 1 < k) st[(i + 1) * FX_LONG_SPLITS + lane] = x[u].y;
       }
     }
   }
-  static_assert(FX_MAX_SPLITS <= 16, "the chunk statistics are reduced over 16 lanes");
   float mx = ms.x;                                                      // lanes >= S hold -inf and 0
 #pragma unroll
-  for (int o = 8; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
-  mx = __shfl_sync(FULL, mx, 0);
+  for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
   double t = 0.0;
   if (ms.y != ms.y) t = (double)ms.y;                                   // NaN or +inf logit in the chunk
   else if (ms.x > -CUDART_INF_F) t = (double)ms.y * (double)exp2f((ms.x - mx) * LOG2E_F);
 #pragma unroll
-  for (int o = 8; o; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
-  t = __shfl_sync(FULL, t, 0);
+  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
   const bool finite = (t > 0.0) && (t < CUDART_INF) && (mx < CUDART_INF_F) && (mx > -CUDART_INF_F);
 
   if (KMAX > 16 && S > 1) {
@@ -866,11 +880,11 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
     // ke-th key of any one chunk, and the ke-th best of the chunk heads (ke different chunks each
     // hold a key at least that large).
     const u64 head = lane < S ? st[lane] : 0ull;
-    u64 tau = lane < S ? st[(ke - 1) * FX_MAX_SPLITS + lane] : 0ull;
+    u64 tau = lane < S ? st[(ke - 1) * FX_LONG_SPLITS + lane] : 0ull;
     if (S >= ke) {
       int cnt = 0;                                 // (lanes past the chunks hold 0 and count for nothing)
 #pragma unroll
-      for (int o = 0; o < FX_MAX_SPLITS; ++o) cnt += (shfl_u64(head, o) > head) ? 1 : 0;
+      for (int o = 0; o < FX_LONG_SPLITS; ++o) cnt += (shfl_u64(head, o) > head) ? 1 : 0;
       if (cnt == ke - 1) tau = umax64(tau, head);
     }
     tau = warp_max_u64(tau);
@@ -878,7 +892,7 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
     // first position where no chunk has one
     int ns = 0;
     for (int i = 0; i < ke; ++i) {
-      const u64 key = lane < S ? st[i * FX_MAX_SPLITS + lane] : 0ull;
+      const u64 key = lane < S ? st[i * FX_LONG_SPLITS + lane] : 0ull;
       const bool ok = key != 0ull && key >= tau;
       const unsigned mk = __ballot_sync(FULL, ok);
       if (mk == 0u) break;
@@ -899,7 +913,7 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
       // many keys at the bound (equal logits): pop the largest head ke times
       int p = 0;
       for (int r = 0; r < ke; ++r) {
-        const u64 cand = (lane < S && p < ke) ? st[p * FX_MAX_SPLITS + lane] : 0ull;
+        const u64 cand = (lane < S && p < ke) ? st[p * FX_LONG_SPLITS + lane] : 0ull;
         const u64 best = warp_max_u64(cand);
         if (best == 0ull) break;
         if (cand == best) ++p;
@@ -921,13 +935,13 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
 // The same for WIDE lists, by the whole CTA: the row's k best keys and scores go straight to
 // key_out / score_out [k] (slot 0 of score_out NaN when the row has no softmax).  st: WIDE_STAGE_WORDS
 // words of shared memory.
-constexpr int WIDE_STAGE_WORDS = 2 * FX_MAX_SPLITS * 128 + 4;
+constexpr int WIDE_STAGE_WORDS = 2 * FX_LONG_SPLITS * 128 + 4;
 __device__ __forceinline__ void merge_row_wide(const ChunkOut &res, size_t item0, int S, int k, int ke, double ps, u64 *st,
                                                u64 *key_out, double *score_out, int *status) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ks = res.key_stride, total = S * ke;
-  u64 *sv = st + FX_MAX_SPLITS * 128;
-  double *s_lse = reinterpret_cast<double *>(sv + FX_MAX_SPLITS * 128);
+  u64 *sv = st + FX_LONG_SPLITS * 128;
+  double *s_lse = reinterpret_cast<double *>(sv + FX_LONG_SPLITS * 128);
   int *s_n = reinterpret_cast<int *>(s_lse + 1);
   u64 *s_tau = reinterpret_cast<u64 *>(s_lse + 2);
   for (int i = tid; i < total; i += EXP_THREADS) {
@@ -1011,6 +1025,7 @@ __device__ __forceinline__ int layer_select(int F, int k, int ke, int want, bool
   const int gl = lane & (G - 1), gbase = lane & ~(G - 1);
   const unsigned gmask = (G == 32 ? FULL : ((1u << (G & 31)) - 1u)) << gbase;
   constexpr int per_pass = THREADS / G;
+  constexpr int FEW = KMAX <= 16 ? 256 / KMAX : 0;
   constexpr int PASSES = 32 * NQ / per_pass > 0 ? 32 * NQ / per_pass : 1;
   const int my_row = tid / G;
 
@@ -1039,7 +1054,7 @@ __device__ __forceinline__ int layer_select(int F, int k, int ke, int want, bool
 #pragma unroll
       for (int i = 0; i < KMAX; ++i) s[i] = score(r, min(i, k - 1));
 #pragma unroll
-      for (int i = 0; i < KMAX; ++i) cnt[q] += (i < ke && s[i] >= thr) ? 1 : 0;
+      for (int i = 0; i < KMAX; ++i) cnt[q] += (int)(i < ke) & (int)(s[i] >= thr);
       if (q * 32 + lane >= F) cnt[q] = 0;
     }
   }
@@ -1084,6 +1099,19 @@ __device__ __forceinline__ int layer_select(int F, int k, int ke, int want, bool
       if (j < F && gl < s_cnt[j]) {
         const double s = score(j, gl);
         int rank = gl;
+        // (a small pool is counted through, loads in flight together; a large one searched row by row)
+        if (F <= FEW) {
+          rank = 0;
+          for (int o = 0; o < F; ++o) {
+            const int h = s_cnt[o];
+            double v[KMAX];
+#pragma unroll
+            for (int i = 0; i < KMAX; ++i) v[i] = score(o, min(i, k - 1));
+#pragma unroll
+            for (int i = 0; i < KMAX; ++i)          // (& and |: no branch per candidate)
+              rank += (int)(i < h) & ((int)(v[i] > s) | ((int)(v[i] == s) & ((int)(o < j) | ((int)(o == j) & (int)(i < gl)))));
+          }
+        } else
         for (int o = 0; o < F && rank < want; ++o) {
           int l = 0, h = o == j ? 0 : s_cnt[o];
           while (l < h) {
@@ -1117,7 +1145,7 @@ __device__ __forceinline__ int layer_select(int F, int k, int ke, int want, bool
     const int t = (gl < c) ? tok(j, gl) : 0x7FFFFFFF;
     int r = 0;
 #pragma unroll
-    for (int i = 0; i < KMAX; ++i) r += __shfl_sync(FULL, t, gbase + i) < t ? 1 : 0;      // unused lanes hold the largest
+    for (int i = 0; i < KMAX; ++i) r += (int)(__shfl_sync(FULL, t, gbase + i) < t);      // unused lanes hold the largest
     if (gl < c) append(o0 + r, j, gl, t, score(j, gl));
   }
   return total;

@@ -27,7 +27,7 @@ namespace {
 struct RowPassArgs {
   const float *draft, *target;        // [B, N] rows
   int64_t draft_stride, target_stride;
-  int B, N, V, k, key_stride, max_split;
+  int B, N, V, k, key_stride;
   int r0, r1;                         // node slots of this round, per sequence
   int t1;                             // target rows of slots r0 .. t1-1 (t1 = r0: none)
   int draft_ctas;                     // CTAs 0 .. draft_ctas-1 take draft rows, the others target rows
@@ -199,7 +199,7 @@ row_pass_kernel(RowPassArgs a) {
   __syncthreads();
 
   const int cta = is_draft ? (int)blockIdx.x : (int)blockIdx.x - a.draft_ctas;
-  const SpanGeom g = span_geom(q.total, a.V, is_draft ? a.draft_ctas : (int)gridDim.x - a.draft_ctas, a.max_split, a.spans);
+  const SpanGeom g = span_geom(q.total, a.V, is_draft ? a.draft_ctas : (int)gridDim.x - a.draft_ctas, a.spans);
   const unsigned long long line_end = (unsigned long long)q.total * g.pitch;
   const float ln_mu = (float)a.log_mu;
   unsigned wt = 0;
@@ -528,8 +528,8 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
   RowPassArgs ra;
   ra.draft = draft; ra.draft_stride = draft_stride;
   ra.target = with_target ? target : nullptr; ra.target_stride = target_stride;
-  ra.B = B; ra.N = N; ra.V = p.vocab; ra.k = k; ra.key_stride = c->key_stride; ra.max_split = c->expand_max_split;
-  ra.init_layers = p.init_layers; ra.log_mu = c->log_mu; ra.spans = span_table(p.vocab);
+  ra.B = B; ra.N = N; ra.V = p.vocab; ra.k = k; ra.key_stride = c->key_stride;
+  ra.init_layers = p.init_layers; ra.log_mu = c->log_mu; ra.spans = span_table(p.vocab, k, c->expand_max_split);
   ra.part_keys = c->d_part_keys; ra.part_ms = c->d_part_ms; ra.row_keys = c->d_row_keys; ra.row_lp = c->d_row_score;
   ra.row_count = c->d_row_count; ra.best = c->d_argmax; ra.row_bad = c->d_row_bad; ra.status = c->d_status;
   GrowArgs ga;
@@ -551,17 +551,14 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
     ra.clear_status = r == 0;
     // CTAs per row: as many as the grid holds, no row cut into less than a CTA step per chunk
     const long long dr = (long long)B * (upto - done), tr = (long long)B * (ra.t1 - done);
-    // (as span_geom cuts them: 4096 elements a chunk at least)
-    int cut = (p.vocab + 3) / 4 * 4 / EXP_TILE;
-    if (cut > c->expand_max_split) cut = c->expand_max_split;
-    if (cut < 1) cut = 1;
+    const int cut = (int)ra.spans.most;
     int grid = c->row_grid;
     if (tr == 0) {
       if (dr * cut < grid) grid = (int)(dr * cut);
       ra.draft_ctas = grid;
     } else {
       int gd = (int)(grid * dr / (dr + tr));
-      const int target_cut = (p.vocab + 4 * EXP_TILE - 1) / (4 * EXP_TILE);
+      const int target_cut = (p.vocab + 8 * EXP_TILE - 1) / (8 * EXP_TILE);
       if (dr * cut + tr * target_cut <= grid) {
         // small rows: the draft rows are cut as finely as a single layer's would be (the same partial
         // sums, so the same scores to the last bit), the target rows share the rest of the grid

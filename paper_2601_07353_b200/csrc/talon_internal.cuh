@@ -27,7 +27,8 @@ constexpr int MAX_BATCH = 1024;
 constexpr int SEL_THREADS = 512;
 // fused expansion kernel (k <= 32)
 constexpr int FX_SURV = 64;                // keys of a row that may pass the merge bound before the slow path
-constexpr int FX_MAX_SPLITS = 16;          // chunks per row, at most (one lane per chunk in the merge)
+constexpr int FX_MAX_SPLITS = 32;          // chunks per row, at most (one lane per chunk in the merge)
+constexpr int FX_LONG_SPLITS = 16;         // the same for lists of more than 16 keys (they are merged in shared memory)
 
 // Order-preserving map fp32 -> u32 (larger float <=> larger integer; -inf > 0).
 __host__ __device__ inline uint32_t f32_ord(float f) {
