@@ -121,9 +121,7 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     if (c->expand_max_split < 1) c->expand_max_split = 1;
     const char *ac = std::getenv("TALON_ATTN_CLUSTER");
     c->attn_cluster = ac ? std::atoi(ac) : 1;
-    for (int i = 0; i < 9; ++i) c->attn_cluster_ok[i] = -1;
-    const char *cc = std::getenv("TALON_ATTN_CLUSTER_CAP");
-    c->attn_cluster_cap = cc ? std::atoi(cc) : 32;
+    std::memset(c->attn_clusters, -1, sizeof(c->attn_clusters));
     const char *cr = std::getenv("TALON_ATTN_CLUSTER_MIN_ROWS");
     c->attn_cluster_min_rows = cr ? std::atoll(cr) : 8192;
     const char *fs = std::getenv("TALON_ATTN_SPLITS");

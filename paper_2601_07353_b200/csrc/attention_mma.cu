@@ -10,6 +10,8 @@
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "talon_internal.cuh"
 
 namespace talon {
@@ -19,7 +21,6 @@ constexpr int AT_BM = 128;     // packed query rows per CTA (16 per warp)
 constexpr int AT_BN = 64;      // keys per tile
 constexpr int AT_D = 128;      // head dimension
 constexpr int AT_TILE_BYTES = AT_BN * AT_D * 2;
-constexpr int TC_MIN_TILES_PER_CTA = 4;   // split-KV of the tensor-core path: key tiles a CTA should at least own
 constexpr int AT_SMEM = AT_BM * AT_D * 2 + 4 * AT_TILE_BYTES;   // Q + 2 stages of (K, V)
 
 struct AttnArgs {
@@ -29,6 +30,7 @@ struct AttnArgs {
   const int32_t *prefix_len, *n_nodes;
   const unsigned long long *mask;
   int B, N, W, Hq, Hkv, g;
+  int npt;                    // combine kernel: nodes per query tile of the partials (0: rows packed without gaps)
   float scale_log2;
   int splits, m_blocks;
   __nv_bfloat16 *out;
@@ -302,14 +304,15 @@ __global__ void attention_combine_kernel(AttnArgs a) {
   const int bh = (int)(gw / rows_total), r = (int)(gw - (int64_t)bh * rows_total);
   const int b = bh / a.Hkv, kvh = bh - b * a.Hkv;
   const int node = r / a.g, qh = r - node * a.g;
+  const int pr = a.npt ? node / a.npt * AT_BM + node % a.npt * a.g + qh : r;      // the packed row
   __nv_bfloat16 *op = a.out + (((int64_t)b * a.N + node) * a.Hq + kvh * a.g + qh) * AT_D + lane * 4;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float lsum = 0.f;
   if (r < a.g * a.n_nodes[b]) {
     float mx = -CUDART_INF_F;
-    for (int s = 0; s < a.splits; ++s) mx = fmaxf(mx, a.part_ml[((int64_t)bh * a.splits + s) * mpad + r].x);
+    for (int s = 0; s < a.splits; ++s) mx = fmaxf(mx, a.part_ml[((int64_t)bh * a.splits + s) * mpad + pr].x);
     for (int s = 0; s < a.splits; ++s) {
-      const int64_t prow = ((int64_t)bh * a.splits + s) * mpad + r;
+      const int64_t prow = ((int64_t)bh * a.splits + s) * mpad + pr;
       const float2 ml = a.part_ml[prow];
       if (ml.x == -CUDART_INF_F) continue;
       const float w = exp2f(ml.x - mx);
@@ -329,9 +332,16 @@ static int attn_m_blocks(const talon_ctx *c) {
   const int g = c->p.n_q_heads / c->p.n_kv_heads;
   return (g * c->p.budget + AT_BM - 1) / AT_BM;
 }
+// the tensor-core kernel packs whole nodes into a query tile
+static int attn_tc_blocks(const talon_ctx *c) {
+  const int g = c->p.n_q_heads / c->p.n_kv_heads;
+  if (g > AT_BM) return attn_m_blocks(c);
+  const int npt = AT_BM / g;
+  return (c->p.budget + npt - 1) / npt;
+}
 
 size_t attention_workspace_elems(const talon_ctx *c, size_t *ml_elems) {
-  const int mb = attn_m_blocks(c);
+  const int mb = attn_tc_blocks(c);
   long long ctas = 2LL * c->p.batch_max * c->p.n_kv_heads * mb;       // room for two key ranges per CTA slot
   if (ctas < 2LL * c->sm_count) ctas = 2LL * c->sm_count;
   *ml_elems = (size_t)ctas * AT_BM;
@@ -357,24 +367,32 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
   a.g = a.Hq / a.Hkv;
   a.scale_log2 = sm_scale * 1.4426950408889634f;
   a.m_blocks = attn_m_blocks(c);
+  a.npt = 0;
   a.out = (__nv_bfloat16 *)out; a.part_o = c->d_attn_o; a.part_ml = c->d_attn_ml;
 
   if (attention_tc_supported(c, stride_t, stride_h, sm_scale)) {
     // tensor-core path: CTAs own two 128-row query tiles and 128-key tiles
+    a.m_blocks = attn_tc_blocks(c);
+    a.npt = AT_BM / a.g;
     const int pairs = (a.m_blocks + 1) / 2;
     const int ctas = pairs * c->B * a.Hkv;
     const int tiles = (max_prefix_len + 127) / 128 + (a.N + 127) / 128;
     int sp = 1;
     if (ctas < c->sm_count) {
-      sp = c->sm_count / ctas;
-      const int by_tiles = (tiles + c->attn_min_tiles - 1) / c->attn_min_tiles;
-      if (sp > by_tiles) sp = by_tiles;
-      if (sp < 1) sp = 1;
-      // up to eight key ranges can merge inside one thread-block cluster, which saves the merge
-      // kernel; a ninth range is worth less than that
-      if (c->attn_cluster && sp > 8 && sp <= c->attn_cluster_cap &&
-          (c->attn_cluster == 2 || (long long)c->B * a.Hkv * a.g * a.N * 8 >= c->attn_cluster_min_rows))
-        sp = 8;
+      // The fewest rounds of key tiles: a CTA of s ranges takes ceil(tiles / s) of them and about three
+      // tiles' worth of prologue and epilogue, merging in a cluster costs another two, the second kernel
+      // (more ranges than a cluster has CTAs, or few rows) four.  Clusters whose CTAs fill SMs only fit a
+      // GPC at a time, so the device says how many it holds: a second round of them doubles the time.
+      const int most = std::min(c->sm_count / ctas, (tiles + c->attn_min_tiles - 1) / c->attn_min_tiles);
+      auto cost = [&](int s) {
+        const bool cluster = s >= 2 && s <= 8 && c->attn_cluster &&
+                             (c->attn_cluster == 2 || (long long)c->B * a.Hkv * a.g * a.N * s >= c->attn_cluster_min_rows);
+        const int held = cluster ? attention_tc_clusters(c, a.m_blocks, s) : 0;
+        const int rounds = held > 0 ? (ctas + held - 1) / held : 1;
+        return rounds * ((tiles + s - 1) / s + 3) + (s == 1 ? 0 : (held > 0 ? 2 : 4));
+      };
+      for (int s = 2; s <= most; ++s)
+        if (cost(s) < cost(sp)) sp = s;
     } else if (ctas % c->sm_count) {
       // More CTAs than SMs and a ragged last wave: halving the key ranges can fill it (512 CTAs on
       // 148 SMs are 4 waves of 257 tiles, 1024 half CTAs are 7 waves of 129).  Cost model in key

@@ -40,21 +40,27 @@ namespace {
 constexpr int TC_BN = 128;                 // keys per tile
 constexpr int TC_D = 128;                  // head dimension
 constexpr int TC_MT = 128;                 // query rows per tile
-constexpr int TC_STAGES = 2;               // K and V ring depth
-constexpr int TC_THREADS = 320;
 constexpr int TC_TILE_BYTES = TC_BN * TC_D * 2;      // 32 KB: one K, V or Q tile
 constexpr int TC_HALF_BYTES = TC_BN * 64 * 2;        // 16 KB: the 64-element half of a tile
-constexpr int TC_NBARS = 16;
-constexpr int TC_SMEM = (2 + 2 * TC_STAGES) * TC_TILE_BYTES + 1024 + TC_NBARS * 8 + 64;
-constexpr uint32_t TC_TMEM_COLS = 512;     // O0 | O1 | S0 | S1, 128 fp32 columns each
+constexpr int TC_NBARS = 24;
+// Per CTA: MT query tiles with four softmax warps each, a producer warp and an MMA warp.  Two query tiles
+// are the rule; a group whose rows fit one tile gets a third K/V stage instead.  With two tiles the block
+// has a third warpgroup so that registers can be split: 216 for the softmax threads (a row of S is 128 of
+// them), 72 for the others, 256 x 216 + 128 x 72 = 384 x 168 in all.
+template <int MT> struct TcShape {
+  static constexpr int STAGES = MT == 1 ? 3 : 2;
+  static constexpr int THREADS = MT == 1 ? 192 : 384;
+  static constexpr int SMEM = (MT + 2 * STAGES) * TC_TILE_BYTES + 1024 + TC_NBARS * 8 + 64;
+  static constexpr uint32_t TMEM_COLS = MT * 256;      // O tiles | S tiles, 128 fp32 columns each
+};
 constexpr float TC_RESCALE_GAP = 8.f;      // raise the reference maximum only beyond 2^8
 constexpr long long TC_WAIT_CYCLES = 4000000000ll;   // ~2 s: far beyond any legitimate wait
 constexpr int TC_XO_PITCH = TC_D + 4;      // floats per row of the partial result a CTA leaves in shared memory
-constexpr int TC_XO_BYTES = 2 * TC_MT * TC_XO_PITCH * 4;        // 256 rows; their (max, sum) pairs follow
-static_assert(TC_XO_BYTES + 2 * TC_MT * 8 <= (2 + 2 * TC_STAGES) * TC_TILE_BYTES, "the partial result reuses the tile buffers");
+constexpr int TC_XO_ROW_BYTES = TC_XO_PITCH * 4;                 // (the rows' (max, sum) pairs follow the rows)
+static_assert(2 * TC_MT * (TC_XO_ROW_BYTES + 8) <= 6 * TC_TILE_BYTES, "the partial result reuses the tile buffers");
 
-// barrier slots
-enum { B_Q = 0, B_KFULL = 1, B_VFULL = 3, B_KEMPTY = 5, B_VEMPTY = 7, B_SFULL = 9, B_PFULL = 11, B_ODONE = 13 };
+// barrier slots: K/V stages (up to three each), S ready, first and second half of P ready, O complete
+enum { B_Q = 0, B_KFULL = 1, B_VFULL = 4, B_KEMPTY = 7, B_VEMPTY = 10, B_SFULL = 13, B_PFULL = 15, B_ODONE = 19 };
 
 struct TcArgs {
   const int64_t *kv_start;
@@ -63,6 +69,7 @@ struct TcArgs {
   const int32_t *prefix_len, *n_nodes;   // prefix_len: the caller's array when early
   const unsigned long long *mask;
   int B, N, W, Hq, Hkv, g;
+  int npt;                     // nodes per query tile, 128 / g (rows from npt * g on hold nothing)
   float scale_log2;
   int splits, m_blocks;
   int early;                   // launched beside the kernel that grows the trees (see the kernel)
@@ -172,6 +179,13 @@ constexpr uint32_t idesc_base = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3
 constexpr uint32_t IDESC_QK = idesc_base;                 // A and B K-major
 constexpr uint32_t IDESC_PV = idesc_base | (1u << 16);    // B MN-major
 
+// true in one lane of a converged warp
+__device__ inline bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xFFFFFFFF;\nselp.b32 %0, 1, 0, p;\n}" : "=r"(p));
+  return p != 0;
+}
+
 __device__ inline float fast_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -228,10 +242,13 @@ __device__ inline void cluster_sync_all() {
 
 }  // namespace
 
-__global__ void __launch_bounds__(TC_THREADS, 1)
+template <int MT>
+__global__ void __launch_bounds__(TcShape<MT>::THREADS, 1)
 tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kp,
                          const __grid_constant__ CUtensorMap map_vp, const __grid_constant__ CUtensorMap map_kt,
                          const __grid_constant__ CUtensorMap map_vt, TcArgs a) {
+  constexpr int STAGES = TcShape<MT>::STAGES, SOFT = MT * 128;      // threads of the softmax warps
+  constexpr int W_LOAD = MT * 4, W_MMA = MT * 4 + 1;
   extern __shared__ unsigned char smem_dyn[];
   __shared__ uint32_t s_tmem_base;
   __shared__ int s_abort;
@@ -248,16 +265,14 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
   // carve shared memory: tiles need 1024-byte alignment for the 128-byte swizzle
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   const uint32_t q_smem = base;
-  const uint32_t k_smem = base + 2 * TC_TILE_BYTES;
-  const uint32_t v_smem = k_smem + TC_STAGES * TC_TILE_BYTES;
-  const uint32_t bars = v_smem + TC_STAGES * TC_TILE_BYTES;
+  const uint32_t k_smem = base + MT * TC_TILE_BYTES;
+  const uint32_t v_smem = k_smem + STAGES * TC_TILE_BYTES;
+  const uint32_t bars = v_smem + STAGES * TC_TILE_BYTES;
   unsigned char *gen_base = smem_dyn + (base - smem_u32(smem_dyn));      // generic pointer to `base`
   auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
 
   const int L = a.prefix_len[b];
-  const int rows_total = a.g * a.N;
-  int nmt = (rows_total - mpair * 2 * TC_MT + TC_MT - 1) / TC_MT;       // query tiles of this CTA with rows
-  nmt = nmt > 2 ? 2 : nmt;
+  const int nmt = min(a.m_blocks - mpair * MT, MT);                      // query tiles of this CTA with rows
 
   const int nP = (L + TC_BN - 1) / TC_BN;
   const int nT = (a.N + TC_BN - 1) / TC_BN;
@@ -270,7 +285,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
   if (tid == 0) {
     s_abort = 0;
     mbar_init(bar(B_Q), 1);
-    for (int s = 0; s < TC_STAGES; ++s) {
+    for (int s = 0; s < STAGES; ++s) {
       mbar_init(bar(B_KFULL + s), 1);
       mbar_init(bar(B_VFULL + s), 1);
       mbar_init(bar(B_KEMPTY + s), 1);
@@ -278,14 +293,15 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar(B_SFULL + i), 1);
-      mbar_init(bar(B_PFULL + i), 128);
+      mbar_init(bar(B_PFULL + 2 * i), 128);
+      mbar_init(bar(B_PFULL + 2 * i + 1), 128);
       mbar_init(bar(B_ODONE + i), 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 9) {          // this warp owns the tensor-memory allocation
+  if (warp == W_MMA) {      // this warp owns the tensor-memory allocation
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)),
-                 "r"(TC_TMEM_COLS) : "memory");
+                 "r"(TcShape<MT>::TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
@@ -294,15 +310,15 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
   const uint32_t tmem = s_tmem_base;
   volatile int *abort_flag = &s_abort;
 
-  if (warp == 8) {
+  if (warp == W_LOAD) {
     // ================= producer =================
+    if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     if (lane == 0 && nt > 0) {
-      const int nodes_per_tile = TC_MT / a.g;
-      mbar_expect_tx(bar(B_Q), (uint32_t)nmt * TC_TILE_BYTES);
+      mbar_expect_tx(bar(B_Q), (uint32_t)(nmt * a.npt * a.g * TC_D * 2));
       for (int i = 0; i < nmt; ++i)
         for (int h = 0; h < 2; ++h)
           tma_load_4d(q_smem + i * TC_TILE_BYTES + h * TC_HALF_BYTES, &map_q, bar(B_Q), h * 64, kvh * a.g,
-                      (mpair * 2 + i) * nodes_per_tile, b);
+                      (mpair * MT + i) * a.npt, b);
       // first cache token of prefix tile tg: a page of TC_BN tokens from the table, or the
       // sequence's contiguous block
       const long long tok0 = a.block_table ? 0ll : a.kv_start[b];
@@ -311,8 +327,8 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       };
       bool ok = true;
       for (int it = 0; it < nt && ok; ++it) {
-        const int s = it % TC_STAGES;
-        const uint32_t par = ((it / TC_STAGES) & 1) ^ 1;
+        const int s = it % STAGES;
+        const uint32_t par = ((it / STAGES) & 1) ^ 1;
         const int tg = t_begin + it;
         ok = mbar_wait(bar(B_KEMPTY + s), par, abort_flag);
         if (!ok) break;
@@ -333,66 +349,91 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       }
     }
     __syncwarp();
-  } else if (warp == 9) {
+  } else if (warp == W_MMA) {
     // ================= MMA issue =================
-    if (lane == 0 && nt > 0) {
-      bool ok = mbar_wait(bar(B_Q), 0, abort_flag);
+    if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    // The whole warp runs the loop and one elected lane issues: with the warp converged the addresses
+    // and descriptors stay in uniform registers.
+    if (nt > 0) {
+      const bool leader = elect_one();
+      constexpr uint32_t T_S = 128 * MT;                 // first S column
+      auto wait = [&](uint32_t bar_addr, uint32_t parity) { return __all_sync(0xFFFFFFFFu, mbar_wait(bar_addr, parity, abort_flag)); };
       auto issue_qk = [&](int i, int s) {
+        const uint64_t qd = desc_kmajor(q_smem + i * TC_TILE_BYTES), kd = desc_kmajor(k_smem + s * TC_TILE_BYTES);
 #pragma unroll
         for (int kk = 0; kk < TC_D / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * TC_HALF_BYTES + (kk & 3) * 32;
-          tc_mma_ss(tmem + 256 + 128 * i, desc_kmajor(q_smem + i * TC_TILE_BYTES + off),
-                    desc_kmajor(k_smem + s * TC_TILE_BYTES + off), IDESC_QK, kk > 0 ? 1u : 0u);
+          const uint32_t off = ((kk >> 2) * TC_HALF_BYTES + (kk & 3) * 32) >> 4;
+          tc_mma_ss(tmem + T_S + 128 * i, qd + off, kd + off, IDESC_QK, kk > 0 ? 1u : 0u);
         }
       };
-      auto issue_pv = [&](int i, int s, bool accumulate) {
+      auto issue_pv = [&](int i, int s, int half, bool accumulate) {
+        const uint64_t vd = desc_mnmajor(v_smem + s * TC_TILE_BYTES);
 #pragma unroll
-        for (int kk = 0; kk < TC_BN / 16; ++kk)
-          tc_mma_ts(tmem + 128 * i, tmem + 256 + 128 * i + kk * 8, desc_mnmajor(v_smem + s * TC_TILE_BYTES + kk * 2048),
-                    IDESC_PV, (accumulate || kk > 0) ? 1u : 0u);
+        for (int kk = 0; kk < TC_BN / 32; ++kk)
+          tc_mma_ts(tmem + 128 * i, tmem + T_S + 128 * i + (half * 4 + kk) * 8, vd + (((half * 4 + kk) * 2048) >> 4),
+                    IDESC_PV, (accumulate || half > 0 || kk > 0) ? 1u : 0u);
       };
-      if (ok) ok = mbar_wait(bar(B_KFULL + 0), 0, abort_flag);
+      bool ok = wait(bar(B_Q), 0);
+      if (ok) ok = wait(bar(B_KFULL + 0), 0);
       if (ok) {
         tc_fence_after();
-        for (int i = 0; i < nmt; ++i) {
-          issue_qk(i, 0);
-          tc_commit(bar(B_SFULL + i));
+        if (leader) {
+          for (int i = 0; i < nmt; ++i) {
+            issue_qk(i, 0);
+            tc_commit(bar(B_SFULL + i));
+          }
+          tc_commit(bar(B_KEMPTY + 0));
         }
-        tc_commit(bar(B_KEMPTY + 0));
       }
+      int s = 0, phase = 0;
       for (int it = 0; it < nt && ok; ++it) {
-        const int s = it % TC_STAGES;
-        ok = mbar_wait(bar(B_VFULL + s), (it / TC_STAGES) & 1, abort_flag);
+        const int s2 = s + 1 == STAGES ? 0 : s + 1, phase2 = s + 1 == STAGES ? phase ^ 1 : phase;
+        ok = wait(bar(B_VFULL + s), phase);
         for (int i = 0; i < nmt && ok; ++i) {
-          ok = mbar_wait(bar(B_PFULL + i), it & 1, abort_flag);
+          // P arrives in two halves of 64 keys: the first half's MMAs run under the exponentials of the second
+          for (int half = 0; half < 2 && ok; ++half) {
+            ok = wait(bar(B_PFULL + 2 * i + half), it & 1);
+            if (!ok) break;
+            tc_fence_after();
+            if (leader) issue_pv(i, s, half, it > 0);
+          }
           if (!ok) break;
-          tc_fence_after();
-          issue_pv(i, s, it > 0);
-          tc_commit(bar(B_ODONE + i));
-          if (i == nmt - 1) tc_commit(bar(B_VEMPTY + s));
+          if (leader) {
+            if (it + 1 == nt) tc_commit(bar(B_ODONE + i));
+            if (i == nmt - 1) tc_commit(bar(B_VEMPTY + s));
+          }
           if (it + 1 < nt) {
-            const int s2 = (it + 1) % TC_STAGES;
             if (i == 0) {
-              ok = mbar_wait(bar(B_KFULL + s2), ((it + 1) / TC_STAGES) & 1, abort_flag);
+              ok = wait(bar(B_KFULL + s2), phase2);
               if (!ok) break;
               tc_fence_after();
             }
-            issue_qk(i, s2);
-            tc_commit(bar(B_SFULL + i));
-            if (i == nmt - 1) tc_commit(bar(B_KEMPTY + s2));
+            if (leader) {
+              issue_qk(i, s2);
+              tc_commit(bar(B_SFULL + i));
+              if (i == nmt - 1) tc_commit(bar(B_KEMPTY + s2));
+            }
           }
         }
+        s = s2;
+        phase = phase2;
       }
     }
     __syncwarp();
+  } else if (MT == 2 && warp > W_MMA) {
+    if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
   } else {
-    // ================= softmax + epilogue: warps 0-3 own query tile 0, warps 4-7 tile 1 =================
+    // ================= softmax + epilogue: warps 4 i .. 4 i + 3 own query tile i =================
+    if (MT == 2) asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
     const int i = warp >> 2;
     const int quarter = warp & 3;
     const int r_local = quarter * 32 + lane;
-    const int R = (mpair * 2 + i) * TC_MT + r_local;            // packed query row
+    const int mt = mpair * MT + i;                              // query tile
+    const int R = mt * TC_MT + r_local;                         // packed query row
+    const int node = mt * a.npt + r_local / a.g, qh = r_local % a.g;
+    const bool in_range = r_local < a.npt * a.g && node < a.N;
     const uint32_t t_lane = tmem + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t t_S = t_lane + 256 + 128 * i;
+    const uint32_t t_S = t_lane + 128 * MT + 128 * i;
     const uint32_t t_O = t_lane + 128 * i;
     // tree size and this row's mask: known before the first tile, or (early) before the tree tile or the epilogue
     int n = 0;
@@ -401,9 +442,9 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     auto load_tree = [&]() {
       if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
       n = __ldcg(a.n_nodes + b);
-      row_valid = R < a.g * n;
+      row_valid = in_range && node < n;
       if (row_valid)
-        for (int w = 0; w < a.W; ++w) mrow[w] = __ldcg(a.mask + ((int64_t)b * a.N + R / a.g) * a.W + w);
+        for (int w = 0; w < a.W; ++w) mrow[w] = __ldcg(a.mask + ((int64_t)b * a.N + node) * a.W + w);
       have_tree = true;
     };
     if (!a.early) load_tree();
@@ -415,15 +456,15 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       const bool tree_tile = tg >= nP;
       if (tree_tile && !have_tree) load_tree();
       const int kvalid = tree_tile ? min(n - (tg - nP) * TC_BN, TC_BN) : min(L - tg * TC_BN, TC_BN);
-      const int s = it % TC_STAGES;
+      const int s = it % STAGES;
       // keys beyond the valid range may hold anything: tile 0's warps clear their V rows so that
       // a zero probability times stale memory cannot produce a NaN
       if (i == 0 && kvalid < TC_BN) {
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(B_VFULL + s), (it / TC_STAGES) & 1, abort_flag));
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(B_VFULL + s), (it / STAGES) & 1, abort_flag));
         if (!ok) break;
         const int zr = max(kvalid, 0) + r_local;
         if (zr < TC_BN) {
-          uint4 *p0 = reinterpret_cast<uint4 *>(gen_base + (2 + TC_STAGES) * TC_TILE_BYTES + s * TC_TILE_BYTES + zr * 128);
+          uint4 *p0 = reinterpret_cast<uint4 *>(gen_base + (MT + STAGES) * TC_TILE_BYTES + s * TC_TILE_BYTES + zr * 128);
           uint4 *p1 = reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(p0) + TC_HALF_BYTES);
 #pragma unroll
           for (int c = 0; c < 8; ++c) { p0[c] = make_uint4(0, 0, 0, 0); p1[c] = make_uint4(0, 0, 0, 0); }
@@ -475,7 +516,22 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       }
       const float m_eff = (m_used == -CUDART_INF_F) ? 0.f : m_used;
 
-      // ---- P = exp2(S * scale - max) as bf16 over S; row sum in four packed chains ----
+      // ---- rare: the reference maximum moved, rescale the accumulator of this row's warp (the MMAs of
+      // the tile before are complete: S of this one was issued after them) ----
+      if (it > 0 && __any_sync(0xFFFFFFFFu, alpha != 1.f)) {
+#pragma unroll
+        for (int c0 = 0; c0 < TC_D; c0 += 32) {
+          uint32_t o[32];
+          tc_ld32(t_O + c0, o);
+          tc_wait_ld();
+#pragma unroll
+          for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha);
+          tc_st32(t_O + c0, o);
+        }
+      }
+
+      // ---- P = exp2(S * scale - max) as bf16 over S, handed over in two halves; row sum in four packed
+      // chains ----
       const unsigned long long scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
       const unsigned long long nmax2 = pack_f32x2(-m_eff, -m_eff);
       unsigned long long sum2[4] = {0ull, 0ull, 0ull, 0ull};          // four pairs of 0.f
@@ -496,6 +552,9 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
           }
         }
         tc_st32(t_S + half * 32, pk);
+        tc_wait_st();
+        tc_fence_before();
+        mbar_arrive(bar(B_PFULL + 2 * i + half));
       }
       float sum4[4];
 #pragma unroll
@@ -506,25 +565,6 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       }
       l_run += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
 
-      // ---- rare: the reference maximum moved, rescale the accumulator of this row's warp ----
-      if (it > 0 && __any_sync(0xFFFFFFFFu, alpha != 1.f)) {
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(B_ODONE + i), (it - 1) & 1, abort_flag));
-        if (ok) {
-          tc_fence_after();
-#pragma unroll
-          for (int c0 = 0; c0 < TC_D; c0 += 32) {
-            uint32_t r[32];
-            tc_ld32(t_O + c0, r);
-            tc_wait_ld();
-#pragma unroll
-            for (int c = 0; c < 32; ++c) r[c] = __float_as_uint(__uint_as_float(r[c]) * alpha);
-            tc_st32(t_O + c0, r);
-          }
-        }
-      }
-      tc_wait_st();
-      tc_fence_before();
-      mbar_arrive(bar(B_PFULL + i));
     }
 
     if (!have_tree) load_tree();
@@ -532,17 +572,16 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     // ---- epilogue: O / l (or the partial result of this key range) ----
     // tcgen05.ld is a warp-wide instruction: every lane of a warp that holds any row takes part
     // in the loads, and only the stores are per lane.
-    if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(B_ODONE + i), (nt - 1) & 1, abort_flag));
-    const bool in_range = R < rows_total;
+    if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(B_ODONE + i), 0, abort_flag));
     if (a.cluster_merge) {
       // The key ranges of this (sequence, head, tile pair) are the CTAs of one cluster: each leaves
       // its partial result in its own shared memory (the tile buffers are free once both query
-      // tiles' MMAs have finished, hence the barrier over the 256 softmax threads) and the merge
+      // tiles' MMAs have finished, hence the barrier over the softmax threads) and the merge
       // reads them from there after the cluster barrier at the end of the kernel.
-      asm volatile("bar.sync 1, 256;" ::: "memory");
+      asm volatile("bar.sync 1, %0;" ::"n"(SOFT) : "memory");
       const int rr = i * TC_MT + r_local;
       float *xo = reinterpret_cast<float *>(gen_base) + (size_t)rr * TC_XO_PITCH;
-      float2 *xml = reinterpret_cast<float2 *>(gen_base + TC_XO_BYTES);
+      float2 *xml = reinterpret_cast<float2 *>(gen_base + SOFT * TC_XO_ROW_BYTES);
       const bool dump = ok && __any_sync(0xFFFFFFFFu, in_range);     // warp-uniform; rows past the last are never read
       if (dump) {
         tc_fence_after();
@@ -559,11 +598,10 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       xml[rr] = (ok && row_valid) ? make_float2(m_used, l_run) : make_float2(-CUDART_INF_F, 0.f);
     } else if (ok && __any_sync(0xFFFFFFFFu, in_range)) {
       tc_fence_after();
-      const int node = in_range ? R / a.g : 0, qh = in_range ? R - node * a.g : 0;
       if (a.splits == 1) {
         const bool live = row_valid && l_run > 0.f;
         const float inv = live ? 1.f / l_run : 0.f;
-        __nv_bfloat16 *op = a.out + (((int64_t)b * a.N + node) * a.Hq + kvh * a.g + qh) * TC_D;
+        __nv_bfloat16 *op = a.out + (((int64_t)b * a.N + (in_range ? node : 0)) * a.Hq + kvh * a.g + qh) * TC_D;
 #pragma unroll
         for (int c0 = 0; c0 < TC_D; c0 += 32) {
           uint32_t r[32];
@@ -596,10 +634,9 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         }
         if (row_valid) a.part_ml[prow] = make_float2(m_used, l_run);
       }
-    } else if (nt == 0 && i < nmt && R < rows_total) {
+    } else if (nt == 0 && i < nmt && in_range) {
       // an empty key range (more splits than tiles): contribute nothing
       if (a.splits == 1) {
-        const int node = R / a.g, qh = R - node * a.g;
         uint4 *op = reinterpret_cast<uint4 *>(a.out + (((int64_t)b * a.N + node) * a.Hq + kvh * a.g + qh) * TC_D);
 #pragma unroll
         for (int c = 0; c < 16; ++c) op[c] = make_uint4(0, 0, 0, 0);
@@ -608,61 +645,84 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         a.part_ml[((int64_t)bh * a.splits + split) * mpad + R] = make_float2(-CUDART_INF_F, 0.f);
       }
     }
+    // (the merge stays inside this branch: past the join the compiler has to get by with the other
+    // warps' registers)
+    if (a.cluster_merge) {
+      // ---- merge of the cluster's partial results: CTA c takes every splits-th share of the packed
+      // rows, one warp per row, lane l the output columns 4l..4l+3.  Two rows at a time with the loads of
+      // all (up to eight) ranges in flight: a trip to a peer's shared memory is most of a microsecond, and
+      // with four loads in flight the merge was 5 us of a short prefix's 18. ----
+      cluster_sync_all();
+      {
+        const int S = a.splits;
+        const int share = (SOFT + S - 1) / S;
+        const int r_lo = split * share, r_hi = min(SOFT, r_lo + share);
+        const uint32_t xo0 = smem_u32(gen_base), xml0 = xo0 + (uint32_t)(SOFT * TC_XO_ROW_BYTES);
+        const int rpt = a.npt * a.g;
+        for (int r0 = r_lo + warp; r0 < r_hi; r0 += 2 * (SOFT / 32)) {
+          int rr[2], rnode[2];
+          bool live[2];
+          float2 ml[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            rr[u] = r0 + u * (SOFT / 32);
+            const int mt = mpair * MT + rr[u] / TC_MT, rl = rr[u] % TC_MT;
+            rnode[u] = mt * a.npt + rl / a.g;
+            live[u] = rr[u] < r_hi && rl < rpt && rnode[u] < a.N;
+            ml[u] = live[u] && lane < S ? cluster_ld_f2(cluster_map(xml0 + (uint32_t)rr[u] * 8u, (uint32_t)lane))
+                                        : make_float2(-CUDART_INF_F, 0.f);
+          }
+          float w[2], lsum[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            float gm = ml[u].x;
+#pragma unroll
+            for (int o = 4; o; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xFFFFFFFFu, gm, o));
+            w[u] = (ml[u].x == -CUDART_INF_F) ? 0.f : fast_exp2(ml[u].x - gm);     // an empty range has no row to read
+            lsum[u] = w[u] * ml[u].y;
+#pragma unroll
+            for (int o = 4; o; o >>= 1) lsum[u] += __shfl_xor_sync(0xFFFFFFFFu, lsum[u], o);
+            lsum[u] = __shfl_sync(0xFFFFFFFFu, lsum[u], 0);
+          }
+          float4 o4[2][8];
+          float ws[2][8];
+#pragma unroll
+          for (int sidx = 0; sidx < 8; ++sidx)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              ws[u][sidx] = __shfl_sync(0xFFFFFFFFu, w[u], sidx);
+              o4[u][sidx] = ws[u][sidx] != 0.f
+                                ? cluster_ld_f4(cluster_map(xo0 + ((uint32_t)rr[u] * TC_XO_PITCH + (uint32_t)lane * 4u) * 4u, (uint32_t)sidx))
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            if (!live[u]) continue;
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int sidx = 0; sidx < 8; ++sidx) {
+              acc.x += ws[u][sidx] * o4[u][sidx].x; acc.y += ws[u][sidx] * o4[u][sidx].y;
+              acc.z += ws[u][sidx] * o4[u][sidx].z; acc.w += ws[u][sidx] * o4[u][sidx].w;
+            }
+            const float inv = lsum[u] > 0.f ? 1.f / lsum[u] : 0.f;
+            uint2 packed;
+            packed.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+            packed.y = pack_bf16x2(acc.z * inv, acc.w * inv);
+            *reinterpret_cast<uint2 *>(a.out + (((int64_t)b * a.N + rnode[u]) * a.Hq + kvh * a.g + rr[u] % TC_MT % a.g) * TC_D +
+                                       lane * 4) = packed;
+          }
+        }
+      }
+      cluster_sync_all();                    // nobody leaves while a peer may still read its shared memory
+    }
   }
+  if (a.cluster_merge && warp >= SOFT / 32) { cluster_sync_all(); cluster_sync_all(); }      // with the two of the merge
 
   tc_fence_before();
   __syncthreads();
-  if (a.cluster_merge) {
-    // ---- merge of the cluster's partial results: CTA c takes every splits-th share of the 256
-    // packed rows, one warp per row, lane l the output columns 4l..4l+3 ----
-    cluster_sync_all();
-    if (warp < 8) {
-      const int S = a.splits;
-      const int share = (2 * TC_MT + S - 1) / S;
-      const int r_lo = split * share, r_hi = min(2 * TC_MT, r_lo + share);
-      const uint32_t xo0 = smem_u32(gen_base), xml0 = smem_u32(gen_base + TC_XO_BYTES);
-      for (int rr = r_lo + warp; rr < r_hi; rr += 8) {
-        const int Rm = mpair * 2 * TC_MT + rr;
-        if (Rm >= rows_total) break;
-        const float2 ml = lane < S ? cluster_ld_f2(cluster_map(xml0 + (uint32_t)rr * 8u, (uint32_t)lane))
-                                   : make_float2(-CUDART_INF_F, 0.f);
-        float gm = ml.x;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xFFFFFFFFu, gm, o));
-        const float w = (ml.x == -CUDART_INF_F) ? 0.f : fast_exp2(ml.x - gm);    // an empty range has no row to read
-        float lsum = w * ml.y;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xFFFFFFFFu, lsum, o);
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        const uint32_t row_off = xo0 + ((uint32_t)rr * TC_XO_PITCH + (uint32_t)lane * 4u) * 4u;
-        for (int s0 = 0; s0 < S; s0 += 4) {        // the loads of four ranges go out before any is used
-          float ws[4];
-          float4 o4[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int sidx = s0 + u;
-            ws[u] = __shfl_sync(0xFFFFFFFFu, w, sidx & 31);
-            if (sidx >= S) ws[u] = 0.f;
-            o4[u] = ws[u] != 0.f ? cluster_ld_f4(cluster_map(row_off, (uint32_t)sidx)) : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            acc.x += ws[u] * o4[u].x; acc.y += ws[u] * o4[u].y; acc.z += ws[u] * o4[u].z; acc.w += ws[u] * o4[u].w;
-          }
-        }
-        const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
-        const int node = Rm / a.g, qh = Rm - node * a.g;
-        uint2 packed;
-        packed.x = pack_bf16x2(acc.x * inv, acc.y * inv);
-        packed.y = pack_bf16x2(acc.z * inv, acc.w * inv);
-        *reinterpret_cast<uint2 *>(a.out + (((int64_t)b * a.N + node) * a.Hq + kvh * a.g + qh) * TC_D + lane * 4) = packed;
-      }
-    }
-    cluster_sync_all();                    // nobody leaves while a peer may still read its shared memory
-  }
-  if (warp == 9) {
+  if (warp == W_MMA) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TcShape<MT>::TMEM_COLS) : "memory");
   }
   if (tid == 0 && s_abort) atomicOr(a.status, STATUS_TIMEOUT);
 }
@@ -707,29 +767,55 @@ bool encode_bf16(CUtensorMap *m, const void *ptr, int rank, const cuuint64_t *di
 bool attention_tc_supported(const talon_ctx *c, int64_t stride_t, int64_t stride_h, float sm_scale) {
   const int g = c->p.n_q_heads / c->p.n_kv_heads;
   if (c->p.head_dim != 128 || c->p.budget > 128) return false;
-  if (g < 1 || g > 128 || (128 % g) != 0) return false;
+  if (g < 1 || g > 128) return false;
   if (!(sm_scale > 0.f)) return false;                     // the lazy maximum assumes a positive scale
   if (stride_t < 128 || stride_h < 1) return false;
   return encode_fn() != nullptr;
 }
 
 talon_status attention_tc_setup() {
-  return cudaFuncSetAttribute(tree_attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM) ==
-                 cudaSuccess ? TALON_OK : TALON_ERR_CUDA;
+  return cudaFuncSetAttribute(tree_attention_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcShape<1>::SMEM) == cudaSuccess &&
+                 cudaFuncSetAttribute(tree_attention_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcShape<2>::SMEM) ==
+                     cudaSuccess
+             ? TALON_OK : TALON_ERR_CUDA;
+}
+
+// How many clusters of `splits` CTAs (one per key range, a whole SM each) the device can hold at once; 0: it
+// cannot place one.  The SMs of a cluster share a GPC, so this is less than SMs / splits.
+int attention_tc_clusters(talon_ctx *c, int m_blocks, int splits) {
+  if (splits < 2 || splits > 8) return 0;
+  const bool one = m_blocks == 1;
+  int &known = c->attn_clusters[one ? 0 : 1][splits];
+  if (known < 0) {
+    cudaLaunchConfig_t q = {};
+    q.gridDim = dim3(1, splits, 1);
+    q.blockDim = dim3(one ? TcShape<1>::THREADS : TcShape<2>::THREADS);
+    q.dynamicSmemBytes = one ? TcShape<1>::SMEM : TcShape<2>::SMEM;
+    cudaLaunchAttribute qa[1];
+    qa[0].id = cudaLaunchAttributeClusterDimension;
+    qa[0].val.clusterDim.x = 1; qa[0].val.clusterDim.y = (unsigned)splits; qa[0].val.clusterDim.z = 1;
+    q.attrs = qa; q.numAttrs = 1;
+    int n = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, one ? tree_attention_tc_kernel<1> : tree_attention_tc_kernel<2>, &q);
+    if (e != cudaSuccess) cudaGetLastError();
+    known = e == cudaSuccess ? n : 0;
+  }
+  return known;
 }
 
 talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *q, const void *kp, const void *vp,
                                  const void *kt, const void *vt, const int64_t *kv_start, const int32_t *block_table,
                                  int bt_stride, int64_t stride_t,
                                  int64_t stride_h, int64_t kv_tokens, int max_prefix_len, float sm_scale, void *out,
-                                 int splits, int m_blocks, cudaStream_t st, int *merged_in_kernel, const int32_t *early_prefix) {
+                                 int splits, int m_blocks, cudaStream_t st, int *merged_in_kernel,
+                                 const int32_t *early_prefix) {
   *merged_in_kernel = 0;
-  const int N = c->p.budget, Hq = c->p.n_q_heads, Hkv = c->p.n_kv_heads, g = Hq / Hkv, B = c->B;
+  const int N = c->p.budget, Hq = c->p.n_q_heads, Hkv = c->p.n_kv_heads, g = Hq / Hkv, B = c->B, npt = 128 / g;
   CUtensorMap mq, mkp, mvp, mkt, mvt;
   {
     const cuuint64_t dims[4] = {128, (cuuint64_t)Hq, (cuuint64_t)N, (cuuint64_t)B};
     const cuuint64_t str[3] = {256, (cuuint64_t)Hq * 256, (cuuint64_t)N * Hq * 256};
-    const cuuint32_t box[4] = {64, (cuuint32_t)g, (cuuint32_t)(128 / g), 1};
+    const cuuint32_t box[4] = {64, (cuuint32_t)g, (cuuint32_t)npt, 1};
     if (!encode_bf16(&mq, q, 4, dims, str, box)) return TALON_ERR_CUDA;
   }
   {
@@ -749,39 +835,27 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
   a.early = early_prefix != nullptr;
   a.prefix_len = early_prefix ? early_prefix : c->d_prefix_len; a.n_nodes = t->n_nodes;
   a.mask = (const unsigned long long *)t->mask;
-  a.B = B; a.N = N; a.W = c->W; a.Hq = Hq; a.Hkv = Hkv; a.g = g;
+  a.B = B; a.N = N; a.W = c->W; a.Hq = Hq; a.Hkv = Hkv; a.g = g; a.npt = npt;
   a.scale_log2 = sm_scale * 1.4426950408889634f;
   a.splits = splits; a.m_blocks = m_blocks;
   a.out = (__nv_bfloat16 *)out; a.part_o = c->d_attn_o; a.part_ml = c->d_attn_ml; a.status = c->d_status;
   (void)max_prefix_len;
+  const bool one = m_blocks == 1;
+  auto kernel = one ? tree_attention_tc_kernel<1> : tree_attention_tc_kernel<2>;
+  const int threads = one ? TcShape<1>::THREADS : TcShape<2>::THREADS, smem = one ? TcShape<1>::SMEM : TcShape<2>::SMEM;
   dim3 grid((m_blocks + 1) / 2, splits, B * Hkv);
   // Two to eight key ranges: they are launched as one thread-block cluster and merge their partial
   // results through distributed shared memory, if the device can place such a cluster (asked once
   // per cluster size; a cluster of full-SM CTAs needs that many SMs free in one GPC).
-  a.cluster_merge = 0;
   // (few rows: the second kernel is cheaper than a cluster launch and two cluster barriers)
   const long long merge_rows = (long long)B * Hkv * g * N * splits;
-  if ((c->attn_cluster == 2 || (c->attn_cluster == 1 && merge_rows >= c->attn_cluster_min_rows)) && splits >= 2 &&
-      splits <= 8) {
-    cudaLaunchConfig_t q = {};
-    q.gridDim = grid; q.blockDim = dim3(TC_THREADS); q.dynamicSmemBytes = TC_SMEM; q.stream = st;
-    cudaLaunchAttribute qa[1];
-    qa[0].id = cudaLaunchAttributeClusterDimension;
-    qa[0].val.clusterDim.x = 1; qa[0].val.clusterDim.y = (unsigned)splits; qa[0].val.clusterDim.z = 1;
-    q.attrs = qa; q.numAttrs = 1;
-    if (c->attn_cluster_ok[splits] < 0) {
-      int n = 0;
-      const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, tree_attention_tc_kernel, &q);
-      if (e != cudaSuccess) cudaGetLastError();
-      c->attn_cluster_ok[splits] = (e == cudaSuccess && n >= 1) ? 1 : 0;
-    }
-    a.cluster_merge = c->attn_cluster_ok[splits];
-  }
+  a.cluster_merge = (c->attn_cluster == 2 || (c->attn_cluster == 1 && merge_rows >= c->attn_cluster_min_rows)) &&
+                    attention_tc_clusters(c, m_blocks, splits) > 0;
   {
     LaunchTimer lt(c, TALON_K_ATTENTION, st);
     if (a.cluster_merge) {
       cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = grid; cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = TC_SMEM; cfg.stream = st;
+      cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
       cudaLaunchAttribute attr[2];
       attr[0].id = cudaLaunchAttributeClusterDimension;
       attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = (unsigned)splits; attr[0].val.clusterDim.z = 1;
@@ -789,10 +863,10 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
       attr[1].val.programmaticStreamSerializationAllowed = 1;
       cfg.attrs = attr;
       cfg.numAttrs = (c->pdl == 1 || (c->pdl < 0 && (c->B <= PDL_AUTO_BATCH || early_prefix))) ? 2 : 1;
-      cudaLaunchKernelEx(&cfg, tree_attention_tc_kernel, mq, mkp, mvp, mkt, mvt, a);
+      cudaLaunchKernelEx(&cfg, kernel, mq, mkp, mvp, mkt, mvt, a);
       *merged_in_kernel = 1;
     } else {
-      launch_kernel_pdl(c, early_prefix != nullptr, tree_attention_tc_kernel, grid, dim3(TC_THREADS), TC_SMEM, st, mq, mkp, mvp, mkt, mvt, a);
+      launch_kernel_pdl(c, early_prefix != nullptr, kernel, grid, dim3(threads), smem, st, mq, mkp, mvp, mkt, mvt, a);
     }
   }
   if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
