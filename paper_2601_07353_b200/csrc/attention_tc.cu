@@ -50,6 +50,8 @@ constexpr int TC_NBARS = 24;
 template <int MT> struct TcShape {
   static constexpr int STAGES = MT == 1 ? 3 : 2;
   static constexpr int THREADS = MT == 1 ? 192 : 384;
+  static constexpr int LAUNCH_REGS = 168, SOFT_REGS = 216, OTHER_REGS = 72;      // the split: MT == 2 only
+  static_assert(MT == 1 || 256 * SOFT_REGS + 128 * OTHER_REGS <= THREADS * LAUNCH_REGS, "setmaxnreg would wait for good");
   static constexpr int SMEM = (MT + 2 * STAGES) * TC_TILE_BYTES + 1024 + TC_NBARS * 8 + 64;
   static constexpr uint32_t TMEM_COLS = MT * 256;      // O tiles | S tiles, 128 fp32 columns each
 };
@@ -312,7 +314,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
 
   if (warp == W_LOAD) {
     // ================= producer =================
-    if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TcShape<2>::OTHER_REGS));
     if (lane == 0 && nt > 0) {
       mbar_expect_tx(bar(B_Q), (uint32_t)(nmt * a.npt * a.g * TC_D * 2));
       for (int i = 0; i < nmt; ++i)
@@ -351,7 +353,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     __syncwarp();
   } else if (warp == W_MMA) {
     // ================= MMA issue =================
-    if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TcShape<2>::OTHER_REGS));
     // The whole warp runs the loop and one elected lane issues: with the warp converged the addresses
     // and descriptors stay in uniform registers.
     if (nt > 0) {
@@ -421,10 +423,10 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     }
     __syncwarp();
   } else if (MT == 2 && warp > W_MMA) {
-    if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TcShape<2>::OTHER_REGS));
   } else {
     // ================= softmax + epilogue: warps 4 i .. 4 i + 3 own query tile i =================
-    if (MT == 2) asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+    if (MT == 2) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TcShape<2>::SOFT_REGS));
     const int i = warp >> 2;
     const int quarter = warp & 3;
     const int r_local = quarter * 32 + lane;
@@ -774,6 +776,9 @@ bool attention_tc_supported(const talon_ctx *c, int64_t stride_t, int64_t stride
 }
 
 talon_status attention_tc_setup() {
+  // (a register split beyond what the block was launched with would never be granted)
+  cudaFuncAttributes at;
+  if (cudaFuncGetAttributes(&at, tree_attention_tc_kernel<2>) != cudaSuccess || at.numRegs != TcShape<2>::LAUNCH_REGS) return TALON_ERR_CUDA;
   return cudaFuncSetAttribute(tree_attention_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcShape<1>::SMEM) == cudaSuccess &&
                  cudaFuncSetAttribute(tree_attention_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcShape<2>::SMEM) ==
                      cudaSuccess
