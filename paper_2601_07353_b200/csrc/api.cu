@@ -141,9 +141,14 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
   c->exp_grid = c->sm_count * talon::EXP_CTAS_PER_SM;
   c->rows_cap = p->batch_max * (p->budget - 1);
   if (c->rows_cap < p->batch_max * p->budget) c->rows_cap = p->batch_max * p->budget;
+  // rows of several steps of talon_loop: as many steps as about 2048 rows are, eight at most
+  c->ahead = 2048 / c->rows_cap;
+  if (c->ahead < 1) c->ahead = 1;
+  if (c->ahead > 8) c->ahead = 8;
+  c->rows_cap *= c->ahead;
   c->items_cap = c->exp_grid + c->rows_cap;
 
-  const size_t nrow = (size_t)p->batch_max * p->budget;
+  const size_t nrow = (size_t)p->batch_max * p->budget * c->ahead;
   // One allocation holds the whole workspace (an allocation is a trip to the driver, tens to hundreds of
   // microseconds, and a program may make a context per model or per request class); what has to start
   // at zero comes first.
@@ -171,7 +176,7 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     take(&c->d_growing, bm);
     take(&c->d_depth_at, bm);
     take(&c->d_target_tok, nrow);
-    take(&c->d_samp_ms, nrow * talon::EXP_MAX_SPLITS);
+    take(&c->d_samp_ms, nrow / c->ahead * talon::EXP_MAX_SPLITS);
     take(&c->d_attn_o, c->attn_o_elems);
     take(&c->d_attn_ml, c->attn_ml_elems);
     if (pass == 0 && cudaMalloc(&c->d_arena, total) != cudaSuccess) break;
@@ -219,6 +224,9 @@ static talon_status check_accept(const talon_ctx *c, const talon_tree *t, const 
   if (!c || !tree_complete(t) || !accept_len || !accept_nodes || !bonus_tok) return TALON_ERR_INVALID_ARG;
   return check_rows(c, target_logits, row_stride);
 }
+
+// Whether a step may prepare the rows of all its node slots in one pass (timed launches are reported per layer).
+static bool rows_at_once(const talon_ctx *c) { return c->step_rows && c->k_cap <= 32 && !(c->ev && !c->ev_paused); }
 
 // Whether somebody is capturing the stream's work into a graph (or it cannot be told).
 static bool being_captured(cudaStream_t st) {
@@ -406,16 +414,40 @@ talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_
   // a caller that captures the loop gets the layered launch sequence, as talon_step's callers do
   const bool layered = being_captured((cudaStream_t)stream);
   const char *qb = static_cast<const char *>(q), *ktb = static_cast<const char *>(k_tree), *vtb = static_cast<const char *>(v_tree);
+  // (the same condition as in step_enqueue, whose argument checks follow)
+  const bool ahead = !layered && n_layers > 0 && rows_at_once(c) && B >= 1 && B <= c->p.batch_max && n_steps > 1;
+  if (ahead) {
+    talon_status r = check_reset(c, t, root_tok, prefix_len, B);
+    if (r == TALON_OK) r = check_rows(c, draft_logits, draft_row_stride);
+    if (r == TALON_OK) r = check_accept(c, t, target_logits, target_row_stride, accept_len, accept_nodes, bonus_tok);
+    if (r != TALON_OK) return r;
+    c->B = B;
+  }
+  const bool batched = ahead && talon::loop_rows_possible(c, n_layers);
   for (int s = 0; s < n_steps; ++s) {
     // step s reads its own slice of the stand-ins for the two model forwards; the tree, the cache,
     // the prefix lengths and the roots are the state the steps hand on to one another on the device
     const void *qs = qb + 2 * q_step_stride * s, *kts = ktb + 2 * kv_tree_step_stride * s, *vts = vtb + 2 * kv_tree_step_stride * s;
     int32_t *al = accept_len + result_step_stride * s, *an = accept_nodes + result_step_stride * (c->p.max_depth + 1) * s;
     int32_t *bt = bonus_tok + result_step_stride * s;
-    talon_status r = step_enqueue(c, t, B, root_tok, prefix_len, draft_logits + draft_step_stride * s, draft_row_stride,
-                                  n_layers, qs, k_prefix, v_prefix, kts, vts, kv_start, kv_tokens, kv_stride_t, kv_stride_h,
-                                  max_prefix_len, sm_scale, out, target_logits + target_step_stride * s, target_row_stride,
-                                  target_tok, al, an, bt, stream, layered);
+    talon_status r = TALON_OK;
+    if (batched) {
+      const int within = s % c->ahead;
+      if (within == 0)
+        r = talon::launch_loop_rows(c, draft_logits + draft_step_stride * s, draft_row_stride, draft_step_stride, n_layers,
+                                    target_logits + target_step_stride * s, target_row_stride, target_step_stride,
+                                    n_steps - s < c->ahead ? n_steps - s : c->ahead, (cudaStream_t)stream);
+      if (r == TALON_OK)
+        r = talon::launch_loop_grow(c, t, root_tok, prefix_len, n_layers, within, target_tok, al, an, bt, (cudaStream_t)stream);
+      if (r == TALON_OK)
+        r = attention_checked(c, t, qs, k_prefix, v_prefix, kts, vts, kv_start, kv_tokens, kv_stride_t, kv_stride_h,
+                              max_prefix_len, sm_scale, out, stream, prefix_len);
+    } else {
+      r = step_enqueue(c, t, B, root_tok, prefix_len, draft_logits + draft_step_stride * s, draft_row_stride,
+                       n_layers, qs, k_prefix, v_prefix, kts, vts, kv_start, kv_tokens, kv_stride_t, kv_stride_h,
+                       max_prefix_len, sm_scale, out, target_logits + target_step_stride * s, target_row_stride,
+                       target_tok, al, an, bt, stream, layered);
+    }
     if (r == TALON_OK)
       r = talon_commit(c, t, al, an, bt, kts, vts, k_prefix, v_prefix, kv_start, kv_limit, kv_tokens, kv_stride_t,
                        kv_stride_h, prefix_len, root_tok, counters, stream);
@@ -522,7 +554,7 @@ static talon_status step_enqueue(talon_ctx *c, const talon_tree *t, int32_t B, c
   talon_status r = TALON_OK;
   bool closed = false, accepted = false;
   // (timed launches are reported per layer, so they take the layered sequence too)
-  if (!layered && c->step_rows && c->k_cap <= 32 && !(c->ev && !c->ev_paused) && n_layers > 0) {
+  if (!layered && n_layers > 0 && rows_at_once(c)) {
     r = check_reset(c, t, root_tok, prefix_len, B);
     if (r == TALON_OK) r = check_rows(c, draft_logits, draft_row_stride);
     if (r == TALON_OK) r = check_accept(c, t, target_logits, target_row_stride, accept_len, accept_nodes, bonus_tok);

@@ -28,6 +28,8 @@ struct RowPassArgs {
   const float *draft, *target;        // [B, N] rows
   int64_t draft_stride, target_stride;
   int B, N, V, k, key_stride;
+  int step_B;                         // sequences per step; the B ones are those of B / step_B steps
+  int64_t draft_step, target_step;    // elements from one step's rows to the next one's
   int r0, r1;                         // node slots of this round, per sequence
   int t1;                             // target rows of slots r0 .. t1-1 (t1 = r0: none)
   int draft_ctas;                     // CTAs 0 .. draft_ctas-1 take draft rows, the others target rows
@@ -216,15 +218,17 @@ row_pass_kernel(RowPassArgs a) {
     const int node = a.r0 + j;
     const size_t slot = (size_t)b * a.N + node;
     const int end = min(a.V, start + len);
+    const int step = b < a.step_B ? 0 : b / a.step_B;
+    const int64_t lrow = (int64_t)slot - (int64_t)step * a.step_B * a.N;
     if (!is_draft) {
       if (start < end)
-        argmax_chunk(a.target + (int64_t)slot * a.target_stride, start, end, a.best + slot, a.row_bad + slot, s_pool);
+        argmax_chunk(a.target + step * a.target_step + lrow * a.target_stride, start, end, a.best + slot, a.row_bad + slot, s_pool);
       continue;
     }
     // a node below the root is gated when every layer but the first is; deeper Top-K layers are not told apart here
     const bool gated = a.init_layers == 0 || (a.init_layers == 1 && node > 0);
     const int item = cta + row;
-    if (!stream_chunk<false>(sh, a.draft + (int64_t)slot * a.draft_stride, start, end, k, k, gated, ln_mu, (size_t)item, res, wt)) return;
+    if (!stream_chunk<false>(sh, a.draft + step * a.draft_step + lrow * a.draft_stride, start, end, k, k, gated, ln_mu, (size_t)item, res, wt)) return;
 
     // the barrier orders this CTA's chunk results before thread 0's device-scope release; whoever
     // brings the row's last elements acquires and merges the row
@@ -314,7 +318,7 @@ grow_kernel(GrowArgs a) {
   // prefix while the trees grow, and what it reads for that has to be complete.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   const int b = blockIdx.x, k = a.k, N = a.N;
   const size_t nb = (size_t)b * N;
   int d = 0, lo = 0, hi = 1;
@@ -504,94 +508,151 @@ static void step_bounds(const talon_ctx *c, int n_layers, int *expandable, int *
   *nodes = (int)(sum + f < N ? sum + f : N);
 }
 
-talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len,
-                              const float *draft, int64_t draft_stride, int n_layers, const float *target,
-                              int64_t target_stride, int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes,
-                              int32_t *bonus_tok, cudaStream_t st, bool *accepted) {
+// How far a step's first round goes and whether the target rows come along.
+struct StepPlan { int expandable, nodes, first; bool with_target; };
+static StepPlan plan_step(const talon_ctx *c, int n_layers) {
   const talon_params &p = c->p;
-  const int B = c->B, N = p.budget, k = c->k_cap;
-  int expandable, nodes;
-  step_bounds(c, n_layers, &expandable, &nodes);
+  StepPlan s;
+  step_bounds(c, n_layers, &s.expandable, &s.nodes);
   // One round with the target rows alongside is the quickest way even where a part of the rows is read
   // for nothing (the pass then runs at the copy bandwidth; a round of its own costs about 20 us: pass
   // start-up, hand-off, growth).  A tree of few layers cannot get near a large budget, though: on
   // confident rows a layer adds one node, on flat ones K, seldom more.  Where the slots beyond
   // 1 + 7/8 K D would cost more to read than a second round, the first round stops there, the second
   // takes the rest for the trees that do go on, and the target rows wait for the trees' sizes.
-  const double row_bytes = 4.0 * p.vocab * B;           // of one slot of every sequence
-  int first = 1 + p.root_topk * n_layers * 7 / 8;
-  if (c->step_first_rows > 0) first = c->step_first_rows;
-  else if (row_bytes * 2.0 * (expandable - first) < STEP_SPLIT_BYTES) first = expandable;
-  if (first > expandable) first = expandable;
-  const bool with_target = first == expandable;
-  *accepted = with_target;
+  const double row_bytes = 4.0 * p.vocab * c->B;          // of one slot of every sequence
+  s.first = 1 + p.root_topk * n_layers * 7 / 8;
+  if (c->step_first_rows > 0) s.first = c->step_first_rows;
+  else if (row_bytes * 2.0 * (s.expandable - s.first) < STEP_SPLIT_BYTES) s.first = s.expandable;
+  if (s.first > s.expandable) s.first = s.expandable;
+  s.with_target = s.first == s.expandable;
+  return s;
+}
+
+static RowPassArgs row_pass_args(talon_ctx *c, const float *draft, int64_t draft_stride, const float *target, int64_t target_stride) {
+  const talon_params &p = c->p;
   RowPassArgs ra;
-  ra.draft = draft; ra.draft_stride = draft_stride;
-  ra.target = with_target ? target : nullptr; ra.target_stride = target_stride;
-  ra.B = B; ra.N = N; ra.V = p.vocab; ra.k = k; ra.key_stride = c->key_stride;
-  ra.init_layers = p.init_layers; ra.log_mu = c->log_mu; ra.spans = span_table(p.vocab, k, c->expand_max_split);
+  ra.draft = draft; ra.draft_stride = draft_stride; ra.target = target; ra.target_stride = target_stride;
+  ra.B = ra.step_B = c->B; ra.draft_step = ra.target_step = 0;
+  ra.N = p.budget; ra.V = p.vocab; ra.k = c->k_cap; ra.key_stride = c->key_stride;
+  ra.init_layers = p.init_layers; ra.log_mu = c->log_mu; ra.spans = span_table(p.vocab, c->k_cap, c->expand_max_split);
+  ra.growing = nullptr;
   ra.part_keys = c->d_part_keys; ra.part_ms = c->d_part_ms; ra.row_keys = c->d_row_keys; ra.row_lp = c->d_row_score;
   ra.row_count = c->d_row_count; ra.best = c->d_argmax; ra.row_bad = c->d_row_bad; ra.status = c->d_status;
+  return ra;
+}
+
+// Launches the pass over slots ra.r0 .. ra.r1 - 1 (draft) and ra.r0 .. ra.t1 - 1 (target).
+static talon_status launch_row_pass(talon_ctx *c, RowPassArgs &ra, cudaStream_t st) {
+  // CTAs per row: as many as the grid holds, no row cut into less than a CTA step per chunk
+  const long long dr = (long long)ra.B * (ra.r1 - ra.r0), tr = (long long)ra.B * (ra.t1 - ra.r0);
+  const int cut = (int)ra.spans.most;
+  int grid = c->row_grid;
+  if (tr == 0) {
+    if (dr * cut < grid) grid = (int)(dr * cut);
+    ra.draft_ctas = grid;
+  } else {
+    int gd = (int)(grid * dr / (dr + tr));
+    const int target_cut = (ra.V + 8 * EXP_TILE - 1) / (8 * EXP_TILE);
+    if (dr * cut + tr * target_cut <= grid) {
+      // small rows: the draft rows are cut as finely as a single layer's would be (the same partial
+      // sums, so the same scores to the last bit), the target rows share the rest of the grid
+      gd = (int)(dr * cut);
+      const int most = (ra.V + EXP_TILE - 1) / EXP_TILE, st_cut = (int)((grid - gd) / tr);
+      grid = gd + (int)(tr * (st_cut < most ? st_cut : most));
+    } else if (dr + tr <= grid) {        // whole chunks per row for both kinds
+      const int both = (int)(grid / ((dr + tr + 1) / 2));
+      int sd = (both + 1) / 2, stt = both / 2;
+      if (stt < 1) stt = 1;
+      if (sd > cut) sd = cut;
+      gd = (int)(dr * sd);
+      grid = gd + (int)(tr * stt);
+    }
+    ra.draft_ctas = gd;
+  }
+  if (grid < 1) grid = 1;
+  {
+    LaunchTimer lt(c, TALON_K_EXPAND_ROWS, st);
+    launch_kernel_pdl(c, false, row_pass_for(c), dim3(grid), dim3(EXP_THREADS), row_pass_smem(c, ra.growing && ra.B > 32), st, ra);
+  }
+  if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
+  c->launches += 1;
+  return TALON_OK;
+}
+
+static GrowArgs grow_args(talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len, int n_layers,
+                          int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes, int32_t *bonus_tok, bool walk) {
+  const talon_params &p = c->p;
   GrowArgs ga;
   ga.t = *t; ga.root_tok = root_tok; ga.prefix_len = prefix_len; ga.prefix_copy = c->d_prefix_len;
-  ga.lo_stride = p.max_depth + 2; ga.B = B; ga.N = N; ga.W = c->W; ga.k = k; ga.key_stride = c->key_stride;
+  ga.lo_stride = p.max_depth + 2; ga.B = c->B; ga.N = p.budget; ga.W = c->W; ga.k = c->k_cap; ga.key_stride = c->key_stride;
   ga.n_layers = n_layers; ga.max_depth = p.max_depth; ga.root_topk = p.root_topk; ga.init_layers = p.init_layers;
   ga.log_mu = c->log_mu;
   ga.row_keys = c->d_row_keys; ga.row_lp = c->d_row_score; ga.growing = c->d_growing; ga.depth_at = c->d_depth_at;
   ga.row_count = c->d_row_count; ga.status = c->d_status;
-  ga.best = with_target ? c->d_argmax : nullptr; ga.row_bad = c->d_row_bad;
+  ga.best = walk ? c->d_argmax : nullptr; ga.row_bad = c->d_row_bad;
   ga.target_tok = target_tok ? target_tok : c->d_target_tok;
   ga.accept_len = accept_len; ga.accept_nodes = accept_nodes; ga.bonus_tok = bonus_tok;
+  return ga;
+}
 
-  int done = 0;
-  for (int r = 0; done < expandable; ++r) {
-    const int upto = r == 0 ? first : expandable;
-    ra.r0 = done; ra.r1 = upto; ra.t1 = with_target ? nodes : done;
+static talon_status launch_grow(talon_ctx *c, GrowArgs &ga, cudaStream_t st) {
+  LaunchTimer lt(c, TALON_K_SELECT, st);
+  launch_kernel(c, grow_kernel_for(c), dim3(ga.B), dim3(GROW_THREADS), grow_smem_bytes(ga.rows, ga.k, ga.N), st, ga);
+  if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
+  c->launches += 1;
+  return TALON_OK;
+}
+
+talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len,
+                              const float *draft, int64_t draft_stride, int n_layers, const float *target,
+                              int64_t target_stride, int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes,
+                              int32_t *bonus_tok, cudaStream_t st, bool *accepted) {
+  const StepPlan plan = plan_step(c, n_layers);
+  *accepted = plan.with_target;
+  RowPassArgs ra = row_pass_args(c, draft, draft_stride, plan.with_target ? target : nullptr, target_stride);
+  GrowArgs ga = grow_args(c, t, root_tok, prefix_len, n_layers, target_tok, accept_len, accept_nodes, bonus_tok, plan.with_target);
+  for (int r = 0, done = 0; done < plan.expandable; ++r) {
+    const int upto = r == 0 ? plan.first : plan.expandable;
+    ra.r0 = done; ra.r1 = upto; ra.t1 = plan.with_target ? plan.nodes : done;
     ra.growing = r ? c->d_growing : nullptr;
     ra.clear_status = r == 0;
-    // CTAs per row: as many as the grid holds, no row cut into less than a CTA step per chunk
-    const long long dr = (long long)B * (upto - done), tr = (long long)B * (ra.t1 - done);
-    const int cut = (int)ra.spans.most;
-    int grid = c->row_grid;
-    if (tr == 0) {
-      if (dr * cut < grid) grid = (int)(dr * cut);
-      ra.draft_ctas = grid;
-    } else {
-      int gd = (int)(grid * dr / (dr + tr));
-      const int target_cut = (p.vocab + 8 * EXP_TILE - 1) / (8 * EXP_TILE);
-      if (dr * cut + tr * target_cut <= grid) {
-        // small rows: the draft rows are cut as finely as a single layer's would be (the same partial
-        // sums, so the same scores to the last bit), the target rows share the rest of the grid
-        gd = (int)(dr * cut);
-        const int most = (p.vocab + EXP_TILE - 1) / EXP_TILE, st_cut = (int)((grid - gd) / tr);
-        grid = gd + (int)(tr * (st_cut < most ? st_cut : most));
-      } else if (dr + tr <= grid) {        // whole chunks per row for both kinds
-        const int both = (int)(grid / ((dr + tr + 1) / 2));
-        int sd = (both + 1) / 2, stt = both / 2;
-        if (stt < 1) stt = 1;
-        if (sd > cut) sd = cut;
-        gd = (int)(dr * sd);
-        grid = gd + (int)(tr * stt);
-      }
-      ra.draft_ctas = gd;
-    }
-    if (grid < 1) grid = 1;
-    {
-      LaunchTimer lt(c, TALON_K_EXPAND_ROWS, st);
-      launch_kernel(c, row_pass_for(c), dim3(grid), dim3(EXP_THREADS), row_pass_smem(c, r > 0 && B > 32), st, ra);
-    }
-    if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
+    talon_status s = launch_row_pass(c, ra, st);
+    if (s != TALON_OK) return s;
     ga.first = r == 0; ga.rows = upto;
-    {
-      LaunchTimer lt(c, TALON_K_SELECT, st);
-      launch_kernel_pdl(c, true, grow_kernel_for(c), dim3(B), dim3(GROW_THREADS), grow_smem_bytes(upto, k, N), st, ga);
-    }
-    if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
-    c->launches += 2;
+    s = launch_grow(c, ga, st);
+    if (s != TALON_OK) return s;
     done = upto;
   }
   c->layers_run = n_layers;
   return TALON_OK;
+}
+
+bool loop_rows_possible(const talon_ctx *c, int n_layers) { return c->ahead > 1 && plan_step(c, n_layers).with_target; }
+
+// One pass for several steps: at small batches a step's rows are a few dozen MB, too few to fill the
+// pass's start and end (four steps of 2 sequences: 4 x 31 us against 80).
+talon_status launch_loop_rows(talon_ctx *c, const float *draft, int64_t draft_stride, int64_t draft_step, int n_layers,
+                              const float *target, int64_t target_stride, int64_t target_step, int steps, cudaStream_t st) {
+  const StepPlan plan = plan_step(c, n_layers);
+  RowPassArgs ra = row_pass_args(c, draft, draft_stride, target, target_stride);
+  ra.B = c->B * steps; ra.draft_step = draft_step; ra.target_step = target_step;
+  ra.r0 = 0; ra.r1 = plan.expandable; ra.t1 = plan.nodes;
+  ra.clear_status = 1;
+  return launch_row_pass(c, ra, st);
+}
+
+talon_status launch_loop_grow(talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len, int n_layers,
+                              int step, int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes, int32_t *bonus_tok,
+                              cudaStream_t st) {
+  const StepPlan plan = plan_step(c, n_layers);
+  GrowArgs ga = grow_args(c, t, root_tok, prefix_len, n_layers, target_tok, accept_len, accept_nodes, bonus_tok, true);
+  const size_t at = (size_t)step * c->B * c->p.budget;
+  ga.row_keys += at * c->key_stride; ga.row_lp += at * c->key_stride;
+  ga.row_count += at; ga.best += at; ga.row_bad += at;
+  ga.first = 1; ga.rows = plan.expandable;
+  c->layers_run = n_layers;
+  return launch_grow(c, ga, st);
 }
 
 }  // namespace talon

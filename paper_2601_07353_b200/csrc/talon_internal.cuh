@@ -121,6 +121,7 @@ struct talon_ctx {
   unsigned int *d_seq_count;         // [batch_max]              chunks finished per sequence (fused kernel)
   int fused_grid;                    // CTAs of the fused kernel at full width
   // whole-step growth (grow_step.cu)
+  int ahead;                         // steps of talon_loop whose rows one pass prepares (the workspace holds them)
   int row_grid;                      // CTAs of the row pass at full width
   int32_t *d_growing, *d_depth_at;   // [batch_max] a sequence's tree still grows; layer it stopped at
   unsigned int *d_row_bad;           // [batch_max * N] NaN in a target row (zero between calls)
@@ -167,14 +168,12 @@ __device__ __forceinline__ void pdl_enter() {
 }
 
 // Launches `kernel` so that it may be scheduled while its predecessor in the stream drains
-// (the kernel itself waits in pdl_enter()); a plain launch when ctx->pdl is off.  In automatic mode
-// (-1) it is used for batches of at most PDL_AUTO_BATCH sequences: there the grids are small and the
-// overlapped launch latency is a gain, while at larger batches the early-scheduled CTAs of the next
-// kernel take SM slots from the running one.
+// (the kernel itself waits in pdl_enter()); a plain launch when ctx->pdl is off.  A step is a chain of
+// dependent kernels, most of them short, so the overlap of launch latency pays at every batch size
+// (sampling verification of 8 sequences: 252 -> 242 us).  The exception, chain = false, is the row pass of a
+// whole step: its CTAs, waiting beside the attention of the step before, slow that down (270 -> 278 us at the
+// shape with 64 query heads), so it is launched this way up to PDL_AUTO_BATCH sequences only.
 constexpr int PDL_AUTO_BATCH = 4;
-// `chain` marks the launches of a chain of short dependent kernels (the expansion layers): there
-// the overlap of launch latency pays at every batch size (a layer that finds every tree full costs
-// little more than its launch), while behind the long verification kernels it does not.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel_pdl(const talon_ctx *c, bool chain, void (*kernel)(KArgs...), dim3 grid, dim3 block,
                                      size_t smem, cudaStream_t st, Args &&...args) {
@@ -193,7 +192,7 @@ inline cudaError_t launch_kernel_pdl(const talon_ctx *c, bool chain, void (*kern
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(const talon_ctx *c, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                  cudaStream_t st, Args &&...args) {
-  return launch_kernel_pdl(c, false, kernel, grid, block, smem, st, static_cast<Args &&>(args)...);
+  return launch_kernel_pdl(c, true, kernel, grid, block, smem, st, static_cast<Args &&>(args)...);
 }
 
 // Brackets one kernel launch with a pair of CUDA events on the launching stream when timing
@@ -227,6 +226,14 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
                               const float *draft, int64_t draft_stride, int n_layers, const float *target,
                               int64_t target_stride, int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes,
                               int32_t *bonus_tok, cudaStream_t st, bool *accepted);
+// The same for talon_loop, whose steps' rows are all there at the start: rows of `steps` steps (ctx->ahead at most)
+// in one pass, then per step the growth and the walk.  False from loop_rows_possible: step by step instead.
+bool loop_rows_possible(const talon_ctx *c, int n_layers);
+talon_status launch_loop_rows(talon_ctx *c, const float *draft, int64_t draft_stride, int64_t draft_step, int n_layers,
+                              const float *target, int64_t target_stride, int64_t target_step, int steps, cudaStream_t st);
+talon_status launch_loop_grow(talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len, int n_layers,
+                              int step, int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes, int32_t *bonus_tok,
+                              cudaStream_t st);
 talon_status launch_build(talon_ctx *c, const talon_tree *t, uint8_t *dense, cudaStream_t st);
 talon_status launch_prune(talon_ctx *c, const talon_tree *t, int keep, cudaStream_t st);
 talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, const void *kp,
