@@ -41,70 +41,64 @@ struct WalkArgs {
   const int32_t *prefix_len;
 };
 
-// The closing pass over the node slots of sequence b (what build_tree_kernel writes there):
-// positions of the tree's nodes, sentinels in the unused slots.  The walk reads none of it.
-__device__ __forceinline__ void close_slots(const WalkArgs &a, int b, int first, int step) {
-  const size_t nb = (size_t)b * a.N;
-  const int n = a.t.n_nodes[b];
-  const int L = a.prefix_len[b];
-  for (int i = first; i < a.N; i += step) {
-    if (i < n) {
-      a.t.position[nb + i] = L + a.t.depth[nb + i];
-    } else {
-      a.t.token[nb + i] = -1;
-      a.t.parent[nb + i] = -1;
-      a.t.depth[nb + i] = -1;
-      a.t.position[nb + i] = -1;
-      a.t.score[nb + i] = -CUDART_INF;
-      for (int w = 0; w < a.W; ++w) a.t.mask[(nb + i) * a.W + w] = ((i >> 6) == w) ? (1ull << (i & 63)) : 0ull;
-    }
-  }
-}
+struct WalkShared {
+  int tgt[MAX_BUDGET];      // the target's choice after each node
+  int next[MAX_BUDGET];     // the child that carries it (siblings have different tokens), or -1
+};
 
-// One warp decodes the keys of sequence b and walks its tree.
-__device__ __forceinline__ void accept_walk(const WalkArgs &a, int b, int lane) {
+// A CTA of at least MAX_BUDGET threads decodes the keys of sequence b and walks its tree: one thread per
+// node, everything a node needs fetched in one trip to L2 (following the path through global memory took
+// three dependent trips, 2 us, per accepted node), then links in shared memory.  With close_tree it also
+// writes what build_tree_kernel writes.
+__device__ __forceinline__ void accept_walk(const WalkArgs &a, int b, WalkShared &sh) {
   const size_t nb = (size_t)b * a.N;
+  const int i = threadIdx.x;
+  const bool slot = i < a.N;
   const int n = a.t.n_nodes[b];
-  if (a.close_tree) {
-    // layers that were never launched: their offsets close at the tree's size (the walk reads them)
-    for (int i = a.layers_run + 2 + lane; i < a.lo_stride; i += 32) a.t.layer_off[b * a.lo_stride + i] = n;
-    __syncwarp();
-  }
-  for (int i = lane; i < a.N; i += 32) {
-    const unsigned long long k = __ldcg(&a.best[nb + i]);
+  const int L = a.close_tree ? a.prefix_len[b] : 0;
+  const bool live = slot && i < n;
+  const unsigned long long key = slot ? __ldcg(&a.best[nb + i]) : 0ull;
+  const int par = live ? a.t.parent[nb + i] : -1, tok = live ? a.t.token[nb + i] : -1;
+  const int dep = live && a.close_tree ? a.t.depth[nb + i] : -1;
+  const int want = live && key != 0ull ? (int)key_tok(key) : -1;
+  if (slot) {
     a.best[nb + i] = 0ull;                                  // leave the workspace clean
-    a.target_tok[nb + i] = (i < n && k != 0ull) ? (int32_t)key_tok(k) : -1;
+    a.target_tok[nb + i] = want;
+    sh.tgt[i] = want;
+    sh.next[i] = -1;
   }
-  __syncwarp();
-  int cur = 0, len = 0;
-  if (lane == 0) a.accept_nodes[(size_t)b * (a.max_depth + 1)] = 0;
-  for (int d = 0; d < a.max_depth; ++d) {
-    const int want = a.target_tok[nb + cur];
-    const int lo = a.t.layer_off[b * a.lo_stride + d + 1];
-    const int hi = a.t.layer_off[b * a.lo_stride + d + 2];
-    int found = -1;
-    for (int c0 = lo; c0 < hi; c0 += 32) {
-      const int c = c0 + lane;
-      const bool hit = c < hi && a.t.parent[nb + c] == cur && a.t.token[nb + c] == want;
-      const unsigned m = __ballot_sync(FULL, hit);
-      if (m) { found = c0 + __ffs(m) - 1; break; }
-    }
-    if (found < 0) break;
-    cur = found;
-    ++len;
-    if (lane == 0) a.accept_nodes[(size_t)b * (a.max_depth + 1) + len] = cur;
-  }
-  for (int i = len + 1 + lane; i <= a.max_depth; i += 32) a.accept_nodes[(size_t)b * (a.max_depth + 1) + i] = -1;
-  if (lane == 0) {
+  __syncthreads();
+  if (par >= 0 && par < n && tok == sh.tgt[par]) sh.next[par] = i;
+  __syncthreads();
+  int32_t *path = a.accept_nodes + (size_t)b * (a.max_depth + 1);
+  if (i == 0) {
+    int cur = 0, len = 0;
+    path[0] = 0;
+    for (int c = sh.next[0]; c >= 0 && len < a.max_depth; c = sh.next[c]) { cur = c; path[++len] = c; }
     a.accept_len[b] = len;
-    a.bonus_tok[b] = a.target_tok[nb + cur];
+    a.bonus_tok[b] = sh.tgt[cur];
+    for (int d = len + 1; d <= a.max_depth; ++d) path[d] = -1;
   }
+  if (!a.close_tree) return;
+  if (live) {
+    a.t.position[nb + i] = L + dep;
+  } else if (slot) {
+    a.t.token[nb + i] = -1;
+    a.t.parent[nb + i] = -1;
+    a.t.depth[nb + i] = -1;
+    a.t.position[nb + i] = -1;
+    a.t.score[nb + i] = -CUDART_INF;
+    for (int w = 0; w < a.W; ++w) a.t.mask[(nb + i) * a.W + w] = ((i >> 6) == w) ? (1ull << (i & 63)) : 0ull;
+  }
+  // layers that were never launched: their offsets close at the tree's size
+  for (int d = a.layers_run + 2 + i; d < a.lo_stride; d += blockDim.x) a.t.layer_off[b * a.lo_stride + d] = n;
 }
 
 __global__ void __launch_bounds__(EXP_THREADS)
 target_argmax_kernel(ArgmaxArgs a, WalkArgs wa, unsigned int *seq_done, int fold) {
   __shared__ unsigned long long s_key[EXP_WARPS];
   __shared__ int s_walk;
+  __shared__ WalkShared s_tree;
   pdl_enter();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_items = a.B * a.N * a.splits;
@@ -193,66 +187,33 @@ target_argmax_kernel(ArgmaxArgs a, WalkArgs wa, unsigned int *seq_done, int fold
     if (fold) {
       __syncthreads();
       if (s_walk >= 0) {
-        if (warp == 0) accept_walk(wa, s_walk, lane);
-        else if (wa.close_tree) close_slots(wa, s_walk, tid - 32, EXP_THREADS - 32);   // beside the walk
+        __threadfence();
+        accept_walk(wa, s_walk, s_tree);
       }
     }
   }
 }
 
-// one warp per sequence
-__global__ void accept_walk_kernel(WalkArgs a) {
+// one CTA per sequence
+__global__ void __launch_bounds__(MAX_BUDGET)
+accept_walk_kernel(WalkArgs a) {
+  __shared__ WalkShared s_tree;
   pdl_enter();
-  const int lane = threadIdx.x & 31;
-  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (b >= a.B) return;
-  // the closing pass needs each node's depth: the loads are issued before the walk (a chain of
-  // dependent L2 trips) and their results are used after it
-  constexpr int PER = (MAX_BUDGET + 31) / 32;
-  int dep[PER];
-  int L = 0, n = 0;
-  if (a.close_tree) {
-    n = a.t.n_nodes[b];
-    L = a.prefix_len[b];
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int i = lane + 32 * k;
-      dep[k] = (i < n) ? a.t.depth[(size_t)b * a.N + i] : -1;
-    }
-  }
-  accept_walk(a, b, lane);
-  if (a.close_tree) {
-    const size_t nb = (size_t)b * a.N;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int i = lane + 32 * k;
-      if (i >= a.N) continue;
-      if (i < n) {
-        a.t.position[nb + i] = L + dep[k];
-      } else {
-        a.t.token[nb + i] = -1;
-        a.t.parent[nb + i] = -1;
-        a.t.depth[nb + i] = -1;
-        a.t.position[nb + i] = -1;
-        a.t.score[nb + i] = -CUDART_INF;
-        for (int w = 0; w < a.W; ++w) a.t.mask[(nb + i) * a.W + w] = ((i >> 6) == w) ? (1ull << (i & 63)) : 0ull;
-      }
-    }
-  }
+  accept_walk(a, blockIdx.x, s_tree);
 }
-
 
 talon_status launch_accept(talon_ctx *c, const talon_tree *t, const float *target_logits, int64_t row_stride,
                            int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes,
                            int32_t *bonus_tok, cudaStream_t st, bool close_tree) {
   const int rows = c->B * c->p.budget;
-  // Fewer rows than CTAs: as many chunks per row as keep rows x chunks within the grid (rounded
-  // down), so that every CTA has one chunk and the last chunk's CTA can do the walk.
+  // Small passes: as many chunks per row as keep rows x chunks within the grid (rounded down), so that
+  // every CTA has one chunk and the last chunk's CTA can do the walk.  Larger ones: finer, about four
+  // chunks per CTA -- with one per CTA and row the SMs that got fewer wait for the others (a third of
+  // the slots may hold no node besides): 364 slots, 240 nodes of 128256, 45 us with whole rows, 27 us
+  // this way.  The line between them is where a CTA's chunk would exceed 64 KB.
   LayerGeom g = make_geom(rows, c->p.vocab, rows <= c->exp_grid ? c->exp_grid - rows + 1 : c->exp_grid);
-  // More rows than half the grid: with one chunk per CTA round the last round leaves most SMs
-  // idle (960 rows on 592 CTAs are 1.6 rounds); finer chunks keep every CTA streaming to the end.
-  if ((long long)rows * g.splits > c->exp_grid && c->argmax_oversplit > 1)
-    g = make_geom(rows, c->p.vocab, c->exp_grid * c->argmax_oversplit);
+  const bool coarse = (long long)rows * g.splits > c->exp_grid || g.chunk_len > 16384;
+  if (coarse && c->argmax_oversplit > 1) g = make_geom(rows, c->p.vocab, c->exp_grid * c->argmax_oversplit);
   ArgmaxArgs aa;
   aa.logits = target_logits; aa.row_stride = row_stride; aa.n_nodes = t->n_nodes;
   aa.B = c->B; aa.N = c->p.budget; aa.V = c->p.vocab;
@@ -275,10 +236,9 @@ talon_status launch_accept(talon_ctx *c, const talon_tree *t, const float *targe
   if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
   c->launches += 1;
   if (fold) return TALON_OK;
-  const int warps_per_block = 4;
   {
     LaunchTimer lt(c, TALON_K_WALK, st);
-    launch_kernel(c, accept_walk_kernel, dim3((c->B + warps_per_block - 1) / warps_per_block), dim3(warps_per_block * 32), 0, st, wa);
+    launch_kernel(c, accept_walk_kernel, dim3(c->B), dim3(MAX_BUDGET), 0, st, wa);
   }
   if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
   c->launches += 1;

@@ -1007,6 +1007,7 @@ __device__ __forceinline__ void merge_row_wide(const ChunkOut &res, size_t item0
 // ---------------------------------------------------------------------------------------
 // Selection of one layer (Eq. 4, Eq. 5, truncation to the budget)
 // ---------------------------------------------------------------------------------------
+constexpr int SELECT_LIST = 256;      // candidates that are ranked in one list
 // Called by all THREADS threads of a CTA.  A frontier of F rows (32 NQ at most), row j's candidates
 // sorted by score: score(j, i) for i < k (-inf: none), tok(j, i) its token.  At most `want` candidates
 // are taken, the best ones, after the gate p(u) >= mu * max p when not `init`; append(slot, j, i, tok,
@@ -1025,7 +1026,8 @@ __device__ __forceinline__ int layer_select(int F, int k, int ke, int want, bool
   const int gl = lane & (G - 1), gbase = lane & ~(G - 1);
   const unsigned gmask = (G == 32 ? FULL : ((1u << (G & 31)) - 1u)) << gbase;
   constexpr int per_pass = THREADS / G;
-  constexpr int FEW = KMAX <= 16 ? 256 / KMAX : 0;
+  __shared__ double s_list[SELECT_LIST];                // eligible scores in (row, position) order
+  __shared__ unsigned char s_row[SELECT_LIST];
   constexpr int PASSES = 32 * NQ / per_pass > 0 ? 32 * NQ / per_pass : 1;
   const int my_row = tid / G;
 
@@ -1082,7 +1084,36 @@ __device__ __forceinline__ int layer_select(int F, int k, int ke, int want, bool
     for (int q = 1; q < NQ; ++q) if ((j >> 5) == q) x = v[q];
     return __shfl_sync(FULL, x, j & 31);
   };
-  if (total > want) {
+  if (total > want && total <= SELECT_LIST) {
+    // ---- truncation of a small pool: the eligible scores go into one list, in the order that decides
+    // ties, and every score's betters are counted by as many threads as there are to spare (searching
+    // the rows for each candidate took 4 us at 100 candidates, this 1 us) ----
+    for (int j0 = 0; j0 < F; j0 += per_pass) {
+      const int j = j0 + my_row;
+      const int c0 = of_row(cnt, j), o0 = of_row(off, j);
+      if (j < F && gl < c0) {
+        s_list[o0 + gl] = score(j, gl);
+        s_row[o0 + gl] = (unsigned char)j;
+      }
+    }
+    for (int j = tid; j < F; j += THREADS) s_cnt[j] = 0;
+    __syncthreads();
+    const int per = total <= THREADS / 8 ? 8 : (total <= THREADS / 4 ? 4 : (total <= THREADS / 2 ? 2 : 1));
+    const int p = tid / per, part = tid & (per - 1);
+    const double s = p < total ? s_list[p] : 0.0;
+    int better = 0;
+#pragma unroll 4
+    for (int o = part; o < total; o += per) {
+      const double v = s_list[o];
+      better += (int)(v > s) | ((int)(v == s) & (int)(o < p));
+    }
+    for (int o = 1; o < per; o <<= 1) better += __shfl_xor_sync(FULL, better, o);
+    if (part == 0 && p < total && better < want) atomicAdd(&s_cnt[s_row[p]], 1);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) cnt[q] = q * 32 + lane < F ? s_cnt[q * 32 + lane] : 0;
+    scan();
+  } else if (total > want) {
     // ---- truncation: rank by (score desc, parent asc, token asc) among the eligible; rows are sorted
     // that way already, so a rank is a sum of binary searches in the rows' prefixes ----
     if (warp == 0)
@@ -1099,19 +1130,6 @@ __device__ __forceinline__ int layer_select(int F, int k, int ke, int want, bool
       if (j < F && gl < s_cnt[j]) {
         const double s = score(j, gl);
         int rank = gl;
-        // (a small pool is counted through, loads in flight together; a large one searched row by row)
-        if (F <= FEW) {
-          rank = 0;
-          for (int o = 0; o < F; ++o) {
-            const int h = s_cnt[o];
-            double v[KMAX];
-#pragma unroll
-            for (int i = 0; i < KMAX; ++i) v[i] = score(o, min(i, k - 1));
-#pragma unroll
-            for (int i = 0; i < KMAX; ++i)          // (& and |: no branch per candidate)
-              rank += (int)(i < h) & ((int)(v[i] > s) | ((int)(v[i] == s) & ((int)(o < j) | ((int)(o == j) & (int)(i < gl)))));
-          }
-        } else
         for (int o = 0; o < F && rank < want; ++o) {
           int l = 0, h = o == j ? 0 : s_cnt[o];
           while (l < h) {
