@@ -49,11 +49,12 @@ constexpr int TC_NBARS = 24;
 // them), 72 for the others, 256 x 216 + 128 x 72 = 384 x 168 in all.
 template <int MT> struct TcShape {
   static constexpr int STAGES = MT == 1 ? 3 : 2;
-  static constexpr int THREADS = MT == 1 ? 192 : 384;
+  static constexpr int THREADS = MT == 1 ? 224 : 384;
   static constexpr int LAUNCH_REGS = 168, SOFT_REGS = 216, OTHER_REGS = 72;      // the split: MT == 2 only
   static_assert(MT == 1 || 256 * SOFT_REGS + 128 * OTHER_REGS <= THREADS * LAUNCH_REGS, "setmaxnreg would wait for good");
   static constexpr int SMEM = (MT + 2 * STAGES) * TC_TILE_BYTES + 1024 + TC_NBARS * 8 + 64;
-  static constexpr uint32_t TMEM_COLS = MT * 256;      // O tiles | S tiles, 128 fp32 columns each
+  // tensor memory: O of each tile (128 fp32 columns), S (128, one for both tiles), P of each tile (64: 128 bf16)
+  static constexpr uint32_t TMEM_COLS = 512, COL_S = 128 * MT, COL_P = 128 * MT + 128;
 };
 constexpr float TC_RESCALE_GAP = 8.f;      // raise the reference maximum only beyond 2^8
 constexpr long long TC_WAIT_CYCLES = 4000000000ll;   // ~2 s: far beyond any legitimate wait
@@ -61,8 +62,9 @@ constexpr int TC_XO_PITCH = TC_D + 4;      // floats per row of the partial resu
 constexpr int TC_XO_ROW_BYTES = TC_XO_PITCH * 4;                 // (the rows' (max, sum) pairs follow the rows)
 static_assert(2 * TC_MT * (TC_XO_ROW_BYTES + 8) <= 6 * TC_TILE_BYTES, "the partial result reuses the tile buffers");
 
-// barrier slots: K/V stages (up to three each), S ready, first and second half of P ready, O complete
-enum { B_Q = 0, B_KFULL = 1, B_VFULL = 4, B_KEMPTY = 7, B_VEMPTY = 10, B_SFULL = 13, B_PFULL = 15, B_ODONE = 19 };
+// barrier slots: K/V stages (up to three each); per query tile S ready, first and second half of P ready, P.V
+// complete; S read out
+enum { B_Q = 0, B_KFULL = 1, B_VFULL = 4, B_KEMPTY = 7, B_VEMPTY = 10, B_SFULL = 13, B_PFULL = 15, B_ODONE = 19, B_SFREE = 21 };
 
 struct TcArgs {
   const int64_t *kv_start;
@@ -250,7 +252,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                          const __grid_constant__ CUtensorMap map_vp, const __grid_constant__ CUtensorMap map_kt,
                          const __grid_constant__ CUtensorMap map_vt, TcArgs a) {
   constexpr int STAGES = TcShape<MT>::STAGES, SOFT = MT * 128;      // threads of the softmax warps
-  constexpr int W_LOAD = MT * 4, W_MMA = MT * 4 + 1;
+  constexpr int W_LOAD = MT * 4, W_QK = MT * 4 + 1, W_PV = MT * 4 + 2;
   extern __shared__ unsigned char smem_dyn[];
   __shared__ uint32_t s_tmem_base;
   __shared__ int s_abort;
@@ -291,17 +293,18 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       mbar_init(bar(B_KFULL + s), 1);
       mbar_init(bar(B_VFULL + s), 1);
       mbar_init(bar(B_KEMPTY + s), 1);
-      mbar_init(bar(B_VEMPTY + s), 1);
+      mbar_init(bar(B_VEMPTY + s), nmt);           // (each tile's P.V)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar(B_SFULL + i), 1);
-      mbar_init(bar(B_PFULL + 2 * i), 128);
-      mbar_init(bar(B_PFULL + 2 * i + 1), 128);
+      mbar_init(bar(B_PFULL + 2 * i), 4);          // (one arrival per softmax warp)
+      mbar_init(bar(B_PFULL + 2 * i + 1), 4);
       mbar_init(bar(B_ODONE + i), 1);
     }
+    mbar_init(bar(B_SFREE), 4);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == W_MMA) {      // this warp owns the tensor-memory allocation
+  if (warp == W_QK) {       // this warp owns the tensor-memory allocation
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)),
                  "r"(TcShape<MT>::TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -351,79 +354,68 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       }
     }
     __syncwarp();
-  } else if (warp == W_MMA) {
-    // ================= MMA issue =================
+  } else if (warp >= W_QK) {
+    // ================= MMA issue: one warp for Q.K, one per query tile for P.V =================
     if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TcShape<2>::OTHER_REGS));
-    // The whole warp runs the loop and one elected lane issues: with the warp converged the addresses
-    // and descriptors stay in uniform registers.
-    if (nt > 0) {
-      const bool leader = elect_one();
-      constexpr uint32_t T_S = 128 * MT;                 // first S column
-      auto wait = [&](uint32_t bar_addr, uint32_t parity) { return __all_sync(0xFFFFFFFFu, mbar_wait(bar_addr, parity, abort_flag)); };
-      auto issue_qk = [&](int i, int s) {
-        const uint64_t qd = desc_kmajor(q_smem + i * TC_TILE_BYTES), kd = desc_kmajor(k_smem + s * TC_TILE_BYTES);
-#pragma unroll
-        for (int kk = 0; kk < TC_D / 16; ++kk) {
-          const uint32_t off = ((kk >> 2) * TC_HALF_BYTES + (kk & 3) * 32) >> 4;
-          tc_mma_ss(tmem + T_S + 128 * i, qd + off, kd + off, IDESC_QK, kk > 0 ? 1u : 0u);
-        }
-      };
-      auto issue_pv = [&](int i, int s, int half, bool accumulate) {
-        const uint64_t vd = desc_mnmajor(v_smem + s * TC_TILE_BYTES);
-#pragma unroll
-        for (int kk = 0; kk < TC_BN / 32; ++kk)
-          tc_mma_ts(tmem + 128 * i, tmem + T_S + 128 * i + (half * 4 + kk) * 8, vd + (((half * 4 + kk) * 2048) >> 4),
-                    IDESC_PV, (accumulate || half > 0 || kk > 0) ? 1u : 0u);
-      };
-      bool ok = wait(bar(B_Q), 0);
-      if (ok) ok = wait(bar(B_KFULL + 0), 0);
-      if (ok) {
-        tc_fence_after();
-        if (leader) {
-          for (int i = 0; i < nmt; ++i) {
-            issue_qk(i, 0);
-            tc_commit(bar(B_SFULL + i));
-          }
-          tc_commit(bar(B_KEMPTY + 0));
-        }
-      }
-      int s = 0, phase = 0;
+    // A warp that has issued a group of MMAs is held up until nearly all of them have run (about 230
+    // clocks on top of 64 each before it can issue the next group); with the groups coming from three
+    // warps the tensor pipe runs another group meanwhile.  Each warp runs its loop converged and one
+    // elected lane issues, so addresses and descriptors stay in uniform registers.
+    const bool leader = elect_one();
+    constexpr uint32_t COL_S = TcShape<MT>::COL_S, COL_P = TcShape<MT>::COL_P;
+    auto wait = [&](uint32_t bar_addr, uint32_t parity) { return __all_sync(0xFFFFFFFFu, mbar_wait(bar_addr, parity, abort_flag)); };
+    int s = 0, phase = 0;
+    if (warp == W_QK) {
+      bool ok = nt > 0 && wait(bar(B_Q), 0);
+      unsigned free_phase = 0;                           // S is free at first, then whenever a tile's softmax has read it out
       for (int it = 0; it < nt && ok; ++it) {
-        const int s2 = s + 1 == STAGES ? 0 : s + 1, phase2 = s + 1 == STAGES ? phase ^ 1 : phase;
-        ok = wait(bar(B_VFULL + s), phase);
+        ok = wait(bar(B_KFULL + s), phase);
         for (int i = 0; i < nmt && ok; ++i) {
-          // P arrives in two halves of 64 keys: the first half's MMAs run under the exponentials of the second
-          for (int half = 0; half < 2 && ok; ++half) {
-            ok = wait(bar(B_PFULL + 2 * i + half), it & 1);
-            if (!ok) break;
-            tc_fence_after();
-            if (leader) issue_pv(i, s, half, it > 0);
+          if (it > 0 || i > 0) {
+            ok = wait(bar(B_SFREE), free_phase);
+            free_phase ^= 1;
           }
           if (!ok) break;
+          tc_fence_after();
           if (leader) {
-            if (it + 1 == nt) tc_commit(bar(B_ODONE + i));
-            if (i == nmt - 1) tc_commit(bar(B_VEMPTY + s));
-          }
-          if (it + 1 < nt) {
-            if (i == 0) {
-              ok = wait(bar(B_KFULL + s2), phase2);
-              if (!ok) break;
-              tc_fence_after();
+            const uint64_t qd = desc_kmajor(q_smem + i * TC_TILE_BYTES), kd = desc_kmajor(k_smem + s * TC_TILE_BYTES);
+#pragma unroll
+            for (int kk = 0; kk < TC_D / 16; ++kk) {
+              const uint32_t off = ((kk >> 2) * TC_HALF_BYTES + (kk & 3) * 32) >> 4;
+              tc_mma_ss(tmem + COL_S, qd + off, kd + off, IDESC_QK, kk > 0 ? 1u : 0u);
             }
-            if (leader) {
-              issue_qk(i, s2);
-              tc_commit(bar(B_SFULL + i));
-              if (i == nmt - 1) tc_commit(bar(B_KEMPTY + s2));
+            tc_commit(bar(B_SFULL + i));
+            if (i == nmt - 1) tc_commit(bar(B_KEMPTY + s));
+          }
+        }
+        if (++s == STAGES) { s = 0; phase ^= 1; }
+      }
+    } else if (warp - W_PV < nmt) {
+      const int i = warp - W_PV;
+      bool ok = true;
+      for (int it = 0; it < nt && ok; ++it) {
+        ok = wait(bar(B_VFULL + s), phase);
+        // P arrives in two halves of 64 keys: the first half's MMAs run under the exponentials of the second
+        for (int half = 0; half < 2 && ok; ++half) {
+          ok = wait(bar(B_PFULL + 2 * i + half), it & 1);
+          if (!ok) break;
+          tc_fence_after();
+          if (leader) {
+            const uint64_t vd = desc_mnmajor(v_smem + s * TC_TILE_BYTES);
+#pragma unroll
+            for (int kk = 0; kk < TC_BN / 32; ++kk)
+              tc_mma_ts(tmem + 128 * i, tmem + COL_P + 64 * i + (half * 4 + kk) * 8, vd + (((half * 4 + kk) * 2048) >> 4),
+                        IDESC_PV, (it > 0 || half > 0 || kk > 0) ? 1u : 0u);
+            if (half) {
+              tc_commit(bar(B_ODONE + i));
+              tc_commit(bar(B_VEMPTY + s));
             }
           }
         }
-        s = s2;
-        phase = phase2;
+        if (++s == STAGES) { s = 0; phase ^= 1; }
       }
     }
     __syncwarp();
-  } else if (MT == 2 && warp > W_MMA) {
-    if (MT == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TcShape<2>::OTHER_REGS));
   } else {
     // ================= softmax + epilogue: warps 4 i .. 4 i + 3 own query tile i =================
     if (MT == 2) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TcShape<2>::SOFT_REGS));
@@ -435,7 +427,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     const int node = mt * a.npt + r_local / a.g, qh = r_local % a.g;
     const bool in_range = r_local < a.npt * a.g && node < a.N;
     const uint32_t t_lane = tmem + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t t_S = t_lane + 128 * MT + 128 * i;
+    const uint32_t t_S = t_lane + TcShape<MT>::COL_S, t_P = t_lane + TcShape<MT>::COL_P + 64 * i;
     const uint32_t t_O = t_lane + 128 * i;
     // tree size and this row's mask: known before the first tile, or (early) before the tree tile or the epilogue
     int n = 0;
@@ -492,6 +484,9 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       tc_ld32(t_S + 64, r[2]);
       tc_ld32(t_S + 96, r[3]);
       tc_wait_ld();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(B_SFREE));           // S may take the next unit
       if (masked) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -518,8 +513,13 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       }
       const float m_eff = (m_used == -CUDART_INF_F) ? 0.f : m_used;
 
-      // ---- rare: the reference maximum moved, rescale the accumulator of this row's warp (the MMAs of
-      // the tile before are complete: S of this one was issued after them) ----
+      // P of the key tile before has been used up (long ago, as a rule) and O is at rest
+      if (it > 0) {
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(B_ODONE + i), (it - 1) & 1, abort_flag));
+        if (!ok) break;
+        tc_fence_after();
+      }
+      // ---- rare: the reference maximum moved, rescale the accumulator of this row's warp ----
       if (it > 0 && __any_sync(0xFFFFFFFFu, alpha != 1.f)) {
 #pragma unroll
         for (int c0 = 0; c0 < TC_D; c0 += 32) {
@@ -532,7 +532,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         }
       }
 
-      // ---- P = exp2(S * scale - max) as bf16 over S, handed over in two halves; row sum in four packed
+      // ---- P = exp2(S * scale - max) as bf16, handed over in two halves; row sum in four packed
       // chains ----
       const unsigned long long scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
       const unsigned long long nmax2 = pack_f32x2(-m_eff, -m_eff);
@@ -553,10 +553,11 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             pk[q * 16 + (c >> 1)] = pack_bf16x2(p0, p1);
           }
         }
-        tc_st32(t_S + half * 32, pk);
+        tc_st32(t_P + half * 32, pk);
         tc_wait_st();
         tc_fence_before();
-        mbar_arrive(bar(B_PFULL + 2 * i + half));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(B_PFULL + 2 * i + half));
       }
       float sum4[4];
 #pragma unroll
@@ -574,7 +575,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     // ---- epilogue: O / l (or the partial result of this key range) ----
     // tcgen05.ld is a warp-wide instruction: every lane of a warp that holds any row takes part
     // in the loads, and only the stores are per lane.
-    if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(B_ODONE + i), 0, abort_flag));
+    if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(B_ODONE + i), (nt - 1) & 1, abort_flag));
     if (a.cluster_merge) {
       // The key ranges of this (sequence, head, tile pair) are the CTAs of one cluster: each leaves
       // its partial result in its own shared memory (the tile buffers are free once both query
@@ -722,7 +723,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
 
   tc_fence_before();
   __syncthreads();
-  if (warp == W_MMA) {
+  if (warp == W_QK) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TcShape<MT>::TMEM_COLS) : "memory");
   }
