@@ -935,18 +935,46 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
 // The same for WIDE lists, by the whole CTA: the row's k best keys and scores go straight to
 // key_out / score_out [k] (slot 0 of score_out NaN when the row has no softmax).  st: WIDE_STAGE_WORDS
 // words of shared memory.
-constexpr int WIDE_STAGE_WORDS = 2 * FX_LONG_SPLITS * 128 + 4;
-__device__ __forceinline__ void merge_row_wide(const ChunkOut &res, size_t item0, int S, int k, int ke, double ps, u64 *st,
-                                               u64 *key_out, double *score_out, int *status) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int ks = res.key_stride, total = S * ke;
-  u64 *sv = st + FX_LONG_SPLITS * 128;
-  double *s_lse = reinterpret_cast<double *>(sv + FX_LONG_SPLITS * 128);
-  int *s_n = reinterpret_cast<int *>(s_lse + 1);
-  u64 *s_tau = reinterpret_cast<u64 *>(s_lse + 2);
-  for (int i = tid; i < total; i += EXP_THREADS) {
-    const int c = i / ke;
-    st[i] = __ldcg(res.part_keys + (item0 + c) * ks + (i - c * ke));
+// The lists are sorted, so they are merged pairwise in registers, R keys a lane (position r * 32 + lane):
+// eight warps, then four, two, one -- 2 us a row, where collecting the keys above a bound and ranking them
+// by counting took 5 us, and 21 us on gated rows, whose short lists give no bound.
+constexpr int WIDE_STAGE_WORDS = EXP_WARPS * 128 + 2;
+
+// a <- the 32 R largest of a and b, both descending, descending
+template <int R>
+__device__ __forceinline__ void merge_wide(u64 (&a)[R], const u64 (&b)[R], int lane) {
+#pragma unroll
+  for (int r = 0; r < R; ++r) a[r] = umax64(a[r], shfl_u64(b[R - 1 - r], 31 - lane));      // bitonic, the largest
+#pragma unroll
+  for (int j = R / 2; j > 0; j >>= 1)
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if ((r & j) == 0) {
+        const u64 hi = umax64(a[r], a[r + j]), lo = umin64(a[r], a[r + j]);
+        a[r] = hi;
+        a[r + j] = lo;
+      }
+#pragma unroll
+  for (int j = 16; j > 0; j >>= 1)
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const u64 o = shfl_xor_u64(a[r], j);
+      a[r] = ((lane & j) == 0) ? umax64(a[r], o) : umin64(a[r], o);
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void merge_row_wide_n(const ChunkOut &res, size_t item0, int S, int k, int ke, double ps, u64 *st,
+                                                 u64 *key_out, double *score_out, int *status) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ks = res.key_stride;
+  double *s_lse = reinterpret_cast<double *>(st + EXP_WARPS * 128);
+  u64 a[R], b[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int p = r * 32 + lane;
+    a[r] = (2 * warp < S && p < ke) ? __ldcg(res.part_keys + (item0 + 2 * warp) * ks + p) : 0ull;
+    b[r] = (2 * warp + 1 < S && p < ke) ? __ldcg(res.part_keys + (item0 + 2 * warp + 1) * ks + p) : 0ull;
   }
   if (warp == EXP_WARPS - 1) {
     const float2 ms = lane < S ? __ldcg(res.part_ms + item0 + lane) : make_float2(-CUDART_INF_F, 0.f);
@@ -959,49 +987,40 @@ __device__ __forceinline__ void merge_row_wide(const ChunkOut &res, size_t item0
 #pragma unroll
     for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
     const bool finite = (t > 0.0) && (t < CUDART_INF) && (mx < CUDART_INF_F) && (mx > -CUDART_INF_F);
-    if (lane == 0) {
-      *s_lse = finite ? (double)mx + log(t) : CUDART_NAN;
-      *s_n = 0;
-    }
+    if (lane == 0) *s_lse = finite ? (double)mx + log(t) : CUDART_NAN;
   }
-  __syncthreads();
-  if (warp == 0) {
-    // Lower bounds of the row's ke-th best key: S chunks hold ceil(ke / S) keys each at least as large
-    // as the smallest of their ceil(ke / S)-th keys; one chunk alone holds ke at least its ke-th.
-    const int p = (ke + S - 1) / S - 1;
-    u64 low = lane < S ? st[lane * ke + p] : ~0ull, own = lane < S ? st[lane * ke + ke - 1] : 0ull;
+  merge_wide<R>(a, b, lane);
+  static_assert(FX_LONG_SPLITS <= 2 * EXP_WARPS, "two lists a warp");
+#pragma unroll 1
+  for (int half = EXP_WARPS / 2; half > 0; half >>= 1) {
+    if (warp >= half && warp < 2 * half)
 #pragma unroll
-    for (int o = 16; o; o >>= 1) { low = umin64(low, shfl_xor_u64(low, o)); own = umax64(own, shfl_xor_u64(own, o)); }
-    if (lane == 0) *s_tau = umax64(low, own);
-  }
-  __syncthreads();
-  const u64 tau = *s_tau;
-  for (int i = tid; i < total; i += EXP_THREADS) {
-    const u64 key = st[i];
-    if (key != 0ull && key >= tau) sv[atomicAdd(s_n, 1)] = key;
-  }
-  __syncthreads();
-  const int ns = *s_n;
-  const double lse = *s_lse;
-  for (int c0 = 0; c0 < ns; c0 += EXP_THREADS / 4) {                     // four lanes count a key's betters
-    const int ci = c0 + (tid >> 2), q = tid & 3;
-    const u64 key = ci < ns ? sv[ci] : 0ull;
-    int r = 0;
-#pragma unroll 4
-    for (int o = q; o < ns; o += 4) r += (sv[o] > key) ? 1 : 0;
-    r += __shfl_xor_sync(FULL, r, 1);
-    r += __shfl_xor_sync(FULL, r, 2);
-    if (q == 0 && ci < ns && r < ke) {
-      const double s = ps + ((double)key_logit(key) - lse);
-      key_out[r] = key;
-      score_out[r] = lse != lse ? (r == 0 ? CUDART_NAN : -CUDART_INF) : (s == s && s > -CUDART_INF ? s : -CUDART_INF);
+      for (int r = 0; r < R; ++r) st[warp * 128 + r * 32 + lane] = a[r];
+    __syncthreads();
+    if (warp < half) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) b[r] = st[(warp + half) * 128 + r * 32 + lane];
+      merge_wide<R>(a, b, lane);
     }
   }
-  for (int r = min(ns, ke) + tid; r < k; r += EXP_THREADS) {
-    key_out[r] = 0ull;
-    score_out[r] = (r == 0 && lse != lse) ? CUDART_NAN : -CUDART_INF;
+  if (warp == 0) {
+    const double lse = *s_lse;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int p = r * 32 + lane;
+      if (p >= k) continue;
+      const u64 key = p < ke ? a[r] : 0ull;
+      const double sc = ps + ((double)key_logit(key) - lse);
+      key_out[p] = key;
+      score_out[p] = lse != lse ? (p == 0 ? CUDART_NAN : -CUDART_INF) : (key != 0ull && sc == sc && sc > -CUDART_INF ? sc : -CUDART_INF);
+    }
+    if (lane == 0 && lse != lse) atomicOr(status, STATUS_NONFINITE);
   }
-  if (tid == 0 && lse != lse) atomicOr(status, STATUS_NONFINITE);
+}
+__device__ __forceinline__ void merge_row_wide(const ChunkOut &res, size_t item0, int S, int k, int ke, double ps, u64 *st,
+                                               u64 *key_out, double *score_out, int *status) {
+  if (k <= 64) merge_row_wide_n<2>(res, item0, S, k, ke, ps, st, key_out, score_out, status);
+  else merge_row_wide_n<4>(res, item0, S, k, ke, ps, st, key_out, score_out, status);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -296,11 +296,12 @@ __host__ __device__ inline size_t grow_smem_bytes(int rows, int k, int N) {
   return (size_t)grow_pitch(rows) * k * 16 + (size_t)N * (8 + 16 + 12) + MAX_BUDGET * 4 + 32;
 }
 
-// One CTA per sequence, a layer per turn of the loop (layer_select), one barrier each.
+// One CTA per sequence: narrow layers by its first warp, wide ones by all (layer_select).
 template <int NQ, int KMAX>  // frontier rows per lane; k rounded up to 8, 16 or 32
 __global__ void __launch_bounds__(GROW_THREADS)
 grow_kernel(GrowArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ int s_state[4];               // layer, frontier, and how warp 0 left its layers
   const int pitch = grow_pitch(a.rows);
   GrowSmem sm;
   {
@@ -368,11 +369,96 @@ grow_kernel(GrowArgs a) {
   }
   __syncthreads();
 
-  bool paused = false;
-  for (; d < a.n_layers; ++d) {
+  // Most layers are a few rows wide, and those one warp does alone, a lane per candidate: no barrier, no
+  // per-row chains, 400 to 700 clocks a layer where the whole CTA takes 1550 (a chain of 12 layers: 11 us
+  // -> 5).  Wider layers, and those where more candidates pass than the budget takes, go to the CTA.
+  constexpr int PER_ROUND = 32 / KMAX, ROUNDS = 4;      // rows a warp takes at a time, and how often
+  enum { WALK_ON = 0, DONE = 1, PAUSED = 2 };
+  for (;;) {
+    if (tid < 32) {
+      const int sub = lane / KMAX, ci = lane & (KMAX - 1), gbase = sub * KMAX;
+      const unsigned before = gbase ? (1u << gbase) - 1u : 0u;
+      int what = WALK_ON;
+      for (;;) {
+        const int F = hi - lo, n = hi;
+        if (d >= a.n_layers || F <= 0 || n >= N) { what = DONE; break; }
+        if (hi > a.rows) { what = PAUSED; break; }      // the frontier's rows are not all there yet
+        if (F > PER_ROUND * ROUNDS) break;
+        const int R = N - n, ke = min(k, R);            // a parent can place at most R children
+        const bool init = d < a.init_layers;
+        double s[ROUNDS];
+        int tok[ROUNDS];
+        bool bad = false;                               // rows without a softmax
+        u64 head = 0ull;
+#pragma unroll
+        for (int q = 0; q < ROUNDS; ++q) {
+          s[q] = -CUDART_INF;
+          if (q * PER_ROUND >= F) continue;
+          const int j = q * PER_ROUND + sub, at = min(ci, k - 1) * pitch + lo + min(j, F - 1);
+          const double lp = sm.lp[at], ps = sm.score[lo + min(j, F - 1)];
+          tok[q] = (int)key_tok(sm.key[at]);
+          bad |= lp != lp;
+          if (j < F && ci < ke) s[q] = ps + lp;
+          if (s[q] > -CUDART_INF) head = umax64(head, f64_ord(s[q]));
+        }
+        if (__any_sync(FULL, bad)) {                    // this sequence adds nothing any more
+          if (lane == 0) {
+            atomicOr(a.status, STATUS_NONFINITE);
+            a.t.layer_off[b * a.lo_stride + d + 2] = n;
+          }
+          ++d;
+          what = DONE;
+          break;
+        }
+        double thr = -1.7976931348623157e308;           // an impossible candidate (-inf) never passes
+        if (!init) {
+          head = warp_redux_max_u64(head);
+          if (head != 0ull) thr = a.log_mu + f64_unord(head);
+        }
+        unsigned m[ROUNDS];
+        int total = 0;
+#pragma unroll
+        for (int q = 0; q < ROUNDS; ++q) {
+          m[q] = 0u;
+          if (q * PER_ROUND >= F) continue;
+          m[q] = __ballot_sync(FULL, s[q] >= thr);
+          total += __popc(m[q]);
+        }
+        if (total > (init ? min(a.root_topk, R) : R)) break;
+        // append in storage order: (parent asc, token asc)
+        int base = n;
+#pragma unroll
+        for (int q = 0; q < ROUNDS; ++q) {
+          if (q * PER_ROUND >= F) continue;
+          const bool in = (m[q] >> lane) & 1u;
+          const int t = in ? tok[q] : 0x7FFFFFFF;
+          int r = 0;
+#pragma unroll
+          for (int i = 0; i < KMAX; ++i) r += (int)(__shfl_sync(FULL, t, gbase + i) < t);
+          if (in) {
+            const int node = base + __popc(m[q] & before) + r, par = lo + q * PER_ROUND + sub;
+            sm.tok[node] = t;
+            sm.parent[node] = par;
+            sm.depth[node] = d + 1;
+            sm.score[node] = s[q];
+            sm.mask[2 * node] = sm.mask[2 * par] | (node < 64 ? 1ull << node : 0ull);
+            sm.mask[2 * node + 1] = sm.mask[2 * par + 1] | (node >= 64 ? 1ull << (node - 64) : 0ull);
+          }
+          base += __popc(m[q]);
+        }
+        __syncwarp();
+        lo = hi;
+        hi = base;
+        if (lane == 0) a.t.layer_off[b * a.lo_stride + d + 2] = hi;
+        ++d;
+      }
+      if (lane == 0) { s_state[0] = d; s_state[1] = lo; s_state[2] = hi; s_state[3] = what; }
+    }
+    __syncthreads();
+    d = s_state[0]; lo = s_state[1]; hi = s_state[2];
+    if (s_state[3] != WALK_ON) break;
+    // ---- a layer by the whole CTA ----
     const int F = hi - lo, n = hi;
-    if (F <= 0 || n >= N) break;
-    if (hi > a.rows) { paused = true; break; }          // the frontier's rows are not all there yet
     const int R = N - n, ke = min(k, R);                // a parent can place at most R children
     bool bad = false;                                   // rows without a softmax
 #pragma unroll
@@ -381,12 +467,14 @@ grow_kernel(GrowArgs a) {
         const double lp = sm.lp[lo + q * 32 + lane];
         bad |= lp != lp;
       }
-    if (__any_sync(FULL, bad)) {                        // this sequence adds nothing any more
+    if (__any_sync(FULL, bad)) {                        // this sequence adds nothing any more (every warp sees it)
       if (tid == 0) {
         atomicOr(a.status, STATUS_NONFINITE);
         a.t.layer_off[b * a.lo_stride + d + 2] = n;
+        s_state[3] = DONE;
       }
       ++d;
+      __syncthreads();
       break;
     }
     const bool init = d < a.init_layers;
@@ -406,8 +494,10 @@ grow_kernel(GrowArgs a) {
     lo = hi;
     hi = n + total;
     if (tid == 0) a.t.layer_off[b * a.lo_stride + d + 2] = hi;
+    ++d;
     __syncthreads();
   }
+  const bool paused = s_state[3] == PAUSED;
 
   // ---- the new nodes, and once the tree is finished what closes it (positions, sentinel slots, the
   // unused tail of the layer offsets) ----
