@@ -124,10 +124,10 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     const char *ac = std::getenv("TALON_ATTN_CLUSTER");
     c->attn_cluster = ac ? std::atoi(ac) : 1;
     std::memset(c->attn_clusters, -1, sizeof(c->attn_clusters));
-    const char *cr = std::getenv("TALON_ATTN_CLUSTER_MIN_ROWS");
-    c->attn_cluster_min_rows = cr ? std::atoll(cr) : 8192;
     const char *fs = std::getenv("TALON_ATTN_SPLITS");
     c->attn_force_splits = fs ? std::atoi(fs) : 0;
+    const char *ft = std::getenv("TALON_ATTN_TILES");
+    c->attn_force_tiles = ft ? std::atoi(ft) : 0;
     const char *ao = std::getenv("TALON_ARGMAX_OVERSPLIT");
     c->argmax_oversplit = ao ? std::atoi(ao) : 4;
     if (c->argmax_oversplit < 1) c->argmax_oversplit = 1;

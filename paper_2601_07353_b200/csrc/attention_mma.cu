@@ -374,25 +374,36 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
     // tensor-core path: CTAs own two 128-row query tiles and 128-key tiles
     a.m_blocks = attn_tc_blocks(c);
     a.npt = AT_BM / a.g;
-    const int pairs = (a.m_blocks + 1) / 2;
-    const int ctas = pairs * c->B * a.Hkv;
-    const int tiles = (max_prefix_len + 127) / 128 + (a.N + 127) / 128;
+    const int tiles = (max_prefix_len + 127) / 128 + (a.N + 127) / 128, heads = c->B * a.Hkv;
+    const int ctas = (a.m_blocks + 1) / 2 * heads;
+    bool one = a.m_blocks == 1;
     int sp = 1;
     if (ctas < c->sm_count) {
-      // The fewest rounds of key tiles: a CTA of s ranges takes ceil(tiles / s) of them and about three
-      // tiles' worth of prologue and epilogue, merging in a cluster costs another two, the second kernel
-      // (more ranges than a cluster has CTAs, or few rows) four.  Clusters whose CTAs fill SMs only fit a
-      // GPC at a time, so the device says how many it holds: a second round of them doubles the time.
-      const int most = std::min(c->sm_count / ctas, (tiles + c->attn_min_tiles - 1) / c->attn_min_tiles);
-      auto cost = [&](int s) {
-        const bool cluster = s >= 2 && s <= 8 && c->attn_cluster &&
-                             (c->attn_cluster == 2 || (long long)c->B * a.Hkv * a.g * a.N * s >= c->attn_cluster_min_rows);
-        const int held = cluster ? attention_tc_clusters(c, a.m_blocks, s) : 0;
-        const int rounds = held > 0 ? (ctas + held - 1) / held : 1;
-        return rounds * ((tiles + s - 1) / s + 3) + (s == 1 ? 0 : (held > 0 ? 2 : 4));
+      // Room for key ranges, or for a CTA per query tile instead of two tiles: the cheapest by a model in
+      // microseconds, fitted to 1 to 4 sequences of 1-3 query tiles over 2048 tokens.  A key tile takes a CTA
+      // 1.2 with one query tile and 1.6 with two, all before the first another 2.6; writing the result of one
+      // range 1.6 a query tile.  Merging ranges in a cluster moves a CTA's partial result, 64 KB a query
+      // tile, between SMs; the second kernel (more ranges than a cluster has CTAs) 8 and 11.  Clusters whose
+      // CTAs fill SMs only fit a GPC at a time, so the device says how many it holds: a second round of them
+      // doubles the time.  Started beside the growth of the trees (about 1.2 a layer), the work on the prefix
+      // counts only where it takes longer than that.
+      const float growing = early_prefix ? 1.2f * c->p.max_depth : 0.f;
+      auto cost = [&](bool single, int s) {
+        const int n = single ? a.m_blocks * heads : ctas;
+        const int held = s >= 2 && s <= 8 && c->attn_cluster ? attention_tc_clusters(c, single, s) : 0;
+        const int slots = held > 0 ? held : std::max(c->sm_count / s, 1);
+        const float end = s == 1 ? (single ? 1.6f : 3.2f) : held == 0 ? (single ? 8.f : 11.f)
+                          : s <= 4 ? (single ? 4.9f : 7.3f) : (single ? 5.9f : 9.f);
+        const float tile = single ? 1.2f : 1.6f, before = 2.6f + ((tiles + s - 1) / s - 1) * tile;
+        return (n + slots - 1) / slots * (std::max(before, growing) + tile) + end;
       };
-      for (int s = 2; s <= most; ++s)
-        if (cost(s) < cost(sp)) sp = s;
+      const int most = std::min((tiles + c->attn_min_tiles - 1) / c->attn_min_tiles, c->attn_cluster == 2 ? 8 : c->sm_count);
+      float best = cost(one, 1);
+      for (int single = a.m_blocks == 1 || c->attn_force_tiles == 1; single <= (c->attn_force_tiles != 2 || a.m_blocks == 1); ++single)
+        for (int s = 1; s <= std::min(most, c->sm_count / (single ? a.m_blocks * heads : ctas)); ++s) {
+          const float t = cost(single, s);
+          if (t < best) { best = t; sp = s; one = single; }
+        }
     } else if (ctas % c->sm_count) {
       // More CTAs than SMs and a ragged last wave: halving the key ranges can fill it (512 CTAs on
       // 148 SMs are 4 waves of 257 tiles, 1024 half CTAs are 7 waves of 129).  Cost model in key
@@ -407,11 +418,12 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
       if (tiles >= 32 && cost(2) < cost(1)) sp = 2;
     }
     if (c->attn_force_splits > 0) sp = c->attn_force_splits;
+    if (c->attn_force_tiles > 0) one = c->attn_force_tiles == 1 || a.m_blocks == 1;
     while (sp > 1 && (size_t)a.m_blocks * c->B * a.Hkv * sp * AT_BM > c->attn_ml_elems) --sp;
     a.splits = sp;
     int merged = 0;
     talon_status r = launch_attention_tc(c, t, q, kp, vp, kt, vt, kv_start, block_table, bt_stride, stride_t, stride_h, kv_tokens,
-                                         max_prefix_len, sm_scale, out, sp, a.m_blocks, st, &merged, early_prefix);
+                                         max_prefix_len, sm_scale, out, sp, a.m_blocks, one, st, &merged, early_prefix);
     if (r != TALON_OK) return r;
     if (sp > 1 && !merged) {
       const int64_t rows = (int64_t)c->B * a.Hkv * a.g * a.N;

@@ -60,7 +60,7 @@ constexpr float TC_RESCALE_GAP = 8.f;      // raise the reference maximum only b
 constexpr long long TC_WAIT_CYCLES = 4000000000ll;   // ~2 s: far beyond any legitimate wait
 constexpr int TC_XO_PITCH = TC_D + 4;      // floats per row of the partial result a CTA leaves in shared memory
 constexpr int TC_XO_ROW_BYTES = TC_XO_PITCH * 4;                 // (the rows' (max, sum) pairs follow the rows)
-static_assert(2 * TC_MT * (TC_XO_ROW_BYTES + 8) <= 6 * TC_TILE_BYTES, "the partial result reuses the tile buffers");
+static_assert(2 * TC_MT * (TC_XO_ROW_BYTES + 8 + 8) + 64 <= 6 * TC_TILE_BYTES, "the partial result reuses the tile buffers");
 
 // barrier slots: K/V stages (up to three each); per query tile S ready, first and second half of P ready, P.V
 // complete; S read out
@@ -239,6 +239,7 @@ __device__ inline float2 cluster_ld_f2(uint32_t addr) {
   asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
   return v;
 }
+template <int Q> struct Ranges { static constexpr int value = Q; };      // most ranges a merge is unrolled for
 // every thread of every CTA of the cluster; orders shared-memory writes before it against reads after it
 __device__ inline void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -435,10 +436,14 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     unsigned long long mrow[2] = {0ull, 0ull};
     auto load_tree = [&]() {
       if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
-      n = __ldcg(a.n_nodes + b);
+      n = __ldcg(a.n_nodes + b);               // (one trip for the size and the mask)
+      if (in_range) {
+        const unsigned long long *m = a.mask + ((int64_t)b * a.N + node) * a.W;
+        mrow[0] = __ldcg(m);
+        if (a.W > 1) mrow[1] = __ldcg(m + 1);
+      }
       row_valid = in_range && node < n;
-      if (row_valid)
-        for (int w = 0; w < a.W; ++w) mrow[w] = __ldcg(a.mask + ((int64_t)b * a.N + node) * a.W + w);
+      if (!row_valid) mrow[0] = mrow[1] = 0ull;
       have_tree = true;
     };
     if (!a.early) load_tree();
@@ -651,70 +656,88 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     // (the merge stays inside this branch: past the join the compiler has to get by with the other
     // warps' registers)
     if (a.cluster_merge) {
-      // ---- merge of the cluster's partial results: CTA c takes every splits-th share of the packed
-      // rows, one warp per row, lane l the output columns 4l..4l+3.  Two rows at a time with the loads of
-      // all (up to eight) ranges in flight: a trip to a peer's shared memory is most of a microsecond, and
-      // with four loads in flight the merge was 5 us of a short prefix's 18. ----
+      // ---- merge of the cluster's partial results: CTA c takes the c-th share of the rows that exist, one warp
+      // per row, lane l the output columns 4l..4l+3.  A trip to a peer's shared memory is most of a microsecond:
+      // a warp has sixteen rows' pieces in flight whatever the number of ranges, the first sixteen while a
+      // thread per row turns the ranges' maxima and sums into weights.  4.9 us from the last P.V to the end with
+      // one query tile (was 8.4: two tiles a CTA, four trips a pair of rows); half of it is 32 bytes a clock out of an SM.
+      // Through the workspace in L2 by bulk copies, and pushed to the merging CTA: the same or slower. ----
       cluster_sync_all();
       {
-        const int S = a.splits;
-        const int share = (SOFT + S - 1) / S;
-        const int r_lo = split * share, r_hi = min(SOFT, r_lo + share);
+        constexpr int NW = SOFT / 32;
+        const int S = a.splits, rpt = a.npt * a.g;
+        const int rows = min(MT * rpt, (a.N - mpair * MT * a.npt) * a.g);
+        const int share = (rows + S - 1) / S, lo = split * share, mine = min(rows - lo, share);
         const uint32_t xo0 = smem_u32(gen_base), xml0 = xo0 + (uint32_t)(SOFT * TC_XO_ROW_BYTES);
-        const int rpt = a.npt * a.g;
-        for (int r0 = r_lo + warp; r0 < r_hi; r0 += 2 * (SOFT / 32)) {
-          int rr[2], rnode[2];
-          bool live[2];
-          float2 ml[2];
+        float *xw = reinterpret_cast<float *>(gen_base + SOFT * (TC_XO_ROW_BYTES + 8));              // weights [range][row]
+        int *xat = reinterpret_cast<int *>(xw + SOFT + 8);                                           // output rows
+        auto tile_row = [&](int r) { r += lo; return (uint32_t)(r >= rpt ? r - rpt + TC_MT : r); };
+        auto merge = [&](auto ranges) {
+          constexpr int Q = decltype(ranges)::value, U = 16 / Q;
+          uint32_t peer[Q];
+          int rank[Q];                       // (each CTA starts at itself, or all would ask the same one at a time)
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            rr[u] = r0 + u * (SOFT / 32);
-            const int mt = mpair * MT + rr[u] / TC_MT, rl = rr[u] % TC_MT;
-            rnode[u] = mt * a.npt + rl / a.g;
-            live[u] = rr[u] < r_hi && rl < rpt && rnode[u] < a.N;
-            ml[u] = live[u] && lane < S ? cluster_ld_f2(cluster_map(xml0 + (uint32_t)rr[u] * 8u, (uint32_t)lane))
-                                        : make_float2(-CUDART_INF_F, 0.f);
+          for (int q = 0; q < Q; ++q) {
+            rank[q] = q >= S ? split : split + q < S ? split + q : split + q - S;
+            peer[q] = cluster_map(xo0 + (uint32_t)lane * 16u, (uint32_t)rank[q]);
           }
-          float w[2], lsum[2];
+          float2 ml[Q];
+          if (tid < mine) {
+            const uint32_t at = xml0 + tile_row(tid) * 8u;
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            float gm = ml[u].x;
-#pragma unroll
-            for (int o = 4; o; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xFFFFFFFFu, gm, o));
-            w[u] = (ml[u].x == -CUDART_INF_F) ? 0.f : fast_exp2(ml[u].x - gm);     // an empty range has no row to read
-            lsum[u] = w[u] * ml[u].y;
-#pragma unroll
-            for (int o = 4; o; o >>= 1) lsum[u] += __shfl_xor_sync(0xFFFFFFFFu, lsum[u], o);
-            lsum[u] = __shfl_sync(0xFFFFFFFFu, lsum[u], 0);
+            for (int q = 0; q < Q; ++q) ml[q] = cluster_ld_f2(cluster_map(at, (uint32_t)rank[q]));
           }
-          float4 o4[2][8];
-          float ws[2][8];
+          float4 o[U][Q];
+          auto load = [&](int r0) {
 #pragma unroll
-          for (int sidx = 0; sidx < 8; ++sidx)
+            for (int q = 0; q < Q; ++q)
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              ws[u][sidx] = __shfl_sync(0xFFFFFFFFu, w[u], sidx);
-              o4[u][sidx] = ws[u][sidx] != 0.f
-                                ? cluster_ld_f4(cluster_map(xo0 + ((uint32_t)rr[u] * TC_XO_PITCH + (uint32_t)lane * 4u) * 4u, (uint32_t)sidx))
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
+              for (int u = 0; u < U; ++u)
+                if (q < S) o[u][q] = cluster_ld_f4(peer[q] + tile_row(min(r0 + u * NW, mine - 1)) * TC_XO_ROW_BYTES);
+          };
+          if (warp < mine) load(warp);
+          if (tid < mine) {
+            const int at = lo + tid;
+            xat[tid] = (b * a.N + mpair * MT * a.npt + at / a.g) * a.Hq + kvh * a.g + at % a.g;
+            float gm = -CUDART_INF_F, lsum = 0.f;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) gm = fmaxf(gm, ml[q].x);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+              ml[q].x = q >= S || ml[q].x == -CUDART_INF_F ? 0.f : fast_exp2(ml[q].x - gm);          // 0: nothing of this row there
+              lsum += ml[q].x * ml[q].y;
             }
+            const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            if (!live[u]) continue;
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int sidx = 0; sidx < 8; ++sidx) {
-              acc.x += ws[u][sidx] * o4[u][sidx].x; acc.y += ws[u][sidx] * o4[u][sidx].y;
-              acc.z += ws[u][sidx] * o4[u][sidx].z; acc.w += ws[u][sidx] * o4[u][sidx].w;
-            }
-            const float inv = lsum[u] > 0.f ? 1.f / lsum[u] : 0.f;
-            uint2 packed;
-            packed.x = pack_bf16x2(acc.x * inv, acc.y * inv);
-            packed.y = pack_bf16x2(acc.z * inv, acc.w * inv);
-            *reinterpret_cast<uint2 *>(a.out + (((int64_t)b * a.N + rnode[u]) * a.Hq + kvh * a.g + rr[u] % TC_MT % a.g) * TC_D +
-                                       lane * 4) = packed;
+            for (int q = 0; q < Q; ++q)
+              if (q < S) xw[q * share + tid] = ml[q].x * inv;
           }
-        }
+          asm volatile("bar.sync 1, %0;" ::"n"(SOFT) : "memory");
+#pragma unroll 1
+          for (int r0 = warp; r0 < mine;) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const int r = r0 + u * NW;
+              if (r >= mine) break;
+              float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+              for (int q = 0; q < Q; ++q) {
+                const float w = q < S ? xw[q * share + r] : 0.f;
+                if (w != 0.f) {
+                  acc.x += w * o[u][q].x; acc.y += w * o[u][q].y;
+                  acc.z += w * o[u][q].z; acc.w += w * o[u][q].w;
+                }
+              }
+              *reinterpret_cast<uint2 *>(a.out + (int64_t)xat[r] * TC_D + lane * 4) =
+                  make_uint2(pack_bf16x2(acc.x, acc.y), pack_bf16x2(acc.z, acc.w));
+            }
+            r0 += U * NW;
+            if (r0 < mine) load(r0);
+          }
+        };
+        if (S <= 2) merge(Ranges<2>{});
+        else if (S <= 4) merge(Ranges<4>{});
+        else merge(Ranges<8>{});
       }
       cluster_sync_all();                    // nobody leaves while a peer may still read its shared memory
     }
@@ -788,9 +811,8 @@ talon_status attention_tc_setup() {
 
 // How many clusters of `splits` CTAs (one per key range, a whole SM each) the device can hold at once; 0: it
 // cannot place one.  The SMs of a cluster share a GPC, so this is less than SMs / splits.
-int attention_tc_clusters(talon_ctx *c, int m_blocks, int splits) {
+int attention_tc_clusters(talon_ctx *c, bool one, int splits) {
   if (splits < 2 || splits > 8) return 0;
-  const bool one = m_blocks == 1;
   int &known = c->attn_clusters[one ? 0 : 1][splits];
   if (known < 0) {
     cudaLaunchConfig_t q = {};
@@ -813,7 +835,7 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
                                  const void *kt, const void *vt, const int64_t *kv_start, const int32_t *block_table,
                                  int bt_stride, int64_t stride_t,
                                  int64_t stride_h, int64_t kv_tokens, int max_prefix_len, float sm_scale, void *out,
-                                 int splits, int m_blocks, cudaStream_t st, int *merged_in_kernel,
+                                 int splits, int m_blocks, bool one, cudaStream_t st, int *merged_in_kernel,
                                  const int32_t *early_prefix) {
   *merged_in_kernel = 0;
   const int N = c->p.budget, Hq = c->p.n_q_heads, Hkv = c->p.n_kv_heads, g = Hq / Hkv, B = c->B, npt = 128 / g;
@@ -846,17 +868,13 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
   a.splits = splits; a.m_blocks = m_blocks;
   a.out = (__nv_bfloat16 *)out; a.part_o = c->d_attn_o; a.part_ml = c->d_attn_ml; a.status = c->d_status;
   (void)max_prefix_len;
-  const bool one = m_blocks == 1;
   auto kernel = one ? tree_attention_tc_kernel<1> : tree_attention_tc_kernel<2>;
   const int threads = one ? TcShape<1>::THREADS : TcShape<2>::THREADS, smem = one ? TcShape<1>::SMEM : TcShape<2>::SMEM;
-  dim3 grid((m_blocks + 1) / 2, splits, B * Hkv);
+  dim3 grid(one ? m_blocks : (m_blocks + 1) / 2, splits, B * Hkv);
   // Two to eight key ranges: they are launched as one thread-block cluster and merge their partial
   // results through distributed shared memory, if the device can place such a cluster (asked once
   // per cluster size; a cluster of full-SM CTAs needs that many SMs free in one GPC).
-  // (few rows: the second kernel is cheaper than a cluster launch and two cluster barriers)
-  const long long merge_rows = (long long)B * Hkv * g * N * splits;
-  a.cluster_merge = (c->attn_cluster == 2 || (c->attn_cluster == 1 && merge_rows >= c->attn_cluster_min_rows)) &&
-                    attention_tc_clusters(c, m_blocks, splits) > 0;
+  a.cluster_merge = c->attn_cluster && attention_tc_clusters(c, one, splits) > 0;
   {
     LaunchTimer lt(c, TALON_K_ATTENTION, st);
     if (a.cluster_merge) {
