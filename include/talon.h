@@ -248,6 +248,8 @@ talon_status talon_poll_status(talon_ctx *ctx, void *stream);
  *  k_tree/v_tree [B,N,Hkv,Dh], all bf16
  *  outputs: out_attn [B,N,Hq,Dh] bf16 (may be null), n_nodes [B], token/parent/depth/position
  *  [B,N] (each may be null), accept_len [B], accept_nodes [B, D_max+1], bonus_tok [B].
+ * The draft rows of expanded nodes and the target rows of the tree's nodes are copied as the tree
+ * grows, and no other rows; q, K and V are copied whole.
  * The first call allocates device staging buffers sized for batch_max inside the context
  * (a later call with a longer total prefix reallocates).  Synchronises `stream` before
  * returning and returns the device status. */
@@ -294,8 +296,9 @@ talon_status talon_step(talon_ctx *ctx, const talon_tree *tree, int32_t B, const
  *  block_table   device [B, table_stride] int32 page numbers; a sequence needs
  *                ceil(prefix_len / 128) entries (talon_commit_paged: up to n_blocks[b])
  *  n_pages       pages in the pool (bounds the tensor map)
- * Otherwise as talon_tree_attention.  Query-group sizes that do not divide 128 return
- * TALON_ERR_UNSUPPORTED here (the warp-MMA kernel reads contiguous blocks only). */
+ * Otherwise as talon_tree_attention.  Every query-group size up to 128 with sm_scale > 0; what
+ * needs the warp-MMA kernel (a scale of zero or less, strides that TMA cannot take) returns
+ * TALON_ERR_UNSUPPORTED here, since that kernel reads contiguous blocks only. */
 #define TALON_PAGE_TOKENS 128
 talon_status talon_tree_attention_paged(talon_ctx *ctx, const talon_tree *tree, const void *q,
                                         const void *k_pages, const void *v_pages, const void *k_tree,
@@ -327,7 +330,9 @@ talon_status talon_commit_paged(talon_ctx *ctx, const talon_tree *tree, const in
  * + s * result_step_stride and accept_nodes at + s * result_step_stride * (D_max + 1) (a stride of 0
  * keeps only the last step's).  root_tok, prefix_len, the cache and counters ([B, 3], as in
  * talon_commit; required) are read and advanced in place.
- *  max_prefix_len  bound on prefix_len[b] over ALL steps (the last step's prefix included) */
+ *  max_prefix_len  bound on prefix_len[b] over ALL steps (the last step's prefix included)
+ * The rows of several steps may be read ahead, and the device status then covers those steps together:
+ * a row that is not finite in one of them is reported after the last. */
 talon_status talon_loop(talon_ctx *ctx, const talon_tree *tree, int32_t B, int32_t n_steps,
                         int32_t *root_tok, int32_t *prefix_len, const float *draft_logits,
                         int64_t draft_row_stride, int64_t draft_step_stride, int32_t n_layers,
