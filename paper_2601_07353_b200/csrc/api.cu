@@ -227,6 +227,15 @@ static talon_status check_accept(const talon_ctx *c, const talon_tree *t, const 
   return check_rows(c, target_logits, row_stride);
 }
 
+// A step or loop that fails once target rows have been read leaves their arg-max keys and NaN flags behind, which
+// the next arg-max of these slots would be taken on top of: the workspace is made clean again.
+static talon_status abandon_rows(talon_ctx *c, talon_status r, void *stream) {
+  const size_t slots = (size_t)c->p.batch_max * c->p.budget * c->ahead;
+  cudaMemsetAsync(c->d_argmax, 0, slots * sizeof(*c->d_argmax), (cudaStream_t)stream);
+  cudaMemsetAsync(c->d_row_bad, 0, slots * sizeof(*c->d_row_bad), (cudaStream_t)stream);
+  return r;
+}
+
 // Whether a step may prepare the rows of all its node slots in one pass (timed launches are reported per layer).
 static bool rows_at_once(const talon_ctx *c) { return c->step_rows && c->k_cap <= 32 && !(c->ev && !c->ev_paused); }
 
@@ -274,20 +283,30 @@ talon_status talon_prune_tree(talon_ctx *c, const talon_tree *t, int32_t keep, v
   return talon::launch_prune(c, t, keep, (cudaStream_t)stream);
 }
 
-static talon_status attention_checked(talon_ctx *c, const talon_tree *t, const void *q, const void *k_prefix,
-                                  const void *v_prefix, const void *k_tree, const void *v_tree,
-                                  const int64_t *kv_start, int64_t kv_tokens, int64_t kv_stride_t,
-                                  int64_t kv_stride_h, int32_t max_prefix_len, float sm_scale, void *out,
-                                  void *stream, const int32_t *early_prefix) {
+static talon_status check_attention(const talon_ctx *c, const talon_tree *t, const void *q, const void *k_prefix,
+                                    const void *v_prefix, const void *k_tree, const void *v_tree,
+                                    const int64_t *kv_start, int64_t kv_tokens, int64_t kv_stride_t,
+                                    int64_t kv_stride_h, int32_t max_prefix_len, float sm_scale, const void *out) {
   if (!c || !tree_complete(t) || !q || !k_tree || !v_tree || !kv_start || !out) return TALON_ERR_INVALID_ARG;
-  if (c->B < 1 || max_prefix_len < 0 || kv_tokens < 0 || kv_tokens > 0x7FFFFFFFll) return TALON_ERR_INVALID_ARG;
+  if (max_prefix_len < 0 || kv_tokens < 0 || kv_tokens > 0x7FFFFFFFll) return TALON_ERR_INVALID_ARG;
   if (max_prefix_len > kv_tokens) return TALON_ERR_INVALID_ARG;
   if (max_prefix_len > 0 && (!k_prefix || !v_prefix)) return TALON_ERR_INVALID_ARG;
   if ((kv_stride_t & 7) || (kv_stride_h & 7) || kv_stride_t < 0 || kv_stride_h < 0) return TALON_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k_prefix) || !aligned16(v_prefix) || !aligned16(k_tree) || !aligned16(v_tree) ||
       !aligned16(out))
     return TALON_ERR_INVALID_ARG;
-  if (!(sm_scale == sm_scale)) return TALON_ERR_INVALID_ARG;
+  return sm_scale == sm_scale ? TALON_OK : TALON_ERR_INVALID_ARG;
+}
+
+static talon_status attention_checked(talon_ctx *c, const talon_tree *t, const void *q, const void *k_prefix,
+                                  const void *v_prefix, const void *k_tree, const void *v_tree,
+                                  const int64_t *kv_start, int64_t kv_tokens, int64_t kv_stride_t,
+                                  int64_t kv_stride_h, int32_t max_prefix_len, float sm_scale, void *out,
+                                  void *stream, const int32_t *early_prefix) {
+  const talon_status ok = check_attention(c, t, q, k_prefix, v_prefix, k_tree, v_tree, kv_start, kv_tokens, kv_stride_t,
+                                          kv_stride_h, max_prefix_len, sm_scale, out);
+  if (ok != TALON_OK) return ok;
+  if (c->B < 1) return TALON_ERR_INVALID_ARG;
   return talon::launch_attention(c, t, q, k_prefix ? k_prefix : k_tree, v_prefix ? v_prefix : v_tree, k_tree,
                                  v_tree, kv_start, nullptr, 0, kv_tokens, kv_stride_t, kv_stride_h, max_prefix_len,
                                  sm_scale, out, (cudaStream_t)stream, early_prefix);
@@ -355,18 +374,30 @@ talon_status talon_accept_sample(talon_ctx *c, const talon_tree *t, const float 
                                      accept_nodes, out_tok, (cudaStream_t)stream);
 }
 
+static talon_status check_commit(const talon_ctx *c, const talon_tree *t, const int32_t *accept_len,
+                                 const int32_t *accept_nodes, const int32_t *next_tok, const void *k_tree,
+                                 const void *v_tree, const void *k_prefix, const void *v_prefix, const int64_t *kv_start,
+                                 int64_t kv_tokens, int64_t kv_stride_t, int64_t kv_stride_h, const int32_t *prefix_len,
+                                 const int32_t *root_tok) {
+  if (!c || !tree_complete(t) || !accept_len || !accept_nodes || !next_tok || !k_tree || !v_tree || !k_prefix ||
+      !v_prefix || !kv_start || !prefix_len || !root_tok)
+    return TALON_ERR_INVALID_ARG;
+  if (kv_tokens < 0 || kv_tokens > 0x7FFFFFFFll) return TALON_ERR_INVALID_ARG;
+  if ((kv_stride_t & 7) || (kv_stride_h & 7) || kv_stride_t < 0 || kv_stride_h < 0) return TALON_ERR_INVALID_ARG;
+  if (!aligned16(k_prefix) || !aligned16(v_prefix) || !aligned16(k_tree) || !aligned16(v_tree))
+    return TALON_ERR_INVALID_ARG;
+  return TALON_OK;
+}
+
 talon_status talon_commit(talon_ctx *c, const talon_tree *t, const int32_t *accept_len, const int32_t *accept_nodes,
                           const int32_t *next_tok, const void *k_tree, const void *v_tree, void *k_prefix,
                           void *v_prefix, const int64_t *kv_start, const int64_t *kv_limit, int64_t kv_tokens,
                           int64_t kv_stride_t, int64_t kv_stride_h, int32_t *prefix_len, int32_t *root_tok,
                           int64_t *counters, void *stream) {
-  if (!c || !tree_complete(t) || !accept_len || !accept_nodes || !next_tok || !k_tree || !v_tree || !k_prefix ||
-      !v_prefix || !kv_start || !prefix_len || !root_tok)
-    return TALON_ERR_INVALID_ARG;
-  if (c->B < 1 || kv_tokens < 0 || kv_tokens > 0x7FFFFFFFll) return TALON_ERR_INVALID_ARG;
-  if ((kv_stride_t & 7) || (kv_stride_h & 7) || kv_stride_t < 0 || kv_stride_h < 0) return TALON_ERR_INVALID_ARG;
-  if (!aligned16(k_prefix) || !aligned16(v_prefix) || !aligned16(k_tree) || !aligned16(v_tree))
-    return TALON_ERR_INVALID_ARG;
+  const talon_status ok = check_commit(c, t, accept_len, accept_nodes, next_tok, k_tree, v_tree, k_prefix, v_prefix, kv_start,
+                                       kv_tokens, kv_stride_t, kv_stride_h, prefix_len, root_tok);
+  if (ok != TALON_OK) return ok;
+  if (c->B < 1) return TALON_ERR_INVALID_ARG;
   return talon::launch_commit(c, t, accept_len, accept_nodes, next_tok, k_tree, v_tree, k_prefix, v_prefix, kv_start,
                               kv_limit, nullptr, 0, nullptr, kv_tokens, kv_stride_t, kv_stride_h, prefix_len, root_tok,
                               counters, (cudaStream_t)stream);
@@ -398,6 +429,23 @@ static talon_status step_enqueue(talon_ctx *c, const talon_tree *t, int32_t B, c
                                  int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes, int32_t *bonus_tok,
                                  void *stream, bool layered);
 
+// What a whole step checks, all of it before its first launch.
+static talon_status check_step(const talon_ctx *c, const talon_tree *t, int32_t B, const int32_t *root_tok,
+                               const int32_t *prefix_len, const float *draft_logits, int64_t draft_row_stride,
+                               int32_t n_layers, const void *q, const void *k_prefix, const void *v_prefix,
+                               const void *k_tree, const void *v_tree, const int64_t *kv_start, int64_t kv_tokens,
+                               int64_t kv_stride_t, int64_t kv_stride_h, int32_t max_prefix_len, float sm_scale,
+                               const void *out, const float *target_logits, int64_t target_row_stride,
+                               const int32_t *accept_len, const int32_t *accept_nodes, const int32_t *bonus_tok) {
+  talon_status r = check_reset(c, t, root_tok, prefix_len, B);
+  if (r == TALON_OK && n_layers > 0) r = check_rows(c, draft_logits, draft_row_stride);
+  if (r == TALON_OK)
+    r = check_attention(c, t, q, k_prefix, v_prefix, k_tree, v_tree, kv_start, kv_tokens, kv_stride_t, kv_stride_h,
+                        max_prefix_len, sm_scale, out);
+  if (r == TALON_OK) r = check_accept(c, t, target_logits, target_row_stride, accept_len, accept_nodes, bonus_tok);
+  return r;
+}
+
 talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_steps, int32_t *root_tok,
                         int32_t *prefix_len, const float *draft_logits, int64_t draft_row_stride,
                         int64_t draft_step_stride, int32_t n_layers, const void *q, int64_t q_step_stride,
@@ -416,15 +464,16 @@ talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_
   // a caller that captures the loop gets the layered launch sequence, as talon_step's callers do
   const bool layered = being_captured((cudaStream_t)stream);
   const char *qb = static_cast<const char *>(q), *ktb = static_cast<const char *>(k_tree), *vtb = static_cast<const char *>(v_tree);
-  // (the same condition as in step_enqueue, whose argument checks follow)
-  const bool ahead = !layered && n_layers > 0 && rows_at_once(c) && B >= 1 && B <= c->p.batch_max && n_steps > 1;
-  if (ahead) {
-    talon_status r = check_reset(c, t, root_tok, prefix_len, B);
-    if (r == TALON_OK) r = check_rows(c, draft_logits, draft_row_stride);
-    if (r == TALON_OK) r = check_accept(c, t, target_logits, target_row_stride, accept_len, accept_nodes, bonus_tok);
-    if (r != TALON_OK) return r;
-    c->B = B;
-  }
+  // every argument of every step is checked before the first launch (the step strides keep the alignment)
+  talon_status ok = check_step(c, t, B, root_tok, prefix_len, draft_logits, draft_row_stride, n_layers, q, k_prefix, v_prefix,
+                               k_tree, v_tree, kv_start, kv_tokens, kv_stride_t, kv_stride_h, max_prefix_len, sm_scale, out,
+                               target_logits, target_row_stride, accept_len, accept_nodes, bonus_tok);
+  if (ok == TALON_OK)
+    ok = check_commit(c, t, accept_len, accept_nodes, bonus_tok, k_tree, v_tree, k_prefix, v_prefix, kv_start, kv_tokens,
+                      kv_stride_t, kv_stride_h, prefix_len, root_tok);
+  if (ok != TALON_OK) return ok;
+  const bool ahead = !layered && n_layers > 0 && rows_at_once(c) && n_steps > 1;
+  if (ahead) c->B = B;
   const bool batched = ahead && talon::loop_rows_possible(c, n_layers);
   for (int s = 0; s < n_steps; ++s) {
     // step s reads its own slice of the stand-ins for the two model forwards; the tree, the cache,
@@ -453,7 +502,7 @@ talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_
     if (r == TALON_OK)
       r = talon_commit(c, t, al, an, bt, kts, vts, k_prefix, v_prefix, kv_start, kv_limit, kv_tokens, kv_stride_t,
                        kv_stride_h, prefix_len, root_tok, counters, stream);
-    if (r != TALON_OK) return r;
+    if (r != TALON_OK) return batched ? abandon_rows(c, r, stream) : r;
   }
   return TALON_OK;
 }
@@ -553,18 +602,18 @@ static talon_status step_enqueue(talon_ctx *c, const talon_tree *t, int32_t B, c
                                  void *out, const float *target_logits, int64_t target_row_stride,
                                  int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes, int32_t *bonus_tok,
                                  void *stream, bool layered) {
-  talon_status r = TALON_OK;
+  talon_status r = check_step(c, t, B, root_tok, prefix_len, draft_logits, draft_row_stride, n_layers, q, k_prefix, v_prefix,
+                              k_tree, v_tree, kv_start, kv_tokens, kv_stride_t, kv_stride_h, max_prefix_len, sm_scale, out,
+                              target_logits, target_row_stride, accept_len, accept_nodes, bonus_tok);
+  if (r != TALON_OK) return r;
   bool closed = false, accepted = false;
   // (timed launches are reported per layer, so they take the layered sequence too)
   if (!layered && n_layers > 0 && rows_at_once(c)) {
-    r = check_reset(c, t, root_tok, prefix_len, B);
-    if (r == TALON_OK) r = check_rows(c, draft_logits, draft_row_stride);
-    if (r == TALON_OK) r = check_accept(c, t, target_logits, target_row_stride, accept_len, accept_nodes, bonus_tok);
-    if (r != TALON_OK) return r;
     c->B = B;
     r = talon::launch_grow_step(c, t, root_tok, prefix_len, draft_logits, draft_row_stride, n_layers, target_logits,
                                 target_row_stride, target_tok, accept_len, accept_nodes, bonus_tok, (cudaStream_t)stream,
                                 &accepted);
+    if (r != TALON_OK) return abandon_rows(c, r, stream);
     closed = true;
   } else {
     r = talon_reset(c, t, root_tok, prefix_len, B, stream);

@@ -1,0 +1,105 @@
+"""What one call leaves behind for the next one, and what a call has to wait for."""
+import math
+
+import pytest
+import torch
+
+from tests.test_gpu_step_paths import DH, Step, _talon
+
+pytestmark = pytest.mark.gpu
+
+
+def _loop(t, s, n, **other):
+    """The first n steps of s as one call; `other` replaces arguments."""
+    a = dict(q=s.q, kp=s.kp, vp=s.vp, tokens=s.tokens, stride=s.hkv * DH, max_len=s.max_len, scale=1 / math.sqrt(DH))
+    a.update(other)
+    t.loop(s.tree, n, s.root, s.plen, s.draft, s.D, a["q"], a["kp"], a["vp"], s.kt, s.vt, s.start, s.limit, a["tokens"],
+           a["stride"], DH, a["max_len"], a["scale"], s.out, s.target, s.tok, s.alen, s.anodes, s.bonus, s.counters)
+
+
+def _results(s):
+    return s.whole() + [s.plen, s.root, s.counters, s.kp, s.vp]
+
+
+# what the attention refuses, and (no prefix, no cache) what only the commit refuses
+REFUSALS = [dict(max_len=1 << 20), dict(scale=float("nan")), dict(stride=2 * DH + 1), dict(q="misaligned"),
+            dict(kp=None, vp=None, max_len=0)]
+
+
+def _other(s, refusal):
+    r = dict(refusal)
+    if r.get("q") == "misaligned":
+        r["q"] = s.q.reshape(-1)[1:].as_strided(s.q.shape, s.q.stride())
+    return r
+
+
+@pytest.mark.parametrize("refusal", REFUSALS)
+def test_a_refused_loop_enqueues_nothing_and_leaves_nothing(refusal):
+    B, V, N, K, D, S = 2, 2003, 20, 5, 4, 6
+    talon, t = _talon(B, V, N, K, D)
+    shape = (t, B, V, N, D, 8, 2, [0, 0] if "kp" in refusal else [90, 33])
+    s = Step(*shape, 3, steps=S)
+    s.q = torch.cat([s.q.reshape(-1), s.q.new_zeros(8)])[:s.q.numel()].view(s.q.shape)     # (room for the shifted view)
+    s.target += 50.0                                     # larger than any row of the loop that follows
+    s.target[:, :, 1, 7] = float("nan")
+    before, launches = [x.clone() for x in _results(s)], t.launch_count()
+    with pytest.raises(talon.TalonError) as e:
+        _loop(t, s, S, **_other(s, refusal))
+    assert e.value.code == talon.ERR_INVALID_ARG
+    assert t.launch_count() == launches
+    torch.cuda.synchronize()
+    for x, y in zip(before, _results(s)):
+        assert torch.equal(x, y)
+    good, ref = Step(*shape, 4, steps=S), Step(*shape, 4, steps=S)
+    _loop(t, good, S)
+    talon, fresh = _talon(B, V, N, K, D)
+    _loop(fresh, ref, S)
+    torch.cuda.synchronize()
+    assert t.poll_status() == fresh.poll_status() == talon.OK
+    for x, y in zip(_results(good), _results(ref)):
+        assert torch.equal(x, y)
+    t.close()
+    fresh.close()
+
+
+@pytest.mark.parametrize("refusal", REFUSALS[:4])
+def test_a_refused_step_enqueues_nothing(refusal):
+    B, V, N, K, D = 2, 2003, 20, 5, 4
+    talon, t = _talon(B, V, N, K, D)
+    s = Step(t, B, V, N, D, 8, 2, [90, 33], 3)
+    s.q = torch.cat([s.q.reshape(-1), s.q.new_zeros(8)])[:s.q.numel()].view(s.q.shape)
+    a = dict(q=s.q, tokens=s.tokens, stride=s.hkv * DH, max_len=s.max_len, scale=1 / math.sqrt(DH))
+    a.update(_other(s, refusal))
+    before, launches = s.whole(), t.launch_count()
+    with pytest.raises(talon.TalonError) as e:
+        t.step(s.tree, s.root, s.plen, s.draft, D, a["q"], s.kp, s.vp, s.kt, s.vt, s.start, a["tokens"], a["stride"], DH,
+               a["max_len"], a["scale"], s.out, s.target, s.tok, s.alen, s.anodes, s.bonus)
+    assert e.value.code == talon.ERR_INVALID_ARG
+    assert t.launch_count() == launches
+    torch.cuda.synchronize()
+    for x, y in zip(before, s.whole()):
+        assert torch.equal(x, y)
+    t.close()
+
+
+def test_a_loop_that_fails_after_its_first_launch_leaves_nothing():
+    """A token stride that no tensor map can hold is only found when the attention is launched."""
+    B, V, N, K, D, S = 2, 2003, 20, 5, 4, 6
+    talon, t = _talon(B, V, N, K, D)
+    shape = (t, B, V, N, D, 8, 2, [90, 33])
+    s = Step(*shape, 3, steps=S)
+    s.target += 50.0
+    s.target[:, :, 1, 7] = float("nan")
+    with pytest.raises(talon.TalonError) as e:
+        _loop(t, s, S, stride=1 << 40)
+    assert e.value.code == talon.ERR_CUDA
+    good, ref = Step(*shape, 4, steps=S), Step(*shape, 4, steps=S)
+    _loop(t, good, S)
+    talon, fresh = _talon(B, V, N, K, D)
+    _loop(fresh, ref, S)
+    torch.cuda.synchronize()
+    assert t.poll_status() == fresh.poll_status() == talon.OK
+    for x, y in zip(_results(good), _results(ref)):
+        assert torch.equal(x, y)
+    t.close()
+    fresh.close()
