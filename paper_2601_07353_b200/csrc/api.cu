@@ -26,7 +26,7 @@ struct HostStage {
   int32_t *accept_len = nullptr, *accept_nodes = nullptr, *bonus = nullptr;
   char *h_scratch = nullptr;       // pinned: kv_start [batch_max] int64, n_nodes [batch_max] int32
   cudaStream_t copy = nullptr;
-  cudaEvent_t rows = nullptr, kv = nullptr, targets = nullptr;
+  cudaEvent_t begin = nullptr, rows = nullptr, kv = nullptr, targets = nullptr;
 };
 
 #define TALON_CUDA_OK(expr)                                                              \
@@ -49,6 +49,7 @@ static void free_stage(HostStage *s) {
   if (!s) return;
   cudaFree(s->arena);
   if (s->h_scratch) cudaFreeHost(s->h_scratch);
+  if (s->begin) cudaEventDestroy(s->begin);
   if (s->rows) cudaEventDestroy(s->rows);
   if (s->kv) cudaEventDestroy(s->kv);
   if (s->targets) cudaEventDestroy(s->targets);
@@ -782,6 +783,7 @@ talon_status talon_step_host(talon_ctx *c, int32_t B, const int32_t *root_tok, c
     }
     TALON_CUDA_OK(cudaMallocHost((void **)&s->h_scratch, bm * 12));
     TALON_CUDA_OK(cudaStreamCreateWithFlags(&s->copy, cudaStreamNonBlocking));
+    TALON_CUDA_OK(cudaEventCreateWithFlags(&s->begin, cudaEventDisableTiming));
     TALON_CUDA_OK(cudaEventCreateWithFlags(&s->rows, cudaEventDisableTiming));
     TALON_CUDA_OK(cudaEventCreateWithFlags(&s->kv, cudaEventDisableTiming));
     TALON_CUDA_OK(cudaEventCreateWithFlags(&s->targets, cudaEventDisableTiming));
@@ -841,6 +843,8 @@ talon_status talon_step_host(talon_ctx *c, int32_t B, const int32_t *root_tok, c
       queue.push_back({s->vp, v_prefix, (size_t)tokens * kvrow});
     }
     kv_pieces = queue.size();
+    // what the caller has enqueued on `stream` (a copy or callback that fills these buffers) comes first
+    if (cudaEventRecord(s->begin, st) != cudaSuccess || cudaStreamWaitEvent(s->copy, s->begin, 0) != cudaSuccess) return TALON_ERR_CUDA;
     if (!copy_in(s->root, root_tok, (size_t)B * 4) || !copy_in(s->plen, prefix_len, (size_t)B * 4) ||
         !copy_in(s->kv_start, h_kv_start, (size_t)B * 8))
       return TALON_ERR_CUDA;

@@ -4,7 +4,7 @@ import math
 import pytest
 import torch
 
-from tests.test_gpu_step_paths import DH, Step, _talon
+from tests.test_gpu_step_paths import ATT_TOL, DH, Step, _talon
 
 pytestmark = pytest.mark.gpu
 
@@ -103,3 +103,33 @@ def test_a_loop_that_fails_after_its_first_launch_leaves_nothing():
         assert torch.equal(x, y)
     t.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("own", [False, True])
+def test_a_host_step_follows_what_its_stream_still_has_to_do(own):
+    """The pinned inputs are filled by copies that are enqueued, behind 50 ms of other work, but not finished."""
+    B, V, N, K, D = 2, 3000, 40, 8, 5
+    talon, t = _talon(B, V, N, K, D)
+    s = Step(t, B, V, N, D, 8, 2, [70, 120], 5)
+    s.draft, s.target = s.draft.contiguous(), s.target.contiguous()
+    s.calls(t)
+    torch.cuda.synchronize()
+    pinned = lambda x: torch.zeros(x.shape, dtype=x.dtype).pin_memory()
+    names = ("draft", "target", "q", "kp", "vp", "kt", "vt")
+    host = {n: pinned(getattr(s, n)) for n in names}
+    res = [pinned(x) for x in (s.out, s.tree.n_nodes, s.tree.token, s.tree.parent, s.tree.depth, s.tree.position, s.alen,
+                               s.anodes, s.bonus)]
+    root, plen = s.root.cpu(), s.plen.cpu()
+    call = lambda: t.step_host(root, plen, *(host[n] for n in names), 1 / math.sqrt(DH), *res)
+    assert call() == talon.OK                            # (allocates the staging buffers, which synchronises)
+    stream = torch.cuda.Stream() if own else torch.cuda.default_stream()
+    with torch.cuda.stream(stream):
+        torch.cuda._sleep(100_000_000)
+        for n in names:
+            host[n].copy_(getattr(s, n), non_blocking=True)
+        assert call() == talon.OK
+    for got, want in zip(res[1:], (s.tree.n_nodes, s.tree.token, s.tree.parent, s.tree.depth, s.tree.position, s.alen, s.anodes,
+                                   s.bonus)):
+        assert torch.equal(got, want.cpu())
+    assert (res[0].float() - s.out.cpu().float()).abs().max() <= ATT_TOL
+    t.close()
