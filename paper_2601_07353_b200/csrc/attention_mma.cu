@@ -378,7 +378,16 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
     const int ctas = (a.m_blocks + 1) / 2 * heads;
     bool one = a.m_blocks == 1;
     int sp = 1;
+    // How exact the rounding of P to bf16 is hangs on the ranges: a row's largest probability in the first tile of
+    // each is 1 and so exact, and its neighbours round with half the error.  `usual`: as many ranges as the SMs and two
+    // tiles a range allow (eight rather than nine or more, where a cluster has enough rows to merge).  With fewer the
+    // reference follows every growth of the maximum (exact_max), which comes closer to 64 bits than the usual number
+    // does (512 keys 2.20e-3 of the norm against 2.25e-3, 2048 keys 2.23e-3 against 2.28e-3; without it 2.30e-3
+    // and 2.33e-3) for a rescale of O now and then, 0.15 us a key tile with one query tile and 0.3 with two.
+    int usual = 1;
     if (ctas < c->sm_count) {
+      usual = std::max(1, std::min(c->sm_count / ctas, (tiles + c->attn_min_tiles - 1) / c->attn_min_tiles));
+      if (usual > 8 && c->attn_cluster && heads * a.g * a.N >= 1024) usual = 8;
       // Room for key ranges, or for a CTA per query tile instead of two tiles: the cheapest by a model in
       // microseconds, fitted to 1 to 4 sequences of 1-3 query tiles over 2048 tokens.  A key tile takes a CTA
       // 1.2 with one query tile and 1.6 with two, all before the first another 2.6; writing the result of one
@@ -394,7 +403,8 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
         const int slots = held > 0 ? held : std::max(c->sm_count / s, 1);
         const float end = s == 1 ? (single ? 1.6f : 3.2f) : held == 0 ? (single ? 8.f : 11.f)
                           : s <= 4 ? (single ? 4.9f : 7.3f) : (single ? 5.9f : 9.f);
-        const float tile = single ? 1.2f : 1.6f, before = 2.6f + ((tiles + s - 1) / s - 1) * tile;
+        const float tile = single ? 1.2f : 1.6f, rescale = s < usual ? (single ? 0.15f : 0.3f) : 0.f;
+        const float before = 2.6f + ((tiles + s - 1) / s - 1) * (tile + rescale);
         return (n + slots - 1) / slots * (std::max(before, growing) + tile) + end;
       };
       const int most = std::min((tiles + c->attn_min_tiles - 1) / c->attn_min_tiles, c->attn_cluster == 2 ? 8 : c->sm_count);
@@ -421,9 +431,10 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
     if (c->attn_force_tiles > 0) one = c->attn_force_tiles == 1 || a.m_blocks == 1;
     while (sp > 1 && (size_t)a.m_blocks * c->B * a.Hkv * sp * AT_BM > c->attn_ml_elems) --sp;
     a.splits = sp;
+    const bool exact_max = sp < usual;
     int merged = 0;
     talon_status r = launch_attention_tc(c, t, q, kp, vp, kt, vt, kv_start, block_table, bt_stride, stride_t, stride_h, kv_tokens,
-                                         max_prefix_len, sm_scale, out, sp, a.m_blocks, one, st, &merged, early_prefix);
+                                         max_prefix_len, sm_scale, out, sp, a.m_blocks, one, exact_max, st, &merged, early_prefix);
     if (r != TALON_OK) return r;
     if (sp > 1 && !merged) {
       const int64_t rows = (int64_t)c->B * a.Hkv * a.g * a.N;

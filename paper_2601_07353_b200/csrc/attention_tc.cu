@@ -14,9 +14,11 @@
 //                   S = Q K^T from tensor memory (tcgen05.ld), applies the ragged-length or
 //                   ancestor-bitmask visibility, keeps a running maximum and sum, and writes
 //                   P = exp2(S*scale - max) as bf16 back to tensor memory over S (tcgen05.st).
-//                   The running maximum is only raised when it grows by more than 2^8, so the
-//                   accumulator in tensor memory is rescaled rarely (the final division by the
-//                   running sum makes any reference maximum exact).
+//                   With many key tiles a CTA the running maximum is only raised when it grows by
+//                   more than 2^8, so the accumulator in tensor memory is rescaled rarely; with few
+//                   it follows every growth (launch_attention has the rule: the final division by
+//                   the running sum makes any reference right, but a row's largest probability is
+//                   exact in bf16 only if the reference is its maximum).
 //   warp 8          producer: TMA loads of Q (once) and of the K / V tiles into a ring of
 //                   128-byte-swizzled shared-memory stages (no multicast).
 //   warp 9          one thread issues tcgen05.mma: S_i = Q_i K^T (both operands in shared
@@ -56,7 +58,7 @@ template <int MT> struct TcShape {
   // tensor memory: O of each tile (128 fp32 columns), S (128, one for both tiles), P of each tile (64: 128 bf16)
   static constexpr uint32_t TMEM_COLS = 512, COL_S = 128 * MT, COL_P = 128 * MT + 128;
 };
-constexpr float TC_RESCALE_GAP = 8.f;      // raise the reference maximum only beyond 2^8
+constexpr float TC_RESCALE_GAP = 8.f;      // the reference maximum is raised beyond 2^8 only, or (exact_max) whenever it grows
 constexpr long long TC_WAIT_CYCLES = 4000000000ll;   // ~2 s: far beyond any legitimate wait
 constexpr int TC_XO_PITCH = TC_D + 4;      // floats per row of the partial result a CTA leaves in shared memory
 constexpr int TC_XO_ROW_BYTES = TC_XO_PITCH * 4;                 // (the rows' (max, sum) pairs follow the rows)
@@ -75,6 +77,7 @@ struct TcArgs {
   int B, N, W, Hq, Hkv, g;
   int npt;                     // nodes per query tile, 128 / g (rows from npt * g on hold nothing)
   float scale_log2;
+  float gap;                   // how far a row's maximum may outgrow the reference before that is raised
   int splits, m_blocks;
   int early;                   // launched beside the kernel that grows the trees (see the kernel)
   int cluster_merge;           // the key ranges of a (sequence, head, tile pair) form a cluster and merge in shared memory
@@ -511,7 +514,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       const float mx_x = mx * a.scale_log2;
       float alpha = 1.f;
       if (m_used == -CUDART_INF_F) m_used = mx_x;
-      else if (mx_x > m_used + TC_RESCALE_GAP) {
+      else if (mx_x > m_used + a.gap) {
         alpha = fast_exp2(m_used - mx_x);
         l_run *= alpha;
         m_used = mx_x;
@@ -835,7 +838,7 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
                                  const void *kt, const void *vt, const int64_t *kv_start, const int32_t *block_table,
                                  int bt_stride, int64_t stride_t,
                                  int64_t stride_h, int64_t kv_tokens, int max_prefix_len, float sm_scale, void *out,
-                                 int splits, int m_blocks, bool one, cudaStream_t st, int *merged_in_kernel,
+                                 int splits, int m_blocks, bool one, bool exact_max, cudaStream_t st, int *merged_in_kernel,
                                  const int32_t *early_prefix) {
   *merged_in_kernel = 0;
   const int N = c->p.budget, Hq = c->p.n_q_heads, Hkv = c->p.n_kv_heads, g = Hq / Hkv, B = c->B, npt = 128 / g;
@@ -865,6 +868,7 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
   a.mask = (const unsigned long long *)t->mask;
   a.B = B; a.N = N; a.W = c->W; a.Hq = Hq; a.Hkv = Hkv; a.g = g; a.npt = npt;
   a.scale_log2 = sm_scale * 1.4426950408889634f;
+  a.gap = exact_max ? 0.f : TC_RESCALE_GAP;
   a.splits = splits; a.m_blocks = m_blocks;
   a.out = (__nv_bfloat16 *)out; a.part_o = c->d_attn_o; a.part_ml = c->d_attn_ml; a.status = c->d_status;
   (void)max_prefix_len;

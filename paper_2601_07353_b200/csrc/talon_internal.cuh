@@ -247,7 +247,7 @@ int attention_tc_clusters(talon_ctx *c, bool one, int splits);
 talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *q, const void *kp, const void *vp,
                                  const void *kt, const void *vt, const int64_t *kv_start, const int32_t *block_table,
                                  int bt_stride, int64_t stride_t, int64_t stride_h, int64_t kv_tokens, int max_prefix_len, float sm_scale, void *out,
-                                 int splits, int m_blocks, bool one, cudaStream_t st, int *merged_in_kernel,
+                                 int splits, int m_blocks, bool one, bool exact_max, cudaStream_t st, int *merged_in_kernel,
                                  const int32_t *early_prefix);
 talon_status launch_accept(talon_ctx *c, const talon_tree *t, const float *target_logits,
                            int64_t row_stride, int32_t *target_tok, int32_t *accept_len,
