@@ -353,6 +353,71 @@ talon_status attention_mma_setup() {
                  cudaSuccess ? TALON_OK : TALON_ERR_CUDA;
 }
 
+// How the tensor-core kernel is launched: its kind, the key ranges, and whether the reference follows the maximum.
+struct AttnPlan { int kind, splits; bool exact_max; };
+static AttnPlan plan_attention(talon_ctx *c, const AttnArgs &a, int tiles, bool early, bool split_p) {
+  const int heads = c->B * a.Hkv;
+  const int ctas = split_p ? a.m_blocks * heads : (a.m_blocks + 1) / 2 * heads;
+  const bool only_one = split_p || a.m_blocks == 1;
+  bool one = only_one;
+  int sp = 1;
+  // How exact the rounding of P to bf16 is hangs on the ranges: a row's largest probability in the first tile of
+  // each is 1 and so exact, and its neighbours round with half the error.  `usual`: as many ranges as the SMs and two
+  // tiles a range allow (eight rather than nine or more, where a cluster has enough rows to merge).  With fewer the
+  // reference follows every growth of the maximum (exact_max), which comes closer to 64 bits than the usual number
+  // does (512 keys 2.20e-3 of the norm against 2.25e-3, 2048 keys 2.23e-3 against 2.28e-3; without it 2.30e-3
+  // and 2.33e-3) for a rescale of O now and then, 0.15 us a key tile with one query tile and 0.3 with two.
+  int usual = 1;
+  if (!split_p && ctas < c->sm_count) {
+    usual = std::max(1, std::min(c->sm_count / ctas, (tiles + c->attn_min_tiles - 1) / c->attn_min_tiles));
+    if (usual > 8 && c->attn_cluster && heads * a.g * a.N >= 1024) usual = 8;
+  }
+  if (ctas < c->sm_count) {
+    // Room for key ranges, or for a CTA per query tile instead of two tiles: the cheapest by a model in
+    // microseconds, fitted to 1 to 4 sequences of 1-3 query tiles over 2048 tokens.  A key tile takes a CTA
+    // 1.2 with one query tile and 1.6 with two, all before the first another 2.6; writing the result of one
+    // range 1.6 a query tile.  Merging ranges in a cluster moves a CTA's partial result, 64 KB a query
+    // tile, between SMs; the second kernel (more ranges than a cluster has CTAs) 8 and 11.  Clusters whose
+    // CTAs fill SMs only fit a GPC at a time, so the device says how many it holds: a second round of them
+    // doubles the time.  Started beside the growth of the trees (about 1.2 a layer), the work on the prefix
+    // counts only where it takes longer than that.
+    const float growing = early ? 1.2f * c->p.max_depth : 0.f;
+    auto cost = [&](bool single, int s) {
+      const int n = single ? a.m_blocks * heads : ctas;
+      const int held = s >= 2 && s <= 8 && c->attn_cluster ? attention_tc_clusters(c, split_p ? TC_SPLIT_P : single ? TC_SINGLE : TC_PAIR, s) : 0;
+      const int slots = held > 0 ? held : std::max(c->sm_count / s, 1);
+      const float end = s == 1 ? (single ? 1.6f : 3.2f) : held == 0 ? (single ? 8.f : 11.f)
+                        : s <= 4 ? (single ? 4.9f : 7.3f) : (single ? 5.9f : 9.f);
+      const float tile = split_p ? 1.4f : single ? 1.2f : 1.6f, rescale = s < usual ? (single ? 0.15f : 0.3f) : 0.f;
+      const float before = 2.6f + ((tiles + s - 1) / s - 1) * (tile + rescale);
+      return (n + slots - 1) / slots * (std::max(before, growing) + tile) + end;
+    };
+    const int most = std::min((tiles + c->attn_min_tiles - 1) / c->attn_min_tiles, c->attn_cluster == 2 ? 8 : c->sm_count);
+    float best = cost(one, 1);
+    for (int single = only_one || c->attn_force_tiles == 1; single <= (c->attn_force_tiles != 2 || only_one); ++single)
+      for (int s = 1; s <= std::min(most, c->sm_count / (single ? a.m_blocks * heads : ctas)); ++s) {
+        const float t = cost(single, s);
+        if (t < best) { best = t; sp = s; one = single; }
+      }
+  } else if (ctas % c->sm_count) {
+    // More CTAs than SMs and a ragged last wave: halving the key ranges can fill it (512 CTAs on
+    // 148 SMs are 4 waves of 257 tiles, 1024 half CTAs are 7 waves of 129).  Cost model in key
+    // tiles: waves x (tiles per CTA + 2 for the prologue and epilogue), plus what merging the
+    // partial results costs, about one tile per 24 CTAs per SM.
+    const long long sm = c->sm_count;
+    auto cost = [&](int s) {
+      const long long n = (long long)ctas * s;
+      const long long waves = (n + sm - 1) / sm;
+      return waves * ((tiles + s - 1) / s + 2) + (s > 1 ? n / (24 * sm) + 3 : 0);
+    };
+    if (tiles >= 32 && cost(2) < cost(1)) sp = 2;
+  }
+  if (c->attn_force_splits > 0) sp = c->attn_force_splits;
+  if (c->attn_force_tiles > 0) one = c->attn_force_tiles == 1 || only_one;
+  while (sp > 1 && (size_t)a.m_blocks * c->B * a.Hkv * sp * AT_BM > c->attn_ml_elems) --sp;
+  return {split_p ? TC_SPLIT_P : one ? TC_SINGLE : TC_PAIR, sp, sp < usual};
+}
+
 talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, const void *kp, const void *vp,
                               const void *kt, const void *vt, const int64_t *kv_start, const int32_t *block_table,
                               int bt_stride, int64_t kv_tokens,
@@ -375,68 +440,26 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
     a.m_blocks = attn_tc_blocks(c);
     a.npt = AT_BM / a.g;
     const int tiles = (max_prefix_len + 127) / 128 + (a.N + 127) / 128, heads = c->B * a.Hkv;
-    const int ctas = (a.m_blocks + 1) / 2 * heads;
-    bool one = a.m_blocks == 1;
-    int sp = 1;
-    // How exact the rounding of P to bf16 is hangs on the ranges: a row's largest probability in the first tile of
-    // each is 1 and so exact, and its neighbours round with half the error.  `usual`: as many ranges as the SMs and two
-    // tiles a range allow (eight rather than nine or more, where a cluster has enough rows to merge).  With fewer the
-    // reference follows every growth of the maximum (exact_max), which comes closer to 64 bits than the usual number
-    // does (512 keys 2.20e-3 of the norm against 2.25e-3, 2048 keys 2.23e-3 against 2.28e-3; without it 2.30e-3
-    // and 2.33e-3) for a rescale of O now and then, 0.15 us a key tile with one query tile and 0.3 with two.
-    int usual = 1;
-    if (ctas < c->sm_count) {
-      usual = std::max(1, std::min(c->sm_count / ctas, (tiles + c->attn_min_tiles - 1) / c->attn_min_tiles));
-      if (usual > 8 && c->attn_cluster && heads * a.g * a.N >= 1024) usual = 8;
-      // Room for key ranges, or for a CTA per query tile instead of two tiles: the cheapest by a model in
-      // microseconds, fitted to 1 to 4 sequences of 1-3 query tiles over 2048 tokens.  A key tile takes a CTA
-      // 1.2 with one query tile and 1.6 with two, all before the first another 2.6; writing the result of one
-      // range 1.6 a query tile.  Merging ranges in a cluster moves a CTA's partial result, 64 KB a query
-      // tile, between SMs; the second kernel (more ranges than a cluster has CTAs) 8 and 11.  Clusters whose
-      // CTAs fill SMs only fit a GPC at a time, so the device says how many it holds: a second round of them
-      // doubles the time.  Started beside the growth of the trees (about 1.2 a layer), the work on the prefix
-      // counts only where it takes longer than that.
-      const float growing = early_prefix ? 1.2f * c->p.max_depth : 0.f;
-      auto cost = [&](bool single, int s) {
-        const int n = single ? a.m_blocks * heads : ctas;
-        const int held = s >= 2 && s <= 8 && c->attn_cluster ? attention_tc_clusters(c, single, s) : 0;
-        const int slots = held > 0 ? held : std::max(c->sm_count / s, 1);
-        const float end = s == 1 ? (single ? 1.6f : 3.2f) : held == 0 ? (single ? 8.f : 11.f)
-                          : s <= 4 ? (single ? 4.9f : 7.3f) : (single ? 5.9f : 9.f);
-        const float tile = single ? 1.2f : 1.6f, rescale = s < usual ? (single ? 0.15f : 0.3f) : 0.f;
-        const float before = 2.6f + ((tiles + s - 1) / s - 1) * (tile + rescale);
-        return (n + slots - 1) / slots * (std::max(before, growing) + tile) + end;
-      };
-      const int most = std::min((tiles + c->attn_min_tiles - 1) / c->attn_min_tiles, c->attn_cluster == 2 ? 8 : c->sm_count);
-      float best = cost(one, 1);
-      for (int single = a.m_blocks == 1 || c->attn_force_tiles == 1; single <= (c->attn_force_tiles != 2 || a.m_blocks == 1); ++single)
-        for (int s = 1; s <= std::min(most, c->sm_count / (single ? a.m_blocks * heads : ctas)); ++s) {
-          const float t = cost(single, s);
-          if (t < best) { best = t; sp = s; one = single; }
-        }
-    } else if (ctas % c->sm_count) {
-      // More CTAs than SMs and a ragged last wave: halving the key ranges can fill it (512 CTAs on
-      // 148 SMs are 4 waves of 257 tiles, 1024 half CTAs are 7 waves of 129).  Cost model in key
-      // tiles: waves x (tiles per CTA + 2 for the prologue and epilogue), plus what merging the
-      // partial results costs, about one tile per 24 CTAs per SM.
-      const long long sm = c->sm_count;
-      auto cost = [&](int s) {
-        const long long n = (long long)ctas * s;
-        const long long waves = (n + sm - 1) / sm;
-        return waves * ((tiles + s - 1) / s + 2) + (s > 1 ? n / (24 * sm) + 3 : 0);
-      };
-      if (tiles >= 32 && cost(2) < cost(1)) sp = 2;
+    const bool odd = AT_BM % a.g != 0;
+    AttnPlan plan = plan_attention(c, a, tiles, early_prefix != nullptr, false);
+    plan.exact_max |= odd;
+    if (odd) {
+      // Query groups that do not divide 128 ran on the warp-MMA kernel once.  Its 64-key tiles, and up to `finer` ranges,
+      // make more of the largest probabilities exact: 2.06e-3 to 2.30e-3 of the norm, and up to 6 % more in 128-key tiles
+      // even if the reference follows every growth.  With sixteen tiles a range and no more than twice our ranges there,
+      // the two are within 0.2 % (two seeds differ by 0.5); elsewhere P goes in as two parts (1.66e-3), 0 to 30 % more
+      // time for a step of 100 to 700 keys.  At 2000 keys and 8 sequences two parts cost 46 %, following the maximum 4 %.
+      const int blocks = attn_m_blocks(c) * heads, keys64 = (max_prefix_len + AT_BN - 1) / AT_BN + (a.N + AT_BN - 1) / AT_BN;
+      const int finer = blocks < c->sm_count ? std::max(1, std::min(c->sm_count / blocks, keys64)) : 1;
+      if (tiles < 16 * plan.splits || finer > 2 * plan.splits) plan = plan_attention(c, a, tiles, early_prefix != nullptr, true);
     }
-    if (c->attn_force_splits > 0) sp = c->attn_force_splits;
-    if (c->attn_force_tiles > 0) one = c->attn_force_tiles == 1 || a.m_blocks == 1;
-    while (sp > 1 && (size_t)a.m_blocks * c->B * a.Hkv * sp * AT_BM > c->attn_ml_elems) --sp;
-    a.splits = sp;
-    const bool exact_max = sp < usual;
+    a.splits = plan.splits;
     int merged = 0;
     talon_status r = launch_attention_tc(c, t, q, kp, vp, kt, vt, kv_start, block_table, bt_stride, stride_t, stride_h, kv_tokens,
-                                         max_prefix_len, sm_scale, out, sp, a.m_blocks, one, exact_max, st, &merged, early_prefix);
+                                         max_prefix_len, sm_scale, out, plan.splits, a.m_blocks, plan.kind, plan.exact_max, st, &merged,
+                                         early_prefix);
     if (r != TALON_OK) return r;
-    if (sp > 1 && !merged) {
+    if (plan.splits > 1 && !merged) {
       const int64_t rows = (int64_t)c->B * a.Hkv * a.g * a.N;
       const int wpb = 8;
       LaunchTimer lt(c, TALON_K_COMBINE, st);

@@ -55,8 +55,9 @@ template <int MT> struct TcShape {
   static constexpr int LAUNCH_REGS = 168, SOFT_REGS = 216, OTHER_REGS = 72;      // the split: MT == 2 only
   static_assert(MT == 1 || 256 * SOFT_REGS + 128 * OTHER_REGS <= THREADS * LAUNCH_REGS, "setmaxnreg would wait for good");
   static constexpr int SMEM = (MT + 2 * STAGES) * TC_TILE_BYTES + 1024 + TC_NBARS * 8 + 64;
-  // tensor memory: O of each tile (128 fp32 columns), S (128, one for both tiles), P of each tile (64: 128 bf16)
-  static constexpr uint32_t TMEM_COLS = 512, COL_S = 128 * MT, COL_P = 128 * MT + 128;
+  // tensor memory: O of each tile (128 fp32 columns), S (128, one for both tiles), P of each tile (64: 128 bf16),
+  // with SPLIT_P what P's rounding left (64)
+  static constexpr uint32_t TMEM_COLS = 512, COL_S = 128 * MT, COL_P = 128 * MT + 128, COL_REST = COL_P + 64 * MT;
 };
 constexpr float TC_RESCALE_GAP = 8.f;      // the reference maximum is raised beyond 2^8 only, or (exact_max) whenever it grows
 constexpr long long TC_WAIT_CYCLES = 4000000000ll;   // ~2 s: far beyond any legitimate wait
@@ -250,7 +251,10 @@ __device__ inline void cluster_sync_all() {
 
 }  // namespace
 
-template <int MT>
+// SPLIT_P: P goes into the product with V as two bf16 numbers, its rounding and what that left (2^-17 of it), so that
+// the output's own rounding is all that is left of the error.  For query groups that do not divide 128 (launch_attention
+// has the rule).
+template <int MT, bool SPLIT_P>
 __global__ void __launch_bounds__(TcShape<MT>::THREADS, 1)
 tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kp,
                          const __grid_constant__ CUtensorMap map_vp, const __grid_constant__ CUtensorMap map_kt,
@@ -410,6 +414,11 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             for (int kk = 0; kk < TC_BN / 32; ++kk)
               tc_mma_ts(tmem + 128 * i, tmem + COL_P + 64 * i + (half * 4 + kk) * 8, vd + (((half * 4 + kk) * 2048) >> 4),
                         IDESC_PV, (it > 0 || half > 0 || kk > 0) ? 1u : 0u);
+            if (SPLIT_P)
+#pragma unroll
+              for (int kk = 0; kk < TC_BN / 32; ++kk)
+                tc_mma_ts(tmem + 128 * i, tmem + TcShape<MT>::COL_REST + 64 * i + (half * 4 + kk) * 8,
+                          vd + (((half * 4 + kk) * 2048) >> 4), IDESC_PV, 1u);
             if (half) {
               tc_commit(bar(B_ODONE + i));
               tc_commit(bar(B_VEMPTY + s));
@@ -547,7 +556,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       unsigned long long sum2[4] = {0ull, 0ull, 0ull, 0ull};          // four pairs of 0.f
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
-        uint32_t pk[32];
+        uint32_t pk[32], rest[SPLIT_P ? 32 : 1];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
 #pragma unroll
@@ -558,10 +567,13 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             unpack_f32x2(x2, x0, x1);
             const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
             sum2[(c >> 1) & 3] = add_f32x2(sum2[(c >> 1) & 3], pack_f32x2(p0, p1));
-            pk[q * 16 + (c >> 1)] = pack_bf16x2(p0, p1);
+            const uint32_t both = pack_bf16x2(p0, p1);
+            pk[q * 16 + (c >> 1)] = both;
+            if (SPLIT_P) rest[q * 16 + (c >> 1)] = pack_bf16x2(p0 - __uint_as_float(both << 16), p1 - __uint_as_float(both & 0xFFFF0000u));
           }
         }
         tc_st32(t_P + half * 32, pk);
+        if constexpr (SPLIT_P) tc_st32(t_lane + TcShape<MT>::COL_REST + 64 * i + half * 32, rest);
         tc_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -793,6 +805,20 @@ bool encode_bf16(CUtensorMap *m, const void *ptr, int rank, const cuuint64_t *di
 
 }  // namespace
 
+namespace {
+
+struct TcLaunch {
+  void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, TcArgs);
+  int threads, smem;
+};
+TcLaunch tc_launch(int kind) {
+  if (kind == TC_PAIR) return {tree_attention_tc_kernel<2, false>, TcShape<2>::THREADS, TcShape<2>::SMEM};
+  if (kind == TC_SINGLE) return {tree_attention_tc_kernel<1, false>, TcShape<1>::THREADS, TcShape<1>::SMEM};
+  return {tree_attention_tc_kernel<1, true>, TcShape<1>::THREADS, TcShape<1>::SMEM};
+}
+
+}  // namespace
+
 bool attention_tc_supported(const talon_ctx *c, int64_t stride_t, int64_t stride_h, float sm_scale) {
   const int g = c->p.n_q_heads / c->p.n_kv_heads;
   if (c->p.head_dim != 128 || c->p.budget > 128) return false;
@@ -805,29 +831,31 @@ bool attention_tc_supported(const talon_ctx *c, int64_t stride_t, int64_t stride
 talon_status attention_tc_setup() {
   // (a register split beyond what the block was launched with would never be granted)
   cudaFuncAttributes at;
-  if (cudaFuncGetAttributes(&at, tree_attention_tc_kernel<2>) != cudaSuccess || at.numRegs != TcShape<2>::LAUNCH_REGS) return TALON_ERR_CUDA;
-  return cudaFuncSetAttribute(tree_attention_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcShape<1>::SMEM) == cudaSuccess &&
-                 cudaFuncSetAttribute(tree_attention_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcShape<2>::SMEM) ==
-                     cudaSuccess
-             ? TALON_OK : TALON_ERR_CUDA;
+  if (cudaFuncGetAttributes(&at, tree_attention_tc_kernel<2, false>) != cudaSuccess || at.numRegs != TcShape<2>::LAUNCH_REGS) return TALON_ERR_CUDA;
+  for (int kind : {TC_PAIR, TC_SINGLE, TC_SPLIT_P}) {
+    const TcLaunch l = tc_launch(kind);
+    if (cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, l.smem) != cudaSuccess) return TALON_ERR_CUDA;
+  }
+  return TALON_OK;
 }
 
 // How many clusters of `splits` CTAs (one per key range, a whole SM each) the device can hold at once; 0: it
 // cannot place one.  The SMs of a cluster share a GPC, so this is less than SMs / splits.
-int attention_tc_clusters(talon_ctx *c, bool one, int splits) {
+int attention_tc_clusters(talon_ctx *c, int kind, int splits) {
   if (splits < 2 || splits > 8) return 0;
-  int &known = c->attn_clusters[one ? 0 : 1][splits];
+  int &known = c->attn_clusters[kind][splits];
   if (known < 0) {
+    const TcLaunch l = tc_launch(kind);
     cudaLaunchConfig_t q = {};
     q.gridDim = dim3(1, splits, 1);
-    q.blockDim = dim3(one ? TcShape<1>::THREADS : TcShape<2>::THREADS);
-    q.dynamicSmemBytes = one ? TcShape<1>::SMEM : TcShape<2>::SMEM;
+    q.blockDim = dim3(l.threads);
+    q.dynamicSmemBytes = l.smem;
     cudaLaunchAttribute qa[1];
     qa[0].id = cudaLaunchAttributeClusterDimension;
     qa[0].val.clusterDim.x = 1; qa[0].val.clusterDim.y = (unsigned)splits; qa[0].val.clusterDim.z = 1;
     q.attrs = qa; q.numAttrs = 1;
     int n = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, one ? tree_attention_tc_kernel<1> : tree_attention_tc_kernel<2>, &q);
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, l.kernel, &q);
     if (e != cudaSuccess) cudaGetLastError();
     known = e == cudaSuccess ? n : 0;
   }
@@ -838,7 +866,7 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
                                  const void *kt, const void *vt, const int64_t *kv_start, const int32_t *block_table,
                                  int bt_stride, int64_t stride_t,
                                  int64_t stride_h, int64_t kv_tokens, int max_prefix_len, float sm_scale, void *out,
-                                 int splits, int m_blocks, bool one, bool exact_max, cudaStream_t st, int *merged_in_kernel,
+                                 int splits, int m_blocks, int kind, bool exact_max, cudaStream_t st, int *merged_in_kernel,
                                  const int32_t *early_prefix) {
   *merged_in_kernel = 0;
   const int N = c->p.budget, Hq = c->p.n_q_heads, Hkv = c->p.n_kv_heads, g = Hq / Hkv, B = c->B, npt = 128 / g;
@@ -872,18 +900,17 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
   a.splits = splits; a.m_blocks = m_blocks;
   a.out = (__nv_bfloat16 *)out; a.part_o = c->d_attn_o; a.part_ml = c->d_attn_ml; a.status = c->d_status;
   (void)max_prefix_len;
-  auto kernel = one ? tree_attention_tc_kernel<1> : tree_attention_tc_kernel<2>;
-  const int threads = one ? TcShape<1>::THREADS : TcShape<2>::THREADS, smem = one ? TcShape<1>::SMEM : TcShape<2>::SMEM;
-  dim3 grid(one ? m_blocks : (m_blocks + 1) / 2, splits, B * Hkv);
+  const TcLaunch l = tc_launch(kind);
+  dim3 grid(kind == TC_PAIR ? (m_blocks + 1) / 2 : m_blocks, splits, B * Hkv);
   // Two to eight key ranges: they are launched as one thread-block cluster and merge their partial
   // results through distributed shared memory, if the device can place such a cluster (asked once
   // per cluster size; a cluster of full-SM CTAs needs that many SMs free in one GPC).
-  a.cluster_merge = c->attn_cluster && attention_tc_clusters(c, one, splits) > 0;
+  a.cluster_merge = c->attn_cluster && attention_tc_clusters(c, kind, splits) > 0;
   {
     LaunchTimer lt(c, TALON_K_ATTENTION, st);
     if (a.cluster_merge) {
       cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+      cfg.gridDim = grid; cfg.blockDim = dim3(l.threads); cfg.dynamicSmemBytes = l.smem; cfg.stream = st;
       cudaLaunchAttribute attr[2];
       attr[0].id = cudaLaunchAttributeClusterDimension;
       attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = (unsigned)splits; attr[0].val.clusterDim.z = 1;
@@ -891,10 +918,10 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
       attr[1].val.programmaticStreamSerializationAllowed = 1;
       cfg.attrs = attr;
       cfg.numAttrs = (c->pdl == 1 || (c->pdl < 0 && (c->B <= PDL_AUTO_BATCH || early_prefix))) ? 2 : 1;
-      cudaLaunchKernelEx(&cfg, kernel, mq, mkp, mvp, mkt, mvt, a);
+      cudaLaunchKernelEx(&cfg, l.kernel, mq, mkp, mvp, mkt, mvt, a);
       *merged_in_kernel = 1;
     } else {
-      launch_kernel_pdl(c, early_prefix != nullptr, kernel, grid, dim3(threads), smem, st, mq, mkp, mvp, mkt, mvt, a);
+      launch_kernel_pdl(c, early_prefix != nullptr, l.kernel, grid, dim3(l.threads), l.smem, st, mq, mkp, mvp, mkt, mvt, a);
     }
   }
   if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;

@@ -128,7 +128,7 @@ struct talon_ctx {
   int step_rows;                     // 0: whole steps expand layer by layer too
   int step_first_rows;               // > 0: slots per sequence the first round of a step prepares (for experiments)
   int attn_cluster;                  // key ranges of the tensor-core attention merge inside a cluster (1; 2: never more of them than it has CTAs) or in a second kernel (0)
-  int attn_clusters[2][9];           // per query tiles of a CTA (1, 2) and cluster size: clusters the device holds at once (-1 not asked yet)
+  int attn_clusters[3][9];           // per kind of the tensor-core attention and cluster size: clusters the device holds at once (-1 not asked yet)
   int attn_force_splits;             // > 0: key ranges per (sequence, head, query tiles), for experiments
   int attn_force_tiles;              // 1, 2: query tiles of a CTA, for experiments
   int argmax_oversplit;              // target argmax: chunk rounds per CTA when the rows outnumber the grid
@@ -243,11 +243,12 @@ talon_status launch_attention(talon_ctx *c, const talon_tree *t, const void *q, 
                               int max_prefix_len, float sm_scale, void *out, cudaStream_t st,
                               const int32_t *early_prefix = nullptr);
 bool attention_tc_supported(const talon_ctx *c, int64_t stride_t, int64_t stride_h, float sm_scale);
-int attention_tc_clusters(talon_ctx *c, bool one, int splits);
+enum { TC_PAIR = 0, TC_SINGLE = 1, TC_SPLIT_P = 2 };      // query tiles of a CTA; one with P in two bf16 parts
+int attention_tc_clusters(talon_ctx *c, int kind, int splits);
 talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *q, const void *kp, const void *vp,
                                  const void *kt, const void *vt, const int64_t *kv_start, const int32_t *block_table,
                                  int bt_stride, int64_t stride_t, int64_t stride_h, int64_t kv_tokens, int max_prefix_len, float sm_scale, void *out,
-                                 int splits, int m_blocks, bool one, bool exact_max, cudaStream_t st, int *merged_in_kernel,
+                                 int splits, int m_blocks, int kind, bool exact_max, cudaStream_t st, int *merged_in_kernel,
                                  const int32_t *early_prefix);
 talon_status launch_accept(talon_ctx *c, const talon_tree *t, const float *target_logits,
                            int64_t row_stride, int32_t *target_tok, int32_t *accept_len,

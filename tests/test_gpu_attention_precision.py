@@ -42,3 +42,19 @@ def test_few_ctas(B, N, L):
         torch.cuda.synchronize()
         assert _error(s, 32, 8) <= 2.27e-3
     t.close()
+
+
+# Groups of 3, 5 and 7.  Short contexts: P in two parts leaves the output's own rounding, 1.65e-3 (the warp-MMA kernel,
+# which these groups once ran on: 2.06e-3 to 2.26e-3).  Long ones: the reference follows the maximum, at most 2.30e-3 as
+# there (2.34e-3 with 2^8 of slack).
+@pytest.mark.parametrize("hq,hkv,B", [(24, 8, 1), (24, 8, 20), (40, 8, 1), (40, 8, 4), (28, 4, 2), (28, 4, 40)])
+@pytest.mark.parametrize("L", [0, 200, 1000, 4100])
+def test_groups_that_do_not_divide_a_query_tile(hq, hkv, B, L):
+    talon, t = _talon(B, 3000, 60, 8, 12, hq=hq, hkv=hkv)
+    s = Step(t, B, 3000, 60, 12, hq, hkv, [L] * B, 12)
+    s.out.fill_(float("nan"))
+    for run in (s.calls, s.step):
+        run(t)
+        torch.cuda.synchronize()
+        assert _error(s, hq, hkv) <= (1.8e-3 if L <= 1000 else 2.3e-3)
+    t.close()
