@@ -78,6 +78,15 @@ __device__ __forceinline__ u64 add_f32x2(u64 a, u64 b) {
   return d;
 }
 
+// A maximum ignores NaN, so a lane that has seen nothing but NaN and -inf (or the fill past the slice) still has -inf
+// for a maximum and takes no exponentials; any other lane's sum shows a NaN.
+__device__ __forceinline__ bool lane_nan(const float (&v)[16]) {
+  bool bad = false;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) bad |= v[i] != v[i];
+  return bad;
+}
+
 // ---- bulk-copy ring ----
 __device__ inline uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ inline void ring_bar_init(uint32_t bar) {
@@ -566,6 +575,8 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
         float s0, s1;
         unpack_f32x2(add_f32x2(acc0, acc1), s0, s1);
         st += s0 + s1;
+      } else if (lane_nan(v)) {
+        st = CUDART_NAN_F;
       }
     }
     // the warp's largest lane maximum and its (share_pos + 1)-th largest
@@ -686,6 +697,8 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
         float s0, s1;
         unpack_f32x2(add_f32x2(acc0, acc1), s0, s1);
         w.s_t += s0 + s1;
+      } else if (lane_nan(v)) {
+        w.s_t = CUDART_NAN_F;
       }
       refreshed = (t & (t + 1)) == 0 || t == 2;  // after tiles 1, 2, 3, 4, 8, 16, ... of the slice
       // (the first tile has nothing but its own lane maxima to go by: their exact ke-th largest)
