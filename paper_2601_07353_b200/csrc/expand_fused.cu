@@ -574,10 +574,7 @@ void (*fused_kernel_for(const talon_ctx *c))(FusedArgs) {
 
 talon_status expand_fused_setup(talon_ctx *c) {
   const size_t bytes = fused_smem_bytes(c);
-  if (cudaFuncSetAttribute(fused_kernel_for(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(bytes + fused_base_bytes(c->p.batch_max))) !=
-      cudaSuccess)
-    return TALON_ERR_CUDA;
+  if (!allow_shared_memory(c, fused_kernel_for(c))) return TALON_ERR_CUDA;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_kernel_for(c), EXP_THREADS, bytes) !=
       cudaSuccess || per_sm < 1)

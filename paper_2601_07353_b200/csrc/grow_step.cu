@@ -571,10 +571,7 @@ static void (*row_pass_for(const talon_ctx *c))(RowPassArgs) {
 }
 
 talon_status grow_step_setup(talon_ctx *c) {
-  if (cudaFuncSetAttribute(row_pass_for(c), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_pass_smem(c, true)) != cudaSuccess ||
-      cudaFuncSetAttribute(grow_kernel_for(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)grow_smem_bytes(c->p.budget, c->k_cap, c->p.budget)) != cudaSuccess)
-    return TALON_ERR_CUDA;
+  if (!allow_shared_memory(c, row_pass_for(c)) || !allow_shared_memory(c, grow_kernel_for(c))) return TALON_ERR_CUDA;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, row_pass_for(c), EXP_THREADS, row_pass_smem(c, false)) != cudaSuccess ||
       per_sm < 1)

@@ -213,6 +213,17 @@ struct LaunchTimer {
   }
 };
 
+// Lets `kernel` be launched with as much dynamic shared memory as the device has.  The bound belongs to the kernel, not to
+// a context: set to what one context needs, it would refuse the launches of an older one that needs more.
+template <typename... KArgs>
+inline bool allow_shared_memory(const talon_ctx *c, void (*kernel)(KArgs...)) {
+  int most = 0;
+  cudaFuncAttributes at;
+  return cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) == cudaSuccess &&
+         cudaFuncGetAttributes(&at, kernel) == cudaSuccess &&
+         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes) == cudaSuccess;
+}
+
 // launchers implemented in the .cu files (all asynchronous on `st`).  launch_attention's early_prefix: the
 // kernel launched just before is grow_kernel, and this array holds the prefix lengths it copies
 talon_status launch_reset(talon_ctx *c, const talon_tree *t, const int32_t *root_tok,

@@ -133,3 +133,23 @@ def test_a_host_step_follows_what_its_stream_still_has_to_do(own):
         assert torch.equal(got, want.cpu())
     assert (res[0].float() - s.out.cpu().float()).abs().max() <= ATT_TOL
     t.close()
+
+
+# (keys a row, budget, batch) of an older context and of a smaller one that uses the same kernels
+@pytest.mark.parametrize("older,newer", [((8, 128, 40), (5, 66, 1)), ((32, 128, 40), (17, 65, 1)), ((60, 128, 40), (33, 40, 1))])
+def test_a_smaller_context_does_not_stop_an_older_one(older, newer):
+    (k, N, B), (k2, N2, B2), V, D = older, newer, 3001, 4
+    talon, t = _talon(B, V, N, 8, D, cand=k)
+    s = Step(t, B, V, N, D, 8, 2, [10] * B, 5)
+    s.step(t)
+    torch.cuda.synchronize()
+    want = s.whole()
+    talon, other = _talon(B2, V, N2, 8, D, cand=k2)
+    for run in (s.step, s.calls):
+        run(t)
+        torch.cuda.synchronize()
+        assert t.poll_status() == talon.OK
+        for a, b in zip(want, s.whole()):
+            assert torch.equal(a, b)
+    other.close()
+    t.close()
