@@ -331,8 +331,8 @@ talon_status talon_commit_paged(talon_ctx *ctx, const talon_tree *tree, const in
  * keeps only the last step's).  root_tok, prefix_len, the cache and counters ([B, 3], as in
  * talon_commit; required) are read and advanced in place.
  *  max_prefix_len  bound on prefix_len[b] over ALL steps (the last step's prefix included)
- * The rows of several steps may be read ahead, and the device status then covers those steps together:
- * a row that is not finite in one of them is reported after the last. */
+ * The rows of several steps may be read ahead.  The device status afterwards is the last step's, as after
+ * separate calls. */
 talon_status talon_loop(talon_ctx *ctx, const talon_tree *tree, int32_t B, int32_t n_steps,
                         int32_t *root_tok, int32_t *prefix_len, const float *draft_logits,
                         int64_t draft_row_stride, int64_t draft_step_stride, int32_t n_layers,

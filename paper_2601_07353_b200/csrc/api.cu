@@ -164,7 +164,7 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
       if (pass) *ptr = reinterpret_cast<std::remove_reference_t<decltype(*ptr)>>(static_cast<char *>(c->d_arena) + total);
       total += (count * sizeof(**ptr) + 255) / 256 * 256;
     };
-    take(&c->d_status, 1);
+    take(&c->d_status, 2);
     take(&c->d_row_count, rows);
     take(&c->d_seq_count, bm);
     take(&c->d_walk_count, bm);
@@ -476,6 +476,7 @@ talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_
   const bool ahead = !layered && n_layers > 0 && rows_at_once(c) && n_steps > 1;
   if (ahead) c->B = B;
   const bool batched = ahead && talon::loop_rows_possible(c, n_layers);
+  int *const status = c->d_status;
   for (int s = 0; s < n_steps; ++s) {
     // step s reads its own slice of the stand-ins for the two model forwards; the tree, the cache,
     // the prefix lengths and the roots are the state the steps hand on to one another on the device
@@ -489,6 +490,9 @@ talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_
         r = talon::launch_loop_rows(c, draft_logits + draft_step_stride * s, draft_row_stride, draft_step_stride, n_layers,
                                     target_logits + target_step_stride * s, target_row_stride, target_step_stride,
                                     n_steps - s < c->ahead ? n_steps - s : c->ahead, (cudaStream_t)stream);
+      // The status is the last step's, as after separate calls, each of which starts by clearing the word; here only the
+      // row pass clears it, so what an earlier step reports goes to the word beside it.
+      c->d_status = s + 1 < n_steps ? status + 1 : status;
       if (r == TALON_OK)
         r = talon::launch_loop_grow(c, t, root_tok, prefix_len, n_layers, within, target_tok, al, an, bt, (cudaStream_t)stream);
       if (r == TALON_OK)
@@ -503,6 +507,7 @@ talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_
     if (r == TALON_OK)
       r = talon_commit(c, t, al, an, bt, kts, vts, k_prefix, v_prefix, kv_start, kv_limit, kv_tokens, kv_stride_t,
                        kv_stride_h, prefix_len, root_tok, counters, stream);
+    c->d_status = status;
     if (r != TALON_OK) return batched ? abandon_rows(c, r, stream) : r;
   }
   return TALON_OK;

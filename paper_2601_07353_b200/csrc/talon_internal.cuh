@@ -107,7 +107,7 @@ struct talon_ctx {
   double log_mu;
 
   void *d_arena;                  // the one allocation behind the pointers below
-  int *d_status;
+  int *d_status;                  // the status word; the one after it takes what talon_loop's earlier steps report
   int32_t *d_prefix_len;          // [batch_max]
   // expansion workspace
   int exp_grid;                   // CTAs of the streaming kernel at full width

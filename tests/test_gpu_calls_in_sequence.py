@@ -153,3 +153,17 @@ def test_a_smaller_context_does_not_stop_an_older_one(older, newer):
             assert torch.equal(a, b)
     other.close()
     t.close()
+
+
+@pytest.mark.parametrize("where", ["draft", "target"])
+@pytest.mark.parametrize("bad", [0, 3, 9, 10])
+def test_the_status_after_a_loop_is_the_last_steps(bad, where):
+    """Eleven steps, whose rows are prepared eight at a time; a NaN in one of them."""
+    B, V, N, K, D, S = 2, 2003, 20, 5, 4, 11
+    talon, t = _talon(B, V, N, K, D)
+    s = Step(t, B, V, N, D, 8, 2, [90, 33], 3, steps=S)
+    getattr(s, where)[bad, 1, 0, 17] = float("nan")
+    _loop(t, s, S)
+    torch.cuda.synchronize()
+    assert t.poll_status() == (talon.ERR_NONFINITE if bad == S - 1 else talon.OK)
+    t.close()
