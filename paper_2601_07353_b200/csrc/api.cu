@@ -57,6 +57,45 @@ static void free_stage(HostStage *s) {
   delete s;
 }
 
+// All of the staging for total prefixes of `tokens`, or null with nothing kept.
+static HostStage *make_stage(const talon_ctx *c, int64_t tokens) {
+  HostStage *s = new (std::nothrow) HostStage();
+  if (!s) return nullptr;
+  const talon_params &p = c->p;
+  const size_t N = p.budget, V = p.vocab, Dh = p.head_dim, bm = p.batch_max, W = c->W, nrow = bm * N;
+  s->prefix_tokens = tokens;
+  const size_t kv = (size_t)tokens * p.n_kv_heads * Dh * 2;
+  cudaError_t e = cudaSuccess;
+  for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+    size_t total = 0;
+    auto take = [&](auto **ptr, size_t bytes) {
+      if (pass) *ptr = reinterpret_cast<std::remove_reference_t<decltype(*ptr)>>(static_cast<char *>(s->arena) + total);
+      total += (bytes + 255) / 256 * 256;
+    };
+    take(&s->draft, nrow * V * 4); take(&s->target, nrow * V * 4);
+    take(&s->q, nrow * p.n_q_heads * Dh * 2); take(&s->out, nrow * p.n_q_heads * Dh * 2);
+    take(&s->kp, kv); take(&s->vp, kv);
+    take(&s->kt, nrow * p.n_kv_heads * Dh * 2); take(&s->vt, nrow * p.n_kv_heads * Dh * 2);
+    take(&s->root, bm * 4); take(&s->plen, bm * 4); take(&s->kv_start, bm * 8);
+    take(&s->tree.n_nodes, bm * 4);
+    take(&s->tree.token, nrow * 4); take(&s->tree.parent, nrow * 4); take(&s->tree.depth, nrow * 4);
+    take(&s->tree.position, nrow * 4);
+    take(&s->tree.layer_off, bm * (p.max_depth + 2) * 4);
+    take(&s->tree.score, nrow * 8); take(&s->tree.mask, nrow * W * 8);
+    take(&s->accept_len, bm * 4); take(&s->accept_nodes, bm * (p.max_depth + 1) * 4); take(&s->bonus, bm * 4);
+    if (!pass) e = cudaMalloc(&s->arena, total);
+  }
+  if (e == cudaSuccess) e = cudaMallocHost((void **)&s->h_scratch, bm * 12);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->copy, cudaStreamNonBlocking);
+  for (cudaEvent_t *ev : {&s->begin, &s->rows, &s->kv, &s->targets})
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+  if (e == cudaSuccess) return s;
+  std::fprintf(stderr, "talon: staging buffers: %s\n", cudaGetErrorString(e));
+  cudaGetLastError();
+  free_stage(s);
+  return nullptr;
+}
+
 extern "C" {
 
 const char *talon_status_string(talon_status s) {
@@ -761,37 +800,9 @@ talon_status talon_step_host(talon_ctx *c, int32_t B, const int32_t *root_tok, c
     TALON_CUDA_OK(cudaStreamSynchronize(st));
     free_stage(s);
     c->stage = nullptr;
-    s = new (std::nothrow) HostStage();
+    s = make_stage(c, tokens > 0 ? tokens : 1);
     if (!s) return TALON_ERR_CUDA;
     c->stage = s;
-    const size_t bm = p.batch_max, W = c->W, nrow = bm * N;
-    s->prefix_tokens = tokens > 0 ? tokens : 1;
-    const size_t kv = (size_t)s->prefix_tokens * p.n_kv_heads * Dh * 2;
-    for (int pass = 0; pass < 2; ++pass) {
-      size_t total = 0;
-      auto take = [&](auto **ptr, size_t bytes) {
-        if (pass) *ptr = reinterpret_cast<std::remove_reference_t<decltype(*ptr)>>(static_cast<char *>(s->arena) + total);
-        total += (bytes + 255) / 256 * 256;
-      };
-      take(&s->draft, nrow * V * 4); take(&s->target, nrow * V * 4);
-      take(&s->q, nrow * p.n_q_heads * Dh * 2); take(&s->out, nrow * p.n_q_heads * Dh * 2);
-      take(&s->kp, kv); take(&s->vp, kv);
-      take(&s->kt, nrow * p.n_kv_heads * Dh * 2); take(&s->vt, nrow * p.n_kv_heads * Dh * 2);
-      take(&s->root, bm * 4); take(&s->plen, bm * 4); take(&s->kv_start, bm * 8);
-      take(&s->tree.n_nodes, bm * 4);
-      take(&s->tree.token, nrow * 4); take(&s->tree.parent, nrow * 4); take(&s->tree.depth, nrow * 4);
-      take(&s->tree.position, nrow * 4);
-      take(&s->tree.layer_off, bm * (p.max_depth + 2) * 4);
-      take(&s->tree.score, nrow * 8); take(&s->tree.mask, nrow * W * 8);
-      take(&s->accept_len, bm * 4); take(&s->accept_nodes, bm * (p.max_depth + 1) * 4); take(&s->bonus, bm * 4);
-      if (!pass) TALON_CUDA_OK(cudaMalloc(&s->arena, total));
-    }
-    TALON_CUDA_OK(cudaMallocHost((void **)&s->h_scratch, bm * 12));
-    TALON_CUDA_OK(cudaStreamCreateWithFlags(&s->copy, cudaStreamNonBlocking));
-    TALON_CUDA_OK(cudaEventCreateWithFlags(&s->begin, cudaEventDisableTiming));
-    TALON_CUDA_OK(cudaEventCreateWithFlags(&s->rows, cudaEventDisableTiming));
-    TALON_CUDA_OK(cudaEventCreateWithFlags(&s->kv, cudaEventDisableTiming));
-    TALON_CUDA_OK(cudaEventCreateWithFlags(&s->targets, cudaEventDisableTiming));
   }
   int64_t *h_kv_start = reinterpret_cast<int64_t *>(s->h_scratch);
   int32_t *h_n = reinterpret_cast<int32_t *>(s->h_scratch + (size_t)p.batch_max * 8);

@@ -167,3 +167,17 @@ def test_the_status_after_a_loop_is_the_last_steps(bad, where):
     torch.cuda.synchronize()
     assert t.poll_status() == (talon.ERR_NONFINITE if bad == S - 1 else talon.OK)
     t.close()
+
+
+def test_a_host_step_whose_staging_does_not_fit_can_be_called_again():
+    """Room for 1024 sequences of 16 rows of four million tokens, twice, is more than any device has."""
+    V, N, D, B = 1 << 22, 16, 2, 1024
+    talon, t = _talon(B, V, N, 4, D)
+    row = torch.zeros(1, N, V)
+    bf = lambda heads: torch.zeros(1, N, heads, DH, dtype=torch.bfloat16)
+    i32 = lambda *shape: torch.zeros(*shape, dtype=torch.int32)
+    for _ in range(2):
+        assert t.step_host(i32(1), i32(1), row, row, bf(8), None, None, bf(2), bf(2), 0.1, bf(8), i32(1), i32(1, N), i32(1, N), i32(1, N),
+                           i32(1, N), i32(1), i32(1, D + 1), i32(1)) == talon.ERR_CUDA
+    torch.zeros(8, device="cuda").sum().item()           # nothing is left behind in the CUDA runtime either
+    t.close()
