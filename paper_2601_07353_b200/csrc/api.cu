@@ -4,7 +4,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
-#include <vector>
 #include <type_traits>
 
 #include "talon_internal.cuh"
@@ -14,8 +13,13 @@ talon_status attention_mma_setup();
 talon_status attention_tc_setup();
 }  // namespace talon
 
+// A copy to the device that is still to be made.
+struct CopyPiece { void *dst; const void *src; size_t bytes; };
+
 // Device staging for talon_step_host: one allocation, a copy stream of its own.
 struct HostStage {
+  CopyPiece *queue = nullptr;      // [5 + batch_max * (max_depth + 1)]
+  int *bounds = nullptr;           // [3 * batch_max]
   int64_t prefix_tokens = 0;
   void *arena = nullptr;
   float *draft = nullptr, *target = nullptr;
@@ -47,6 +51,8 @@ static bool tree_complete(const talon_tree *t) {
 
 static void free_stage(HostStage *s) {
   if (!s) return;
+  std::free(s->queue);
+  std::free(s->bounds);
   cudaFree(s->arena);
   if (s->h_scratch) cudaFreeHost(s->h_scratch);
   if (s->begin) cudaEventDestroy(s->begin);
@@ -64,8 +70,11 @@ static HostStage *make_stage(const talon_ctx *c, int64_t tokens) {
   const talon_params &p = c->p;
   const size_t N = p.budget, V = p.vocab, Dh = p.head_dim, bm = p.batch_max, W = c->W, nrow = bm * N;
   s->prefix_tokens = tokens;
+  // (host memory too: nothing that a call needs may be left to throw in it)
+  s->queue = static_cast<CopyPiece *>(std::malloc((5 + bm * (p.max_depth + 1)) * sizeof(CopyPiece)));
+  s->bounds = static_cast<int *>(std::malloc(3 * bm * sizeof(int)));
   const size_t kv = (size_t)tokens * p.n_kv_heads * Dh * 2;
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = s->queue && s->bounds ? cudaSuccess : cudaErrorMemoryAllocation;
   for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
     size_t total = 0;
     auto take = [&](auto **ptr, size_t bytes) {
@@ -819,18 +828,18 @@ talon_status talon_step_host(talon_ctx *c, int32_t B, const int32_t *root_tok, c
   // layer at a time as its frontier's rows arrive, and while the host waits to learn the next frontier
   // the copy stream works off what is needed in any case (queries, cache, target rows of the nodes so
   // far).  One sequence of 2048 tokens, N 60, V 128256: 78 MB -> 61 MB, 1523 -> 1200 us.
-  struct Piece { void *dst; const void *src; size_t bytes; };
-  std::vector<Piece> queue;
-  size_t next = 0, kv_pieces = 0;
+  CopyPiece *const queue = s->queue;
+  size_t queued = 0, next = 0, kv_pieces = 0;
   bool kv_marked = false;
-  std::vector<int> lo(B, 0), hi(B, 1), targets(B, 0);
+  int *const lo = s->bounds, *const hi = lo + B, *const targets = hi + B;
+  for (int b = 0; b < B; ++b) { lo[b] = 0; hi[b] = 1; targets[b] = 0; }
   auto copy_in = [&](void *dst, const void *src, size_t bytes) {
     return bytes == 0 || cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s->copy) == cudaSuccess;
   };
   // copies up to `bytes` from the queue; marks the moment the attention's operands are there
   auto feed = [&](size_t bytes) {
-    while (next < queue.size() && bytes > 0) {
-      Piece &x = queue[next];
+    while (next < queued && bytes > 0) {
+      CopyPiece &x = queue[next];
       const size_t n = x.bytes < bytes ? x.bytes : bytes;
       if (!copy_in(x.dst, x.src, n)) return false;
       x.dst = static_cast<char *>(x.dst) + n;
@@ -851,14 +860,14 @@ talon_status talon_step_host(talon_ctx *c, int32_t B, const int32_t *root_tok, c
   // Enough to cover a layer's turn-around: its kernel, the read-back of the sizes, the next copy's start.
   constexpr size_t TURN_BYTES = 3u << 20;
   auto run = [&]() -> talon_status {
-    queue.push_back({s->q, q, rows * p.n_q_heads * Dh * 2});
-    queue.push_back({s->kt, k_tree, rows * kvrow});
-    queue.push_back({s->vt, v_tree, rows * kvrow});
+    queue[queued++] = {s->q, q, rows * p.n_q_heads * Dh * 2};
+    queue[queued++] = {s->kt, k_tree, rows * kvrow};
+    queue[queued++] = {s->vt, v_tree, rows * kvrow};
     if (tokens > 0) {
-      queue.push_back({s->kp, k_prefix, (size_t)tokens * kvrow});
-      queue.push_back({s->vp, v_prefix, (size_t)tokens * kvrow});
+      queue[queued++] = {s->kp, k_prefix, (size_t)tokens * kvrow};
+      queue[queued++] = {s->vp, v_prefix, (size_t)tokens * kvrow};
     }
-    kv_pieces = queue.size();
+    kv_pieces = queued;
     // what the caller has enqueued on `stream` (a copy or callback that fills these buffers) comes first
     if (cudaEventRecord(s->begin, st) != cudaSuccess || cudaStreamWaitEvent(s->copy, s->begin, 0) != cudaSuccess) return TALON_ERR_CUDA;
     if (!copy_in(s->root, root_tok, (size_t)B * 4) || !copy_in(s->plen, prefix_len, (size_t)B * 4) ||
@@ -878,7 +887,7 @@ talon_status talon_step_host(talon_ctx *c, int32_t B, const int32_t *root_tok, c
       for (int b = 0; b < B; ++b)
         if (targets[b] < hi[b]) {
           const size_t at = ((size_t)b * N + targets[b]) * V;
-          queue.push_back({s->target + at, target_logits + at, (size_t)(hi[b] - targets[b]) * row_bytes});
+          queue[queued++] = {s->target + at, target_logits + at, (size_t)(hi[b] - targets[b]) * row_bytes};
           targets[b] = hi[b];
         }
       if (!feed(TURN_BYTES)) return TALON_ERR_CUDA;
@@ -897,7 +906,7 @@ talon_status talon_step_host(talon_ctx *c, int32_t B, const int32_t *root_tok, c
     for (int b = 0; b < B; ++b)
       if (targets[b] < hi[b]) {
         const size_t at = ((size_t)b * N + targets[b]) * V;
-        queue.push_back({s->target + at, target_logits + at, (size_t)(hi[b] - targets[b]) * row_bytes});
+        queue[queued++] = {s->target + at, target_logits + at, (size_t)(hi[b] - targets[b]) * row_bytes};
       }
     if (!feed(~(size_t)0) || cudaEventRecord(s->targets, s->copy) != cudaSuccess) return TALON_ERR_CUDA;
     if (cudaStreamWaitEvent(st, s->kv, 0) != cudaSuccess) return TALON_ERR_CUDA;

@@ -71,3 +71,17 @@ def test_the_product_has_no_cpu_route():
         from paper_2601_07353_b200 import talon
         with pytest.raises(RuntimeError):
             talon.Talon(batch_max=1, vocab=100, budget=8, root_topk=4, cand_topk=4, max_depth=4, n_q_heads=4, n_kv_heads=2)
+
+
+def test_no_allocation_in_the_library_can_throw_through_its_c_entries():
+    """The C entries catch nothing, so the library must not import what throws when memory runs out."""
+    import shutil
+    import subprocess
+
+    import pytest
+    from paper_2601_07353_b200 import build
+    if not shutil.which("nm"):
+        pytest.skip("needs nm")
+    names = subprocess.run(["nm", "-D", "--undefined-only", build.build()], capture_output=True, text=True, check=True).stdout
+    for thrower in ("_Znwm@", "_Znam@", "__throw_length_error", "__throw_bad_alloc", "bad_array_new_length"):
+        assert thrower not in names, thrower
