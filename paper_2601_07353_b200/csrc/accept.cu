@@ -43,7 +43,7 @@ struct WalkArgs {
 
 struct WalkShared {
   int tgt[MAX_BUDGET];      // the target's choice after each node
-  int next[MAX_BUDGET];     // the child that carries it (siblings have different tokens), or -1
+  int next[MAX_BUDGET];     // the first child that carries it, or MAX_BUDGET
 };
 
 // A CTA of at least MAX_BUDGET threads decodes the keys of sequence b and walks its tree: one thread per
@@ -65,16 +65,17 @@ __device__ __forceinline__ void accept_walk(const WalkArgs &a, int b, WalkShared
     a.best[nb + i] = 0ull;                                  // leave the workspace clean
     a.target_tok[nb + i] = want;
     sh.tgt[i] = want;
-    sh.next[i] = -1;
+    sh.next[i] = MAX_BUDGET;
   }
   __syncthreads();
-  if (par >= 0 && par < n && tok == sh.tgt[par]) sh.next[par] = i;
+  // (the library's siblings have different tokens; a caller's own tree may not, and there the first one counts)
+  if (par >= 0 && par < n && tok == sh.tgt[par]) atomicMin(&sh.next[par], i);
   __syncthreads();
   int32_t *path = a.accept_nodes + (size_t)b * (a.max_depth + 1);
   if (i == 0) {
     int cur = 0, len = 0;
     path[0] = 0;
-    for (int c = sh.next[0]; c >= 0 && len < a.max_depth; c = sh.next[c]) { cur = c; path[++len] = c; }
+    for (int c = sh.next[0]; c < MAX_BUDGET && len < a.max_depth; c = sh.next[c]) { cur = c; path[++len] = c; }
     a.accept_len[b] = len;
     a.bonus_tok[b] = sh.tgt[cur];
     for (int d = len + 1; d <= a.max_depth; ++d) path[d] = -1;
