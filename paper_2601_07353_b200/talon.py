@@ -156,9 +156,15 @@ class Tree:
         return TalonTreeStruct(*(t.data_ptr() for t in (self.n_nodes, self.token, self.parent, self.depth,
                                                           self.position, self.layer_off, self.score, self.mask)))
 
+    _kept = None                                         # not a field: see address()
+
     def __setattr__(self, name, value):
         object.__setattr__(self, name, value)
         object.__setattr__(self, "_kept", None)          # another array: the struct is made anew
+
+    def __getstate__(self):
+        """What copies and pickles take along: the arrays, not the struct that points into them."""
+        return {k: v for k, v in self.__dict__.items() if k != "_kept"}
 
     def address(self) -> int:
         """Address of a ``talon_tree`` for this tree.  The struct is kept between calls and made anew when
