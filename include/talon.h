@@ -268,8 +268,9 @@ talon_status talon_step_host(talon_ctx *ctx, int32_t B, const int32_t *root_tok,
  * the layout of the call it is handed to: talon_reset (root_tok, prefix_len), talon_expand_layer
  * with rows BY_NODE (draft_logits, draft_row_stride, N rows per sequence), talon_tree_attention
  * (q .. out), talon_accept (target_logits .. bonus_tok; target_tok may be null).
- * n_layers  expansion layers to enqueue, 0..D_max (layers after the tree is full cost one
- *           frontier check each and read no logits)
+ * n_layers  expansion layers to enqueue, 0..D_max
+ * The draft and target rows of all N slots have to be readable, whatever they hold in slots that the tree does not
+ * reach: with lists of up to 32 keys the rows may be prepared for all slots at once, before the trees are known.
  * Enqueues only; no synchronisation.
  * A step is a chain of small dependent kernels, so from the second call with exactly the same
  * arguments the library captures these launches into a CUDA graph once and replays it on later

@@ -662,7 +662,7 @@ static talon_status step_enqueue(talon_ctx *c, const talon_tree *t, int32_t B, c
   if (r != TALON_OK) return r;
   bool closed = false, accepted = false;
   // (timed launches are reported per layer, so they take the layered sequence too)
-  if (!layered && n_layers > 0 && rows_at_once(c)) {
+  if (!layered && n_layers > 0 && rows_at_once(c) && talon::step_rows_pay(c, B, n_layers)) {
     c->B = B;
     r = talon::launch_grow_step(c, t, root_tok, prefix_len, draft_logits, draft_row_stride, n_layers, target_logits,
                                 target_row_stride, target_tok, accept_len, accept_nodes, bonus_tok, (cudaStream_t)stream,

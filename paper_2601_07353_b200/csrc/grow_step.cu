@@ -16,8 +16,10 @@
 //                     accepted path too.
 //
 // Rows of slots that the tree turns out not to use, or not to expand, are read for nothing.  Where that
-// could cost more than it saves (launch_grow_step has the rule) the step takes two rounds: the second
-// prepares the remaining rows of the sequences whose trees still grow.
+// could cost more than it saves (plan_step has the rule) the step takes two rounds, the second of which
+// prepares the remaining rows of the sequences whose trees still grow, or goes layer by layer after all.
+#include <algorithm>
+
 #include "expand_stream.cuh"
 
 namespace talon {
@@ -279,7 +281,9 @@ struct GrowArgs {
   int32_t *target_tok, *accept_len, *accept_nodes, *bonus_tok;
 };
 
-constexpr double STEP_SPLIT_BYTES = 150e6;    // about 25 us at the copy bandwidth
+// For the choice between one round, two and a launch per layer (plan_step), in microseconds: the copy bandwidth, what a
+// layer with a launch of its own costs beyond its bytes, what a second round costs beyond its own.
+constexpr double STEP_BYTES_PER_US = 6.5e6, STEP_LAYER_US = 13.5, STEP_ROUND_US = 25.0;
 constexpr int GROW_THREADS = 256;
 
 struct GrowSmem {
@@ -595,26 +599,49 @@ static void step_bounds(const talon_ctx *c, int n_layers, int *expandable, int *
   *nodes = (int)(sum + f < N ? sum + f : N);
 }
 
-// How far a step's first round goes and whether the target rows come along.
+// The fewest nodes a tree can have after n_layers layers: Top-K layers take K, a gated one at least its best candidate.
+static int fewest_nodes(const talon_ctx *c, int n_layers) {
+  const int N = c->p.budget;
+  long long n = 1, width = 1;
+  for (int d = 0; d < n_layers && n < N; ++d) {
+    width = d < c->p.init_layers ? std::min((long long)c->p.root_topk, width * c->k_cap) : 1;
+    n += width;
+  }
+  return (int)(n < N ? n : N);
+}
+
+// How a whole step goes: all rows in one round with the target rows alongside, the draft rows in two rounds, or (first = 0)
+// a launch per layer.
 struct StepPlan { int expandable, nodes, first; bool with_target; };
-static StepPlan plan_step(const talon_ctx *c, int n_layers) {
-  const talon_params &p = c->p;
+static StepPlan plan_step(const talon_ctx *c, int B, int n_layers) {
   StepPlan s;
   step_bounds(c, n_layers, &s.expandable, &s.nodes);
-  // One round with the target rows alongside is the quickest way even where a part of the rows is read
-  // for nothing (the pass then runs at the copy bandwidth; a round of its own costs about 20 us: pass
-  // start-up, hand-off, growth).  A tree of few layers cannot get near a large budget, though: on
-  // confident rows a layer adds one node, on flat ones K, seldom more.  Where the slots beyond
-  // 1 + 7/8 K D would cost more to read than a second round, the first round stops there, the second
-  // takes the rest for the trees that do go on, and the target rows wait for the trees' sizes.
-  const double row_bytes = 4.0 * p.vocab * c->B;          // of one slot of every sequence
-  s.first = 1 + p.root_topk * n_layers * 7 / 8;
-  if (c->step_first_rows > 0) s.first = c->step_first_rows;
-  else if (row_bytes * 2.0 * (s.expandable - s.first) < STEP_SPLIT_BYTES) s.first = s.expandable;
-  if (s.first > s.expandable) s.first = s.expandable;
+  // One round with the target rows alongside is the quickest way even where a part of the rows is read for nothing, as
+  // long as that part, on the smallest tree there can be, costs no more than the layers' own launches would.  (16 sequences,
+  // N 60, 12 layers, rows of 128256: 195 us on trees of 20 nodes and 197 on trees of 51; by layers 218 and 335.)
+  // Beyond that two rounds, with a first one that bounds its own and the second one's loss the same way; between the
+  // bounds it takes what a tree of this depth usually expands, or the least where that is the whole budget.  32
+  // sequences, N 128, 24 layers: 318 us on trees of 32 nodes and 784 on trees of 115, in one round 775 and 790, by layers
+  // 498 and 1063.  And where a slot costs too much for that too, the layers: 32 sequences, N 60, 6 layers: 241 us on
+  // trees of 14 nodes, 374 on trees of 33, in two rounds (43 slots first) 280 and 355.  One round for all of them took up to
+  // 27 % longer on the smallest trees than a launch per layer.
+  const double slot_us = 4.0 * c->p.vocab * B / STEP_BYTES_PER_US, saved = STEP_LAYER_US * n_layers;
+  const int fewest = fewest_nodes(c, n_layers);
+  s.first = s.expandable;
+  if (c->step_first_rows > 0) {
+    s.first = std::min(c->step_first_rows, s.expandable);
+  } else if (slot_us * (s.expandable + s.nodes - 2 * fewest) > saved) {
+    const double spare = saved - STEP_ROUND_US;
+    const int reach = spare > 0.0 ? (int)std::min(spare / slot_us, 1.0 * c->p.budget) : 0;
+    const int least = std::max(fewest, s.expandable - reach), most = std::min(fewest + reach, s.expandable - 1);
+    const int usual = 1 + c->p.root_topk * n_layers * 3 / 4;
+    s.first = reach == 0 || least > most ? 0 : usual < s.expandable ? std::min(std::max(usual, least), most) : least;
+  }
   s.with_target = s.first == s.expandable;
   return s;
 }
+
+bool step_rows_pay(const talon_ctx *c, int B, int n_layers) { return plan_step(c, B, n_layers).first > 0; }
 
 static RowPassArgs row_pass_args(talon_ctx *c, const float *draft, int64_t draft_stride, const float *target, int64_t target_stride) {
   const talon_params &p = c->p;
@@ -695,7 +722,7 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
                               const float *draft, int64_t draft_stride, int n_layers, const float *target,
                               int64_t target_stride, int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes,
                               int32_t *bonus_tok, cudaStream_t st, bool *accepted) {
-  const StepPlan plan = plan_step(c, n_layers);
+  const StepPlan plan = plan_step(c, c->B, n_layers);
   *accepted = plan.with_target;
   RowPassArgs ra = row_pass_args(c, draft, draft_stride, plan.with_target ? target : nullptr, target_stride);
   GrowArgs ga = grow_args(c, t, root_tok, prefix_len, n_layers, target_tok, accept_len, accept_nodes, bonus_tok, plan.with_target);
@@ -715,13 +742,13 @@ talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *
   return TALON_OK;
 }
 
-bool loop_rows_possible(const talon_ctx *c, int n_layers) { return c->ahead > 1 && plan_step(c, n_layers).with_target; }
+bool loop_rows_possible(const talon_ctx *c, int n_layers) { return c->ahead > 1 && plan_step(c, c->B, n_layers).with_target; }
 
 // One pass for several steps: at small batches a step's rows are a few dozen MB, too few to fill the
 // pass's start and end (four steps of 2 sequences: 4 x 31 us against 80).
 talon_status launch_loop_rows(talon_ctx *c, const float *draft, int64_t draft_stride, int64_t draft_step, int n_layers,
                               const float *target, int64_t target_stride, int64_t target_step, int steps, cudaStream_t st) {
-  const StepPlan plan = plan_step(c, n_layers);
+  const StepPlan plan = plan_step(c, c->B, n_layers);
   RowPassArgs ra = row_pass_args(c, draft, draft_stride, target, target_stride);
   ra.B = c->B * steps; ra.draft_step = draft_step; ra.target_step = target_step;
   ra.r0 = 0; ra.r1 = plan.expandable; ra.t1 = plan.nodes;
@@ -732,7 +759,7 @@ talon_status launch_loop_rows(talon_ctx *c, const float *draft, int64_t draft_st
 talon_status launch_loop_grow(talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len, int n_layers,
                               int step, int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes, int32_t *bonus_tok,
                               cudaStream_t st) {
-  const StepPlan plan = plan_step(c, n_layers);
+  const StepPlan plan = plan_step(c, c->B, n_layers);
   GrowArgs ga = grow_args(c, t, root_tok, prefix_len, n_layers, target_tok, accept_len, accept_nodes, bonus_tok, true);
   const size_t at = (size_t)step * c->B * c->p.budget;
   ga.row_keys += at * c->key_stride; ga.row_lp += at * c->key_stride;

@@ -233,6 +233,7 @@ talon_status launch_expand(talon_ctx *c, const talon_tree *t, const float *logit
 // The draft phase of a whole step (reset, n_layers layers, closing pass) from the draft rows of all node
 // slots; k_cap <= 32.  *accepted: the target rows' arg-max and the walk are done as well.
 talon_status grow_step_setup(talon_ctx *c);
+bool step_rows_pay(const talon_ctx *c, int B, int n_layers);      // false: go layer by layer
 talon_status launch_grow_step(talon_ctx *c, const talon_tree *t, const int32_t *root_tok, const int32_t *prefix_len,
                               const float *draft, int64_t draft_stride, int n_layers, const float *target,
                               int64_t target_stride, int32_t *target_tok, int32_t *accept_len, int32_t *accept_nodes,
