@@ -10,7 +10,7 @@
 
 namespace talon {
 talon_status attention_mma_setup();
-talon_status attention_tc_setup();
+talon_status attention_tc_setup(talon_ctx *c);
 }  // namespace talon
 
 // A copy to the device that is still to be made.
@@ -233,7 +233,7 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     if (pass == 0 && cudaMalloc(&c->d_arena, total) != cudaSuccess) break;
   }
   const bool ok = c->d_arena && cudaMemset(c->d_arena, 0, zeroed) == cudaSuccess && 
-                  talon::attention_mma_setup() == TALON_OK && talon::attention_tc_setup() == TALON_OK &&
+                  talon::attention_mma_setup() == TALON_OK && talon::attention_tc_setup(c) == TALON_OK &&
                   talon::expand_fused_setup(c) == TALON_OK && (c->k_cap > 32 || talon::grow_step_setup(c) == TALON_OK);
   if (!ok) {
     std::fprintf(stderr, "talon: context creation failed: %s\n", cudaGetErrorString(cudaGetLastError()));

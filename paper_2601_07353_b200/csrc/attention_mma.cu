@@ -357,8 +357,8 @@ talon_status attention_mma_setup() {
 struct AttnPlan { int kind, splits; bool exact_max; };
 static AttnPlan plan_attention(talon_ctx *c, const AttnArgs &a, int tiles, bool early, bool split_p) {
   const int heads = c->B * a.Hkv;
-  const int ctas = split_p ? a.m_blocks * heads : (a.m_blocks + 1) / 2 * heads;
-  const bool only_one = split_p || a.m_blocks == 1;
+  const bool only_one = split_p || a.m_blocks == 1 || c->attn_force_tiles == 1;
+  const int ctas = only_one ? a.m_blocks * heads : (a.m_blocks + 1) / 2 * heads;
   bool one = only_one;
   int sp = 1;
   // How exact the rounding of P to bf16 is hangs on the ranges: a row's largest probability in the first tile of
@@ -394,7 +394,7 @@ static AttnPlan plan_attention(talon_ctx *c, const AttnArgs &a, int tiles, bool 
     };
     const int most = std::min((tiles + c->attn_min_tiles - 1) / c->attn_min_tiles, c->attn_cluster == 2 ? 8 : c->sm_count);
     float best = cost(one, 1);
-    for (int single = only_one || c->attn_force_tiles == 1; single <= (c->attn_force_tiles != 2 || only_one); ++single)
+    for (int single = only_one; single <= (c->attn_force_tiles != 2 || only_one); ++single)
       for (int s = 1; s <= std::min(most, c->sm_count / (single ? a.m_blocks * heads : ctas)); ++s) {
         const float t = cost(single, s);
         if (t < best) { best = t; sp = s; one = single; }
@@ -413,7 +413,7 @@ static AttnPlan plan_attention(talon_ctx *c, const AttnArgs &a, int tiles, bool 
     if (tiles >= 32 && cost(2) < cost(1)) sp = 2;
   }
   if (c->attn_force_splits > 0) sp = c->attn_force_splits;
-  if (c->attn_force_tiles > 0) one = c->attn_force_tiles == 1 || only_one;
+  if (c->attn_force_tiles == 2) one = only_one;
   while (sp > 1 && (size_t)a.m_blocks * c->B * a.Hkv * sp * AT_BM > c->attn_ml_elems) --sp;
   return {split_p ? TC_SPLIT_P : one ? TC_SINGLE : TC_PAIR, sp, sp < usual};
 }

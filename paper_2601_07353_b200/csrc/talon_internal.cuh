@@ -130,7 +130,7 @@ struct talon_ctx {
   int attn_cluster;                  // key ranges of the tensor-core attention merge inside a cluster (1; 2: never more of them than it has CTAs) or in a second kernel (0)
   int attn_clusters[3][9];           // per kind of the tensor-core attention and cluster size: clusters the device holds at once (-1 not asked yet)
   int attn_force_splits;             // > 0: key ranges per (sequence, head, query tiles), for experiments
-  int attn_force_tiles;              // 1, 2: query tiles of a CTA, for experiments
+  int attn_force_tiles;              // 1, 2: query tiles of a CTA, for experiments (1 also where two cannot be had)
   int argmax_oversplit;              // target argmax: chunk rounds per CTA when the rows outnumber the grid
   int expand_max_split;              // fused kernel: chunks a row is cut into at most when the grid has room
   int attn_min_tiles;                // split-KV: key tiles a CTA should at least own
