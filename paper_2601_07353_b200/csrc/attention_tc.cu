@@ -267,6 +267,9 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
   // `early`: the kernel before this one only grows the trees (grow_step.cu).  Everything about the
   // prefix is complete then, so the CTA starts on its prefix tiles at once; the softmax warps wait for
   // that kernel before they look at tree sizes and mask rows, and so before anything is written.
+  // Why the prefix is complete: every CTA of that kernel first waits for all that came before it (the commit that
+  // wrote prefix lengths and cache rows among it) to have finished and be visible, and only then triggers; this grid
+  // starts when the last of them has.  The lengths are read past L1, which may hold the step before's.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -282,7 +285,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
   unsigned char *gen_base = smem_dyn + (base - smem_u32(smem_dyn));      // generic pointer to `base`
   auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
 
-  const int L = a.prefix_len[b];
+  const int L = __ldcg(a.prefix_len + b);
   const int nmt = min(a.m_blocks - mpair * MT, MT);                      // query tiles of this CTA with rows
 
   const int nP = (L + TC_BN - 1) / TC_BN;
