@@ -381,7 +381,7 @@ static AttnPlan plan_attention(talon_ctx *c, const AttnArgs &a, int tiles, bool 
     // CTAs fill SMs only fit a GPC at a time, so the device says how many it holds: a second round of them
     // doubles the time.  Started beside the growth of the trees (about 1.2 a layer), the work on the prefix
     // counts only where it takes longer than that.
-    const float growing = early ? 1.2f * c->p.max_depth : 0.f;
+    const float growing = early ? 1.2f * c->layers_run : 0.f;
     auto cost = [&](bool single, int s) {
       const int n = single ? a.m_blocks * heads : ctas;
       const int held = s >= 2 && s <= 8 && c->attn_cluster ? attention_tc_clusters(c, split_p ? TC_SPLIT_P : single ? TC_SINGLE : TC_PAIR, s) : 0;
