@@ -214,6 +214,7 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
     };
     take(&c->d_status, 2);
     take(&c->d_row_count, rows);
+    take(&c->d_pass_count, rows);
     take(&c->d_seq_count, bm);
     take(&c->d_walk_count, bm);
     take(&c->d_argmax, nrow);

@@ -652,7 +652,7 @@ static RowPassArgs row_pass_args(talon_ctx *c, const float *draft, int64_t draft
   ra.init_layers = p.init_layers; ra.log_mu = c->log_mu; ra.spans = span_table(p.vocab, c->k_cap, c->expand_max_split);
   ra.growing = nullptr;
   ra.part_keys = c->d_part_keys; ra.part_ms = c->d_part_ms; ra.row_keys = c->d_row_keys; ra.row_lp = c->d_row_score;
-  ra.row_count = c->d_row_count; ra.best = c->d_argmax; ra.row_bad = c->d_row_bad; ra.status = c->d_status;
+  ra.row_count = c->d_pass_count; ra.best = c->d_argmax; ra.row_bad = c->d_row_bad; ra.status = c->d_status;
   return ra;
 }
 
@@ -703,7 +703,7 @@ static GrowArgs grow_args(talon_ctx *c, const talon_tree *t, const int32_t *root
   ga.n_layers = n_layers; ga.max_depth = p.max_depth; ga.root_topk = p.root_topk; ga.init_layers = p.init_layers;
   ga.log_mu = c->log_mu;
   ga.row_keys = c->d_row_keys; ga.row_lp = c->d_row_score; ga.growing = c->d_growing; ga.depth_at = c->d_depth_at;
-  ga.row_count = c->d_row_count; ga.status = c->d_status;
+  ga.row_count = c->d_pass_count; ga.status = c->d_status;
   ga.best = walk ? c->d_argmax : nullptr; ga.row_bad = c->d_row_bad;
   ga.target_tok = target_tok ? target_tok : c->d_target_tok;
   ga.accept_len = accept_len; ga.accept_nodes = accept_nodes; ga.bonus_tok = bonus_tok;

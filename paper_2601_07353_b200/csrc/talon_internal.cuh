@@ -117,7 +117,8 @@ struct talon_ctx {
   float2 *d_part_ms;                 // [items_cap]              per-chunk (max, sum exp)
   unsigned long long *d_row_keys;    // [rows_cap, key_stride]   per-row top-k
   double *d_row_score;               // [rows_cap, key_stride]   per-row candidate scores (fused kernel, wide frontiers)
-  unsigned int *d_row_count;         // [rows_cap]               chunks finished per row
+  unsigned int *d_row_count;         // [rows_cap]               chunks finished per row, layer by layer (zeroed by a reset)
+  unsigned int *d_pass_count;        // [rows_cap]               the same for the row pass (zeroed by the growth kernel after it)
   unsigned int *d_seq_count;         // [batch_max]              chunks finished per sequence (fused kernel)
   int fused_grid;                    // CTAs of the fused kernel at full width
   // whole-step growth (grow_step.cu)
