@@ -1,6 +1,6 @@
 """GPU parity on the layouts and shapes the other tests do not reach: vocabularies that are not a
 multiple of four, row strides wider than the vocabulary (NaN between the rows), a sequence with an
-empty prefix inside a batch, and query-group sizes that take the warp-MMA attention kernel."""
+empty prefix inside a batch, and query-group sizes whose rows do not fill a query tile."""
 import math
 
 import numpy as np
@@ -102,8 +102,8 @@ def test_all_prefixes_empty():
 
 @pytest.mark.parametrize("hq,hkv,batch", [(24, 8, 1), (24, 8, 24), (28, 4, 2), (12, 2, 40), (40, 8, 3)])
 def test_group_sizes_that_do_not_divide_128(hq, hkv, batch):
-    """g = 3, 5, 6, 7: packed query rows do not tile 128-row blocks by whole nodes, so the warp-MMA
-    kernel runs, with split-KV (few CTAs) and without (many sequences)."""
+    """g = 3, 5, 6, 7: packed query rows do not tile 128-row blocks by whole nodes, so a query tile of the
+    tcgen05 kernel ends in empty rows; with split-KV (few CTAs) and without (many sequences)."""
     talon, workload = _mods()
     cfg = synth.CONFIGS["tiny"].scaled(n_q_heads=hq, n_kv_heads=hkv, batch=batch, prefix_min=100, prefix_max=700,
                                        vocab=8000)

@@ -1,6 +1,6 @@
 """The kernels behind whole steps and behind odd sizes of single calls: the row pass with the growth
-kernel (talon_step, talon_loop, talon_step_host), wide candidate lists, chunks at the edges of what
-stays resident, and the tensor-core attention with one and two query tiles per CTA."""
+kernel (talon_step, talon_loop), the host step's layer by layer copies, wide candidate lists, chunks at the
+edges of what stays resident, and the tensor-core attention with one and two query tiles per CTA."""
 import math
 
 import numpy as np
@@ -184,7 +184,7 @@ def test_loop_longer_than_the_rows_prepared_at_once():
 
 @pytest.mark.parametrize("B,K,N", [(3, 8, 40), (2, 40, 50), (1, 16, 128)])
 def test_host_step_copies_every_row_the_tree_reads(B, K, N):
-    """Rows are fetched as the tree grows (lists up to 32 keys) or up front (wider lists)."""
+    """Rows are fetched as the tree grows, for lists of any length."""
     V, D = 3001, 5
     talon, t = _talon(B, V, N, K, D)
     s = Step(t, B, V, N, D, 8, 2, [70 + 50 * b for b in range(B)], 5)
