@@ -20,10 +20,12 @@ than half a second the region is repeated and the median repeat is reported (``r
 ``spread``), so that clock samples fall inside it.  With more than one GPU every rank runs its own
 replicas (sequences are independent: no data-path collective).
 
-Rank 0 prints one JSON line.  Beside the contract's keys it carries ``kernels`` (each kernel family
-timed alone: one event pair around at least 20 back-to-back graph replays of just those launches,
-inputs rotated, so no event bracket sits between two kernels), ``roofline`` (the dominant kernel's
-algorithmic bytes or flops over that duration, against the measured peaks), ``cpu_baseline`` (the
+Rank 0 prints one JSON line.  Beside the contract's keys it carries ``kernels`` (each kernel family of
+the single calls timed alone: one event pair around at least 20 back-to-back graph replays of just
+those launches, inputs rotated, so no event bracket sits between two kernels; ``rows_and_growth``,
+what a whole step launches instead of the expansion layers, by difference), ``roofline`` (algorithmic
+bytes or flops over that duration of the dominant family of the timed step, against the measured peaks),
+``cpu_baseline`` (the
 fp64 CPU oracle on all host cores, one core beside it, with its per-stage split and the count of
 tolerated selection ties), ``e2e`` (the same step through ``talon_step_host`` with pinned host
 buffers), ``tree_shapes`` and ``configs``.  ``--impl reference`` times the CPU oracle alone.
@@ -508,7 +510,7 @@ def measure(cfg, args, info, dev, dev_index, peaks, headline: bool, sampler=None
         "value": value, "ms_per_step": seconds / K * 1e3, "steps": K, "repeats": len(reps),
         "spread": (max(reps) - min(reps)) / seconds if len(reps) > 1 else 0.0,
         "warmup": warm, "warmup_requested": args.warmup, "gpu_launches": int(gpu_launches),
-        "sequence_steps_per_s": value * B, "tree_shapes": shapes, "algorithmic_per_step": work,
+        "launches_per_step": gpu_launches / K, "sequence_steps_per_s": value * B, "tree_shapes": shapes, "algorithmic_per_step": work,
         "l2": f"inputs larger than L2: steps rotate over {n_sets} input sets of {per_set / 1e6:.1f} MB "
               f"({n_sets * per_set / 1e6:.0f} MB vs 126 MB L2)",
         "input_sets": n_sets, "timed_wall": (wall0, wall1),
@@ -543,12 +545,28 @@ def measure(cfg, args, info, dev, dev_index, peaks, headline: bool, sampler=None
     ksum = ms["reset+expand"] + ms["tree_attention"] + ms["accept"]
     res["kernels"] = kernels
     res["kernels_sum_ms"] = ksum
-    res["kernels_sum_over_step"] = ksum / res["ms_per_step"]
-    res["kernel_timing"] = (f"each family alone: one event pair around {replays} back-to-back graph replays of its launches, "
-                            "inputs rotated over the input sets; layers that find the tree full are launched and counted")
+    res["kernel_timing"] = (f"each family of the single calls alone: one event pair around {replays} back-to-back graph replays of its "
+                            "launches, inputs rotated over the input sets; layers that find the tree full are launched and counted")
+    # A whole step whose rows are prepared at once launches none of the expansion layers; what it launches instead (row pass,
+    # growth, an arg-max where the target rows do not ride along) is the step less the attention.
+    families = ["expand_rows", "tree_attention", "accept"]
+    if res["launches_per_step"] < D + 3:
+        rows_ms = max(res["ms_per_step"] - ms["tree_attention"], 1e-6)
+        work["rows_and_growth"] = work["expand_rows"] + work["accept"]
+        kernels["rows_and_growth"] = {
+            "ms_per_step": rows_ms, "launches_per_step": res["launches_per_step"] - launches["tree_attention"],
+            "algorithmic_gbs": gbs(work["rows_and_growth"], rows_ms),
+            "note": "row_pass_kernel + grow_kernel, and the arg-max where it is a launch of its own: the step less the attention "
+                    "alone (part of which runs beside the growth); bytes of the rows the trees need, not of all rows read"}
+        kernels["rows_and_growth"]["frac_of_hbm_peak"] = kernels["rows_and_growth"]["algorithmic_gbs"] / peaks["hbm_gbs"]
+        families = ["rows_and_growth", "tree_attention"]
+        res["kernels_sum_over_step"] = None
+        res["kernel_timing"] += "; rows_and_growth by difference; expand_rows and accept are not what the timed step launches"
+    else:
+        res["kernels_sum_over_step"] = ksum / res["ms_per_step"]
 
     # ---- roofline of the dominant kernel ----
-    dominant = max(("expand_rows", "tree_attention", "accept"), key=lambda k: kernels[k]["ms_per_step"])
+    dominant = max(families, key=lambda k: kernels[k]["ms_per_step"])
     kd = kernels[dominant]
     intensity = work["attention_flops"] / max(1.0, work["tree_attention"])
     ridge = peaks["bf16_tflops_sustained"] * 1e12 / (peaks["hbm_gbs"] * 1e9)
@@ -729,8 +747,12 @@ def run_talon(args):
             "repeats": head["repeats"], "spread": head["spread"],
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": DTYPE, "data": "synthetic",
             "config": {"workload": workload_text(cfg), "l2": head["l2"],
-                       "step": f"talon_step: reset + {cfg.max_depth} expand-layer calls + tree attention + accept (whose walk closes the tree) "
-                               "(the library replays its own captured graph of these launches)",
+                       "step": f"talon_step, {head['launches_per_step']:.0f} launches: "
+                               + ("draft rows of all node slots in one pass or two, trees grown in a kernel of their own, tree attention, "
+                                  "target arg-max and walk (in the pass and the growth kernel where one pass does)"
+                                  if head["launches_per_step"] < cfg.max_depth + 3 else
+                                  f"reset + {cfg.max_depth} expansion layers + tree attention + accept (whose walk closes the tree)")
+                               + " (the library replays its own captured graph of these launches)",
                        "sequences_per_rank": cfg.batch, "input_sets": head["input_sets"]},
             "clocks": clocks, "e2e": head.get("e2e"), "gpu_launches": head["gpu_launches"], "roofline": head["roofline"],
             "cpu_baseline": head.get("cpu_baseline"), "selection_ties": head.get("selection_ties"),

@@ -272,12 +272,12 @@ talon_status talon_step_host(talon_ctx *ctx, int32_t B, const int32_t *root_tok,
  * The draft and target rows of all N slots have to be readable, whatever they hold in slots that the tree does not
  * reach: with lists of up to 32 keys the rows may be prepared for all slots at once, before the trees are known.
  * Enqueues only; no synchronisation.
- * A step is a chain of small dependent kernels, so from the second call with exactly the same
- * arguments the library captures these launches into a CUDA graph once and replays it on later
+ * A step is a chain of dependent kernels, three where the rows are prepared at once, so from the second call with
+ * exactly the same arguments the library captures these launches into a CUDA graph once and replays it on later
  * calls (same kernels, same memory, one submission; up to 64 argument sets are kept, least
  * recently used first out).  The plain launch sequence is used on the legacy default stream, while
- * `stream` is being captured by the caller, while launches are timed (talon_timing_enable without
- * pause), and always when the environment has TALON_STEP_GRAPH=0. */
+ * launches are timed (talon_timing_enable without pause), and always when the environment has
+ * TALON_STEP_GRAPH=0.  A caller that captures `stream` gets the launches of the single calls, one per layer. */
 talon_status talon_step(talon_ctx *ctx, const talon_tree *tree, int32_t B, const int32_t *root_tok,
                         const int32_t *prefix_len, const float *draft_logits,
                         int64_t draft_row_stride, int32_t n_layers, const void *q,

@@ -162,8 +162,7 @@ talon_status talon_create(talon_ctx **out_ctx, const talon_params *p, int device
   c->key_stride = (k + 3) & ~3;
   c->log_mu = std::log(p->mu);
   {
-    // Programmatic dependent launch: measured on B200 it gains about 3 % at batch 1 and loses
-    // 3-10 % at batch 16, so by default it is used for small batches only (TALON_PDL=1 / 0 forces it).
+    // (TALON_PDL: programmatic dependent launch for every kernel, 1, or none, 0; launch_kernel_pdl has the rule)
     const char *mt = std::getenv("TALON_ATTN_MIN_TILES");
     c->attn_min_tiles = mt ? std::atoi(mt) : 2;
     if (c->attn_min_tiles < 1) c->attn_min_tiles = 1;
@@ -511,7 +510,9 @@ talon_status talon_loop(talon_ctx *c, const talon_tree *t, int32_t B, int32_t n_
       result_step_stride < 0 || (q_step_stride & 7) || (kv_tree_step_stride & 7) || (draft_step_stride & 3) ||
       (target_step_stride & 3))
     return TALON_ERR_INVALID_ARG;
-  // a caller that captures the loop gets the layered launch sequence, as talon_step's callers do
+  // A caller that captures gets a launch per layer, here and in talon_step: the launches of the single calls, so that the
+  // graph gives what those give to the last bit (whole steps cut rows and choose key ranges otherwise), at the cost of
+  // the launches (a captured long step 3.08 ms where an uncaptured one is 2.78).
   const bool layered = being_captured((cudaStream_t)stream);
   const char *qb = static_cast<const char *>(q), *ktb = static_cast<const char *>(k_tree), *vtb = static_cast<const char *>(v_tree);
   // every argument of every step is checked before the first launch (the step strides keep the alignment)
@@ -700,8 +701,8 @@ talon_status talon_step(talon_ctx *c, const talon_tree *t, int32_t B, const int3
       kv_start, kv_tokens, kv_stride_t, kv_stride_h, max_prefix_len, sm_scale, out, target_logits, target_row_stride, \
       target_tok, accept_len, accept_nodes, bonus_tok, stream
   cudaStream_t st = (cudaStream_t)stream;
-  // A step is a chain of small dependent kernels, so a caller that repeats it pays mostly for
-  // launches.  From the second call with the very same arguments the launches are captured once
+  // A step is a chain of three to a few dozen dependent kernels, so a caller that repeats small ones pays mostly
+  // for launches.  From the second call with the very same arguments the launches are captured once
   // into a CUDA graph and replayed from then on: the same kernels on the same memory, one
   // submission.  Not on the legacy default stream (it cannot be captured), not while the stream is
   // already being captured by the caller, and not while launches are being timed with events.
@@ -828,7 +829,8 @@ talon_status talon_step_host(talon_ctx *c, int32_t B, const int32_t *root_tok, c
   // expanded, the target rows of the nodes there are -- and the bus is never left idle: the tree grows a
   // layer at a time as its frontier's rows arrive, and while the host waits to learn the next frontier
   // the copy stream works off what is needed in any case (queries, cache, target rows of the nodes so
-  // far).  One sequence of 2048 tokens, N 60, V 128256: 78 MB -> 61 MB, 1523 -> 1200 us.
+  // far).  One sequence of 2048 tokens, N 60, V 128256: 78 MB -> 61 MB, 1558 -> 1308 us on one machine, whose single
+  // runs were up to a fifth apart.
   CopyPiece *const queue = s->queue;
   size_t queued = 0, next = 0, kv_pieces = 0;
   bool kv_marked = false;

@@ -9,21 +9,22 @@
 // distributed shared memory -- or, for more than eight ranges or very few rows, by a second kernel
 // from fp32 partials in global memory (split-KV).
 //
-// Roles inside a CTA (320 threads):
-//   warps 0-3, 4-7  softmax of query tile 0 / 1: thread r owns row r.  It reads its row of
+// Roles inside a CTA (MT query tiles; 224 threads with one, 384 with two, the last warp of which is spare):
+//   warps 4 i .. 4 i + 3  softmax of query tile i: thread r owns row r.  It reads its row of
 //                   S = Q K^T from tensor memory (tcgen05.ld), applies the ragged-length or
 //                   ancestor-bitmask visibility, keeps a running maximum and sum, and writes
-//                   P = exp2(S*scale - max) as bf16 back to tensor memory over S (tcgen05.st).
+//                   P = exp2(S*scale - max) as bf16 to columns of tensor memory of its own
+//                   (tcgen05.st), in two halves; both tiles share the columns of S.
 //                   With many key tiles a CTA the running maximum is only raised when it grows by
 //                   more than 2^8, so the accumulator in tensor memory is rescaled rarely; with few
 //                   it follows every growth (launch_attention has the rule: the final division by
 //                   the running sum makes any reference right, but a row's largest probability is
 //                   exact in bf16 only if the reference is its maximum).
-//   warp 8          producer: TMA loads of Q (once) and of the K / V tiles into a ring of
+//   warp 4 MT       producer: TMA loads of Q (once) and of the K / V tiles into a ring of
 //                   128-byte-swizzled shared-memory stages (no multicast).
-//   warp 9          one thread issues tcgen05.mma: S_i = Q_i K^T (both operands in shared
-//                   memory) and O_i += P_i V (P from tensor memory, V from shared memory), with
-//                   tcgen05.commit arriving on mbarriers that the other roles wait on.
+//   warp 4 MT + 1   one thread issues S_i = Q_i K^T (tcgen05.mma, both operands in shared memory);
+//   the MT after it one thread each issues O_i += P_i V (P from tensor memory, V from shared memory);
+//                   tcgen05.commit arrives on mbarriers that the other roles wait on.
 // Every wait is bounded: a role that gives up raises a flag that makes the other roles leave
 // too, tensor memory is released, and the device status word reports a timeout.
 #include <cuda.h>

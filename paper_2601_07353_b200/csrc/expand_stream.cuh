@@ -1,4 +1,4 @@
-// Streaming of fp32 logit rows for the expansion kernels (k <= 32 candidates per row): the row is
+// Streaming of fp32 logit rows for the expansion kernels (up to 128 candidates per row): the row is
 // read once, in chunks, and a chunk leaves its k best (logit, token) keys and its share of the
 // softmax normaliser.  Shared by the kernel that expands one layer (expand_fused.cu) and by the one
 // that prepares every row of a whole step (grow_step.cu).
@@ -170,7 +170,7 @@ __device__ inline u64 warp_merge_desc(u64 list, u64 q, int lane) {
   return x;
 }
 
-// Exclusive scan of the per-sequence frontier sizes: s_base[b] = first packed row of sequence
+// The sequence of packed row `row`: s_base[b] is the first packed row of sequence b, s_base[B] their number.
 __device__ inline int seq_of_row(const int *s_base, int B, int row) {
   int lo = 0, hi = B;   // s_base[lo] <= row < s_base[hi]
   while (hi - lo > 1) {
@@ -233,7 +233,7 @@ inline SpanTable span_table(int vocab, int k, int max_split) {
 }
 __device__ inline unsigned div_small(unsigned a, unsigned b) { return (unsigned)__fdividef((float)a + 0.5f, (float)b); }
 
-// ceil(a / b) for quotients up to 16 of larger numbers
+// min(ceil(a / b), 8) of larger numbers
 __device__ inline int div_up_small(int a, int b) {
   int q = 0;
 #pragma unroll

@@ -1,5 +1,5 @@
 // The draft phase of a whole step in two kernels (k <= 32), for callers that hand in the draft logits
-// of every node slot at once (talon_step, talon_loop, talon_step_host).
+// of every node slot at once (talon_step, talon_loop).
 //
 // What a logit row contributes to the tree -- its k best tokens and their log-probabilities -- does
 // not depend on where its node sits in the tree.  Expanding layer by layer (expand_fused.cu) makes

@@ -25,7 +25,7 @@ constexpr int EXP_CTAS_PER_SM = 4;
 constexpr int MAX_BUDGET = 128;
 constexpr int MAX_BATCH = 1024;
 constexpr int SEL_THREADS = 512;
-// fused expansion kernel (k <= 32)
+// chunks and lists of the expansion kernels
 constexpr int FX_SURV = 64;                // keys of a row that may pass the merge bound before the slow path
 constexpr int FX_MAX_SPLITS = 32;          // chunks per row, at most (one lane per chunk in the merge)
 constexpr int FX_LONG_SPLITS = 16;         // the same for lists of more than 16 keys (they are merged in shared memory)
@@ -171,9 +171,10 @@ __device__ __forceinline__ void pdl_enter() {
 // Launches `kernel` so that it may be scheduled while its predecessor in the stream drains
 // (the kernel itself waits in pdl_enter()); a plain launch when ctx->pdl is off.  A step is a chain of
 // dependent kernels, most of them short, so the overlap of launch latency pays at every batch size
-// (sampling verification of 8 sequences: 252 -> 242 us).  The exception, chain = false, is the row pass of a
-// whole step: its CTAs, waiting beside the attention of the step before, slow that down (270 -> 278 us at the
-// shape with 64 query heads), so it is launched this way up to PDL_AUTO_BATCH sequences only.
+// (sampling verification of 8 sequences: 252 -> 242 us).  The exceptions, chain = false, are launched this way
+// up to PDL_AUTO_BATCH sequences only: the row pass of a whole step, whose CTAs, waiting beside the attention of the
+// step before, slow that down (270 -> 278 us at the shape with 64 query heads), and an attention that does not start
+// beside the growth of the trees, whose CTAs fill SMs and so would take them from the kernel before.
 constexpr int PDL_AUTO_BATCH = 4;
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel_pdl(const talon_ctx *c, bool chain, void (*kernel)(KArgs...), dim3 grid, dim3 block,
