@@ -848,6 +848,34 @@ __device__ __forceinline__ u64 merge_lists(const u64 *lists, int stride, int S, 
   return r[0];
 }
 
+// The ke <= k best of S <= 32 descending lists of k <= K keys, in lanes 0 .. ke - 1 descending: lane c keeps list c in registers
+// and the largest head is taken off ke times.  A short loop rather than the fewest steps: a warp merges a row or two a
+// layer and finds the instructions cold, so that fetching 5 KB of them, which the merge by pairs above unrolls to, costs what it
+// saves.  Lists of 8, one conversation: a whole step 43.5 -> 42.5 us, twelve layers one by one 127.3 -> 126.5.  With lists of 16 the
+// loop is longer and the pairs remain (static trees of four sequences 228.5 us, 229.5 this way).
+template <int K>
+__device__ __forceinline__ u64 pop_lists(const u64 *lists, int stride, int S, int k, int ke, int lane) {
+  u64 r[K];
+  const ulonglong2 *own = reinterpret_cast<const ulonglong2 *>(lists + (size_t)min(lane, S - 1) * stride);      // (slots k .. stride - 1 hold zero)
+#pragma unroll
+  for (int i = 0; i < K; i += 2) {
+    const ulonglong2 x = lane < S && i < k ? __ldcg(own + i / 2) : make_ulonglong2(0ull, 0ull);
+    r[i] = x.x; r[i + 1] = x.y;
+  }
+  u64 out = 0ull;
+#pragma unroll 1
+  for (int i = 0; i < ke; ++i) {
+    const u64 best = warp_redux_max_u64(r[0]);
+    if (lane == i) out = best;
+    if (r[0] == best) {
+#pragma unroll
+      for (int u = 0; u + 1 < K; ++u) r[u] = r[u + 1];
+      r[K - 1] = 0ull;
+    }
+  }
+  return out;
+}
+
 // One warp merges the S chunk results of a row, st: its stage_words(k) words of shared memory (KMAX 32).
 // Afterwards lane i < k holds the row's i-th best key and the score ps + (z - lse), with ps the
 // log-probability of the row's node (Eq. 2-3; -inf for an empty slot or one past the ke children the
@@ -868,7 +896,8 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
   if (KMAX <= 16) {
     constexpr int K = KMAX <= 16 ? KMAX : 16;
     const u64 *lists = res.part_keys + item0 * ks;
-    own = S <= 16 ? merge_lists<K, 16>(lists, ks, S, k, lane) : merge_lists<K, FX_MAX_SPLITS>(lists, ks, S, k, lane);
+    if constexpr (K == 8) own = pop_lists<8>(lists, ks, S, k, ke, lane);
+    else own = S <= 16 ? merge_lists<K, 16>(lists, ks, S, k, lane) : merge_lists<K, FX_MAX_SPLITS>(lists, ks, S, k, lane);
   } else if (S == 1) {
     const u64 key = lane < k ? __ldcg(res.part_keys + item0 * ks + lane) : 0ull;
     if (lane < k) rk[lane] = key;
