@@ -60,6 +60,7 @@ template <int MT> struct TcShape {
   static constexpr uint32_t TMEM_COLS = 512, COL_S = 128 * MT, COL_P = 128 * MT + 128, COL_REST = COL_P + 64 * MT;
 };
 constexpr float TC_RESCALE_GAP = 8.f;      // the reference maximum is raised beyond 2^8 only, or (exact_max) whenever it grows
+constexpr double TC_LATE_US = 400.0;       // an attention longer than this waits for the trees
 constexpr long long TC_WAIT_CYCLES = 4000000000ll;   // ~2 s: far beyond any legitimate wait
 constexpr int TC_XO_PITCH = TC_D + 4;      // floats per row of the partial result a CTA leaves in shared memory
 constexpr int TC_XO_ROW_BYTES = TC_XO_PITCH * 4;                 // (the rows' (max, sum) pairs follow the rows)
@@ -287,7 +288,10 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
   auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
 
   const int L = __ldcg(a.prefix_len + b);
-  const int nmt = min(a.m_blocks - mpair * MT, MT);                      // query tiles of this CTA with rows
+  // query tiles of this CTA with rows, and with nodes where the tree is known by now: a tile of slots that hold none is
+  // nothing but zeros
+  const int row_tiles = min(a.m_blocks - mpair * MT, MT);
+  const int nmt = a.early ? row_tiles : max(min(row_tiles, (__ldcg(a.n_nodes + b) + a.npt - 1) / a.npt - mpair * MT), 0);
 
   const int nP = (L + TC_BN - 1) / TC_BN;
   const int nT = (a.N + TC_BN - 1) / TC_BN;
@@ -295,7 +299,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
   const int tps = (tt + a.splits - 1) / a.splits;
   const int t_begin = split * tps;
   const int t_end = min(tt, t_begin + tps);
-  const int nt = max(t_end - t_begin, 0);
+  const int nt = nmt > 0 ? max(t_end - t_begin, 0) : 0;
 
   if (tid == 0) {
     s_abort = 0;
@@ -304,7 +308,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       mbar_init(bar(B_KFULL + s), 1);
       mbar_init(bar(B_VFULL + s), 1);
       mbar_init(bar(B_KEMPTY + s), 1);
-      mbar_init(bar(B_VEMPTY + s), nmt);           // (each tile's P.V)
+      mbar_init(bar(B_VEMPTY + s), max(nmt, 1));   // (each tile's P.V)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar(B_SFULL + i), 1);
@@ -660,8 +664,8 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         }
         if (row_valid) a.part_ml[prow] = make_float2(m_used, l_run);
       }
-    } else if (nt == 0 && i < nmt && in_range) {
-      // an empty key range (more splits than tiles): contribute nothing
+    } else if ((nt == 0 || i >= nmt) && i < row_tiles && in_range) {
+      // an empty key range (more splits than tiles) or a tile without nodes: contribute nothing
       if (a.splits == 1) {
         uint4 *op = reinterpret_cast<uint4 *>(a.out + (((int64_t)b * a.N + node) * a.Hq + kvh * a.g + qh) * TC_D);
 #pragma unroll
@@ -896,15 +900,20 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
   }
   TcArgs a;
   a.kv_start = kv_start; a.block_table = block_table; a.bt_stride = bt_stride;
-  a.early = early_prefix != nullptr;
-  a.prefix_len = early_prefix ? early_prefix : c->d_prefix_len; a.n_nodes = t->n_nodes;
+  // A long attention does not start beside the growth of the trees but after it: the growth is some 25 us, and which query
+  // tiles hold no node, a tenth of its work where trees fill three quarters of their slots, is known only then (32
+  // sequences of 32768 tokens, trees of 72 to 128 nodes in 128 slots: a step of 2897 us takes 2834).  The line lies where the
+  // wait is at most a sixteenth of it.
+  const double us = 2.0 * ((max_prefix_len + TC_BN - 1) / TC_BN + 1) * ((m_blocks + 1) / 2) * Hkv * B / c->sm_count;
+  const bool early = early_prefix && !(m_blocks > 1 && us > TC_LATE_US);
+  a.early = early;
+  a.prefix_len = early ? early_prefix : c->d_prefix_len; a.n_nodes = t->n_nodes;
   a.mask = (const unsigned long long *)t->mask;
   a.B = B; a.N = N; a.W = c->W; a.Hq = Hq; a.Hkv = Hkv; a.g = g; a.npt = npt;
   a.scale_log2 = sm_scale * 1.4426950408889634f;
   a.gap = exact_max ? 0.f : TC_RESCALE_GAP;
   a.splits = splits; a.m_blocks = m_blocks;
   a.out = (__nv_bfloat16 *)out; a.part_o = c->d_attn_o; a.part_ml = c->d_attn_ml; a.status = c->d_status;
-  (void)max_prefix_len;
   const TcLaunch l = tc_launch(kind);
   dim3 grid(kind == TC_PAIR ? (m_blocks + 1) / 2 : m_blocks, splits, B * Hkv);
   // Two to eight key ranges: they are launched as one thread-block cluster and merge their partial
@@ -922,11 +931,11 @@ talon_status launch_attention_tc(talon_ctx *c, const talon_tree *t, const void *
       attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
       attr[1].val.programmaticStreamSerializationAllowed = 1;
       cfg.attrs = attr;
-      cfg.numAttrs = (c->pdl == 1 || (c->pdl < 0 && (c->B <= PDL_AUTO_BATCH || early_prefix))) ? 2 : 1;
+      cfg.numAttrs = (c->pdl == 1 || (c->pdl < 0 && (c->B <= PDL_AUTO_BATCH || early))) ? 2 : 1;
       cudaLaunchKernelEx(&cfg, l.kernel, mq, mkp, mvp, mkt, mvt, a);
       *merged_in_kernel = 1;
     } else {
-      launch_kernel_pdl(c, early_prefix != nullptr, l.kernel, grid, dim3(l.threads), l.smem, st, mq, mkp, mvp, mkt, mvt, a);
+      launch_kernel_pdl(c, early, l.kernel, grid, dim3(l.threads), l.smem, st, mq, mkp, mvp, mkt, mvt, a);
     }
   }
   if (cudaGetLastError() != cudaSuccess) return TALON_ERR_CUDA;
