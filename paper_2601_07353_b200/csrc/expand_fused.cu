@@ -21,6 +21,8 @@ namespace {
 
 // Frontiers wider than this merge their rows all over the grid.  Up to two rows per warp the CTA that
 // completes the sequence is quicker: no second hand-off, no row results to publish and collect (2 us).
+// With lists of more than 8, whose merge takes twice as long, one row per warp (nine layers of four static trees, ten rows each, 145.7 ->
+// 144.9 us).
 constexpr int XS_TWO_LEVEL = 2 * EXP_WARPS;
 
 struct FusedArgs {
@@ -378,7 +380,7 @@ expand_fused_kernel(FusedArgs a) {
     // ---- hand-off.  The barrier orders this CTA's writes before thread 0's device-scope
     // release; the last arrival acquires.  Narrow frontiers count chunks per sequence, wide ones
     // chunks per row and then rows per sequence. ----
-    const bool two_level = WIDE || rl.F > XS_TWO_LEVEL;
+    const bool two_level = WIDE || rl.F > (KMAX > 8 ? EXP_WARPS : XS_TWO_LEVEL);
     __syncthreads();
     chunk_clear(sh);
     if (tid == 0) {

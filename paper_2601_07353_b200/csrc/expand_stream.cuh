@@ -766,17 +766,35 @@ __device__ __forceinline__ bool stream_chunk(const ChunkShared &sh, const float 
     }
   }
 
-  // ---- the chunk's ke best keys: four lanes count each candidate's betters (keys are unique) ----
+  // ---- the chunk's ke best keys: a few lanes count each candidate's betters (keys are unique): eight lanes a key, four
+  // comparisons each and no loop, where all of them are one pass (the usual pool of a list of 8; twelve layers of one
+  // conversation 105.6 -> 104.8 us), else four ----
   const int nc = *sh.pool_n;
-  for (int c0 = 0; c0 < nc; c0 += EXP_THREADS / 4) {
-    const int ci = c0 + (tid >> 2), q = tid & 3;
+  static_assert(EXP_THREADS / 8 == 32 && POOL >= 32, "one pass of eight lanes a key");
+  if (nc <= 32) {
+    const int ci = tid >> 3, q = tid & 7;
     const u64 key = ci < nc ? sh.pool[ci] : 0ull;
+    u64 other[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) other[i] = sh.pool[q + 8 * i];           // (past the pool's keys: not counted)
     int r = 0;
-#pragma unroll 4
-    for (int o = q; o < nc; o += 4) r += (sh.pool[o] > key) ? 1 : 0;
-    r += __shfl_xor_sync(FULL, r, 1);
-    r += __shfl_xor_sync(FULL, r, 2);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r += q + 8 * i < nc && other[i] > key ? 1 : 0;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) r += __shfl_xor_sync(FULL, r, o);
     if (q == 0 && ci < nc && r < ke) res.part_keys[item * res.key_stride + r] = key;
+  } else {
+#pragma unroll 1
+    for (int c0 = 0; c0 < nc; c0 += EXP_THREADS / 4) {
+      const int ci = c0 + (tid >> 2), q = tid & 3;
+      const u64 key = ci < nc ? sh.pool[ci] : 0ull;
+      int r = 0;
+#pragma unroll 4
+      for (int o = q; o < nc; o += 4) r += (sh.pool[o] > key) ? 1 : 0;
+      r += __shfl_xor_sync(FULL, r, 1);
+      r += __shfl_xor_sync(FULL, r, 2);
+      if (q == 0 && ci < nc && r < ke) res.part_keys[item * res.key_stride + r] = key;
+    }
   }
   if (tid < k && tid >= min(nc, ke)) res.part_keys[item * res.key_stride + tid] = 0ull;
   if (warp == EXP_WARPS - 1) {
@@ -916,9 +934,8 @@ __device__ __forceinline__ bool merge_row(const ChunkOut &res, size_t item0, int
       }
     }
   }
-  float mx = ms.x;                                                      // lanes >= S hold -inf and 0
-#pragma unroll
-  for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
+  // (lanes >= S hold -inf and 0; one reduction of the ordered bits, not five shuffles: 105.6 -> 104.8 us as above)
+  const float mx = f32_unord(__reduce_max_sync(FULL, f32_ord(ms.x)));
   double t = 0.0;
   if (ms.y != ms.y) t = (double)ms.y;                                   // NaN or +inf logit in the chunk
   else if (ms.x > -CUDART_INF_F) t = (double)ms.y * (double)exp2f((ms.x - mx) * LOG2E_F);
@@ -1031,9 +1048,7 @@ __device__ __forceinline__ void merge_row_wide_n(const ChunkOut &res, size_t ite
   }
   if (warp == EXP_WARPS - 1) {
     const float2 ms = lane < S ? __ldcg(res.part_ms + item0 + lane) : make_float2(-CUDART_INF_F, 0.f);
-    float mx = ms.x;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
+    const float mx = f32_unord(__reduce_max_sync(FULL, f32_ord(ms.x)));
     double t = 0.0;
     if (ms.y != ms.y) t = (double)ms.y;                                 // NaN or +inf logit in the chunk
     else if (ms.x > -CUDART_INF_F) t = (double)ms.y * (double)exp2f((ms.x - mx) * LOG2E_F);
