@@ -20,7 +20,7 @@
 // prepares the remaining rows of the sequences whose trees still grow, or goes layer by layer after all.
 #include <algorithm>
 
-#include "expand_stream.cuh"
+#include "target_rows.cuh"
 
 namespace talon {
 
@@ -101,59 +101,6 @@ __device__ __forceinline__ void locate_active(const RowPassArgs &a, const Active
   }
 }
 
-// Arg-max of elements [start, end) of a target row into best[slot] (lowest index among equal maxima,
-// a NaN never wins but sets bad[slot]): 16 elements per thread and step, the next step's loads issued
-// before the current one is worked on, the index looked for only in a step that raises the maximum.
-__device__ __forceinline__ void argmax_chunk(const float *rowp, int start, int end, u64 *best, unsigned int *bad_flag,
-                                             u64 *s_key) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float bestv = -CUDART_INF_F;
-  uint32_t besti = 0xFFFFFFFFu;
-  bool bad = false;
-  float4 nx[EXP_UNROLL];
-  auto load = [&](int base) {
-#pragma unroll
-    for (int u = 0; u < EXP_UNROLL; ++u) {
-      const int idx = base + u * EXP_CHUNK_ALIGN + tid * EXP_VEC;
-      if (idx + EXP_VEC <= end) nx[u] = __ldcs(reinterpret_cast<const float4 *>(rowp + idx));
-      else {
-        nx[u].x = idx < end ? __ldcs(rowp + idx) : -CUDART_INF_F;
-        nx[u].y = idx + 1 < end ? __ldcs(rowp + idx + 1) : -CUDART_INF_F;
-        nx[u].z = idx + 2 < end ? __ldcs(rowp + idx + 2) : -CUDART_INF_F;
-        nx[u].w = -CUDART_INF_F;
-      }
-    }
-  };
-  load(start);
-  for (int base = start; base < end; base += EXP_TILE) {
-    float v[EXP_UNROLL * EXP_VEC];
-#pragma unroll
-    for (int u = 0; u < EXP_UNROLL; ++u) { v[4 * u] = nx[u].x; v[4 * u + 1] = nx[u].y; v[4 * u + 2] = nx[u].z; v[4 * u + 3] = nx[u].w; }
-    if (base + EXP_TILE < end) load(base + EXP_TILE);
-    float bm = -CUDART_INF_F;
-#pragma unroll
-    for (int e = 0; e < EXP_UNROLL * EXP_VEC; ++e) { bad |= (v[e] != v[e]); bm = fmaxf(bm, v[e]); }
-    if (bm > bestv || besti == 0xFFFFFFFFu) {
-      uint32_t first = 0xFFFFFFFFu;
-#pragma unroll
-      for (int e = EXP_UNROLL * EXP_VEC - 1; e >= 0; --e) {
-        const int idx = base + (e / EXP_VEC) * EXP_CHUNK_ALIGN + tid * EXP_VEC + e % EXP_VEC;
-        if (idx < end && v[e] == bm) first = (uint32_t)idx;
-      }
-      if (first != 0xFFFFFFFFu) { bestv = bm; besti = first; }
-    }
-  }
-  u64 key = warp_max_u64(besti == 0xFFFFFFFFu ? 0ull : cand_key(bestv, besti));
-  if (__any_sync(FULL, bad) && lane == 0) atomicOr(bad_flag, 1u);
-  if (lane == 0) s_key[warp] = key;
-  __syncthreads();
-  if (warp == 0) {
-    key = warp_max_u64(lane < EXP_WARPS ? s_key[lane] : 0ull);
-    if (lane == 0 && key) atomicMax(best, key);
-  }
-  __syncthreads();
-}
-
 template <int KMAX>          // k rounded up to 8, 16 or 32
 __global__ void __launch_bounds__(EXP_THREADS, 3)
 row_pass_kernel(RowPassArgs a) {
@@ -224,7 +171,7 @@ row_pass_kernel(RowPassArgs a) {
     const int64_t lrow = (int64_t)slot - (int64_t)step * a.step_B * a.N;
     if (!is_draft) {
       if (start < end)
-        argmax_chunk(a.target + step * a.target_step + lrow * a.target_stride, start, end, a.best + slot, a.row_bad + slot, s_pool);
+        argmax_chunk(a.target + step * a.target_step + lrow * a.target_stride, start, end, a.best + slot, a.row_bad + slot, 1u, s_pool);
       continue;
     }
     // a node below the root is gated when every layer but the first is; deeper Top-K layers are not told apart here

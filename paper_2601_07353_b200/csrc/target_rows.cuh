@@ -1,0 +1,146 @@
+// The target rows of a batch as the verification streams them (accept.cu): the rows of the nodes that the trees have, laid
+// end to end on one line that is shared out over the CTAs.
+#pragma once
+
+#include "expand_stream.cuh"
+
+namespace talon {
+
+namespace {
+
+// Arg-max of elements [start, end) of a target row into *best (lowest index among equal maxima, a NaN never wins but
+// sets `bit` of *flag): 16 elements per thread and step, the next step's loads issued
+// before the current one is worked on, the index looked for only in a step that raises the maximum.
+__device__ __forceinline__ void argmax_chunk(const float *rowp, int start, int end, u64 *best, unsigned int *flag, unsigned bit,
+                                             u64 *s_key) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float bestv = -CUDART_INF_F;
+  uint32_t besti = 0xFFFFFFFFu;
+  bool bad = false;
+  float4 nx[EXP_UNROLL];
+  auto load = [&](int base) {
+#pragma unroll
+    for (int u = 0; u < EXP_UNROLL; ++u) {
+      const int idx = base + u * EXP_CHUNK_ALIGN + tid * EXP_VEC;
+      if (idx + EXP_VEC <= end) nx[u] = __ldcs(reinterpret_cast<const float4 *>(rowp + idx));
+      else {
+        nx[u].x = idx < end ? __ldcs(rowp + idx) : -CUDART_INF_F;
+        nx[u].y = idx + 1 < end ? __ldcs(rowp + idx + 1) : -CUDART_INF_F;
+        nx[u].z = idx + 2 < end ? __ldcs(rowp + idx + 2) : -CUDART_INF_F;
+        nx[u].w = -CUDART_INF_F;
+      }
+    }
+  };
+  load(start);
+  for (int base = start; base < end; base += EXP_TILE) {
+    float v[EXP_UNROLL * EXP_VEC];
+#pragma unroll
+    for (int u = 0; u < EXP_UNROLL; ++u) { v[4 * u] = nx[u].x; v[4 * u + 1] = nx[u].y; v[4 * u + 2] = nx[u].z; v[4 * u + 3] = nx[u].w; }
+    if (base + EXP_TILE < end) load(base + EXP_TILE);
+    float bm = -CUDART_INF_F;
+#pragma unroll
+    for (int e = 0; e < EXP_UNROLL * EXP_VEC; ++e) { bad |= (v[e] != v[e]); bm = fmaxf(bm, v[e]); }
+    if (bm > bestv || besti == 0xFFFFFFFFu) {
+      uint32_t first = 0xFFFFFFFFu;
+#pragma unroll
+      for (int e = EXP_UNROLL * EXP_VEC - 1; e >= 0; --e) {
+        const int idx = base + (e / EXP_VEC) * EXP_CHUNK_ALIGN + tid * EXP_VEC + e % EXP_VEC;
+        if (idx < end && v[e] == bm) first = (uint32_t)idx;
+      }
+      if (first != 0xFFFFFFFFu) { bestv = bm; besti = first; }
+    }
+  }
+  u64 key = warp_max_u64(besti == 0xFFFFFFFFu ? 0ull : cand_key(bestv, besti));
+  if (__any_sync(FULL, bad) && lane == 0) atomicOr(flag, bit);
+  if (lane == 0) s_key[warp] = key;
+  __syncthreads();
+  if (warp == 0) {
+    key = warp_max_u64(lane < EXP_WARPS ? s_key[lane] : 0ull);
+    if (lane == 0 && key) atomicMax(best, key);
+  }
+  __syncthreads();
+}
+
+// ---- rows of the nodes there are ----
+struct LiveRows {
+  int base_l, n_l;       // B <= 32: first packed row and number of rows of sequence `lane`
+  int total;
+  const int *s_base;     // B > 32: [B + 1]
+  bool in_regs;
+};
+
+// All threads of the CTA (a multiple of 32); s_base: B + 1 ints and s_warp: 32, for B > 32.
+__device__ __forceinline__ LiveRows live_rows(const int32_t *n_nodes, int B, int N, int *s_base, int *s_warp) {
+  LiveRows r;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
+  r.in_regs = B <= 32;
+  r.s_base = s_base;
+  r.base_l = r.n_l = 0;
+  if (r.in_regs) {
+    r.n_l = lane < B ? min(max(n_nodes[lane], 0), N) : 0;
+    int inc = r.n_l;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(FULL, inc, o);
+      if (lane >= o) inc += t;
+    }
+    r.base_l = inc - r.n_l;
+    r.total = __shfl_sync(FULL, inc, 31);
+    return r;
+  }
+  int run = 0;
+  for (int b0 = 0; b0 < B; b0 += blockDim.x) {
+    const int b = b0 + tid;
+    int inc = b < B ? min(max(n_nodes[b], 0), N) : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(FULL, inc, o);
+      if (lane >= o) inc += t;
+    }
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int w = 0; w < warps; ++w) { before += w < warp ? s_warp[w] : 0; all += s_warp[w]; }
+    if (b < B) s_base[b + 1] = run + before + inc;
+    run += all;
+    __syncthreads();
+  }
+  if (tid == 0) s_base[0] = 0;
+  __syncthreads();
+  r.total = run;
+  return r;
+}
+// Sequence of packed row `row`, its number of rows and its first packed row.
+__device__ __forceinline__ void locate_live(const LiveRows &r, int B, int row, int &b, int &n, int &base) {
+  if (r.in_regs) {
+    b = 31 - __clz(__ballot_sync(FULL, (int)(threadIdx.x & 31) < B && r.base_l <= row && r.n_l > 0));
+    n = __shfl_sync(FULL, r.n_l, b);
+    base = __shfl_sync(FULL, r.base_l, b);
+  } else {
+    b = seq_of_row(r.s_base, B, row);
+    base = r.s_base[b];
+    n = r.s_base[b + 1] - base;
+  }
+}
+
+// How the line is cut: rows `pitch` elements apart, CTA c takes elements [c span, (c + 1) span).  With four CTAs or more
+// a row the spans are whole fractions of a row, else equal shares of the line, of a CTA step (4096 elements) at least: a
+// CTA has few pieces either way, and a piece costs a reduction and a trip to L2 at its end.
+struct LineCut { unsigned span, pitch; };
+__device__ __forceinline__ LineCut line_cut(int rows, int vocab, int ctas) {
+  LineCut c;
+  const unsigned vp = ((unsigned)vocab + 3u) & ~3u;
+  if (rows > 0 && 4 * rows <= ctas) {
+    const unsigned S = min((unsigned)ctas / (unsigned)rows, (vp + EXP_TILE - 1u) / EXP_TILE);
+    c.span = ((vp + S - 1u) / S + 3u) & ~3u;
+    c.pitch = S * c.span;
+  } else {
+    c.span = max((div_u64((unsigned long long)rows * vp + ctas - 1, (unsigned)ctas) + 3u) & ~3u, (unsigned)EXP_TILE);
+    c.pitch = vp;
+  }
+  return c;
+}
+
+}  // namespace
+
+}  // namespace talon

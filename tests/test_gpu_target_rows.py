@@ -1,0 +1,51 @@
+"""The target's arg-max over the rows of the nodes there are, and the walk behind it: vocabularies around a chunk and off four,
+few rows (whole fractions of a row per CTA) and many (equal shares of all rows), batches around a warp's lanes, sequences
+without a node, NaN in rows of nodes and of empty slots."""
+import pytest
+import torch
+
+from tests.test_gpu_step_paths import _rows, _talon
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("V", [7, 4095, 4097, 50001])
+@pytest.mark.parametrize("B,N", [(1, 2), (1, 37), (4, 37), (3, 128), (32, 24), (33, 24)])
+def test_argmax_and_walk(V, B, N):
+    talon, t = _talon(B, V, N, 4, 8)
+    gen = torch.Generator(device="cuda").manual_seed(V + B)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    target = _rows(gen, B, N, V)
+    tree = t.alloc_tree(B)
+    t.reset(tree, torch.zeros(B, **i32), torch.zeros(B, **i32))
+    alen, nodes, bonus, tok = torch.zeros(B, **i32), torch.zeros(B, 9, **i32), torch.zeros(B, **i32), torch.zeros(B, N, **i32)
+    for fill in (1, N // 2 + 1, N):
+        n = [max(fill - b % 3, 0) for b in range(B)]             # some without a node at the first
+        best = torch.stack([target[b].argmax(-1) for b in range(B)]).to(torch.int32)
+        # a chain that follows the target for two nodes, then departs
+        tree.n_nodes.copy_(torch.tensor(n, **i32))
+        tree.parent.copy_(torch.arange(-1, N - 1, **i32).expand(B, N))
+        tree.token[:, 0] = 0
+        tree.token[:, 1:] = best[:, :-1]
+        if N > 3:
+            tree.token[:, 3] = (best[:, 2] + 1) % V
+        for x in (alen, nodes, bonus, tok):
+            x.fill_(-7)
+        t.accept(tree, target, alen, nodes, bonus, tok)
+        torch.cuda.synchronize()
+        assert t.poll_status() == talon.OK
+        for b in range(B):
+            assert torch.equal(tok[b, :n[b]], best[b, :n[b]]) and (tok[b, n[b]:] == -1).all()
+            length = max(min(n[b] - 1, 2), 0)
+            assert int(alen[b]) == length and nodes[b, :length + 1].tolist() == list(range(length + 1))
+            assert int(bonus[b]) == (int(best[b, length]) if n[b] else -1)
+    if B > 1:
+        n = int(tree.n_nodes[1])
+        if n < N:
+            target[1, n:, V // 2] = float("nan")                 # no node there
+            t.accept(tree, target, alen, nodes, bonus, tok)
+            assert t.poll_status() == talon.OK
+        target[1, n - 1, V - 1] = float("nan")
+        t.accept(tree, target, alen, nodes, bonus, tok)
+        assert t.poll_status() == talon.ERR_NONFINITE
+    t.close()
