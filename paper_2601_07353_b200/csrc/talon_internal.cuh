@@ -132,7 +132,7 @@ struct talon_ctx {
   int attn_clusters[3][9];           // per kind of the tensor-core attention and cluster size: clusters the device holds at once (-1 not asked yet)
   int attn_force_splits;             // > 0: key ranges per (sequence, head, query tiles), for experiments
   int attn_force_tiles;              // 1, 2: query tiles of a CTA, for experiments (1 also where two cannot be had)
-  int argmax_oversplit;              // target argmax: chunk rounds per CTA when the rows outnumber the grid
+  int argmax_oversplit;              // softmax statistics of target rows: chunk rounds per CTA when the rows outnumber the grid
   int expand_max_split;              // fused kernel: chunks a row is cut into at most when the grid has room
   int attn_min_tiles;                // split-KV: key tiles a CTA should at least own
   int pdl;                           // programmatic stream serialization: 1 on, 0 off, -1 on for small batches
