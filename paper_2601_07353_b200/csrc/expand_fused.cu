@@ -4,8 +4,8 @@
 // Streaming phase: expand_stream.cuh.  The frontier's fp32 logit rows are cut into equal chunks, one
 // CTA per chunk at a time; a chunk leaves its k best keys and its share of the normaliser.
 //
-// Selection phase.  Frontiers of at most sixteen rows: the CTA that finishes a sequence's last chunk
-// merges that sequence's rows, one warp per row.  Wider frontiers: the CTA that finishes a row's
+// Selection phase.  Frontiers of at most sixteen rows (eight where lists are longer than 8): the CTA that
+// finishes a sequence's last chunk merges that sequence's rows, one warp per row.  Wider frontiers: the CTA that finishes a row's
 // last chunk merges that row (rows of one sequence finish all over the grid, so the merges run in
 // parallel), and the CTA that finishes the sequence's last row collects the row results.  Either
 // way that CTA then scores the pooled candidates with log p(u) = log p(v) + log P(w | v)
