@@ -4,8 +4,8 @@
 // Streaming phase: expand_stream.cuh.  The frontier's fp32 logit rows are cut into equal chunks, one
 // CTA per chunk at a time; a chunk leaves its k best keys and its share of the normaliser.
 //
-// Selection phase.  Frontiers of at most sixteen rows (eight where lists are longer than 8): the CTA that
-// finishes a sequence's last chunk merges that sequence's rows, one warp per row.  Wider frontiers: the CTA that finishes a row's
+// Selection phase.  Frontiers of at most sixteen rows: the CTA that finishes a sequence's last chunk
+// merges that sequence's rows, one warp per row.  Wider frontiers: the CTA that finishes a row's
 // last chunk merges that row (rows of one sequence finish all over the grid, so the merges run in
 // parallel), and the CTA that finishes the sequence's last row collects the row results.  Either
 // way that CTA then scores the pooled candidates with log p(u) = log p(v) + log P(w | v)
@@ -21,8 +21,8 @@ namespace {
 
 // Frontiers wider than this merge their rows all over the grid.  Up to two rows per warp the CTA that
 // completes the sequence is quicker: no second hand-off, no row results to publish and collect (2 us).
-// With lists of more than 8, whose merge takes twice as long, one row per warp (nine layers of four static trees, ten rows each, 145.7 ->
-// 144.9 us).
+// (Lists of more than 8, whose merge takes twice as long, gain a little from one row per warp where rows are long: nine layers of four
+// static trees, ten rows of 128256 each, 145.7 -> 144.9 us; one tree of five layers of nine rows of 31152 loses: 90.3 -> 92.9.)
 constexpr int XS_TWO_LEVEL = 2 * EXP_WARPS;
 
 struct FusedArgs {
@@ -380,7 +380,7 @@ expand_fused_kernel(FusedArgs a) {
     // ---- hand-off.  The barrier orders this CTA's writes before thread 0's device-scope
     // release; the last arrival acquires.  Narrow frontiers count chunks per sequence, wide ones
     // chunks per row and then rows per sequence. ----
-    const bool two_level = WIDE || rl.F > (KMAX > 8 ? EXP_WARPS : XS_TWO_LEVEL);
+    const bool two_level = WIDE || rl.F > XS_TWO_LEVEL;
     __syncthreads();
     chunk_clear(sh);
     if (tid == 0) {
