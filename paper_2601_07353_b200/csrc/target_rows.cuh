@@ -123,20 +123,24 @@ __device__ __forceinline__ void locate_live(const LiveRows &r, int B, int row, i
   }
 }
 
-// How the line is cut: rows `pitch` elements apart, CTA c takes elements [c span, (c + 1) span).  With four CTAs or more
-// a row the spans are whole fractions of a row, else equal shares of the line, of a CTA step (4096 elements) at least: a
-// CTA has few pieces either way, and a piece costs a reduction and a trip to L2 at its end.
+// How the line is cut: rows `pitch` elements apart, CTA c takes elements [c span, (c + 1) span).  Whole fractions of a row, one
+// piece a CTA, where their span is at most two CTA steps (4096 elements each) longer than an equal share of the
+// line: the second piece that a share has costs its reduction and its trips to L2, about what a CTA reads of 8000 elements
+// (18 trees of 22 slots, rows of 14892: 197.6 -> 195.9 us a step against fractions only from four CTAs a row on; four
+// sequences of 50001: 145.05 -> 144.6).  Else equal shares, of a CTA step at least.
 struct LineCut { unsigned span, pitch; };
 __device__ __forceinline__ LineCut line_cut(int rows, int vocab, int ctas) {
   LineCut c;
   const unsigned vp = ((unsigned)vocab + 3u) & ~3u;
-  if (rows > 0 && 4 * rows <= ctas) {
+  c.pitch = vp;
+  c.span = max((div_u64((unsigned long long)rows * vp + ctas - 1, (unsigned)ctas) + 3u) & ~3u, (unsigned)EXP_TILE);
+  if (rows > 0 && rows <= ctas) {
     const unsigned S = min((unsigned)ctas / (unsigned)rows, (vp + EXP_TILE - 1u) / EXP_TILE);
-    c.span = ((vp + S - 1u) / S + 3u) & ~3u;
-    c.pitch = S * c.span;
-  } else {
-    c.span = max((div_u64((unsigned long long)rows * vp + ctas - 1, (unsigned)ctas) + 3u) & ~3u, (unsigned)EXP_TILE);
-    c.pitch = vp;
+    const unsigned part = ((vp + S - 1u) / S + 3u) & ~3u;
+    if (part <= c.span + 2u * EXP_TILE) {
+      c.span = part;
+      c.pitch = S * part;
+    }
   }
   return c;
 }
